@@ -100,11 +100,11 @@ typedef enum { IFEM_FP32 = 0, IFEM_FP64 = 1 } ifem_precision;
 typedef enum { IFEM_KERNEL_PESKIN4 = 0, IFEM_KERNEL_MLS27 = 1 } ifem_kernel;
 
 /* Summation order of the FP32 scatters (IFEM_FP64 is always deterministic).
- * DET: forces are a fixed-order sum per node over its incident elements;
- * spreading sums each lattice value from the node lists of its own tile
+ * Forces are a fixed-order sum per node over its incident elements in both.
+ * DET: spreading sums each lattice value from the node lists of its own tile
  * (every node binned into each tile its stencil reaches), so repeated runs
  * give identical results.
- * ATOMIC: forces by atomic adds. With PESKIN4, spreading visits each node
+ * ATOMIC: with PESKIN4, spreading visits each node
  * once, in the tile holding its cell, accumulates into the tile plus a
  * 2-cell halo (4 in x) and adds that to the grid with atomic L2 adds, so the
  * order in which neighbouring tiles' halos combine is not reproducible. */

@@ -304,7 +304,119 @@ static void incidence(int nn, int ne, int nv, const int32_t *el, std::vector<int
             idx[cur[el[nv * e + v]]++] = e * 4 + v;
 }
 
-static int tmpl_upload(ifem_ctx ctx, ifem_tmpl t, int nv, const int32_t *el, const std::vector<double> &ref)
+// Order of a node's incident triangles as fans: from a triangle whose first
+// neighbour j no other triangle ends on (an open ring), else from the first
+// one, each triangle followed by the one whose j is its l. pairs: (j, l) per
+// incidence; the permutation is written to order.
+static void fan_order(const std::vector<int2> &pairs, std::vector<int> &order)
+{
+    const int n = (int)pairs.size();
+    std::vector<char> used(n, 0);
+    order.clear();
+    while ((int)order.size() < n) {
+        int start = -1;
+        for (int i = 0; i < n; ++i) {
+            if (used[i])
+                continue;
+            bool follows = false;
+            for (int k = 0; k < n; ++k)
+                follows = follows || (!used[k] && k != i && pairs[k].y == pairs[i].x);
+            if (start < 0 || !follows)
+                start = i;
+            if (!follows)
+                break;
+        }
+        for (int cur = start; cur >= 0;) {
+            used[cur] = 1;
+            order.push_back(cur);
+            int next = -1;
+            for (int k = 0; k < n && next < 0; ++k)
+                if (!used[k] && pairs[k].x == pairs[cur].y)
+                    next = k;
+            cur = next;
+        }
+    }
+}
+
+// The FP32 nodal force kernel's incidences (see TmplDev): reference values in
+// FP64 from X, rounded once. el: the mesh; off, idx: node -> element incidence.
+static int nodal_upload(ifem_ctx ctx, ifem_tmpl t, int nv, const int32_t *el, const double *X,
+                        const std::vector<double> &ref, const std::vector<int> &off, const std::vector<int> &idx)
+{
+    const int nn = t->n_nodes, slices = (nn + 31) / 32;
+    if (nn > kNodalMaxNodes)
+        return IFEM_OK;
+    std::vector<int> base(slices + 1, 0);
+    for (int s = 0; s < slices; ++s) {
+        int width = 0;
+        for (int k = 32 * s; k < std::min(nn, 32 * s + 32); ++k)
+            width = std::max(width, off[k + 1] - off[k]);
+        base[s + 1] = base[s] + 32 * width;
+    }
+    const int per = nv == 3 ? 2 : 4;
+    std::vector<float4> r(base[slices], make_float4(0.f, 0.f, 0.f, 0.f));
+    std::vector<unsigned short> id((size_t)base[slices] * per, 0);
+    std::vector<int2> pairs;
+    std::vector<int> order;
+    auto sub = [&](int i, int j, double d[3]) {
+        for (int a = 0; a < 3; ++a)
+            d[a] = X[3 * (size_t)i + a] - X[3 * (size_t)j + a];
+    };
+    auto dot = [](const double *p, const double *q) { return p[0] * q[0] + p[1] * q[1] + p[2] * q[2]; };
+    for (int k = 0; k < nn; ++k) {
+        const int deg = off[k + 1] - off[k];
+        if (nv == 3) {
+            pairs.resize(deg);
+            for (int q = 0; q < deg; ++q) {
+                const int e = idx[off[k] + q] >> 2, c = idx[off[k] + q] & 3;
+                pairs[q] = make_int2(el[3 * (size_t)e + (c + 1) % 3], el[3 * (size_t)e + (c + 2) % 3]);
+            }
+            fan_order(pairs, order);
+        }
+        for (int s = 0; s < deg; ++s) {
+            const int code = idx[off[k] + (nv == 3 ? order[s] : s)];
+            const int e = code >> 2, c = code & 3;
+            const size_t at = (size_t)base[k / 32] + 32 * s + k % 32;
+            if (nv == 3) {
+                const int j = pairs[order[s]].x, l = pairs[order[s]].y;
+                double e1[3], e2[3], e3[3];
+                sub(j, k, e1);
+                sub(l, k, e2);
+                sub(l, j, e3);
+                id[2 * at] = (unsigned short)j;
+                id[2 * at + 1] = (unsigned short)l;
+                r[at] = make_float4((float)dot(e1, e2), (float)-dot(e1, e3), (float)dot(e2, e3),
+                                    (float)(0.5 / ref[5 * (size_t)e + 4]));
+            } else {
+                // even permutations that bring corner c to the front
+                static const int rot[4][4] = {{0, 1, 2, 3}, {1, 0, 3, 2}, {2, 0, 1, 3}, {3, 0, 2, 1}};
+                const double *g = ref.data() + 10 * (size_t)e;   // grad N_1..3, V0
+                double gr[4][3], sum[3];
+                for (int a = 0; a < 3; ++a) {
+                    for (int v = 1; v < 4; ++v)
+                        gr[v][a] = g[3 * (v - 1) + a];
+                    gr[0][a] = -((gr[1][a] + gr[2][a]) + gr[3][a]);
+                }
+                double h[3];
+                for (int a = 0; a < 3; ++a)
+                    sum[a] = -gr[c][a];   // the other three corners' sum
+                for (int v = 1; v < 4; ++v) {
+                    id[4 * at + v - 1] = (unsigned short)el[4 * (size_t)e + rot[c][v]];
+                    h[v - 1] = g[9] * dot(gr[rot[c][v]], sum);
+                }
+                id[4 * at + 3] = c == 0;
+                r[at] = make_float4((float)h[0], (float)h[1], (float)h[2], (float)(1.0 / (6.0 * g[9])));
+            }
+        }
+    }
+    CK(upload(&t->d_nod_off, base.data(), base.size()));
+    CK(upload(&t->d_nod_ref, r.data(), r.size()));
+    CK(upload(&t->d_nod_idx, id.data(), id.size()));
+    return IFEM_OK;
+}
+
+static int tmpl_upload(ifem_ctx ctx, ifem_tmpl t, int nv, const int32_t *el, const double *X,
+                       const std::vector<double> &ref)
 {
     std::vector<float> reff(ref.begin(), ref.end());
     std::vector<int> off, idx;
@@ -324,6 +436,8 @@ static int tmpl_upload(ifem_ctx ctx, ifem_tmpl t, int nv, const int32_t *el, con
         }
         CK(upload(&t->d_ring, ring.data(), ring.size()));
     }
+    if (ctx->cfg.precision == IFEM_FP32)
+        return nodal_upload(ctx, t, nv, el, X, ref, off, idx);
     return IFEM_OK;
 }
 
@@ -381,7 +495,7 @@ extern "C" int ifem_tmpl_create_membrane(ifem_ctx ctx, int n_nodes, int n_tris, 
     t->c0 = p->c0;
     t->lam = 0.0;
     CK(cudaSetDevice(ctx->cfg.device));
-    int rc = tmpl_upload(ctx, t, 3, tris, ref);
+    int rc = tmpl_upload(ctx, t, 3, tris, X_ref, ref);
     if (rc != IFEM_OK) {
         ifem_tmpl_destroy(t);
         return rc;
@@ -414,7 +528,7 @@ extern "C" int ifem_tmpl_create_solid(ifem_ctx ctx, int n_nodes, int n_tets, con
     t->c0 = 0.0;
     t->lam = p->lambda;
     CK(cudaSetDevice(ctx->cfg.device));
-    int rc = tmpl_upload(ctx, t, 4, tets, ref);
+    int rc = tmpl_upload(ctx, t, 4, tets, X_ref, ref);
     if (rc != IFEM_OK) {
         ifem_tmpl_destroy(t);
         return rc;
@@ -434,6 +548,9 @@ extern "C" int ifem_tmpl_destroy(ifem_tmpl t)
     cudaFree(t->d_inc_off);
     cudaFree(t->d_inc_idx);
     cudaFree(t->d_ring);
+    cudaFree(t->d_nod_off);
+    cudaFree(t->d_nod_ref);
+    cudaFree(t->d_nod_idx);
     delete t;
     return IFEM_OK;
 }
@@ -544,7 +661,7 @@ extern "C" int ifem_batch_create(ifem_ctx ctx, int n_tmpl, const ifem_tmpl *tmpl
     }
     b->N = N;
     b->n_elems = E;
-    b->fused_ok = fused_smem_bytes(b->max_nodes) <= (size_t)kFusedMaxSmemBytes;
+    b->nodal_ok = b->max_nodes <= kNodalMaxNodes;
     split_origins(b, grid);
     std::vector<TmplDev> td(n_tmpl);
     for (int t = 0; t < n_tmpl; ++t) {
@@ -560,17 +677,37 @@ extern "C" int ifem_batch_create(ifem_ctx ctx, int n_tmpl, const ifem_tmpl *tmpl
         d.inc_off = s->d_inc_off;
         d.inc_idx = s->d_inc_idx;
         d.ring = s->d_ring;
+        d.nod_off = s->d_nod_off;
+        d.nod_ref = s->d_nod_ref;
+        d.nod_idx = s->d_nod_idx;
         d.mu = s->mu;
         d.C = s->C;
         d.kb = s->kb;
         d.c0 = s->c0;
         d.lam = s->lam;
+        d.mu_f = (float)s->mu;
+        d.half_muD_f = 0.5f * ((float)s->C * d.mu_f);
+        d.kb_f = (float)s->kb;
+        d.kH0_f = -0.5f * (float)s->c0;
+        d.half_lam_f = 0.5f * (float)s->lam;
     }
+    // element corners, twice where the bending passes visit them again; with
+    // the largest particles last the force kernel ended on them (64 boxes of
+    // mixed particles: step 628 us, largest first 603)
+    auto force_work = [&](int i) {
+        const ifem_tmpl t = tmpls[inst[i].tmpl];
+        return (long long)t->n_elems * (t->kind ? 4 : (t->kb != 0.0 ? 6 : 3));
+    };
+    std::vector<int> order(n_inst);
+    for (int i = 0; i < n_inst; ++i)
+        order[i] = i;
+    std::stable_sort(order.begin(), order.end(), [&](int i, int j) { return force_work(i) > force_work(j); });
     cudaSetDevice(ctx->cfg.device);
     size_t rs = real_size(ctx);
     if (upload(&b->d_tmpl, td.data(), td.size()) != cudaSuccess ||
         upload(&b->d_inst, b->h_inst.data(), b->h_inst.size()) != cudaSuccess ||
         upload(&b->d_node_inst, node_inst.data(), node_inst.size()) != cudaSuccess ||
+        upload(&b->d_inst_order, order.data(), order.size()) != cudaSuccess ||
         cudaMalloc(&b->d_elem_buf, std::max<size_t>(1, (size_t)E * 12 * rs)) != cudaSuccess ||
         cudaMalloc(&b->d_bend_buf, std::max<size_t>(1, (size_t)N * 6 * rs)) != cudaSuccess) {
         ifem_batch_destroy(b);
@@ -598,6 +735,7 @@ extern "C" int ifem_batch_destroy(ifem_batch b)
     cudaFree(b->d_inst);
     cudaFree(b->d_tmpl);
     cudaFree(b->d_node_inst);
+    cudaFree(b->d_inst_order);
     cudaFree(b->d_elem_buf);
     cudaFree(b->d_bend_buf);
     delete b;
@@ -783,7 +921,7 @@ static int do_forces(ifem_ctx ctx, ifem_batch b, const void *x, void *F, const v
     a.x = x;
     a.F = F;
     a.wv = wv;
-    a.scatter = ctx->cfg.scatter;
+    a.n_sm = ctx->n_sm;
     a.hvp = hvp;
     a.stream = (cudaStream_t)stream;
     cudaError_t e = ctx->cfg.precision == IFEM_FP64 ? launch_forces_f64(a) : launch_forces_f32(a);
@@ -1097,13 +1235,12 @@ struct HostIO {
     size_t red_n;   // doubles of red
 };
 
-// The FP32 one-CTA-per-particle force kernel takes a particle range, so the
-// forces of the particles whose positions have arrived can start while the
-// rest are still being copied in.
+// The FP32 nodal force kernel takes a particle range, so the forces of the
+// particles whose positions have arrived can start while the rest are still
+// being copied in.
 static bool forces_ranged_ok(ifem_ctx ctx, ifem_batch b)
 {
-    return ctx->cfg.precision == IFEM_FP32 && ctx->cfg.scatter == IFEM_SCATTER_ATOMIC && b->fused_ok &&
-           b->inst.size() >= 2;
+    return ctx->cfg.precision == IFEM_FP32 && b->nodal_ok && b->inst.size() >= 2;
 }
 
 // Copy node rows [n0, n1) of the 3 x N host array into the device array.

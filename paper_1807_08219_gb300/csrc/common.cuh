@@ -22,10 +22,11 @@ constexpr int kScanThreads = 512;  // tile-count scan: threads per block
 constexpr int kScanPer = 4;        // and values per thread
 constexpr int kScanBlock = kScanThreads * kScanPer;
 constexpr int kCounters = 16;      // DevWork::counters entries
-// FP32 fused force kernel: 7 floats of shared memory per template node
 constexpr int kMaxCtaSmemBytes = 227 * 1024;   // opt-in dynamic shared memory of one CTA
-constexpr int kFusedMaxSmemBytes = kMaxCtaSmemBytes;
-__host__ __device__ inline size_t fused_smem_bytes(int n_nodes) { return (size_t)7 * n_nodes * sizeof(float); }
+// FP32 nodal force kernel: a float4 (position, mean curvature) of shared
+// memory per template node, 16-bit node ids
+constexpr int kNodalMaxNodes = kMaxCtaSmemBytes / 16;
+__host__ __device__ inline size_t nodal_smem_bytes(int n_nodes) { return (size_t)n_nodes * sizeof(float4); }
 constexpr int kStatusWords = 8;
 enum StatusWord {
     ST_INVERTED = 0,
@@ -49,7 +50,13 @@ struct TmplDev {
     const int *inc_idx;    // element*4 + local vertex, ascending element id
     const int2 *ring;      // membranes: per incidence, the other two vertices (j, k) of the
                            // triangle in its orientation order starting at the vertex
+    // FP32 nodal force kernel (templates of at most kNodalMaxNodes nodes, else null): incidences in
+    // slices of 32 nodes, slot s of node k at nod_off[k / 32] + 32 s + k % 32
+    const int *nod_off;
+    const float4 *nod_ref;   // membranes: reference edge dots r_k, r_j, r_l and 1/(2 A0); solids: h1, h2, h3, 1/(6 V0)
+    const void *nod_idx;     // membranes: ushort2 (j, l); solids: ushort4 (1, 2, 3, 1 at the tet's first corner)
     double mu, C, kb, c0, lam;
+    float mu_f, half_muD_f, kb_f, kH0_f, half_lam_f;   // FP32 nodal kernel: mu, C mu/2, kb, -c0/2, lam/2
 };
 
 struct InstDev {
@@ -87,10 +94,11 @@ struct DevBatch {
     int max_elems;
     long long n_elems_total;
     int any_bending;       // some membrane template has kb != 0
-    int fused_ok;          // every template fits the FP32 fused shared-memory kernel
+    int nodal_ok;          // every template fits the FP32 nodal force kernel
     const InstDev *inst;
     const TmplDev *tmpl;
     const int *node_inst;
+    const int *inst_order; // instances by decreasing force work (the force kernel's CTAs: small ones fill the tail)
 };
 
 struct DevGrid {
@@ -334,10 +342,10 @@ struct ForcesArgs {
     const void *x;
     void *F;
     const void *wv;   // HVP direction (or null)
-    int scatter;      // 0 det, 1 atomic
+    int n_sm;
     int hvp;          // 1: compute Hw instead of F
     int inst0, inst_n;  // particle range [inst0, inst0 + inst_n) (inst_n = 0: all); the FP32
-                        // one-CTA-per-particle kernel only (forces_ranged_ok)
+                        // nodal kernel only (forces_ranged_ok)
     cudaStream_t stream;
 };
 

@@ -759,211 +759,355 @@ __global__ void bend_pass2_kernel(DevBatch b, const real *__restrict__ x, const 
     }
 }
 
-// ------------------------------------------------------- FP32 bending helpers
-// The same discrete operators as bend_vertex_pass1/2 (Meyer et al. 2003),
-// arranged for FP32 throughput. Per incident triangle (k, j, l) with
-// e1 = x_j - x_k, e2 = x_l - x_k: 2A = |e1 x e2| from one rsqrt, the corner
-// dots d_k = e1.e2, d_j = |e1|^2 - d_k, d_l = |e2|^2 - d_k, cotangents d/2A.
-// The corner-angle sum enters only through 2 pi - sum(theta); it is taken as
-// -arg(prod_t (cos theta_t + i sin theta_t)), one atan2 per vertex, which
-// equals the deficit while it lies in (-pi, pi) (any vertex of a closed mesh
-// that is not folded onto itself).
+// ------------------------------------------------------------ FP32 nodal path
+// Thread per node: the node's force is gathered over its incident elements in
+// a fixed order, so there are no atomics, no element buffer and no second
+// pass over the elements, and the result is the same from run to run. Each
+// element is evaluated once per corner (3 or 4 times), in forms that need only
+// the corner's own row:
+//
+// Membranes, triangle (k, j, l) at node k, e1 = x_j - x_k, e2 = x_l - x_k: the
+// laws depend on the metric G = [e_a . e_b] alone. With R the metric of the
+// reference triangle, m = Dm^-1 and m m^T = R^-1, det m^2 = 1/det R:
+//   I1 = tr(G R^-1), I2 = det G / det R,
+//   F_k = A0 [e1 e2] (a R^-1 + b adj(G)/det R) (1, 1)^T
+//       = (w/2) [e1 (a r_l + b d_l) + e2 (a r_j + b d_j)],   w = 1/(2 A0),
+// d_k = e1.e2, d_j = |e1|^2 - d_k, d_l = |e2|^2 - d_k the edge dots at the
+// three corners, r_* the same of the reference triangle, and S^ = a I + b adj C^:
+//   NH a = mu, b = -mu/I2^2;  Skalak a = mu (I1 - 1), b = (C mu/2)(I2 - 1) - mu;
+//   I1 = w^2 (|e1|^2 r_l + |e2|^2 r_j + (d_j + d_l) r_k), I2 = w^2 |e1 x e2|^2.
+// These are the dots and the cross product that the bending operators take.
+//
+// Solids, tet (0, 1, 2, 3) rotated (an even permutation) so that the node is
+// corner 0, d_c = x_c - x_0: with P = mu F + beta cof F, beta = (lam/2 (J^2 - 1)
+// - mu)/J, and sum_c cof(F) grad N_c = (d2 x d3 + d3 x d1 + d1 x d2)/(6 V0) =: n/(6 V0),
+//   F_0 = mu (h1 d1 + h2 d2 + h3 d3) + (beta/6) n,  h_c = V0 grad N_c . sum grad N,
+//   J = d1 . (d2 x d3)/(6 V0).
+//
+// Layout: incidences in slices of 32 nodes (a warp), slot by slot, so that a
+// warp's reads are consecutive: reference values (float4: r_k, r_j, r_l, w or
+// h1, h2, h3, 1/(6 V0)) and the other corners as 16-bit node ids. A closed
+// surface's incidences are ordered as a fan around the node (l of one triangle
+// is j of the next), so a triangle takes one new position and edge instead of
+// two.
+//
+// Bending (Meyer et al. 2003) per incident triangle: 2A = |e1 x e2| from one
+// rsqrt, cotangents d/2A. The corner-angle sum enters only through 2 pi -
+// sum(theta); it is taken as -arg(prod_t (cos theta_t + i sin theta_t)), one
+// atan2 per node, which equals the deficit while it lies in (-pi, pi) (any
+// vertex of a closed mesh that is not folded onto itself).
 struct RingF {
-    float e1[3], e2[3], fn[3], inv2A, dk, dj, dl, l1, l2;
+    float fn[3], q, inv2A, dk, dj, dl;   // q = |e1 x e2|^2
 };
-__device__ __forceinline__ void ring_tri_f32(const float xk[3], const float xj[3], const float xl[3], RingF &t)
+__device__ __forceinline__ void ring_edge_f32(const float4 xk, const float4 xj, float e[3], float &l)
 {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        t.e1[a] = xj[a] - xk[a];
-        t.e2[a] = xl[a] - xk[a];
-    }
-    t.fn[0] = t.e1[1] * t.e2[2] - t.e1[2] * t.e2[1];
-    t.fn[1] = t.e1[2] * t.e2[0] - t.e1[0] * t.e2[2];
-    t.fn[2] = t.e1[0] * t.e2[1] - t.e1[1] * t.e2[0];
-    t.inv2A = rsqrtf(t.fn[0] * t.fn[0] + t.fn[1] * t.fn[1] + t.fn[2] * t.fn[2]);
-    t.l1 = t.e1[0] * t.e1[0] + t.e1[1] * t.e1[1] + t.e1[2] * t.e1[2];
-    t.l2 = t.e2[0] * t.e2[0] + t.e2[1] * t.e2[1] + t.e2[2] * t.e2[2];
-    t.dk = t.e1[0] * t.e2[0] + t.e1[1] * t.e2[1] + t.e1[2] * t.e2[2];
-    t.dj = t.l1 - t.dk;
-    t.dl = t.l2 - t.dk;
+    e[0] = xj.x - xk.x;
+    e[1] = xj.y - xk.y;
+    e[2] = xj.z - xk.z;
+    l = e[0] * e[0] + e[1] * e[1] + e[2] * e[2];
+}
+__device__ __forceinline__ void ring_tri_f32(const float e1[3], float l1, const float e2[3], float l2, RingF &t)
+{
+    t.fn[0] = e1[1] * e2[2] - e1[2] * e2[1];
+    t.fn[1] = e1[2] * e2[0] - e1[0] * e2[2];
+    t.fn[2] = e1[0] * e2[1] - e1[1] * e2[0];
+    t.q = t.fn[0] * t.fn[0] + t.fn[1] * t.fn[1] + t.fn[2] * t.fn[2];
+    t.inv2A = rsqrtf(t.q);
+    t.dk = e1[0] * e2[0] + e1[1] * e2[1] + e1[2] * e2[2];
+    t.dj = l1 - t.dk;
+    t.dl = l2 - t.dk;
 }
 
-// Pass 1 at vertex k (positions in shared memory, SoA with stride nn):
-// mixed area A, kH = (K.n)/2 with K the cotangent mean-curvature vector over
-// 2A, kG = deficit / A, unit normal n (area-weighted face normals).
-__device__ __forceinline__ void bend1_f32(const TmplDev &T, int k, const float *xs, int nn, float &A_out,
-                                          float &kH_out, float &kG_out, float n_out[3])
+// Pass 1 of a membrane node: elastic force and, with BEND, the part of the
+// bending force that needs no neighbour's curvature, 2 kb * 2 (kH - kH0)
+// (kH^2 - kG + kH0 kH) A n; kH receives the mean curvature. Along a fan the
+// second edge of a triangle is the first of the next: its vector and length
+// are kept, and the two triangles' coefficients are added before they
+// multiply it.
+template <bool BEND>
+__device__ __forceinline__ void nodal_membrane(const TmplDev &T, int k, const float4 *xs, float F[3], float &kH)
 {
-    float K[3] = {0.f, 0.f, 0.f}, nrm[3] = {0.f, 0.f, 0.f}, A = 0.f, zr = 1.f, zi = 0.f;
-    const float xk[3] = {xs[k], xs[nn + k], xs[2 * nn + k]};
-    for (int q = T.inc_off[k]; q < T.inc_off[k + 1]; ++q) {
-        const int2 jl = T.ring[q];
-        const float xj[3] = {xs[jl.x], xs[nn + jl.x], xs[2 * nn + jl.x]};
-        const float xl[3] = {xs[jl.y], xs[nn + jl.y], xs[2 * nn + jl.y]};
-        RingF t;
-        ring_tri_f32(xk, xj, xl, t);
-        const float cj = t.dj * t.inv2A, cl = t.dl * t.inv2A;
-        // K += cot_l (x_k - x_j) + cot_j (x_k - x_l)
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            K[a] -= cl * t.e1[a] + cj * t.e2[a];
-        const float twoA = (t.fn[0] * t.fn[0] + t.fn[1] * t.fn[1] + t.fn[2] * t.fn[2]) * t.inv2A;
-        float Ai;
-        if (t.dk >= 0.f && t.dj >= 0.f && t.dl >= 0.f)
-            Ai = (cl * t.l1 + cj * t.l2) * 0.125f;
-        else
-            Ai = t.dk < 0.f ? twoA * 0.25f : twoA * 0.125f;
-        A += Ai;
-        // unit (cos, sin) of the corner angle at k, |e1||e2| = sqrt(l1 l2)
-        const float r = rsqrtf(t.l1 * t.l2);
-        const float cr = t.dk * r, ci = twoA * r;
-        const float nr = zr * cr - zi * ci;
-        zi = zr * ci + zi * cr;
-        zr = nr;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            nrm[a] += t.fn[a];
+    const float mu = T.mu_f, half_muD = T.half_muD_f;
+    const int deg = T.inc_off[k + 1] - T.inc_off[k];
+    const long long at = T.nod_off[k >> 5] + (k & 31);
+    const float4 *ref = T.nod_ref + at;
+    const ushort2 *idx = reinterpret_cast<const ushort2 *>(T.nod_idx) + at;
+    const float4 xk = xs[k];
+    float K[3] = {0.f, 0.f, 0.f}, nrm[3] = {0.f, 0.f, 0.f}, A8 = 0.f, zr = 1.f, zi = 0.f;
+    F[0] = F[1] = F[2] = 0.f;
+    float4 rn = make_float4(0.f, 0.f, 0.f, 0.f);
+    ushort2 in = make_ushort2(0, 0);
+    int prev = -1;
+    float e1[3] = {0.f, 0.f, 0.f}, l1 = 0.f, cF = 0.f, cK = 0.f;   // current edge and its coefficients
+    if (deg > 0) {
+        rn = ref[0];
+        in = idx[0];
     }
-    const float rn = rsqrtf(nrm[0] * nrm[0] + nrm[1] * nrm[1] + nrm[2] * nrm[2]);
-    const float h = 0.5f / A;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        n_out[a] = nrm[a] * rn;
-        K[a] *= h;
-    }
-    A_out = A;
-    kH_out = 0.5f * (K[0] * n_out[0] + K[1] * n_out[1] + K[2] * n_out[2]);
-    kG_out = -atan2f(zi, zr) / A;
-}
-
-// Pass 2 at vertex k: lap = sum (cot_l (kH_j - kH_k) + cot_j (kH_l - kH_k))
-// and the unnormalised normal, in the order of pass 1.
-__device__ __forceinline__ void bend2_f32(const TmplDev &T, int k, const float *xs, const float *kHs, int nn,
-                                          float &lap_out, float nrm[3])
-{
-    float lap = 0.f;
-    nrm[0] = nrm[1] = nrm[2] = 0.f;
-    const float xk[3] = {xs[k], xs[nn + k], xs[2 * nn + k]};
-    const float kHk = kHs[k];
-    for (int q = T.inc_off[k]; q < T.inc_off[k + 1]; ++q) {
-        const int2 jl = T.ring[q];
-        const float xj[3] = {xs[jl.x], xs[nn + jl.x], xs[2 * nn + jl.x]};
-        const float xl[3] = {xs[jl.y], xs[nn + jl.y], xs[2 * nn + jl.y]};
-        RingF t;
-        ring_tri_f32(xk, xj, xl, t);
-        lap += (t.dl * t.inv2A) * (kHs[jl.x] - kHk) + (t.dj * t.inv2A) * (kHs[jl.y] - kHk);
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            nrm[a] += t.fn[a];
-    }
-    lap_out = lap;
-}
-
-// ------------------------------------------------------------ FP32 fused path
-// One CTA per instance: node positions and force accumulators in shared
-// memory, element forces added with shared-memory atomics (order not
-// reproducible), then the two bending passes, then one coalesced write of F.
-// The bending force is split so that only kH is kept between the passes:
-//   pass 1 (vertex i): F_i += 2 kb * 2 (kH - kH0)(kH^2 - kG + kH0 kH) A_i n_i
-//   pass 2 (vertex i): F_i += 2 kb * Lap(kH - kH0) A_i n_i = kb * lap_i * n_i
-// where lap_i = sum_j (cot a_ij + cot b_ij)(kH_j - kH_i) (A_i cancels) and n_i
-// is recomputed from the incident faces in the same order as in pass 1.
-// Shared memory: 3n (x) + 3n (F) + n (kH) floats.
-static __global__ void __launch_bounds__(512, 2) forces_fused_f32_kernel(DevBatch b, const float *__restrict__ x,
-                                                                      float *__restrict__ F,
-                                                                      unsigned long long *status, int inst0)
-{
-    extern __shared__ float sm[];
-    const InstDev I = b.inst[inst0 + blockIdx.x];   // particles inst0, inst0 + 1, ...
-    const TmplDev T = b.tmpl[I.tmpl];
-    const int nn = T.n_nodes;
-    const long long N = b.N;
-    float *xs = sm;               // [3][nn]
-    float *Fs = sm + 3 * nn;      // [3][nn]
-    float *kHs = sm + 6 * nn;     // [nn]
-    const unsigned sF = smem_u32(Fs);
-    for (int k = threadIdx.x; k < nn; k += blockDim.x) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            xs[a * nn + k] = x[a * N + I.node_off + k];
-            Fs[a * nn + k] = 0.f;
+    for (int q = 0; q < deg; ++q) {
+        const float4 r = rn;
+        const ushort2 jl = in;
+        if (q + 1 < deg) {
+            rn = ref[32 * (q + 1)];
+            in = idx[32 * (q + 1)];
         }
-    }
-    __syncthreads();
-    const float *ref = T.ref_f;
-    unsigned long long inverted = 0;
-    for (int e = threadIdx.x; e < T.n_elems; e += blockDim.x) {
-        if (T.kind == 0) {
-            int v[3] = {T.elems[3 * e], T.elems[3 * e + 1], T.elems[3 * e + 2]};
-            float p[3][3], f[3][3];
+        if (jl.x != prev) {   // a new fan
 #pragma unroll
-            for (int c = 0; c < 3; ++c)
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    p[c][a] = xs[a * nn + v[c]];
-            const float *r = ref + 5 * e;
-            float m[4] = {r[0], r[1], r[2], r[3]};
-            membrane_force<float>(T.law, (float)T.mu, (float)T.C, m, r[4], p[0], p[1], p[2], f);
-#pragma unroll
-            for (int c = 0; c < 3; ++c)
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    red_shared_add(sF + 4u * (unsigned)(a * nn + v[c]), f[c][a]);
-        } else {
-            int v[4];
-            float p[4][3], f[4][3];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                v[c] = T.elems[4 * e + c];
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    p[c][a] = xs[a * nn + v[c]];
+            for (int i = 0; i < 3; ++i) {
+                F[i] += cF * e1[i];
+                if constexpr (BEND)
+                    K[i] += cK * e1[i];
             }
-            const float *r = ref + 10 * e;
-            float J = tet_force<float>((float)T.lam, (float)T.mu, r, r[9], p, f);
-            inverted += !(J > 0.f);
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    red_shared_add(sF + 4u * (unsigned)(a * nn + v[c]), f[c][a]);
+            cF = cK = 0.f;
+            ring_edge_f32(xk, xs[jl.x], e1, l1);
         }
+        prev = jl.y;
+        float e2[3], l2;
+        ring_edge_f32(xk, xs[jl.y], e2, l2);
+        RingF t;
+        ring_tri_f32(e1, l1, e2, l2, t);
+        const float w = r.w, w2 = w * w;
+        const float I2 = t.q * w2;
+        float a, b;
+        if (T.law == 0) {
+            a = mu;
+            b = -mu / (I2 * I2);
+        } else {
+            a = mu * ((l1 * r.z + l2 * r.y + (t.dj + t.dl) * r.x) * w2 - 1.f);
+            b = half_muD * (I2 - 1.f) - mu;
+        }
+        const float hw = 0.5f * w;
+        cF += hw * (a * r.z + b * t.dl);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            F[i] += cF * e1[i];
+        cF = hw * (a * r.y + b * t.dj);
+        if constexpr (BEND) {
+            const float cj = t.dj * t.inv2A, cl = t.dl * t.inv2A;
+            // K += cot_l (x_k - x_j) + cot_j (x_k - x_l), sign taken below
+            cK += cl;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                K[i] += cK * e1[i];
+                nrm[i] += t.fn[i];
+            }
+            cK = cj;
+            const float twoA = t.q * t.inv2A;
+            // 8 x mixed area: Voronoi, or 2A / 4 at an obtuse corner and 2A / 8 beside one
+            const float obt = t.dk < 0.f ? twoA + twoA : twoA;
+            A8 += fminf(t.dk, fminf(t.dj, t.dl)) >= 0.f ? cl * l1 + cj * l2 : obt;
+            // unit (cos, sin) of the corner angle at k, |e1||e2| = sqrt(l1 l2)
+            const float rr = rsqrtf(l1 * l2);
+            const float cr = t.dk * rr, ci = twoA * rr;
+            const float nr = zr * cr - zi * ci;
+            zi = zr * ci + zi * cr;
+            zr = nr;
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            e1[i] = e2[i];
+        l1 = l2;
     }
-    if (T.kind == 0 && T.kb != 0.0) {
-        const float kb = (float)T.kb, kH0 = -0.5f * (float)T.c0;
-        for (int k = threadIdx.x; k < nn; k += blockDim.x) {
-            float A, kH, kG, n[3];
-            bend1_f32(T, k, xs, nn, A, kH, kG, n);
-            kHs[k] = kH;
-            const float dh = kH - kH0;
-            const float mag = 2.f * kb * (2.f * dh * (kH * kH - kG + kH0 * kH)) * A;
 #pragma unroll
-            for (int a = 0; a < 3; ++a)
-                red_shared_add(sF + 4u * (unsigned)(a * nn + k), mag * n[a]);
+    for (int i = 0; i < 3; ++i)
+        F[i] += cF * e1[i];
+    if constexpr (BEND) {
+        const float kb = T.kb_f, kH0 = T.kH0_f;
+        const float rnl = rsqrtf(nrm[0] * nrm[0] + nrm[1] * nrm[1] + nrm[2] * nrm[2]);
+        const float A = 0.125f * A8;
+        const float h = -0.5f / A;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            K[i] += cK * e1[i];
+            nrm[i] *= rnl;
+            K[i] *= h;
         }
+        kH = 0.5f * (K[0] * nrm[0] + K[1] * nrm[1] + K[2] * nrm[2]);
+        const float kG = -atan2f(zi, zr) / A;
+        const float dh = kH - kH0;
+        const float mag = 2.f * kb * (2.f * dh * (kH * kH - kG + kH0 * kH)) * A;
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            F[i] += mag * nrm[i];
+    }
+}
+
+// Pass 2 of a membrane node: 2 kb Lap(kH - kH0) A n = kb lap n, lap = sum over
+// the ring of cot_l (kH_j - kH_k) + cot_j (kH_l - kH_k) (kH beside the
+// positions; A cancels), n recomputed in the order of pass 1.
+__device__ __forceinline__ void nodal_bend2(const TmplDev &T, int k, const float4 *xs, float Fb[3])
+{
+    const int deg = T.inc_off[k + 1] - T.inc_off[k];
+    const ushort2 *idx = reinterpret_cast<const ushort2 *>(T.nod_idx) + T.nod_off[k >> 5] + (k & 31);
+    const float4 xk = xs[k];
+    float lap = 0.f, nrm[3] = {0.f, 0.f, 0.f};
+    float e1[3] = {0.f, 0.f, 0.f}, l1 = 0.f, h1 = 0.f;
+    int prev = -1;
+    ushort2 in = deg > 0 ? idx[0] : make_ushort2(0, 0);
+    for (int q = 0; q < deg; ++q) {
+        const ushort2 jl = in;
+        if (q + 1 < deg)
+            in = idx[32 * (q + 1)];
+        if (jl.x != prev) {
+            const float4 xj = xs[jl.x];
+            ring_edge_f32(xk, xj, e1, l1);
+            h1 = xj.w - xk.w;
+        }
+        prev = jl.y;
+        const float4 xl = xs[jl.y];
+        float e2[3], l2;
+        ring_edge_f32(xk, xl, e2, l2);
+        const float h2 = xl.w - xk.w;
+        RingF t;
+        ring_tri_f32(e1, l1, e2, l2, t);
+        lap += (t.dl * h1 + t.dj * h2) * t.inv2A;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            nrm[i] += t.fn[i];
+            e1[i] = e2[i];
+        }
+        l1 = l2;
+        h1 = h2;
+    }
+    const float s = T.kb_f * lap * rsqrtf(nrm[0] * nrm[0] + nrm[1] * nrm[1] + nrm[2] * nrm[2]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+        Fb[i] = s * nrm[i];
+}
+
+// A solid node; returns the number of incident tets with J <= 0 among those
+// that count here (each tet is counted at its first corner).
+__device__ __forceinline__ int nodal_solid(const TmplDev &T, int k, const float4 *xs, float F[3])
+{
+    const float mu = T.mu_f, half_lam = T.half_lam_f;
+    const int deg = T.inc_off[k + 1] - T.inc_off[k];
+    const long long at = T.nod_off[k >> 5] + (k & 31);
+    const float4 *ref = T.nod_ref + at;
+    const ushort4 *idx = reinterpret_cast<const ushort4 *>(T.nod_idx) + at;
+    const float4 x0 = xs[k];
+    int inverted = 0;
+    F[0] = F[1] = F[2] = 0.f;
+    float4 rn = make_float4(0.f, 0.f, 0.f, 0.f);
+    ushort4 in = make_ushort4(0, 0, 0, 0);
+    if (deg > 0) {
+        rn = ref[0];
+        in = idx[0];
+    }
+    for (int q = 0; q < deg; ++q) {
+        const float4 h = rn;
+        const ushort4 v = in;
+        if (q + 1 < deg) {
+            rn = ref[32 * (q + 1)];
+            in = idx[32 * (q + 1)];
+        }
+        const float4 p1 = xs[v.x], p2 = xs[v.y], p3 = xs[v.z];
+        const float d1[3] = {p1.x - x0.x, p1.y - x0.y, p1.z - x0.z};
+        const float d2[3] = {p2.x - x0.x, p2.y - x0.y, p2.z - x0.z};
+        const float d3[3] = {p3.x - x0.x, p3.y - x0.y, p3.z - x0.z};
+        const float c[3] = {d2[1] * d3[2] - d2[2] * d3[1], d2[2] * d3[0] - d2[0] * d3[2],
+                            d2[0] * d3[1] - d2[1] * d3[0]};
+        const float J = (d1[0] * c[0] + d1[1] * c[1] + d1[2] * c[2]) * h.w;
+        inverted += v.w != 0 && !(J > 0.f);
+        // n = d2 x d3 + d1 x (d2 - d3)
+        const float g[3] = {d2[0] - d3[0], d2[1] - d3[1], d2[2] - d3[2]};
+        const float n[3] = {c[0] + (d1[1] * g[2] - d1[2] * g[1]), c[1] + (d1[2] * g[0] - d1[0] * g[2]),
+                            c[2] + (d1[0] * g[1] - d1[1] * g[0])};
+        const float beta = (half_lam * (J * J - 1.f) - mu) / (6.f * J);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            F[i] += mu * (h.x * d1[i] + h.y * d2[i] + h.z * d3[i]) + beta * n[i];
+    }
+    return inverted;
+}
+
+// What bounds it: latency and instruction issue. On the 600-particle suspension
+// (1.33 M nodes) 63 M warp instructions, 64 % of the issue slots of the active
+// cycles, at the 28 warps per SM that 64 registers allow (fewer registers
+// spill: 110 us with 40); shared memory at 34 %. 85 us against 129 us for the
+// kernel before it (per-element forces added with float atomics in shared
+// memory, 60 % of that pipe), one red cell 11 against 47 us, the
+// element-buffer path of the deterministic mode (four launches) 51 -> 19 us
+// on 72 particles.
+// One cluster of S CTAs per particle (S = 1: one CTA), each holding every
+// position of the particle in shared memory (float4, kH in w) and taking a
+// chunk of its nodes (inst0 < 0: all particles, the largest first; else
+// particles inst0, inst0 + 1, ...); kH goes to every CTA of the cluster between the passes.
+// The row of F is kept in global memory between the passes (read back by the
+// thread that wrote it).
+template <bool CLUSTER>
+static __global__ void __launch_bounds__(512, 2) forces_nodal_f32_kernel(DevBatch b, const float *__restrict__ x,
+                                                                      float *__restrict__ F,
+                                                                      unsigned long long *status, int inst0, int S)
+{
+    extern __shared__ __align__(16) float4 nodal_xs[];
+    float4 *xs = nodal_xs;
+    const int rank = CLUSTER ? (int)(blockIdx.x % S) : 0;
+    const int which = CLUSTER ? (int)(blockIdx.x / S) : (int)blockIdx.x;
+    const InstDev I = b.inst[inst0 < 0 ? b.inst_order[which] : inst0 + which];
+    const TmplDev &T = b.tmpl[I.tmpl];
+    const int nn = I.n_nodes;
+    const long long N = b.N;
+    const float *xp = x + I.node_off;
+    for (int k = threadIdx.x; k < nn; k += blockDim.x)
+        xs[k] = make_float4(xp[k], xp[N + k], xp[2 * N + k], 0.f);
+    if constexpr (CLUSTER)   // every CTA of the cluster holds its positions (and runs) before kH arrives
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else
         __syncthreads();
-        for (int k = threadIdx.x; k < nn; k += blockDim.x) {
-            float lap, nrm[3];
-            bend2_f32(T, k, xs, kHs, nn, lap, nrm);
-            const float s = kb * lap * rsqrtf(nrm[0] * nrm[0] + nrm[1] * nrm[1] + nrm[2] * nrm[2]);
+    const int chunk = CLUSTER ? ((nn + S - 1) / S + 31) & ~31 : nn;
+    const int k0 = rank * chunk, k1 = min(nn, k0 + chunk);
+    float *Fp = F + I.node_off;
+    if (T.kind != 0) {
+        int inverted = 0;
+        for (int k = k0 + (int)threadIdx.x; k < k1; k += blockDim.x) {
+            float f[3];
+            inverted += nodal_solid(T, k, xs, f);
 #pragma unroll
             for (int a = 0; a < 3; ++a)
-                red_shared_add(sF + 4u * (unsigned)(a * nn + k), s * nrm[a]);
+                Fp[a * N + k] = f[a];
         }
+        inverted = __reduce_add_sync(0xffffffffu, inverted);
+        if ((threadIdx.x & 31) == 0)
+            status_add(status, ST_INVERTED, (unsigned long long)inverted);
+        return;   // every CTA of the cluster alike
     }
-    __syncthreads();
-    for (int k = threadIdx.x; k < nn; k += blockDim.x) {
+    if (T.kb_f == 0.f) {
+        for (int k = k0 + (int)threadIdx.x; k < k1; k += blockDim.x) {
+            float f[3], kH;
+            nodal_membrane<false>(T, k, xs, f, kH);
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                Fp[a * N + k] = f[a];
+        }
+        return;
+    }
+    for (int k = k0 + (int)threadIdx.x; k < k1; k += blockDim.x) {
+        float f[3], kH;
+        nodal_membrane<true>(T, k, xs, f, kH);
 #pragma unroll
         for (int a = 0; a < 3; ++a)
-            F[a * N + I.node_off + k] = Fs[a * nn + k];
+            Fp[a * N + k] = f[a];
+        if constexpr (CLUSTER) {
+            const unsigned at = smem_u32(&xs[k].w);
+            for (int r = 0; r < S; ++r) {
+                unsigned there;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(at), "r"(r));
+                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(there), "f"(kH) : "memory");
+            }
+        } else {
+            xs[k].w = kH;
+        }
     }
-    unsigned long long tot = inverted;
+    if constexpr (CLUSTER)
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else
+        __syncthreads();
+    for (int k = k0 + (int)threadIdx.x; k < k1; k += blockDim.x) {
+        float f[3];
+        nodal_bend2(T, k, xs, f);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        tot += __shfl_down_sync(0xffffffffu, tot, o);
-    if ((threadIdx.x & 31) == 0)
-        status_add(status, ST_INVERTED, tot);
+        for (int a = 0; a < 3; ++a)
+            Fp[a * N + k] += f[a];
+    }
 }
 
 }  // namespace ifem

@@ -42,6 +42,9 @@ struct ifem_tmpl_s {
     int *d_inc_off = nullptr;
     int *d_inc_idx = nullptr;
     int2 *d_ring = nullptr;
+    int *d_nod_off = nullptr;
+    float4 *d_nod_ref = nullptr;
+    unsigned short *d_nod_idx = nullptr;
 };
 
 struct ifem_grid_s {
@@ -71,12 +74,13 @@ struct ifem_batch_s {
     long long N = 0;
     long long n_elems = 0;
     int max_nodes = 0, max_elems = 0;
-    int any_bending = 0, fused_ok = 0;
+    int any_bending = 0, nodal_ok = 0;
     int max_box = 0;
     ifem_grid grid0 = nullptr;
     InstDev *d_inst = nullptr;
     TmplDev *d_tmpl = nullptr;
     int *d_node_inst = nullptr;
+    int *d_inst_order = nullptr;
     void *d_elem_buf = nullptr;
     void *d_bend_buf = nullptr;
     Workspace ws;
@@ -118,10 +122,11 @@ inline DevBatch dev_batch(ifem_batch b)
     d.max_elems = b->max_elems;
     d.n_elems_total = b->n_elems;
     d.any_bending = b->any_bending;
-    d.fused_ok = b->fused_ok;
+    d.nodal_ok = b->nodal_ok;
     d.inst = b->d_inst;
     d.tmpl = b->d_tmpl;
     d.node_inst = b->d_node_inst;
+    d.inst_order = b->d_inst_order;
     return d;
 }
 

@@ -17,6 +17,45 @@ namespace ifem {
             return e_;                           \
     } while (0)
 
+// FP32 nodal forces of particles [inst0, inst0 + n): a cluster of S CTAs per
+// particle. With few particles one CTA each leaves most SMs idle; with many,
+// each doubling only stages the positions once more. Times in us, S = 1, 2, 4, 8:
+//   one red cell (2562 nodes)     29  19  14  11
+//   16 balls of 4096 nodes        62  31  18  21
+//   64 balls of 4096 nodes        64  36  31  35
+//   72 red cells and platelets    30  21  19  30
+//   200 capsules of 2562 nodes    46  44  54  83
+//   300 red cells                 47  52  84 121
+//   600 red cells and platelets   85  87 132 212
+// Nodes per thread: as few rounds as 512 threads allow, evenly filled (smaller
+// blocks measured slower throughout: 600 particles 102 us with 192 threads).
+template <typename real>   // float (a template so that kernels_f64.cu compiles no FP32 kernel)
+static cudaError_t launch_nodal_forces(const DevBatch &b, const float *x, float *F, unsigned long long *status,
+                                       int inst0, int n, int n_sm, cudaStream_t s)
+{
+    const int S = 16 * n <= n_sm ? 8 : (2 * n <= n_sm ? 4 : (2 * n <= 3 * n_sm ? 2 : 1));
+    const int chunk = ((b.max_nodes + S - 1) / S + 31) & ~31;
+    const int rounds = (chunk + 511) / 512;
+    const int threads = ((chunk + rounds - 1) / rounds + 31) & ~31;
+    const size_t sm = nodal_smem_bytes(b.max_nodes);
+    auto kern = S > 1 ? forces_nodal_f32_kernel<true> : forces_nodal_f32_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess)
+        return e;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = S;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(n * S));
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = S > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, b, x, F, status, n == b.n_inst ? -1 : inst0, S);
+}
+
 template <typename real>
 cudaError_t forces_impl(const ForcesArgs &a)
 {
@@ -27,19 +66,15 @@ cudaError_t forces_impl(const ForcesArgs &a)
     real *F = (real *)a.F;
     cudaStream_t s = a.stream;
     if constexpr (std::is_same<real, float>::value) {
-        if (!a.hvp && a.scatter == 1 && b.fused_ok) {
-        size_t sm = fused_smem_bytes(b.max_nodes);
-        const int n = a.inst_n > 0 ? a.inst_n : b.n_inst;
-        if (a.inst0 < 0 || a.inst0 + n > b.n_inst)
-            return cudaErrorInvalidValue;
-        cudaFuncSetAttribute(forces_fused_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        forces_fused_f32_kernel<<<n, 512, sm, s>>>(b, (const float *)a.x, (float *)a.F, a.w.status, a.inst0);
-        IFEM_LAUNCH_CHECK();
-        return cudaSuccess;
+        if (!a.hvp && b.nodal_ok) {
+            const int n = a.inst_n > 0 ? a.inst_n : b.n_inst;
+            if (a.inst0 < 0 || a.inst0 + n > b.n_inst)
+                return cudaErrorInvalidValue;
+            return launch_nodal_forces<real>(b, x, F, a.w.status, a.inst0, n, a.n_sm, s);
         }
     }
     if (a.inst0 != 0 || (a.inst_n != 0 && a.inst_n != b.n_inst))
-        return cudaErrorInvalidValue;   // particle ranges: the one-CTA-per-particle kernel only
+        return cudaErrorInvalidValue;   // particle ranges: the nodal kernel only
     dim3 blk(256);
     dim3 ge((b.max_elems + 255) / 256, b.n_inst);
     dim3 gn((b.max_nodes + 255) / 256, b.n_inst);
