@@ -99,12 +99,6 @@ extern "C" int ifem_ctx_create(const ifem_config *cfg, ifem_ctx *out)
     // 64-bit fixed point (slower shared-memory atomics), anything else 32-bit
     if (const char *acc = std::getenv("IFEM_SPREAD_ACC"))
         ctx->acc64 = std::string(acc) == "64" ? 1 : 0;
-    // fused FP32 transfer kernel (tuning knob): the velocity box of each item
-    // is staged in shared memory (transfer_staged_kernel) unless
-    // IFEM_TRANSFER=halo selects the kernel that gathers velocities through L1
-    ctx->staged = 1;
-    if (const char *tr = std::getenv("IFEM_TRANSFER"))
-        ctx->staged = std::string(tr) == "halo" ? 0 : 1;
     if (cudaSetDevice(cfg->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess ||
         cudaMalloc((void **)&ctx->d_status, sizeof(unsigned long long) * kStatusWords) != cudaSuccess ||
@@ -780,7 +774,9 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
         BoxDev &B = boxes[i];
         B.n = g->n[i];
         B.t = std::min(tile, B.n);
-        B.T = tiles_per_axis(B.n, B.t);
+        // candidate lists need tiles of at least 5 cells; own lists do not, and
+        // keep every tile within the tile edge
+        B.T = use_halo(ctx) ? (B.n + B.t - 1) / B.t : tiles_per_axis(B.n, B.t);
         B.tile_base = nt;
         B.grid_off = g->off[i];
         B.L = g->L[i];
@@ -817,13 +813,13 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
     CK(alloc((void **)&w.own_count, sizeof(int) * (no + 1 + 4 * nt)));
     w.own_flag = w.own_count + no + 1;
     w.tile_fsum = reinterpret_cast<float *>(w.own_flag + nt);
-    CK(alloc((void **)&w.own_off, sizeof(int) * (no + 1)));
     CK(alloc((void **)&w.own_cursor, sizeof(int) * (no + 1)));
-    CK(alloc((void **)&w.own_nodes, sizeof(int) * (size_t)std::max<long long>(N, 1)));
-    CK(alloc((void **)&w.own_rec, sizeof(float4) * (size_t)std::max<long long>(N, 1)));
-    w.node_key = nullptr;
-    w.node_rec = nullptr;
-    if (use_halo(ctx)) {
+    if (!use_halo(ctx)) {
+        CK(alloc((void **)&w.own_off, sizeof(int) * (no + 1)));
+        CK(alloc((void **)&w.own_nodes, sizeof(int) * (size_t)std::max<long long>(N, 1)));
+    } else {
+        CK(alloc((void **)&w.own_rec, 2 * sizeof(float4) * (size_t)std::max<long long>(N, 1)));
+        CK(alloc((void **)&w.tile_desc, sizeof(TileDesc) * (size_t)(nt + 1)));
         CK(alloc((void **)&w.node_key, sizeof(int2) * (size_t)std::max<long long>(N, 1)));
         CK(alloc((void **)&w.node_rec, sizeof(float4) * (size_t)std::max<long long>(N, 1)));
     }
@@ -831,7 +827,6 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
     if (ctx->cfg.precision == IFEM_FP64 && ctx->cfg.kernel == IFEM_KERNEL_PESKIN4)
         CK(alloc((void **)&w.wtab, sizeof(DetW) * (size_t)std::max<long long>(N, 1)));
     CK(alloc((void **)&w.active, sizeof(int) * (nt + 1)));
-    CK(alloc((void **)&w.own_tiles, sizeof(int) * (nt + 1)));
     CK(alloc((void **)&w.counters, sizeof(int) * kCounters));
     CK(alloc((void **)&w.scan_blocks, sizeof(int) * 2 * (nb + 1)));
     CK(alloc((void **)&w.red_tile, sizeof(double) * 3 * (nt + 1)));
@@ -900,7 +895,7 @@ static TransferArgs transfer_args(ifem_ctx ctx, ifem_batch b, const void *x, con
     a.support = ctx->cfg.mls_support;
     a.n_sm = ctx->n_sm;
     a.acc64 = ctx->acc64;
-    a.halo = use_halo(ctx) ? (ctx->staged ? 2 : 1) : 0;
+    a.halo = use_halo(ctx);
     a.lattice = -1;
     a.stream = (cudaStream_t)stream;
     return a;
@@ -929,8 +924,8 @@ static int do_forces(ifem_ctx ctx, ifem_batch b, const void *x, void *F, const v
 }
 
 // stages other than BIN_ALL: the FP32 halo path only. F (FP32 halo path):
-// the placement also sums |F| per tile, which the fused transfer requires
-// (every do_spread_interp follows a binning given the same forces).
+// the placement also sums |F| per tile, which the tile transfer's spread
+// requires (every spread follows a binning given the same forces).
 static int do_bin(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, void *stream, int stages = BIN_ALL,
                   const void *F = nullptr)
 {
@@ -1058,7 +1053,7 @@ extern "C" int ifem_spread(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *
         return fail(ctx, IFEM_ERR_ARG, "spread: null array or grid");
     if (flags & ~(IFEM_SPREAD_FORCE | IFEM_SPREAD_OVERWRITE))
         return fail(ctx, IFEM_ERR_ARG, "spread: unknown flags");
-    if ((rc = do_bin(ctx, b, g, x, stream)) != IFEM_OK)
+    if ((rc = do_bin(ctx, b, g, x, stream, BIN_ALL, F)) != IFEM_OK)
         return rc;
     return do_spread(ctx, b, g, x, F, f, flags, stream);
 }
@@ -1141,7 +1136,7 @@ extern "C" int ifem_indicator_source(ifem_ctx ctx, ifem_batch b, ifem_grid g, co
                                                     : launch_area_normals_f32(db, x, nA, (cudaStream_t)stream);
     if ((rc = launch_rc(ctx, e, "indicator_source")) != IFEM_OK)
         return rc;
-    if ((rc = do_bin(ctx, b, g, x, stream)) != IFEM_OK)
+    if ((rc = do_bin(ctx, b, g, x, stream, BIN_ALL, nA)) != IFEM_OK)
         return rc;
     return do_spread(ctx, b, g, x, nA, G, flags, stream);
 }
@@ -1407,7 +1402,7 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
     // programmatic serialization: their CTAs start on the SMs that the
     // previous lattice's CTAs leave when its items run out (they read nothing
     // it writes), so the three launches share one tail instead of one each
-    const bool v_rows = fused && io && ctx->staged && node_bytes > 0 && !(flags & IFEM_SPREAD_OVERWRITE);
+    const bool v_rows = fused && io && node_bytes > 0 && !(flags & IFEM_SPREAD_OVERWRITE);
     if (v_rows) {
         const size_t row = node_bytes / 3;
         for (int d = 0; d < 3; ++d) {

@@ -120,6 +120,17 @@ struct DetW {
 };
 static_assert(sizeof(DetW) == 336, "DetW layout");
 
+// A tile with own nodes (FP32 halo path), as the transfer needs it.
+struct alignas(16) TileDesc {
+    int tile, n, beg, end;   // tile number, cells per box side, own records [beg, end)
+    int start[3], edge[3];   // first cell and cells per axis
+    long long grid_off;      // the box's offset in a grid field
+    double h3;               // (L/n)^3
+    float scale_f;           // (n/L)^3
+    int pad;
+};
+static_assert(sizeof(TileDesc) == 64, "TileDesc layout");
+
 struct DevWork {
     int *cand_count;    // n_tiles + 1
     int *cand_off;      // n_tiles + 1
@@ -130,17 +141,18 @@ struct DevWork {
     int *own_flag;      // n_tiles (FP32 halo path): 1 where the tile owns a node
     float *tile_fsum;   // 3 per tile (FP32 halo path): sum of |F_d| over the tile's own nodes, from the
                         // placement when it is given the forces (the fused transfer's fixed-point scale)
-    int *own_off;       // n_tiles * kOwnSub3 + 1 offsets; the FP32 halo path finalises the tile
-                        // boundaries only (entries t * kOwnSub3)
+    int *own_off;       // n_tiles * kOwnSub3 + 1 offsets (not in the FP32 halo path)
     int *own_cursor;    // fill cursors; local (per scan block) offsets in the FP32 halo path
-    int *own_nodes;     // N entries: nodes grouped by the tile (and sub-block) of their cell
-    float4 *own_rec;    // beside own_nodes (FP32 halo path): fractional cell coordinates x, y, z of
-                        // the node and, in w, its cell within the tile packed as 8-bit x | y << 8 | z << 16
+    int *own_nodes;     // N entries: nodes grouped by the tile (and sub-block) of their cell (not in
+                        // the FP32 halo path)
+    float4 *own_rec;    // FP32 halo path, 2 per node in that grouping: fractional cell coordinates
+                        // x, y, z of the node and, in w, its cell within the tile packed as 8-bit
+                        // x | y << 8 | z << 16; its force and, in w, its id
     int2 *node_key;     // N entries, by node (FP32 halo path): own-list key (-1: not binned) and
                         // the node's rank among the nodes of that key
-    float4 *node_rec;   // N entries, by node (FP32 halo path): the own_rec entry of the node
+    float4 *node_rec;   // N entries, by node (FP32 halo path): the first float4 of its own_rec entry
     int *active;        // tiles with candidate pairs
-    int *own_tiles;     // tiles with own nodes (FP32 halo path), counters[3] of them
+    TileDesc *tile_desc;  // tiles with own nodes (FP32 halo path), counters[3] of them
     int *counters;      // kCounters: [0] n_active, [2] work counter, [3] tiles with own nodes,
                         // [4] total pairs, [5] total own nodes, [1] [6] [7] work counters of
                         // one-lattice launches, [8] scan blocks finished
@@ -363,12 +375,11 @@ struct TransferArgs {
     double support;
     int n_sm;
     int acc64;        // FP32 spread: 64-bit (1) or 32-bit (0) fixed-point accumulators
-    int halo;         // FP32 Peskin spread with halo scatter (IFEM_SCATTER_ATOMIC): 1; 2 with the
-                      // velocity box staged in shared memory when interpolation is fused
+    int halo;         // FP32 Peskin, IFEM_SCATTER_ATOMIC: the tile transfer over own lists
     int binned;       // the binning of this step ran just before on the same stream (own tiles
                       // listed, work counter and per-tile sums cleared)
-    int lattice;      // staged fused transfer: -1 all three lattices, else that lattice only
-    int pdl;          // staged fused transfer: may start before the previous kernel in the stream ends
+    int lattice;      // tile transfer: -1 all three lattices, else that lattice only
+    int pdl;          // tile transfer: may start before the previous kernel in the stream ends
     int use_wtab;     // FP64 Peskin interpolation: read the stencils the binning of x tabulated
     const void *vp;   // fused position update (halo spread + interpolation only):
     void *xn;         //   xn = x + dt (3/2 v - 1/2 vp) when xn is not null

@@ -144,10 +144,10 @@ cudaError_t bin_impl(const TransferArgs &a, int det_sort, int with_cand, int sta
         bin_kernel<real, true><<<gn, 256, 0, s>>>(b, a.g, w, (const real *)a.x);
         IFEM_LAUNCH_CHECK();
     } else {
-        // enough threads for every tile boundary as well as every node
-        const long long per_inst = ((nt + 1 + 255) / 256 + b.n_inst - 1) / b.n_inst;
+        // enough threads for every tile as well as every node
+        const long long per_inst = ((nt + 255) / 256 + b.n_inst - 1) / b.n_inst;
         dim3 gs((unsigned)std::max<long long>(g1.x, per_inst), b.n_inst);
-        own_scatter_kernel<<<gs, 256, 0, s>>>(b, w, nt, (const float *)a.F);
+        own_scatter_kernel<<<gs, 256, 0, s>>>(b, a.g, w, (const float *)a.F);
         IFEM_LAUNCH_CHECK();
     }
     if (det_sort) {
@@ -161,6 +161,50 @@ cudaError_t bin_impl(const TransferArgs &a, int det_sort, int with_cand, int sta
         }
     }
     return cudaSuccess;
+}
+
+// The FP32 Peskin tile transfer over the own lists of the binning just before
+// it: spreading (SPREAD), interpolation (INTERP) or both, with the position
+// update (AB2) on request. One resident wave of CTAs takes the items.
+template <int W, bool SPREAD, bool INTERP, bool AB2>
+cudaError_t launch_tile_w(const TransferArgs &a)
+{
+    auto kern = transfer_tile_kernel<W, SPREAD, INTERP, AB2>;
+    constexpr int kKinds = (SPREAD ? 1 : 0) + (INTERP ? 1 : 0), T = TileShape<W>::kThreads;
+    const size_t sm = (size_t)4 * TileShape<W>::kWords * 2 * kKinds;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess)
+        return e;
+    int occ = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, T, sm);
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    // programmatic dependent launch: the CTAs of this grid may start once
+    // every CTA of the previous kernel in the stream has signalled
+    // (griddepcontrol.launch_dependents, at its start); they read nothing it
+    // writes
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(a.n_sm * (occ < 1 ? 1 : occ));
+    cfg.blockDim = dim3(T);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = a.stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, a.b, a.w, (const float *)a.x, (float *)a.f, a.density, (const float *)a.u,
+                              (float *)a.v, (const float *)a.vp, (float *)a.xn, (float)a.dt, a.lattice);
+}
+template <bool SPREAD, bool INTERP, bool AB2>
+cudaError_t launch_tile(const TransferArgs &a)
+{
+    switch (tile_width(a.g.max_edge)) {
+    case 12:
+        return launch_tile_w<12, SPREAD, INTERP, AB2>(a);
+    case 16:
+        return launch_tile_w<16, SPREAD, INTERP, AB2>(a);
+    default:
+        return launch_tile_w<20, SPREAD, INTERP, AB2>(a);
+    }
 }
 
 template <typename real>
@@ -183,52 +227,9 @@ cudaError_t spread_impl(const TransferArgs &a)
         if (a.halo) {
             // with u and v given, interpolation is fused into the spread, and
             // with xn also the position update
-            const bool fused = a.u != nullptr && a.v != nullptr;
-            if (fused && a.halo == 2) {
-                auto kp = a.xn ? transfer_staged_kernel<true> : transfer_staged_kernel<false>;
-                const size_t sm = (size_t)pair_smem_bytes(E);
-                cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-                int occ = 1;
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kp, kStagedThreads, sm);
-                occ = occ < 1 ? 1 : occ;
-                if (!a.pdl) {
-                    kp<<<a.n_sm * occ, kStagedThreads, sm, s>>>(b, a.g, a.w, (const float *)a.x,
-                                                              (const float *)a.F, (float *)a.f, a.density,
-                                                              (const float *)a.u, (float *)a.v, (const float *)a.vp,
-                                                              (float *)a.xn, (float)a.dt, a.lattice);
-                    IFEM_LAUNCH_CHECK();
-                    return cudaSuccess;
-                }
-                // programmatic dependent launch: the CTAs of this grid may start once
-                // every CTA of the previous kernel in the stream has signalled
-                // (griddepcontrol.launch_dependents, at its start); they read
-                // nothing it writes
-                cudaLaunchConfig_t cfg{};
-                cudaLaunchAttribute attr[1];
-                attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-                attr[0].val.programmaticStreamSerializationAllowed = 1;
-                cfg.gridDim = dim3(a.n_sm * occ);
-                cfg.blockDim = dim3(kStagedThreads);
-                cfg.dynamicSmemBytes = sm;
-                cfg.stream = s;
-                cfg.attrs = attr;
-                cfg.numAttrs = 1;
-                return cudaLaunchKernelEx(&cfg, kp, b, a.g, a.w, (const float *)a.x, (const float *)a.F,
-                                          (float *)a.f, a.density, (const float *)a.u, (float *)a.v,
-                                          (const float *)a.vp, (float *)a.xn, (float)a.dt, a.lattice);
-            }
-            auto kern = !fused ? spread_halo_kernel<false>
-                               : (a.xn ? spread_halo_kernel<true, true> : spread_halo_kernel<true>);
-            size_t sm = sizeof(int) * (size_t)halo_ints(E);
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            int occ = 1;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 256, sm);
-            occ = occ < 1 ? 1 : occ;
-            kern<<<a.n_sm * occ, 256, sm, s>>>(b, a.g, a.w, (const float *)a.x, (const float *)a.F, (float *)a.f,
-                                               a.density, (const float *)a.u, (float *)a.v,
-                                               (const float *)a.vp, (float *)a.xn, (float)a.dt);
-            IFEM_LAUNCH_CHECK();
-            return cudaSuccess;
+            if (!(a.u && a.v))
+                return launch_tile<true, false, false>(a);
+            return a.xn ? launch_tile<true, true, true>(a) : launch_tile<true, true, false>(a);
         }
         size_t acc = a.acc64 ? sizeof(long long) : sizeof(int);
         size_t sm = acc * 3 * (size_t)acc_stride(E, E, E);
@@ -280,6 +281,8 @@ cudaError_t interp_impl(const TransferArgs &a)
         return cudaSuccess;
     if constexpr (std::is_same<real, float>::value) {
         unsigned grid = (unsigned)((3 * b.N + 255) / 256);
+        if (a.halo)
+            return launch_tile<false, true, false>(a);
         if (a.kernel == 0)
             interp_direct_kernel<0><<<grid, 256, 0, a.stream>>>(b, a.g, a.w, (const float *)a.u, (const float *)a.x,
                                                                (float *)a.v, (float)a.support);

@@ -872,59 +872,29 @@ __global__ void __launch_bounds__(256) spread_fast_kernel(DevBatch b, DevGrid g,
     }
 }
 
-// ------------------------------------------- spread, FP32, halo scatter
-// IFEM_SCATTER_ATOMIC, Peskin kernel. Work item = (tile, lattice) taken from
-// a global counter over every tile. Each node is visited only by the tile
-// that holds its cell (no candidate lists): the CTA accumulates the 64
-// contributions of each own node into a buffer covering the tile plus a
-// halo of 4 cells in x (keeps 16-byte quads aligned) and 2 cells in y and z,
-// so every stencil point of every node lands in the buffer. Accumulation is
-// int32 fixed point with shared-memory atomics (scale from the bound
-// sum_k |g_k| / 8 over the tile's own nodes); the flush adds every non-zero
-// value to the grid with L2 reductions, where neighbouring tiles' halos
-// combine atomically (summation order of a value across tiles is not fixed).
-// ST_TOUCHED counts the non-zero sums inside the tile itself.
-// INTERP = true fuses the interpolation S of the same step: each (node,
-// lattice) unit also gathers u at the 64 stencil points with the unscaled
-// weights it has just computed, v_d = sum phi u_d (Algorithm step 4).
-// AB2 = true (with INTERP) also takes the position update of Eq.
-// Bashforth_eqn from the velocity it has just gathered, out of place:
-// xn_d = x_d + dt (3/2 v_d - 1/2 vp_d), rounded as in ab2_kernel.
-constexpr int kHaloX = 4, kHaloYZ = 2;
-
-// Buffer pitches: the row pitch is 8 mod 16 and the plane pitch 4 mod 8, so
-// the 4 x 4 x 4 cells around a group of neighbouring nodes fall on all 32
-// banks, two cells per bank; both stay multiples of 4 for 16-byte rows.
-__host__ __device__ inline int halo_px(int bx) { return bx + (24 - bx % 16) % 16; }
-__host__ __device__ inline int halo_pp(int by, int px) { return by * px + 4; }
-__host__ __device__ inline int halo_ints(int E)
-{
-    const int px = halo_px(E + 2 * kHaloX);
-    return halo_pp(E + 2 * kHaloYZ, px) * (E + 2 * kHaloYZ);
-}
-
 // FP32 halo path, after the scan: every binned node goes to its slot (the
-// scanned offset of its key plus its rank from own_count_kernel) with its
-// record, kBinPer nodes per thread as in own_count_kernel (loads first, then
-// the offsets, then the stores); the tile boundaries of the own lists are
-// finalised (own_off[t * kOwnSub3] = local offset + block offset, the total
-// at t = n_tiles: the only entries the halo kernels read); the per-tile FP64
-// sums of the spread are cleared for every tile (the transfer writes them
-// for the listed tiles only) and the tiles that own nodes are listed,
-// counters[3] of them. The fused transfer kernels take their (tile,
-// lattice) items from that list, so no CTA walks empty tiles; it keeps
-// roughly the tile order (in order within each warp's append), so items
-// running at the same time are spatial neighbours whose velocity rows and
-// grid lines share L2 (listing the largest tiles first measured slower).
+// scanned offset of its key plus its rank from own_count_kernel) as one
+// 32-byte record: what own_count_kernel kept of it, its force (0 without F)
+// and its id, kBinPer nodes per thread as in own_count_kernel (loads first,
+// then the offsets, then the stores). With the force in the record the
+// transfer reads its nodes in two consecutive 16-byte loads, without a gather
+// through the node id. The per-tile FP64 sums of the spread are cleared for
+// every tile (the transfer writes them for the listed tiles only) and the
+// tiles that own nodes are listed, counters[3] of them, with everything the
+// transfer needs of a tile: it fetches an item in one copy, without walking
+// empty tiles or decoding tile numbers. The list keeps roughly the tile order
+// (in order within each warp's append), so items running at the same time are
+// spatial neighbours whose velocity rows and grid lines share L2 (listing the
+// largest tiles first measured slower).
 // With the forces F given, the placement also sums |F_d| over each tile's
-// own nodes into tile_fsum (zeroed with the counts): the fused transfer's
+// own nodes into tile_fsum (zeroed with the counts): the transfer's
 // fixed-point scale of item (tile, d) comes from that sum instead of a pass
 // over the item's forces. Lanes of a warp hold consecutive nodes, so the
 // tiles come in runs: a segmented shuffle scan sums each run and its last
 // lane adds it with one atomic per lattice (the order of those atomics is
 // not fixed; the transfer's bound allows for it).
-// Grid: as own_count_kernel along x and y, at least n_tiles + 1 threads in all.
-static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, DevWork w, long long n_tiles,
+// Grid: as own_count_kernel along x and y, at least n_tiles threads in all.
+static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, DevGrid g, DevWork w,
                                                                  const float *__restrict__ F)
 {
     const InstDev I = b.inst[blockIdx.y];
@@ -944,10 +914,22 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
             kr[j] = w.node_key[node[j]];
             rec[j] = w.node_rec[node[j]];
             if (F) {
-                fa[j][0] = fabsf(F[node[j]]);
-                fa[j][1] = fabsf(F[N + node[j]]);
-                fa[j][2] = fabsf(F[2 * N + node[j]]);
+                fa[j][0] = F[node[j]];
+                fa[j][1] = F[N + node[j]];
+                fa[j][2] = F[2 * N + node[j]];
             }
+        }
+    }
+    int off[kBinPer];
+#pragma unroll
+    for (int j = 0; j < kBinPer; ++j)
+        off[j] = kr[j].x >= 0 ? w.own_cursor[kr[j].x] + w.scan_blocks[2 * (kr[j].x / kScanBlock) + 1] : 0;
+#pragma unroll
+    for (int j = 0; j < kBinPer; ++j) {
+        if (kr[j].x >= 0) {
+            float4 *slot = w.own_rec + 2LL * (off[j] + kr[j].y);
+            slot[0] = rec[j];
+            slot[1] = make_float4(fa[j][0], fa[j][1], fa[j][2], __int_as_float(node[j]));
         }
     }
     if (F) {   // the same for every thread of the grid
@@ -959,6 +941,9 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
             const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || prev != tile);
             // first lane of this lane's run
             const int seg = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                fa[j][d] = fabsf(fa[j][d]);
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
 #pragma unroll
@@ -975,42 +960,88 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
             }
         }
     }
-    int off[kBinPer];
-#pragma unroll
-    for (int j = 0; j < kBinPer; ++j)
-        off[j] = kr[j].x >= 0 ? w.own_cursor[kr[j].x] + w.scan_blocks[2 * (kr[j].x / kScanBlock) + 1] : 0;
-#pragma unroll
-    for (int j = 0; j < kBinPer; ++j) {
-        if (kr[j].x >= 0) {
-            const int slot = off[j] + kr[j].y;
-            w.own_nodes[slot] = node[j];
-            w.own_rec[slot] = rec[j];
-        }
-    }
     const long long nthr = (long long)gridDim.x * gridDim.y * blockDim.x;
     const long long tid = ((long long)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
-    for (long long t0 = tid - lane; t0 <= n_tiles; t0 += nthr) {   // warp-uniform bounds
+    for (long long t0 = tid - lane; t0 < g.n_tiles; t0 += nthr) {   // warp-uniform bounds
         const long long t = t0 + lane;
         bool has = false;
-        if (t < n_tiles) {
-            const long long i = t * kOwnSub3;
-            w.own_off[i] = w.own_cursor[i] + w.scan_blocks[2 * (i / kScanBlock) + 1];
+        if (t < g.n_tiles) {
             has = w.own_flag[t] != 0;
             w.red_tile[3 * t] = 0.0;
             w.red_tile[3 * t + 1] = 0.0;
             w.red_tile[3 * t + 2] = 0.0;
-        } else if (t == n_tiles) {
-            w.own_off[t * kOwnSub3] = w.counters[5];
         }
         const unsigned m = __ballot_sync(0xffffffffu, has);
         int base = 0;
         if (lane == 0 && m)
             base = atomicAdd(&w.counters[3], __popc(m));
         base = __shfl_sync(0xffffffffu, base, 0);
-        if (has)
-            w.own_tiles[base + __popc(m & ((1u << lane) - 1u))] = (int)t;
+        if (has) {
+            const TileInfo ti = decode_tile(g, t);
+            const BoxDev &B = g.boxes[ti.box];
+            const long long i = t * kOwnSub3, j = i + kOwnSub3;
+            TileDesc td;
+            td.tile = (int)t;
+            td.n = B.n;
+            td.beg = w.own_cursor[i] + w.scan_blocks[2 * (i / kScanBlock) + 1];
+            td.end = t + 1 < g.n_tiles ? w.own_cursor[j] + w.scan_blocks[2 * (j / kScanBlock) + 1] : w.counters[5];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                td.start[a] = ti.start[a];
+                td.edge[a] = ti.edge[a];
+            }
+            td.grid_off = B.grid_off;
+            td.h3 = 1.0 / B.scale;
+            td.scale_f = B.scale_f;
+            td.pad = 0;
+            w.tile_desc[base + __popc(m & ((1u << lane) - 1u))] = td;
+        }
     }
 }
+
+// ------------------------------- tile transfer, FP32 Peskin, own nodes only
+// IFEM_SCATTER_ATOMIC, Peskin kernel: spreading, interpolation, or both fused
+// (Algorithm steps 2 and 4 use the same stencil weights of the same
+// positions), with the position update of Eq. Bashforth_eqn on request. Work
+// item = (tile, lattice) over the tiles with own nodes (own_scatter_kernel),
+// taken from a global counter. Each node is visited only by the tile that
+// holds its cell. Boxes of shared memory cover the tile plus a halo, 2 cells
+// in y and z and 4 in x (so that its 16-byte quads are quads of the grid),
+// which holds every stencil point of every own node: U, the velocity values
+// the item's stencils read, and A, the spread accumulator (int32 fixed point,
+// scale from the bound sum_k |g_k| / 8 over the tile's own nodes, from the sum
+// of |F_d| that the binning's placement keeps per tile; integer addition is
+// associative, so a box does not depend on the order of its nodes).
+//
+// Two boxes of each kind, and two kinds of warps. While the node warps work on
+// item i (one (node, lattice) unit per thread: the Peskin weights, v_d = sum
+// phi u_d from U, 64 contributions added to A with shared-memory reductions),
+// the box warps copy the velocities of item i + 1 into the other U (cp.async)
+// and flush the other A, of item i - 1: every non-zero value is added to the
+// grid with an L2 reduction (the halos of neighbouring tiles combine there;
+// the order of a value's terms across tiles is not fixed) and cleared. One
+// barrier per item. With the copy, the node loop and the flush one after the
+// other, each waited out its own memory latency.
+//
+// Measured, 600-particle suspension (1.33 M nodes, 256^3, 16-cell tiles, fused):
+// 291 us against 375 us for the kernel before it (one box of each kind, three
+// CTAs of 128 threads per SM, stencils in z-y-x order, a status atomic per warp
+// and item); 64 boxes of 32 to 96 cells 240 against 437 us. What bounds it now:
+// instruction issue (51 %) and the shared-memory pipe (44 %) of an SM whose two
+// kinds of warps wait for each other once per item; alone, the node loops take
+// 174 us, the copies 172, the flushes' scans 121.
+//
+// The boxes store the cell (x, y, z) in bank (x & 3) | (z & 3) << 2 | (y & 1)
+// << 4 of the 128-byte line (x >> 2, z >> 2, y >> 1). A unit's 4 x 4 x 4 points
+// fall on every bank exactly twice, and each lane walks its points starting
+// from its own bank: lane l takes, at step (t0, t1, t2), the point in bank
+// ((l + t0) & 3) | ((l >> 2) + t1 & 3) << 2 | ((l >> 4) + t2 & 1) << 4, so the
+// 32 lanes are on 32 different banks at every step wherever their nodes lie.
+// (In plain z-y-x order the lanes' banks are random: 2.7 wavefronts per load
+// and 3.4 per reduction on the 600-particle suspension, by a count over its
+// stencils.) The weights are rotated into that order once per unit; the
+// interpolation adds its terms in pairs that no rotation separates, so v does
+// not depend on the lane.
 
 // red.shared.add without a compiler memory clobber: for accumulators that
 // no thread reads before the next barrier (the caller places a compiler
@@ -1025,254 +1056,68 @@ __device__ __forceinline__ void cp_async16(unsigned dst, const void *src)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(__cvta_generic_to_global(src))
                  : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// Next (tile, lattice) item of the fused transfer kernels (thread 0): items
-// are the three lattices of each listed tile, in list order (lattice < 0,
-// work counter counters[2]), or lattice d of each listed tile (work
-// counters[1], [6], [7] for d = 0, 1, 2), so that one launch per lattice
-// completes row d of v at its end.
-__device__ __forceinline__ void staged_next(const DevGrid &g, const DevWork &w, int lattice, int &item,
-                                            TileInfo &ti, BoxDev &B)
-{
-    const int n_tiles = w.counters[3];
-    int tile = -1, d = 0;
-    if (lattice < 0) {
-        const int it = atomicAdd(&w.counters[2], 1);
-        if (it < 3 * n_tiles) {
-            const int q = it / 3;
-            tile = w.own_tiles[q];
-            d = it - 3 * q;
-        }
-    } else {
-        const int it = atomicAdd(&w.counters[lattice == 0 ? 1 : (lattice == 1 ? 6 : 7)], 1);
-        if (it < n_tiles) {
-            tile = w.own_tiles[it];
-            d = lattice;
-        }
-    }
-    item = -1;
-    if (tile >= 0) {
-        item = 3 * tile + d;
-        ti = decode_tile(g, tile);
-        B = g.boxes[ti.box];
-    }
-}
-
-__device__ __forceinline__ void cp_async8(unsigned dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(__cvta_generic_to_global(src))
-                 : "memory");
-}
 __device__ __forceinline__ void cp_async4(unsigned dst, const void *src)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(__cvta_generic_to_global(src))
                  : "memory");
 }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Periodic wrap of a box coordinate in [-n, 2n): the boxes of a grid have
 // at least 8 cells and the halos at most 4, so one correction suffices.
 __device__ __forceinline__ int wrap1(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
-// Shared buffers of the fused transfer kernel. A, the spread accumulator,
-// covers the tile plus the halo of spread_halo_kernel (4 cells in x, so
-// that the flush adds 16-byte quads, and 2 in y and z). U, the staged
-// velocities, covers exactly the cells the stencils read, 2 cells on every
-// side of the tile: rows of ex + 4 values from x = sx - 2, plane pitch 12
-// floats above the plane size. U starts 8 bytes past a 16-byte boundary, so
-// that the values of x = sx .. sx + ex - 1 fill 16-byte quads. Both rounded
-// to 16 bytes; the pair fits three CTAs per SM for 16-cell tiles.
-constexpr int kStagedThreads = 128;
-__host__ __device__ inline int pair_buf_bytes(int E) { return ((halo_ints(E) * 4 + 15) / 16) * 16; }
-__host__ __device__ inline int pair_u_px(int ex) { return ex + 4; }
-__host__ __device__ inline int pair_u_pp(int ey, int pxu) { return pxu * (ey + 4) + 12; }
-__host__ __device__ inline int pair_u_bytes(int E)
+// Work counter of a launch: the three lattices of each listed tile, in list
+// order (lattice < 0, counters[2]), or lattice d of each listed tile
+// (counters[1], [6], [7] for d = 0, 1, 2), so that one launch per lattice
+// completes row d of v at its end.
+__device__ __forceinline__ int *tile_counter(const DevWork &w, int lattice)
 {
-    return ((8 + 4 * pair_u_pp(E, pair_u_px(E)) * (E + 4) + 15) / 16) * 16;
+    return &w.counters[lattice < 0 ? 2 : (lattice == 0 ? 1 : (lattice == 1 ? 6 : 7))];
 }
-__host__ __device__ inline int pair_smem_bytes(int E) { return pair_u_bytes(E) + pair_buf_bytes(E); }
 
-// One (tile, lattice) item of the fused transfer kernel, in registers.
-struct PairItem {
-    int item, tile, d;
+// Shapes by the width W = 20, 16, 12 of the boxes in y and z (tiles of at most
+// 16, 12, 8 cells): lines per axis, node and box threads. A box thread keeps
+// one (x >> 2, z, y & 1) and walks y in kYStep phases; two phases where that
+// measured faster (64 boxes of odd sizes, 16-cell tiles: 243 against 284 us;
+// 600 particles 292 against 291).
+__host__ __device__ inline int tile_width(int max_edge) { return max_edge <= 8 ? 12 : (max_edge <= 12 ? 16 : 20); }
+template <int W>
+struct TileShape {
+    static constexpr int NX = W / 4 + 1, NZ = W / 4, NY = W / 2;
+    static constexpr int kWords = 32 * NX * NZ * NY;                  // of one box
+    static constexpr int kColumn = (8 * NX * NZ + 31) / 32 * 32;       // box threads per y phase: 256, 160, 96
+    static constexpr int kYStep = W == 16 ? 1 : 2;                    // phases
+    static constexpr int kBoxThreads = kColumn * kYStep;
+    static constexpr int kNodeThreads = W == 20 ? 384 : (W == 16 ? 256 : 64);
+    static constexpr int kThreads = kBoxThreads + kNodeThreads;
+    static constexpr int kCtas = W == 20 ? 1 : (W == 16 ? 2 : 4);     // resident per SM, fused
+};
+
+struct TileItem {
+    int tile, d, beg, end;
     int sx, sy, sz, ex, ey, ez;
-    int n, bx, by, bz, px, pp;
-    int pxu, ppu;   // pitches of the U box
+    int n;
     long long grid_off;
     float sd;
-    double box_scale;
 };
-__device__ __forceinline__ PairItem pair_item(int item, const TileInfo &ti, const BoxDev &B, int density)
+__device__ __forceinline__ TileItem tile_item(const TileDesc &td, int d, int density)
 {
-    PairItem it;
-    it.item = item;
-    it.tile = item / 3;
-    it.d = item - 3 * it.tile;
-    it.sx = ti.start[0];
-    it.sy = ti.start[1];
-    it.sz = ti.start[2];
-    it.ex = ti.edge[0];
-    it.ey = ti.edge[1];
-    it.ez = ti.edge[2];
-    it.n = B.n;
-    it.bx = it.ex + 2 * kHaloX;
-    it.by = it.ey + 2 * kHaloYZ;
-    it.bz = it.ez + 2 * kHaloYZ;
-    it.px = halo_px(it.bx);
-    it.pp = halo_pp(it.by, it.px);
-    it.pxu = pair_u_px(it.ex);
-    it.ppu = pair_u_pp(it.ey, it.pxu);
-    it.grid_off = B.grid_off;
-    it.sd = density ? B.scale_f : 1.f;
-    it.box_scale = B.scale;
-    return it;
+    return TileItem{td.tile, d, td.beg, td.end, td.start[0], td.start[1], td.start[2], td.edge[0], td.edge[1],
+                    td.edge[2], td.n, td.grid_off, density ? td.scale_f : 1.f};
+}
+// 16-byte access to the grid's quads: n, the tile's start and edge multiples of 4, the lattice aligned.
+__device__ __forceinline__ bool tile_vec(const TileItem &it, const float *lat)
+{
+    return ((it.sx | it.n | it.ex) & 3) == 0 && (reinterpret_cast<uintptr_t>(lat) & 15) == 0;
 }
 
-// Rows of a (tile + halo) box walked by the warps of a CTA: a lane takes x
-// unit qx = lq (+ multiples of nql) of every row it visits; rows advance by
-// a fixed (y, z) step, so no index is divided in the loop. fn(lz, ly, gz, gy, qx)
-// receives the row's box coordinates and its wrapped grid coordinates.
-// a / b for 0 <= a < 2^21 and b >= 1, exactly, through a float reciprocal:
-// (a + 1/2) / b lies at least 1/(2b) from the nearest integer, while the
-// rounding of the reciprocal and the product moves it by at most about
-// (a/b) 2^-22 < 1/(2b).
-__device__ __forceinline__ int small_div(int a, int b) { return (int)(((float)a + 0.5f) * __frcp_rn((float)b)); }
-
-// Columns of a (tile + halo) box walked by the threads of a CTA: a column is
-// one x unit (quad or value) qx of one y row ly; each thread takes one column
-// and steps through the z planes (several planes at a time when the CTA has
-// threads for more than one plane's columns), so the loop carries only a
-// plane index. fn(lz, ly, gz, gy, qx) receives the box coordinates and the
-// wrapped grid coordinates. Boxes with more columns than threads take the
-// generic walk (one division per value).
-template <typename Fn>
-__device__ __forceinline__ void box_cols(const PairItem &it, int bz, int by, int nq, Fn fn)
+// Fixed-point scale of an item: the largest power of two that keeps the bound
+// sum |g_k| / 8 below 2^30. fsum: the placement's atomic float sum of |F_d|
+// over n nodes, within (n - 1) 2^-24 of the exact one in any order.
+__device__ __forceinline__ float tile_scale(const TileItem &it, float fsum)
 {
-    const int C = by * nq, T = blockDim.x, t = threadIdx.x;
-    if (C <= T) {
-        const int P = small_div(T, C);
-        const int pz = small_div(t, C);
-        if (pz >= P)
-            return;
-        const int c = t - pz * C;
-        const int ly = small_div(c, nq), qx = c - ly * nq;
-        const int gy = wrap1(it.sy - kHaloYZ + ly, it.n);
-        int gz = wrap1(it.sz - kHaloYZ + pz, it.n);
-        for (int lz = pz; lz < bz; lz += P) {
-            fn(lz, ly, gz, gy, qx);
-            gz += P;
-            gz -= gz >= it.n ? it.n : 0;
-        }
-    } else {
-        for (int q = t; q < C * bz; q += T) {
-            const int lz = small_div(q, C), c = q - lz * C;
-            const int ly = small_div(c, nq), qx = c - ly * nq;
-            fn(lz, ly, wrap1(it.sz - kHaloYZ + lz, it.n), wrap1(it.sy - kHaloYZ + ly, it.n), qx);
-        }
-    }
-}
-
-// The same over a box of bz x by rows starting 2 cells below the tile in y
-// and z (the A box and the U box both do).
-template <typename Fn>
-__device__ __forceinline__ void box_rows(const PairItem &it, int bz, int by, int nq, int lane, int wid, int nw,
-                                         Fn fn)
-{
-    const int nql = nq <= 32 ? nq : 32;
-    const int rpw = small_div(32, nql);
-    const int lr = small_div(lane, nql), lq = lane - lr * nql;
-    if (lr >= rpw)
-        return;
-    const int rstep = nw * rpw;
-    const int r0 = wid * rpw + lr;
-    int lz = small_div(r0, by), ly = r0 - lz * by;
-    const int dz = small_div(rstep, by), dy = rstep - dz * by;
-    while (lz < bz) {
-        const int gz = wrap1(it.sz - kHaloYZ + lz, it.n), gy = wrap1(it.sy - kHaloYZ + ly, it.n);
-        for (int qx = lq; qx < nq; qx += nql)
-            fn(lz, ly, gz, gy, qx);
-        ly += dy;
-        lz += dz;
-        if (ly >= by) {
-            ly -= by;
-            ++lz;
-        }
-    }
-}
-
-template <typename Fn>
-__device__ __forceinline__ void pair_rows(const PairItem &it, int nq, int lane, int wid, int nw, Fn fn)
-{
-    box_rows(it, it.bz, it.by, nq, lane, wid, nw, fn);
-}
-// Copies the velocity box of an item's lattice into the U buffer (value i
-// of a row is x = sx - 2 + i, rows from y and z = tile start - 2)
-// asynchronously with cp.async, waited for before the next node loop. When
-// n, the tile start and edge are multiples of 4 and the lattice is 16-byte
-// aligned, the ex values x = sx .. sx + ex - 1 of every row move as 16-byte
-// quads and the two values at each end as 8-byte pairs (two column walks,
-// so no thread branches per copy); otherwise single values.
-__device__ __forceinline__ void pair_stage(const PairItem &it, const float *__restrict__ u, unsigned sU)
-{
-    const long long n3 = (long long)it.n * it.n * it.n;
-    const float *ud = u + it.grid_off + it.d * n3;
-    const bool vec = ((it.sx | it.n | it.ex) & 3) == 0 && ((reinterpret_cast<uintptr_t>(ud)) & 15) == 0;
-    const int n = it.n, bzu = it.ez + 4, byu = it.ey + 4;
-    if (vec) {
-        box_cols(it, bzu, byu, it.ex >> 2, [&](int lz, int ly, int gz, int gy, int qx) {
-            cp_async16(sU + 4u * (unsigned)(lz * it.ppu + ly * it.pxu + 2 + 4 * qx),
-                       ud + (gz * n + gy) * n + it.sx + 4 * qx);
-        });
-        box_cols(it, bzu, byu, 2, [&](int lz, int ly, int gz, int gy, int e) {
-            cp_async8(sU + 4u * (unsigned)(lz * it.ppu + ly * it.pxu + (e ? it.ex + 2 : 0)),
-                      ud + (gz * n + gy) * n + wrap1(e ? it.sx + it.ex : it.sx - 2, n));
-        });
-    } else {
-        box_cols(it, bzu, byu, it.ex + 4, [&](int lz, int ly, int gz, int gy, int qx) {
-            cp_async4(sU + 4u * (unsigned)(lz * it.ppu + ly * it.pxu + qx),
-                      ud + (gz * n + gy) * n + wrap1(it.sx - 2 + qx, n));
-        });
-    }
-}
-
-// The first own unit of this thread in an item (node id, binning record,
-// F_d), loaded ahead of the item's node loop.
-struct PairUnit {
-    int node;
-    float4 rec;
-    float f;
-};
-
-// The first unit of this thread for an item's node loop; thread 0 also puts
-// into s_part[0] an upper bound of sum |F_d| over the item's own nodes: the
-// placement's atomic float sum, whose rounding in any order is below
-// (n - 1) 2^-24 of the exact sum for n nodes, times 1.0001 + n 2^-23.
-__device__ __forceinline__ PairUnit pair_first(const PairItem &it, const DevWork &w, const float *__restrict__ F,
-                                               long long N, float *s_part)
-{
-    const int beg = w.own_off[(long long)it.tile * kOwnSub3], end = w.own_off[(long long)(it.tile + 1) * kOwnSub3];
-    PairUnit u0{0, make_float4(0.f, 0.f, 0.f, 0.f), 0.f};
-    const int q = beg + (int)threadIdx.x;
-    if (q < end) {
-        u0.node = w.own_nodes[q];
-        u0.rec = w.own_rec[q];
-        u0.f = F[it.d * N + u0.node];
-    }
-    if (threadIdx.x == 0)
-        s_part[0] = w.tile_fsum[3LL * it.tile + it.d] * (1.0001f + (float)(end - beg) * 1.1920929e-7f);
-    return u0;
-}
-
-// Fixed-point scale of a (tile, lattice) accumulator: the largest power of
-// two that keeps wmax * sum_k |g_k| (wmax = 1/8 for Peskin, sd the density
-// factor) below the int32 range, from the per-warp partial sums of |F_d|.
-// Every thread computes the same value.
-__device__ __forceinline__ float halo_scale(const float *s_part, int nw, float sd)
-{
-    float tot = 0.f;
-    for (int q = 0; q < nw; ++q)
-        tot += s_part[q];
-    const float bound = tot * sd * 0.125f * 1.0001f;
+    const float bound = fsum * (1.0001f + (float)(it.end - it.beg) * 1.1920929e-7f) * it.sd * 0.125f;
     float scale = 1.f;
     if (bound > 0.f && isfinite(bound)) {
         int e = (int)floorf(log2f(FixedPoint<int>::kRange / bound));
@@ -1282,462 +1127,377 @@ __device__ __forceinline__ float halo_scale(const float *s_part, int nw, float s
     return scale;
 }
 
-template <bool INTERP, bool AB2 = false>
-__global__ void __launch_bounds__(256, 5) spread_halo_kernel(DevBatch b, DevGrid g, DevWork w,
-                                                          const float *__restrict__ x,
-                                                          const float *__restrict__ F, float *__restrict__ f,
-                                                          int density, const float *__restrict__ u,
-                                                          float *__restrict__ v, const float *__restrict__ vp,
-                                                          float *__restrict__ xn, float dt)
+// Copies the velocity box of an item's lattice into U asynchronously: quads
+// where the grid's quads are aligned, else single values. bt: box thread.
+template <int W>
+__device__ __forceinline__ void tile_stage(const TileItem &it, const float *__restrict__ u, unsigned sU, int bt)
 {
-    const int lattice = -1;   // every lattice in one launch
-    static_assert(INTERP || !AB2, "the position update needs the fused interpolation");
-    extern __shared__ __align__(16) unsigned char halo_smem[];
-    int *acc = reinterpret_cast<int *>(halo_smem);
-    const unsigned sacc = smem_u32(acc);
-    __shared__ float s_part[8];
-    __shared__ long long s_red[8];
-    // the next item, published by thread 0 in slot (k + 1) & 1 during the
-    // flush of item k and read after that flush's barrier (two slots: the
-    // slot of item k is rewritten only during item k + 1's flush)
-    __shared__ int s_item[2];
-    __shared__ TileInfo s_ti[2];
-    __shared__ BoxDev s_B[2];
-    const long long N = b.N;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int i = threadIdx.x; i < halo_ints(g.max_edge); i += blockDim.x)
-        acc[i] = 0;
-    if (threadIdx.x == 0)
-        staged_next(g, w, lattice, s_item[0], s_ti[0], s_B[0]);
-    __syncthreads();
-    for (int slot = 0;; slot ^= 1) {
-        if (s_item[slot] < 0)
-            break;
-        // item fields for the node loop, from the shared slot (it stays
-        // valid until the next item's flush; the flush re-reads it)
-        const int tile = s_item[slot] / 3, d = s_item[slot] - 3 * tile;
-        const int sx = s_ti[slot].start[0], sy = s_ti[slot].start[1], sz = s_ti[slot].start[2];
-        const int bx = s_ti[slot].edge[0] + 2 * kHaloX, by = s_ti[slot].edge[1] + 2 * kHaloYZ,
-                  bz = s_ti[slot].edge[2] + 2 * kHaloYZ;
-        const int px = halo_px(bx), pp = halo_pp(by, px);
-        const int n = s_B[slot].n;
-        const float sd = density ? s_B[slot].scale_f : 1.f;
-        const int beg = w.own_off[(long long)tile * kOwnSub3], end = w.own_off[(long long)(tile + 1) * kOwnSub3];
-        // fixed-point scale from sum |F_d| over the own nodes
-        float gs = 0.f;
-        for (int q = beg + threadIdx.x; q < end; q += blockDim.x)
-            gs += fabsf(F[d * N + w.own_nodes[q]]);
+    using S = TileShape<W>;
+    const int n = it.n, nn = n * n;
+    const float *ud = u + it.grid_off + (long long)it.d * nn * n;
+    if (tile_vec(it, ud)) {
+        const int y0 = bt / S::kColumn;
+        bt -= y0 * S::kColumn;
+        const int zl = bt & 3, yl = (bt >> 2) & 1, line = bt >> 3, gx = line % S::NX, lz = 4 * (line / S::NX) + zl;
+        if (line >= S::NX * S::NZ || 4 * gx >= it.ex + 8 || lz >= it.ez + 4)
+            return;
+        const float *src = ud + wrap1(it.sz - 2 + lz, n) * nn + wrap1(it.sx - 4 + 4 * gx, n);
+        const unsigned dst = sU + 16u * (unsigned)bt;   // (line, yl, zl) in this order
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            gs += __shfl_down_sync(0xffffffffu, gs, o);
-        if (lane == 0)
-            s_part[wid] = gs;
-        __syncthreads();
-        const float gsc = sd * halo_scale(s_part, nw, sd);
-        for (int q = beg + threadIdx.x; q < end; q += blockDim.x) {
-            const int node = w.own_nodes[q];
-            const float4 rec = w.own_rec[q];   // written by the binning
-            const float gq = F[d * N + node] * gsc;
-            const unsigned pk = __float_as_uint(rec.w);
-            const float fr[3] = {rec.x, rec.y, rec.z};
-            float ph[3][4];
-            int l0[3];
-            bool inside = true;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                // lattice d sits at the cell coordinate, the other two half a
-                // cell lower: s = t - 1/2 has floor(t) - 1 and fraction r + 1/2
-                // below r = 1/2, so the stencil starts 2 (not 1) cells below
-                const int c = (int)((pk >> (8 * a)) & 255u);   // cell within the tile
-                int sh = -1;
-                float r = fr[a];
-                if (a != d) {
-                    const bool low = r < 0.5f;
-                    r = low ? r + 0.5f : r - 0.5f;
-                    sh = low ? -2 : -1;
-                }
-                peskin_frac(r, ph[a]);
-                l0[a] = c + (a == 0 ? kHaloX : kHaloYZ) + sh;
-                const int lim = (a == 0 ? bx : (a == 1 ? by : bz)) - 4;
-                inside = inside && (unsigned)l0[a] <= (unsigned)lim;
-            }
-            if (!inside) {   // a record inconsistent with this tile: never expected
-                status_add(w.status, ST_DOMAIN, 1);
+        for (int k = 0; k < S::NY / S::kYStep; ++k) {
+            const int yb = y0 + k * S::kYStep;
+            const int ly = 2 * yb + yl;
+            if (ly < it.ey + 4)
+                cp_async16(dst + 128u * (unsigned)(yb * S::NZ * S::NX), src + wrap1(it.sy - 2 + ly, n) * n);
+        }
+    } else {
+        // lanes take the 32 cells of a line, warps the lines
+        const int xl = bt & 3, zl = (bt >> 2) & 3, yl = (bt >> 4) & 1;
+        for (int c = bt >> 5; c < S::NX * S::NY; c += S::kBoxThreads / 32) {
+            const int yb = c / S::NX, gx = c - yb * S::NX, ly = 2 * yb + yl, lx = 4 * gx + xl;
+            if (lx < 2 || lx >= it.ex + 6 || ly >= it.ey + 4)
                 continue;
-            }
-            const unsigned base = sacc + 4u * (unsigned)(l0[2] * pp + l0[1] * px + l0[0]);
-            if constexpr (INTERP) {
-                // grid indices of the stencil (the buffer origin is the tile
-                // start minus the halo); per z plane the 16 gathers are issued
-                // before that plane's shared-memory reductions
-                const float *ud = u + s_B[slot].grid_off + (long long)d * n * n * n;
-                int gx[4], gy[4], gz[4];
+            const float *row = ud + wrap1(it.sy - 2 + ly, n) * n + wrap1(it.sx - 4 + lx, n);
+            const unsigned dst = sU + 4u * (unsigned)(bt & 31) + 128u * (unsigned)(yb * S::NZ * S::NX + gx);
 #pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    gx[m] = wrap_near(sx - kHaloX + l0[0] + m, n);
-                    gy[m] = wrap_near(sy - kHaloYZ + l0[1] + m, n);
-                    gz[m] = wrap_near(sz - kHaloYZ + l0[2] + m, n);
-                }
-                float out = 0.f;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    float uv[4][4];
-#pragma unroll
-                    for (int bb = 0; bb < 4; ++bb) {
-                        const float *row = ud + (gz[c] * n + gy[bb]) * n;
-#pragma unroll
-                        for (int a = 0; a < 4; ++a)
-                            uv[bb][a] = __ldg(row + gx[a]);
-                    }
-                    const float wz = ph[2][c] * gq;
-#pragma unroll
-                    for (int bb = 0; bb < 4; ++bb) {
-                        const float wyz = ph[1][bb] * wz;
-                        const unsigned row = base + 4u * (unsigned)(c * pp + bb * px);
-#pragma unroll
-                        for (int a = 0; a < 4; ++a)
-                            red_shared_add(row + 4u * a, __float2int_rn(ph[0][a] * wyz));
-                    }
-                    float accz = 0.f;
-#pragma unroll
-                    for (int bb = 0; bb < 4; ++bb) {
-                        float accy = ph[0][0] * uv[bb][0];
-#pragma unroll
-                        for (int a = 1; a < 4; ++a)
-                            accy += ph[0][a] * uv[bb][a];
-                        accz += ph[1][bb] * accy;
-                    }
-                    out += ph[2][c] * accz;
-                }
-                v[d * N + node] = out;
-                if constexpr (AB2) {
-                    const long long i = d * N + node;
-                    xn[i] = ab2_value(x[i], out, vp[i], dt);
-                }
-            } else {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const float wz = ph[2][c] * gq;
-#pragma unroll
-                    for (int bb = 0; bb < 4; ++bb) {
-                        const float wyz = ph[1][bb] * wz;
-                        const unsigned row = base + 4u * (unsigned)(c * pp + bb * px);
-#pragma unroll
-                        for (int a = 0; a < 4; ++a)
-                            red_shared_add(row + 4u * a, __float2int_rn(ph[0][a] * wyz));
-                    }
-                }
+            for (int zb = 0; zb < S::NZ; ++zb) {
+                const int lz = 4 * zb + zl;
+                if (lz < it.ez + 4)
+                    cp_async4(dst + 128u * (unsigned)(zb * S::NX), row + wrap1(it.sz - 2 + lz, n) * nn);
             }
         }
-        __syncthreads();
-        // flush: every non-zero sum is added to the grid with an L2 reduction
-        // (quads of x when rows are 16-byte aligned) and cleared; meanwhile
-        // thread 0 fetches the next item
-        if (threadIdx.x == 0)
-            staged_next(g, w, lattice, s_item[slot ^ 1], s_ti[slot ^ 1], s_B[slot ^ 1]);
-        const PairItem cur = pair_item(s_item[slot], s_ti[slot], s_B[slot], density);
-        const float scale = halo_scale(s_part, nw, cur.sd);   // the node loop's scale, recomputed
-        {
-            const long long n3 = (long long)n * n * n;
-            float *fd = f + cur.grid_off + d * n3;
-            const bool vec = ((sx | n | bx) & 3) == 0 && ((reinterpret_cast<uintptr_t>(fd)) & 15) == 0;
-            const float inv = 1.f / scale;
-            long long qsum = 0;
-            unsigned touched = 0;
-            if (vec) {
-                pair_rows(cur, bx >> 2, lane, wid, nw, [&](int lz, int ly, int gz, int gy, int qx) {
-                    int4 *sp = reinterpret_cast<int4 *>(acc + lz * pp + ly * px + 4 * qx);
-                    const int4 qv = *sp;
-                    if ((qv.x | qv.y | qv.z | qv.w) != 0) {
-                        *sp = make_int4(0, 0, 0, 0);
-                        const int x0 = 4 * qx;
-                        red_add_v4(fd + (gz * n + gy) * n + wrap1(sx - kHaloX + x0, n), (float)qv.x * inv,
-                                   (float)qv.y * inv, (float)qv.z * inv, (float)qv.w * inv);
-                        qsum += (long long)qv.x + (long long)qv.y + (long long)qv.z + (long long)qv.w;
-                        if ((unsigned)(lz - kHaloYZ) < (unsigned)cur.ez && (unsigned)(ly - kHaloYZ) < (unsigned)cur.ey &&
-                            (unsigned)(x0 - kHaloX) < (unsigned)cur.ex)
-                            touched += (qv.x != 0) + (qv.y != 0) + (qv.z != 0) + (qv.w != 0);
-                    }
-                });
-            } else {
-                pair_rows(cur, bx, lane, wid, nw, [&](int lz, int ly, int gz, int gy, int qx) {
-                    int *sp = acc + lz * pp + ly * px + qx;
-                    const int qv = *sp;
-                    if (qv != 0) {
-                        *sp = 0;
-                        red_add(fd + (gz * n + gy) * n + wrap1(sx - kHaloX + qx, n), (float)qv * inv);
-                        qsum += qv;
-                        touched += (unsigned)(lz - kHaloYZ) < (unsigned)cur.ez &&
-                                   (unsigned)(ly - kHaloYZ) < (unsigned)cur.ey && (unsigned)(qx - kHaloX) < (unsigned)cur.ex;
-                    }
-                });
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                qsum += __shfl_down_sync(0xffffffffu, qsum, o);
-                touched += __shfl_down_sync(0xffffffffu, touched, o);
-            }
-            if (lane == 0) {
-                s_red[wid] = qsum;
-                if (touched)
-                    status_add(w.status, ST_TOUCHED, touched);
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            long long vsum = 0;
-            for (int q = 0; q < nw; ++q)
-                vsum += s_red[q];
-            // exact: |vsum| < 2^53, 1/scale a power of two
-            w.red_tile[3LL * tile + d] = (double)vsum * (double)(1.f / scale) / cur.box_scale;
-        }
-        // s_part and s_red are written again only after the next barriers
     }
 }
 
-// ---------------------------------- spread + interp, FP32, staged velocity
-// IFEM_SCATTER_ATOMIC, Peskin kernel, with the interpolation of the same
-// step fused (Algorithm steps 2 and 4 use the same stencil weights of the
-// same positions). Work item = (tile, lattice) over the tiles with own
-// nodes (own_scatter_kernel), taken from a global counter; thread 0 fetches
-// the next item during the node loop. Two shared buffers per CTA: U, the
-// velocity values the item's stencils read (2 cells around the tile), and A,
-// the spread accumulator over the tile plus the halo of spread_halo_kernel
-// (int32 fixed point, scale from the bound sum_k |g_k| / 8 over the tile's
-// own nodes, from the sum of |F_d| that the binning's placement keeps per
-// tile). Per item:
-//   1. node loop, one (node, lattice) unit per thread: the Peskin weights
-//      of the unit; interpolation from U (64 shared-memory loads at
-//      immediate offsets, v_d = sum phi u_d in z-y-x order), then the 64
-//      contributions added to A with shared-memory reductions;
-//   2. the next item's velocity box is copied into U (cp.async), each
-//      thread's first unit of it loaded and its scale bound read, while A
-//      is flushed: every non-zero value is added to the
-//      grid with an L2 reduction (halos of neighbouring tiles combine there)
-//      and cleared.
-// CTAs are small (kStagedThreads): an item has a few hundred units, and the
-// last round of the node loop leaves threads idle at the barrier; with
-// fewer threads per CTA that round is a smaller share of the item.
-// AB2 = true also writes the position update of Eq. Bashforth_eqn from each
-// interpolated velocity, out of place. lattice >= 0 restricts the launch to
-// that lattice's items (see staged_next).
-template <bool AB2>
-__global__ void __launch_bounds__(kStagedThreads, 3) transfer_staged_kernel(DevBatch b, DevGrid g, DevWork w,
-                                                                     const float *__restrict__ x,
-                                                                     const float *__restrict__ F,
-                                                                     float *__restrict__ f, int density,
-                                                                     const float *__restrict__ u,
-                                                                     float *__restrict__ v,
-                                                                     const float *__restrict__ vp,
-                                                                     float *__restrict__ xn, float dt,
-                                                                     int lattice)
+// Adds every non-zero value of A to the grid and clears it; returns the exact
+// integer sum and counts the non-zero values inside the tile itself. Two
+// neighbours' sum fits 32 bits: their weights add up to at most 0.22, against
+// the 1/8 of the bound. bt: box thread.
+template <int W>
+__device__ __forceinline__ long long tile_flush(const TileItem &it, float *__restrict__ f, int4 *A, float inv,
+                                                int bt, unsigned &touched)
 {
-    extern __shared__ __align__(16) unsigned char pair_smem[];
-    __shared__ float s_part[kStagedThreads / 32];
-    __shared__ long long s_red[kStagedThreads / 32];
-    // the next item, published by thread 0 in slot (k + 1) & 1 during the
-    // node loop of item k and read after that loop's barrier (two slots: the
-    // slot of item k is rewritten only during item k + 1's node loop)
-    __shared__ int s_item[2];
-    __shared__ TileInfo s_ti[2];
-    __shared__ BoxDev s_B[2];
-    const int ubytes = pair_u_bytes(g.max_edge), buf = pair_buf_bytes(g.max_edge);
-    const float *U = reinterpret_cast<const float *>(pair_smem + 8);
-    int *A = reinterpret_cast<int *>(pair_smem + ubytes);
-    const unsigned sU = smem_u32(pair_smem) + 8u, sA = smem_u32(pair_smem) + (unsigned)ubytes;
+    using S = TileShape<W>;
+    const int n = it.n;
+    float *fd = f + it.grid_off + (long long)it.d * n * n * n;
+    const bool vec = tile_vec(it, fd);
+    const int y0 = bt / S::kColumn;
+    bt -= y0 * S::kColumn;
+    const int zl = bt & 3, yl = (bt >> 2) & 1, line = bt >> 3, gx = line % S::NX, lz = 4 * (line / S::NX) + zl;
+    if (line >= S::NX * S::NZ || lz >= it.ez + 4)   // cells beyond the box stay zero
+        return 0;
+    float *plane = fd + wrap1(it.sz - 2 + lz, n) * n * n;
+    const bool in_z = (unsigned)(lz - 2) < (unsigned)it.ez;
+    const bool in_xz = in_z && (unsigned)(4 * gx - 4) < (unsigned)it.ex;
+    if (vec)
+        plane += wrap1(it.sx - 4 + 4 * gx, n);
+    long long qsum = 0;
+    A += bt;
+#pragma unroll
+    for (int k = 0; k < S::NY / S::kYStep; ++k) {
+        const int yb = y0 + k * S::kYStep;
+        const int4 q = A[8 * yb * S::NZ * S::NX];
+        if ((q.x | q.y | q.z | q.w) == 0)
+            continue;
+        A[8 * yb * S::NZ * S::NX] = make_int4(0, 0, 0, 0);
+        const int ly = 2 * yb + yl;
+        float *row = plane + wrap1(it.sy - 2 + ly, n) * n;
+        qsum += (long long)(q.x + q.y) + (long long)(q.z + q.w);
+        const float v0 = (float)q.x * inv, v1 = (float)q.y * inv, v2 = (float)q.z * inv, v3 = (float)q.w * inv;
+        const bool in_y = (unsigned)(ly - 2) < (unsigned)it.ey;
+        if (vec) {
+            red_add_v4(row, v0, v1, v2, v3);
+            if (in_xz && in_y)
+                touched += min((unsigned)q.x, 1u) + min((unsigned)q.y, 1u) + min((unsigned)q.z, 1u) +
+                           min((unsigned)q.w, 1u);
+        } else {
+            const int qc[4] = {q.x, q.y, q.z, q.w};
+            const float vc[4] = {v0, v1, v2, v3};
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (qc[c] != 0) {
+                    red_add(row + wrap1(it.sx - 4 + 4 * gx + c, n), vc[c]);
+                    touched += in_z && in_y && (unsigned)(4 * gx + c - 4) < (unsigned)it.ex;
+                }
+        }
+    }
+    return qsum;
+}
+
+// A node's binning record, force and id (see own_scatter_kernel).
+struct TileUnit {
+    float4 rec, fn;
+};
+__device__ __forceinline__ TileUnit tile_unit(const DevWork &w, int q)
+{
+    const float4 *r = w.own_rec + 2LL * q;
+    return TileUnit{r[0], r[1]};
+}
+
+// p[t] = p[(r + t) & 3]
+__device__ __forceinline__ void rotate4(float p[4], int r)
+{
+    const bool one = r & 1, two = r & 2;
+    const float a0 = one ? p[1] : p[0], a1 = one ? p[2] : p[1], a2 = one ? p[3] : p[2], a3 = one ? p[0] : p[3];
+    p[0] = two ? a2 : a0;
+    p[1] = two ? a3 : a1;
+    p[2] = two ? a0 : a2;
+    p[3] = two ? a1 : a3;
+}
+
+// One (node, lattice) unit: spreads into A, interpolates from U, or both
+// (gq: the node's force times the item's fixed-point scale).
+template <int W, bool SPREAD, bool INTERP, bool AB2>
+__device__ __forceinline__ void tile_node(const TileItem &cur, const DevWork &w, const TileUnit &un, float gsc,
+                                          const unsigned char *U, unsigned sA, float *__restrict__ v,
+                                          const float *__restrict__ x, const float *__restrict__ vp,
+                                          float *__restrict__ xn, float dt, long long N)
+{
+    using S = TileShape<W>;
+    const int lane = threadIdx.x & 31, d = cur.d;
+    const int node = __float_as_int(un.fn.w);
+    const float gq = (d == 0 ? un.fn.x : (d == 1 ? un.fn.y : un.fn.z)) * gsc;
+    const unsigned pk = __float_as_uint(un.rec.w);
+    const float fr[3] = {un.rec.x, un.rec.y, un.rec.z};
+    float ph[3][4];
+    int l0[3];
+    bool inside = true;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        // lattice d sits at the cell coordinate, the other two half a
+        // cell lower: s = t - 1/2 has floor(t) - 1 and fraction r + 1/2
+        // below r = 1/2, so the stencil starts 2 (not 1) cells below
+        const int c = (int)((pk >> (8 * ax)) & 255u);   // cell within the tile
+        int sh = 1;
+        float r = fr[ax];
+        if (ax != d) {
+            const bool low = r < 0.5f;
+            r = low ? r + 0.5f : r - 0.5f;
+            sh = low ? 0 : 1;
+        }
+        peskin_frac(r, ph[ax]);
+        l0[ax] = c + sh;   // first stencil cell, from 2 cells below the tile
+        inside = inside && l0[ax] <= (ax == 0 ? cur.ex : (ax == 1 ? cur.ey : cur.ez));
+    }
+    if (!inside) {   // a record inconsistent with this tile: never expected
+        status_add(w.status, ST_DOMAIN, 1);
+        return;
+    }
+    // byte offsets of the lane's points in step order (see above)
+    int xo[4], zo[4], yo[2];
+    const int xl = (l0[0] + 2) & 3, xq = (l0[0] + 2) >> 2;   // the box starts 4 cells below in x
+    const int zl = l0[2] & 3, zq = l0[2] >> 2, yl = l0[1] & 1, yq = l0[1] >> 1;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const int tx = (lane + t) & 3, tz = ((lane >> 2) + t) & 3;
+        xo[t] = 4 * tx + 128 * (xq + (tx < xl));
+        zo[t] = 16 * tz + 128 * S::NX * (zq + (tz < zl));
+    }
+    const int ry = ((lane >> 4) ^ yl) & 1;   // y offset (0 or 1) of step t2 = 0
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+        yo[t] = 64 * ((lane >> 4) ^ t) + 128 * S::NX * S::NZ * (yq + (yl & (ry ^ t)));
+    rotate4(ph[0], lane - xl);
+    rotate4(ph[2], (lane >> 2) - zl);
+    const float py0 = ry ? ph[1][1] : ph[1][0], py2 = ry ? ph[1][3] : ph[1][2];
+    const float py1 = ry ? ph[1][0] : ph[1][1], py3 = ry ? ph[1][2] : ph[1][3];
+    constexpr int kRow2 = 128 * S::NX * S::NZ;   // two y rows further
+    float p[4];
+#pragma unroll
+    for (int t0 = 0; t0 < 4; ++t0) {
+        float qz[4];
+        const float gx = ph[0][t0] * gq;
+#pragma unroll
+        for (int t1 = 0; t1 < 4; ++t1) {
+            const int oa = xo[t0] + zo[t1] + yo[0], ob = xo[t0] + zo[t1] + yo[1];
+            if constexpr (INTERP) {
+                const float ua = *reinterpret_cast<const float *>(U + oa);
+                const float uc = *reinterpret_cast<const float *>(U + oa + kRow2);
+                const float ub = *reinterpret_cast<const float *>(U + ob);
+                const float ue = *reinterpret_cast<const float *>(U + ob + kRow2);
+                const float sa = fmaf(py2, uc, __fmul_rn(py0, ua)), sb = fmaf(py3, ue, __fmul_rn(py1, ub));
+                qz[t1] = __fmul_rn(ph[2][t1], __fadd_rn(sa, sb));
+            }
+            if constexpr (SPREAD) {
+                const float gz = gx * ph[2][t1];
+                const unsigned aa = sA + (unsigned)oa, ab = sA + (unsigned)ob;
+                red_shared_add_nc(aa, __float2int_rn(py0 * gz));
+                red_shared_add_nc(aa + kRow2, __float2int_rn(py2 * gz));
+                red_shared_add_nc(ab, __float2int_rn(py1 * gz));
+                red_shared_add_nc(ab + kRow2, __float2int_rn(py3 * gz));
+            }
+        }
+        if constexpr (INTERP)
+            p[t0] = __fmul_rn(ph[0][t0], __fadd_rn(__fadd_rn(qz[0], qz[2]), __fadd_rn(qz[1], qz[3])));
+    }
+    if constexpr (INTERP) {
+        const float out = __fadd_rn(__fadd_rn(p[0], p[2]), __fadd_rn(p[1], p[3]));
+        const long long i = d * N + node;
+        v[i] = out;
+        if constexpr (AB2)
+            xn[i] = ab2_value(x[i], out, vp[i], dt);
+    }
+}
+
+template <int W, bool SPREAD, bool INTERP, bool AB2>
+__global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
+    transfer_tile_kernel(DevBatch b, DevWork w, const float *__restrict__ x, float *__restrict__ f, int density,
+                         const float *__restrict__ u, float *__restrict__ v, const float *__restrict__ vp,
+                         float *__restrict__ xn, float dt, int lattice)
+{
+    static_assert(INTERP || !AB2, "the position update needs the interpolation");
+    using S = TileShape<W>;
+    constexpr int kBox = 4 * S::kWords, kBoxWarps = S::kBoxThreads / 32, kRing = 8;
+    extern __shared__ __align__(128) unsigned char tile_smem[];
+    unsigned char *U = tile_smem, *A = tile_smem + (INTERP ? 2 * kBox : 0);
+    __shared__ long long s_red[2][kBoxWarps];
+    __shared__ float s_scale[4];   // fixed-point scale of item i in i % 4
+    // items i of this CTA in slot i % kRing: lattice (-1: none) and descriptor
+    __shared__ int s_d[kRing];
+    __shared__ __align__(16) TileDesc s_desc[kRing];
     const long long N = b.N;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const bool box = threadIdx.x < S::kBoxThreads;
+    const int bt = threadIdx.x, nt = (int)threadIdx.x - S::kBoxThreads;
     // a kernel launched after this one with programmatic serialization (the
     // next lattice of the same step, which reads nothing this one writes) may
     // start at once: the grid is sized to be resident, so its CTAs take the
     // SMs that this grid's CTAs leave when the items run out
     asm volatile("griddepcontrol.launch_dependents;");
-    for (int i = threadIdx.x; i < buf / 16; i += blockDim.x)
-        reinterpret_cast<int4 *>(A)[i] = make_int4(0, 0, 0, 0);
-    if (threadIdx.x == 0)
-        staged_next(g, w, lattice, s_item[0], s_ti[0], s_B[0]);
-    __syncthreads();
-    if (s_item[0] < 0)
-        return;
-    PairUnit u0;
-    {
-        const PairItem first = pair_item(s_item[0], s_ti[0], s_B[0], density);
-        pair_stage(first, u, sU);
-        u0 = pair_first(first, w, F, N, s_part);
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    for (int slot = 0;; slot ^= 1) {
-        const PairItem cur = pair_item(s_item[slot], s_ti[slot], s_B[slot], density);
-        // fixed-point scale of this item from the bound of sum |F_d|
-        float scale = 1.f;
-        {
-            const float bound = s_part[0] * cur.sd * 0.125f;
-            if (bound > 0.f && isfinite(bound)) {
-                int e = (int)floorf(log2f(FixedPoint<int>::kRange / bound));
-                e = e > 120 ? 120 : (e < -120 ? -120 : e);
-                scale = exp2f((float)e);
-            }
-        }
-        const float gsc = cur.sd * scale;
-        if (threadIdx.x == 0)
-            staged_next(g, w, lattice, s_item[slot ^ 1], s_ti[slot ^ 1], s_B[slot ^ 1]);
-        const int d = cur.d;
-        const int beg = w.own_off[(long long)cur.tile * kOwnSub3];
-        const int end = w.own_off[(long long)(cur.tile + 1) * kOwnSub3];
-        const int px = cur.px, pp = cur.pp;
-        // 1. node loop: one (node, lattice) unit per thread; the first unit
-        // was loaded ahead (pair_first)
-        PairUnit un = u0;
-        for (int q = beg + (int)threadIdx.x; q < end;) {
-            const int node = un.node;
-            const float4 rec = un.rec;   // written by the binning
-            const float gq = un.f * gsc;
-            q += blockDim.x;
-            if (q < end) {
-                un.node = w.own_nodes[q];
-                un.rec = w.own_rec[q];
-                un.f = F[d * N + un.node];
-            }
-            const unsigned pk = __float_as_uint(rec.w);
-            const float fr[3] = {rec.x, rec.y, rec.z};
-            float ph[3][4];
-            int l0[3];
-            bool inside = true;
-#pragma unroll
-            for (int ax = 0; ax < 3; ++ax) {
-                // lattice d sits at the cell coordinate, the other two half a
-                // cell lower: s = t - 1/2 has floor(t) - 1 and fraction r + 1/2
-                // below r = 1/2, so the stencil starts 2 (not 1) cells below
-                const int c = (int)((pk >> (8 * ax)) & 255u);   // cell within the tile
-                int sh = -1;
-                float r = fr[ax];
-                if (ax != d) {
-                    const bool low = r < 0.5f;
-                    r = low ? r + 0.5f : r - 0.5f;
-                    sh = low ? -2 : -1;
-                }
-                peskin_frac(r, ph[ax]);
-                l0[ax] = c + (ax == 0 ? kHaloX : kHaloYZ) + sh;
-                // inside both boxes: in x within [2, ex + 2] of A (U starts
-                // 2 cells later), in y and z within [0, e]
-                const int lo = ax == 0 ? 2 : 0;
-                const int hi = ax == 0 ? cur.ex + 2 : (ax == 1 ? cur.ey : cur.ez);
-                inside = inside && (unsigned)(l0[ax] - lo) <= (unsigned)(hi - lo);
-            }
-            if (!inside) {   // a record inconsistent with this tile: never expected
-                status_add(w.status, ST_DOMAIN, 1);
-                continue;
-            }
-            const int off = l0[2] * pp + l0[1] * px + l0[0];
-            const float *ub = U + (l0[2] * cur.ppu + l0[1] * cur.pxu + (l0[0] - 2));
-            const unsigned ab = sA + 4u * (unsigned)off;
-            // interpolation first (all 64 loads can be in flight), then the
-            // 64 fixed-point reductions; the reductions carry no compiler
-            // memory clobber, so they do not hold back the loads of the next
-            // unit (the barrier after the loop orders them)
-            float out = 0.f;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                float accz = 0.f;
-#pragma unroll
-                for (int bb = 0; bb < 4; ++bb) {
-                    const float *row = ub + c * cur.ppu + bb * cur.pxu;
-                    float accy = ph[0][0] * row[0];
-#pragma unroll
-                    for (int a = 1; a < 4; ++a)
-                        accy += ph[0][a] * row[a];
-                    accz += ph[1][bb] * accy;
-                }
-                out += ph[2][c] * accz;
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const float wz = ph[2][c] * gq;
-#pragma unroll
-                for (int bb = 0; bb < 4; ++bb) {
-                    const float wyz = ph[1][bb] * wz;
-                    const unsigned arow = ab + 4u * (unsigned)(c * pp + bb * px);
-#pragma unroll
-                    for (int a = 0; a < 4; ++a)
-                        red_shared_add_nc(arow + 4u * a, __float2int_rn(ph[0][a] * wyz));
-                }
-            }
-            v[d * N + node] = out;
-            if constexpr (AB2) {
-                const long long i = d * N + node;
-                xn[i] = ab2_value(x[i], out, vp[i], dt);
-            }
-        }
-        asm volatile("" ::: "memory");   // the reductions above stay before the barrier
-        __syncthreads();   // A complete, U free, the next item published
-
-        // 2. next item's velocities and scale bound; flush of A
-        const int next = s_item[slot ^ 1];
-        if (next >= 0) {
-            const PairItem nxt = pair_item(next, s_ti[slot ^ 1], s_B[slot ^ 1], density);
-            pair_stage(nxt, u, sU);
-            u0 = pair_first(nxt, w, F, N, s_part);
-        }
-        {
-            const long long n3 = (long long)cur.n * cur.n * cur.n;
-            float *fd = f + cur.grid_off + d * n3;
-            const bool vec = ((cur.sx | cur.n | cur.bx) & 3) == 0 && ((reinterpret_cast<uintptr_t>(fd)) & 15) == 0;
-            const float inv = 1.f / scale;
-            const int n = cur.n;
-            long long qsum = 0;
-            unsigned touched = 0;
-            if (vec) {
-                box_cols(cur, cur.bz, cur.by, cur.bx >> 2, [&](int lz, int ly, int gz, int gy, int qx) {
-                    int4 *sp = reinterpret_cast<int4 *>(A + lz * pp + ly * px + 4 * qx);
-                    const int4 qv = *sp;
-                    if ((qv.x | qv.y | qv.z | qv.w) != 0) {
-                        *sp = make_int4(0, 0, 0, 0);
-                        const int x0 = 4 * qx;
-                        red_add_v4(fd + (gz * n + gy) * n + wrap1(cur.sx - kHaloX + x0, n), (float)qv.x * inv,
-                                   (float)qv.y * inv, (float)qv.z * inv, (float)qv.w * inv);
-                        qsum += (long long)qv.x + (long long)qv.y + (long long)qv.z + (long long)qv.w;
-                        if ((unsigned)(lz - kHaloYZ) < (unsigned)cur.ez && (unsigned)(ly - kHaloYZ) < (unsigned)cur.ey &&
-                            (unsigned)(x0 - kHaloX) < (unsigned)cur.ex)
-                            touched += (qv.x != 0) + (qv.y != 0) + (qv.z != 0) + (qv.w != 0);
-                    }
-                });
-            } else {
-                box_cols(cur, cur.bz, cur.by, cur.bx, [&](int lz, int ly, int gz, int gy, int qx) {
-                    int *sp = A + lz * pp + ly * px + qx;
-                    const int qv = *sp;
-                    if (qv != 0) {
-                        *sp = 0;
-                        red_add(fd + (gz * n + gy) * n + wrap1(cur.sx - kHaloX + qx, n), (float)qv * inv);
-                        qsum += qv;
-                        touched += (unsigned)(lz - kHaloYZ) < (unsigned)cur.ez &&
-                                   (unsigned)(ly - kHaloYZ) < (unsigned)cur.ey && (unsigned)(qx - kHaloX) < (unsigned)cur.ex;
-                    }
-                });
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                qsum += __shfl_down_sync(0xffffffffu, qsum, o);
-                touched += __shfl_down_sync(0xffffffffu, touched, o);
-            }
-            if (lane == 0) {
-                s_red[wid] = qsum;
-                if (touched)
-                    status_add(w.status, ST_TOUCHED, touched);
-            }
-        }
+    if constexpr (SPREAD)
+        for (int i = threadIdx.x; i < 2 * kBox / 16; i += S::kThreads)
+            reinterpret_cast<int4 *>(A)[i] = make_int4(0, 0, 0, 0);
+    // the first box warp takes the items: the counter's answer for item i + 3
+    // travels during item i, the descriptor of item i + 2 is copied during it
+    const int n_items = w.counters[3] * (lattice < 0 ? 3 : 1);
+    int *counter = tile_counter(w, lattice);
+    int ahead = 0;   // its lane 0: number of the next item to be copied
+    auto fetch = [&](int it, int i) {
+        const int q = lattice < 0 ? it / 3 : it, slot = i % kRing;
+        if (lane == 0)
+            s_d[slot] = it < n_items ? (lattice < 0 ? it - 3 * q : lattice) : -1;
+        if (lane < (int)sizeof(TileDesc) / 16 && it < n_items)
+            cp_async16(smem_u32(&s_desc[slot]) + 16u * lane,
+                       reinterpret_cast<const char *>(w.tile_desc + q) + 16 * lane);
+    };
+    if (threadIdx.x < 32) {
+        int first = 0;
+        if (lane == 0)
+            first = atomicAdd(counter, 3);   // the first items of a CTA are neighbours
+        first = __shfl_sync(0xffffffffu, first, 0);
+        ahead = first + 2;
+        fetch(first, 0);
+        fetch(first + 1, 1);
         cp_async_wait_all();
-        __syncthreads();   // U holds the next box, A is clear, s_part and s_red are written
-        if (threadIdx.x == 0) {
-            long long vsum = 0;
-            for (int q = 0; q < nw; ++q)
-                vsum += s_red[q];
-            // exact: |vsum| < 2^53, 1/scale a power of two
-            w.red_tile[3LL * cur.tile + d] = (double)vsum * (double)(1.f / scale) / cur.box_scale;
+    }
+    __syncthreads();
+    if (s_d[0] < 0)
+        return;
+    if (INTERP && box) {
+        tile_stage<W>(tile_item(s_desc[0], s_d[0], density), u, smem_u32(U), bt);
+        cp_async_wait_all();
+    }
+    // a node thread's first unit of the next item
+    TileUnit un{};
+    auto unit_ahead = [&](int i) {
+        if (s_d[i % kRing] < 0)
+            return;
+        const TileDesc &td = s_desc[i % kRing];
+        if (td.beg + nt < td.end)
+            un = tile_unit(w, td.beg + nt);
+    };
+    auto put_scale = [&](int i, float fsum) {   // one thread
+        s_scale[i & 3] = tile_scale(tile_item(s_desc[i % kRing], s_d[i % kRing], density), fsum);
+    };
+    auto get_fsum = [&](int i) { return w.tile_fsum[3LL * s_desc[i % kRing].tile + s_d[i % kRing]]; };
+    auto write_sum = [&](int i) {   // one thread: the exact sum of a flushed item, times h^3
+        const TileDesc &td = s_desc[i % kRing];
+        long long vsum = 0;
+#pragma unroll
+        for (int q = 0; q < kBoxWarps; ++q)
+            vsum += s_red[i & 1][q];
+        // |vsum| < 2^53, the scale a power of two: one rounding
+        w.red_tile[3LL * td.tile + s_d[i % kRing]] = (double)vsum * (double)(1.f / s_scale[i & 3]) * td.h3;
+    };
+    if (!box)
+        unit_ahead(0);
+    if (SPREAD && threadIdx.x == 32)
+        put_scale(0, get_fsum(0));
+    __syncthreads();
+    unsigned touched = 0;
+    int i = 0;
+    for (;; ++i) {
+        const bool valid = s_d[i % kRing] >= 0;
+        if (!box) {
+            if (SPREAD && i > 1 && nt == S::kNodeThreads - 1)
+                write_sum(i - 2);
+            if (valid) {
+                const TileItem cur = tile_item(s_desc[i % kRing], s_d[i % kRing], density);
+                const float gsc = SPREAD ? cur.sd * s_scale[i & 3] : 0.f;
+                TileUnit mine = un;
+                int q = cur.beg + nt;
+                const bool more = q + S::kNodeThreads < cur.end;
+                if (more)
+                    un = tile_unit(w, q + S::kNodeThreads);
+                else
+                    unit_ahead(i + 1);
+                const unsigned char *Ui = U + (i & 1) * kBox;
+                const unsigned sA = smem_u32(A) + (unsigned)((i & 1) * kBox);
+                if (q < cur.end)
+                    tile_node<W, SPREAD, INTERP, AB2>(cur, w, mine, gsc, Ui, sA, v, x, vp, xn, dt, N);
+                if (more) {
+#pragma unroll 1
+                    for (q += S::kNodeThreads; q < cur.end; q += S::kNodeThreads) {
+                        mine = un;
+                        if (q + S::kNodeThreads < cur.end)
+                            un = tile_unit(w, q + S::kNodeThreads);
+                        tile_node<W, SPREAD, INTERP, AB2>(cur, w, mine, gsc, Ui, sA, v, x, vp, xn, dt, N);
+                    }
+                    unit_ahead(i + 1);
+                }
+            }
+        } else {
+            const bool scales = SPREAD && threadIdx.x == 32 && s_d[(i + 1) % kRing] >= 0;
+            const float fsum = scales ? get_fsum(i + 1) : 0.f;
+            if (valid) {
+                if (threadIdx.x < 32) {
+                    fetch(__shfl_sync(0xffffffffu, ahead, 0), i + 2);
+                    if (lane == 0)
+                        ahead = atomicAdd(counter, 1);
+                }
+                if (INTERP && s_d[(i + 1) % kRing] >= 0)
+                    tile_stage<W>(tile_item(s_desc[(i + 1) % kRing], s_d[(i + 1) % kRing], density), u,
+                                  smem_u32(U) + (unsigned)(((i + 1) & 1) * kBox), bt);
+            }
+            if (SPREAD && i > 0) {
+                // this flush's sum is written during the next item, by a node
+                // thread; the next item's scale by a thread of the second warp
+                const TileItem old = tile_item(s_desc[(i - 1) % kRing], s_d[(i - 1) % kRing], density);
+                long long qsum = tile_flush<W>(old, f, reinterpret_cast<int4 *>(A + ((i - 1) & 1) * kBox),
+                                               1.f / s_scale[(i - 1) & 3], bt, touched);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+                    qsum += __shfl_down_sync(0xffffffffu, qsum, o);
+                if (lane == 0)
+                    s_red[(i - 1) & 1][threadIdx.x >> 5] = qsum;
+            }
+            if (scales)
+                put_scale(i + 1, fsum);
+            cp_async_wait_all();
         }
-        if (next < 0)
+        asm volatile("" ::: "memory");   // the node threads' reductions stay before the barrier
+        __syncthreads();
+        if (!valid)
             break;
-        // s_red and s_part are written again only after the next node loop's barrier
+    }
+    if constexpr (SPREAD) {
+        if (threadIdx.x == 0)
+            write_sum(i - 1);   // i >= 1: the CTA had an item
+        // one update per warp and launch: one per warp and item, all on this
+        // one word, took longer than the rest of the kernel
+        touched = __reduce_add_sync(0xffffffffu, touched);
+        if (lane == 0)
+            status_add(w.status, ST_TOUCHED, touched);
     }
 }
 
