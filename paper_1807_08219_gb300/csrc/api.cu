@@ -372,34 +372,31 @@ static int nodal_upload(ifem_ctx ctx, ifem_tmpl t, int nv, const int32_t *el, co
             const int e = code >> 2, c = code & 3;
             const size_t at = (size_t)base[k / 32] + 32 * s + k % 32;
             if (nv == 3) {
-                const int j = pairs[order[s]].x, l = pairs[order[s]].y;
-                double e1[3], e2[3], e3[3];
-                sub(j, k, e1);
-                sub(l, k, e2);
-                sub(l, j, e3);
-                id[2 * at] = (unsigned short)j;
-                id[2 * at + 1] = (unsigned short)l;
-                r[at] = make_float4((float)dot(e1, e2), (float)-dot(e1, e3), (float)dot(e2, e3),
-                                    (float)(0.5 / ref[5 * (size_t)e + 4]));
+                const int32_t *v = el + 3 * (size_t)e;
+                id[2 * at] = (unsigned short)(pairs[order[s]].x | c << kNodBits);
+                id[2 * at + 1] = (unsigned short)pairs[order[s]].y;
+                float d[3];
+                for (int i = 0; i < 3; ++i) {
+                    double p[3], q[3];
+                    sub(v[(i + 1) % 3], v[i], p);
+                    sub(v[(i + 2) % 3], v[i], q);
+                    d[i] = (float)dot(p, q);
+                }
+                r[at] = make_float4(d[0], d[1], d[2], (float)(0.5 / ref[5 * (size_t)e + 4]));
             } else {
-                // even permutations that bring corner c to the front
-                static const int rot[4][4] = {{0, 1, 2, 3}, {1, 0, 3, 2}, {2, 0, 1, 3}, {3, 0, 2, 1}};
                 const double *g = ref.data() + 10 * (size_t)e;   // grad N_1..3, V0
-                double gr[4][3], sum[3];
+                double gr[4][3];
                 for (int a = 0; a < 3; ++a) {
                     for (int v = 1; v < 4; ++v)
                         gr[v][a] = g[3 * (v - 1) + a];
                     gr[0][a] = -((gr[1][a] + gr[2][a]) + gr[3][a]);
                 }
-                double h[3];
-                for (int a = 0; a < 3; ++a)
-                    sum[a] = -gr[c][a];   // the other three corners' sum
-                for (int v = 1; v < 4; ++v) {
-                    id[4 * at + v - 1] = (unsigned short)el[4 * (size_t)e + rot[c][v]];
-                    h[v - 1] = g[9] * dot(gr[rot[c][v]], sum);
+                float h[4];
+                for (int v = 0; v < 4; ++v) {
+                    id[4 * at + v] = (unsigned short)(el[4 * (size_t)e + v] | (v == 0 ? c << kNodBits : 0));
+                    h[v] = (float)(v == c ? 1.0 / (6.0 * g[9]) : -(g[9] * dot(gr[v], gr[c])));
                 }
-                id[4 * at + 3] = c == 0;
-                r[at] = make_float4((float)h[0], (float)h[1], (float)h[2], (float)(1.0 / (6.0 * g[9])));
+                r[at] = make_float4(h[0], h[1], h[2], h[3]);
             }
         }
     }
@@ -806,13 +803,23 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
     w.cand_cap = 8 * N;
     CK(alloc((void **)&ws.d_boxes, sizeof(BoxDev) * boxes.size()));
     CK(cudaMemcpy(ws.d_boxes, boxes.data(), sizeof(BoxDev) * boxes.size(), cudaMemcpyHostToDevice));
-    CK(alloc((void **)&w.cand_count, sizeof(int) * (nt + 1)));
+    // what a binning clears, in one piece: the spread's per-tile sums (by a
+    // spread's binning only), then the counters and counts
+    const size_t zero_ints = kCounters + (size_t)(no + 1) + (use_halo(ctx) ? 4 * nt : nt + 1);
+    CK(alloc((void **)&w.red_tile, sizeof(double) * 3 * (size_t)nt + sizeof(int) * zero_ints));
+    CK(cudaMemset(w.red_tile, 0, sizeof(double) * 3 * (size_t)nt));
+    w.counters = reinterpret_cast<int *>(w.red_tile + 3 * nt);
+    w.zero_bytes = sizeof(int) * zero_ints;
+    w.own_count = w.counters + kCounters;
     CK(alloc((void **)&w.cand_off, sizeof(int) * (nt + 1)));
     CK(alloc((void **)&w.cand_cursor, sizeof(int) * (nt + 1)));
     CK(alloc((void **)&w.cand_nodes, sizeof(int) * (size_t)w.cand_cap));
-    CK(alloc((void **)&w.own_count, sizeof(int) * (no + 1 + 4 * nt)));
-    w.own_flag = w.own_count + no + 1;
-    w.tile_fsum = reinterpret_cast<float *>(w.own_flag + nt);
+    if (use_halo(ctx)) {
+        w.own_flag = w.own_count + no + 1;
+        w.tile_fsum = reinterpret_cast<float *>(w.own_flag + nt);
+    } else {
+        w.cand_count = w.own_count + no + 1;
+    }
     CK(alloc((void **)&w.own_cursor, sizeof(int) * (no + 1)));
     if (!use_halo(ctx)) {
         CK(alloc((void **)&w.own_off, sizeof(int) * (no + 1)));
@@ -827,10 +834,7 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
     if (ctx->cfg.precision == IFEM_FP64 && ctx->cfg.kernel == IFEM_KERNEL_PESKIN4)
         CK(alloc((void **)&w.wtab, sizeof(DetW) * (size_t)std::max<long long>(N, 1)));
     CK(alloc((void **)&w.active, sizeof(int) * (nt + 1)));
-    CK(alloc((void **)&w.counters, sizeof(int) * kCounters));
     CK(alloc((void **)&w.scan_blocks, sizeof(int) * 2 * (nb + 1)));
-    CK(alloc((void **)&w.red_tile, sizeof(double) * 3 * (nt + 1)));
-    CK(cudaMemset(w.red_tile, 0, sizeof(double) * 3 * (nt + 1)));
     w.elem_buf = b->d_elem_buf;
     w.bend_buf = b->d_bend_buf;
     w.status = ctx->d_status;
@@ -926,26 +930,32 @@ static int do_forces(ifem_ctx ctx, ifem_batch b, const void *x, void *F, const v
 // stages other than BIN_ALL: the FP32 halo path only. F (FP32 halo path):
 // the placement also sums |F| per tile, which the tile transfer's spread
 // requires (every spread follows a binning given the same forces).
+// sums: a spread follows (the binning clears its per-tile sums, which an
+// interpolation's binning leaves for ifem_reduce).
 static int do_bin(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, void *stream, int stages = BIN_ALL,
-                  const void *F = nullptr)
+                  const void *F = nullptr, int sums = 1)
 {
     int rc = ws_ensure(ctx, b, g, ctx->tile);
     if (rc != IFEM_OK)
         return rc;
     TransferArgs a = transfer_args(ctx, b, x, F, nullptr, nullptr, nullptr, 0, stream);
+    a.clear_sums = sums;
     cudaError_t e = ctx->cfg.precision == IFEM_FP64 ? launch_bin_f64(a, 1, 1, stages)
                                                     : launch_bin_f32(a, 0, !use_halo(ctx), stages);
     return launch_rc(ctx, e, "binning");
 }
 
-static int do_spread(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, const void *F, void *f, int flags,
-                     void *stream)
+// f = 0 where the flags ask for it, before a spread into it.
+static int do_overwrite(ifem_ctx ctx, ifem_grid g, void *f, int flags, void *stream)
 {
-    if (flags & IFEM_SPREAD_OVERWRITE) {
-        cudaError_t e = cudaMemsetAsync(f, 0, (size_t)g->total * real_size(ctx), (cudaStream_t)stream);
-        if (e != cudaSuccess)
-            return launch_rc(ctx, e, "spread overwrite");
-    }
+    if (!(flags & IFEM_SPREAD_OVERWRITE))
+        return IFEM_OK;
+    return launch_rc(ctx, cudaMemsetAsync(f, 0, (size_t)g->total * real_size(ctx), (cudaStream_t)stream),
+                     "spread overwrite");
+}
+
+static int do_spread(ifem_ctx ctx, ifem_batch b, const void *x, const void *F, void *f, int flags, void *stream)
+{
     TransferArgs a = transfer_args(ctx, b, x, F, nullptr, f, nullptr, flags, stream);
     cudaError_t e = ctx->cfg.precision == IFEM_FP64 ? launch_spread_f64(a) : launch_spread_f32(a);
     return launch_rc(ctx, e, "spread");
@@ -955,20 +965,14 @@ static int do_spread(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
 // halo-scatter configuration only): one launch per step for both transfers.
 // With xn given the launch also writes the position update from the
 // velocities it gathers (xn = x + dt (3/2 v - 1/2 vp)).
-static int do_spread_interp(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, const void *F, const void *u,
-                            void *f, void *v, int flags, void *stream, const void *vp = nullptr,
-                            void *xn = nullptr, double dt = 0.0, int lattice = -1, int pdl = 0)
+static int do_spread_interp(ifem_ctx ctx, ifem_batch b, const void *x, const void *F, const void *u, void *f,
+                            void *v, int flags, void *stream, const void *vp = nullptr, void *xn = nullptr,
+                            double dt = 0.0, int lattice = -1, int pdl = 0)
 {
-    if (flags & IFEM_SPREAD_OVERWRITE) {
-        cudaError_t e = cudaMemsetAsync(f, 0, (size_t)g->total * real_size(ctx), (cudaStream_t)stream);
-        if (e != cudaSuccess)
-            return launch_rc(ctx, e, "spread overwrite");
-    }
     TransferArgs a = transfer_args(ctx, b, x, F, u, f, v, flags, stream);
     a.vp = vp;
     a.xn = xn;
     a.dt = dt;
-    a.binned = 1;   // every caller bins just before, on this stream or one joined to it
     a.lattice = lattice;
     a.pdl = pdl;
     return launch_rc(ctx, launch_spread_f32(a), "spread + interpolate");
@@ -1053,9 +1057,10 @@ extern "C" int ifem_spread(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *
         return fail(ctx, IFEM_ERR_ARG, "spread: null array or grid");
     if (flags & ~(IFEM_SPREAD_FORCE | IFEM_SPREAD_OVERWRITE))
         return fail(ctx, IFEM_ERR_ARG, "spread: unknown flags");
-    if ((rc = do_bin(ctx, b, g, x, stream, BIN_ALL, F)) != IFEM_OK)
+    if ((rc = do_overwrite(ctx, g, f, flags, stream)) != IFEM_OK ||
+        (rc = do_bin(ctx, b, g, x, stream, BIN_ALL, F)) != IFEM_OK)
         return rc;
-    return do_spread(ctx, b, g, x, F, f, flags, stream);
+    return do_spread(ctx, b, x, F, f, flags, stream);
 }
 
 static LagrangeArgs lagrange_args(ifem_ctx ctx, ifem_batch b, void *x, void *stream)
@@ -1136,9 +1141,10 @@ extern "C" int ifem_indicator_source(ifem_ctx ctx, ifem_batch b, ifem_grid g, co
                                                     : launch_area_normals_f32(db, x, nA, (cudaStream_t)stream);
     if ((rc = launch_rc(ctx, e, "indicator_source")) != IFEM_OK)
         return rc;
-    if ((rc = do_bin(ctx, b, g, x, stream, BIN_ALL, nA)) != IFEM_OK)
+    if ((rc = do_overwrite(ctx, g, G, flags, stream)) != IFEM_OK ||
+        (rc = do_bin(ctx, b, g, x, stream, BIN_ALL, nA)) != IFEM_OK)
         return rc;
-    return do_spread(ctx, b, g, x, nA, G, flags, stream);
+    return do_spread(ctx, b, x, nA, G, flags, stream);
 }
 
 extern "C" int ifem_interpolate_cc(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *field, int ncomp,
@@ -1199,7 +1205,7 @@ extern "C" int ifem_interpolate(ifem_ctx ctx, ifem_batch b, ifem_grid g, const v
         return fail(ctx, IFEM_ERR_ARG, "interpolate: null array or grid");
     if (ctx->cfg.precision == IFEM_FP32) {
         // the FP32 kernel walks the nodes in tile order (locality)
-        if ((rc = do_bin(ctx, b, g, x, stream)) != IFEM_OK)
+        if ((rc = do_bin(ctx, b, g, x, stream, BIN_ALL, nullptr, 0)) != IFEM_OK)
             return rc;
     } else if ((rc = ws_ensure(ctx, b, g, ctx->tile)) != IFEM_OK) {
         return rc;
@@ -1275,13 +1281,15 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
         if ((rc = do_bin(ctx, b, g, x, stream, BIN_ALL, F)) != IFEM_OK)
             return rc;
         mark(ctx, 2, stream);
+        if ((rc = do_overwrite(ctx, g, f, flags, stream)) != IFEM_OK)
+            return rc;
         ctx->ev_fused = use_halo(ctx);
         if (ctx->ev_fused) {
-            if ((rc = do_spread_interp(ctx, b, g, x, F, u, f, v, flags, stream, vp, xn, dt)) != IFEM_OK)
+            if ((rc = do_spread_interp(ctx, b, x, F, u, f, v, flags, stream, vp, xn, dt)) != IFEM_OK)
                 return rc;
             mark(ctx, 3, stream);
         } else {
-            if ((rc = do_spread(ctx, b, g, x, F, f, flags, stream)) != IFEM_OK)
+            if ((rc = do_spread(ctx, b, x, F, f, flags, stream)) != IFEM_OK)
                 return rc;
             mark(ctx, 3, stream);
             if ((rc = do_interp(ctx, b, u, x, v, stream, 1)) != IFEM_OK)
@@ -1313,7 +1321,7 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
     //   s:    bin ----------------------- wait(forces) spread  wait(interp) sums of v, boxes  wait(sums)
     //   aux0: forces --/ wait(bin) sums of x, F ---------------------------------------------/
     //   aux1:       wait(bin) interp [ab2] -------/
-    // With the fused spread + interpolation [+ ab2] the aux1 branch is absent,
+    // With the fused spread + interpolation [+ ab2] aux1 carries no interpolation,
     // and the binning's placement, which sums |F| per tile for the transfer's
     // fixed-point scales, waits for the forces:
     //   s:    count, scan -- wait(forces) placement  spread+interp  sums of v, boxes  wait(sums)
@@ -1327,6 +1335,25 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
     //   aux1:                                           wait(v) copy v ------------------/
     const bool fused = use_halo(ctx) != 0;
     if ((rc = ws_ensure(ctx, b, g, ctx->tile)) != IFEM_OK)
+        return rc;
+    // the clearing of f runs on aux1 beside the host copies, or beside the
+    // forces and the binning: then launched after the forces, whose blocks
+    // leave it room (before them it takes every SM and they wait)
+    const bool clear_f = (flags & IFEM_SPREAD_OVERWRITE) != 0;
+    if ((e = cudaEventRecord(ctx->fork[0], s)) != cudaSuccess)
+        return launch_rc(ctx, e, "step_coupling fork");
+    auto start_clear = [&]() -> int {
+        if (!clear_f)
+            return IFEM_OK;
+        cudaError_t ce = cudaStreamWaitEvent(ctx->aux[1], ctx->fork[0], 0);
+        if (ce != cudaSuccess)
+            return launch_rc(ctx, ce, "step_coupling fork");
+        int crc = do_overwrite(ctx, g, f, flags, ctx->aux[1]);
+        if (crc != IFEM_OK)
+            return crc;
+        return launch_rc(ctx, cudaEventRecord(ctx->fork[10], ctx->aux[1]), "step_coupling fork");
+    };
+    if (io && (rc = start_clear()) != IFEM_OK)
         return rc;
     const bool split = io && forces_ranged_ok(ctx, b);
     if (split) {
@@ -1350,14 +1377,15 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
         if ((rc = do_forces(ctx, b, x, F, nullptr, 0, ctx->aux[0], h, ni - h)) != IFEM_OK)
             return rc;
     } else {
-        if (io && (e = copy_nodes_in(ctx, b, io->x_host, const_cast<void *>(x), 0, b->N, s)) != cudaSuccess)
+        // (with host arrays the event moves behind the copy; the clearing has been forked already)
+        if (io && ((e = copy_nodes_in(ctx, b, io->x_host, const_cast<void *>(x), 0, b->N, s)) != cudaSuccess ||
+                   (e = cudaEventRecord(ctx->fork[0], s)) != cudaSuccess))
             return launch_rc(ctx, e, "step_coupling_host: copy in");
-        e = cudaEventRecord(ctx->fork[0], s);
-        if (e == cudaSuccess)
-            e = cudaStreamWaitEvent(ctx->aux[0], ctx->fork[0], 0);
-        if (e != cudaSuccess)
+        if ((e = cudaStreamWaitEvent(ctx->aux[0], ctx->fork[0], 0)) != cudaSuccess)
             return launch_rc(ctx, e, "step_coupling fork");
         if ((rc = do_forces(ctx, b, x, F, nullptr, 0, ctx->aux[0])) != IFEM_OK)
+            return rc;
+        if (!io && (rc = start_clear()) != IFEM_OK)
             return rc;
     }
     if ((e = cudaEventRecord(ctx->fork[1], ctx->aux[0])) != cudaSuccess)
@@ -1394,19 +1422,21 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
         if ((e = cudaEventRecord(ctx->fork[3], ctx->aux[1])) != cudaSuccess)
             return launch_rc(ctx, e, "step_coupling fork");
     }
-    if ((e = cudaStreamWaitEvent(s, ctx->fork[1], 0)) != cudaSuccess)
+    if (!fused && (e = cudaStreamWaitEvent(s, ctx->fork[1], 0)) != cudaSuccess)
         return launch_rc(ctx, e, "step_coupling join");
-    // with host arrays and the staged transfer, one launch per lattice: row d
+    if (clear_f && (e = cudaStreamWaitEvent(s, ctx->fork[10], 0)) != cudaSuccess)
+        return launch_rc(ctx, e, "step_coupling join");
+    // with host arrays and the fused transfer, one launch per lattice: row d
     // of v goes back to the host on aux1 as soon as lattice d's launch ends,
     // beside the later lattices. Lattices 1 and 2 are launched with
     // programmatic serialization: their CTAs start on the SMs that the
     // previous lattice's CTAs leave when its items run out (they read nothing
     // it writes), so the three launches share one tail instead of one each
-    const bool v_rows = fused && io && node_bytes > 0 && !(flags & IFEM_SPREAD_OVERWRITE);
+    const bool v_rows = fused && io && node_bytes > 0;
     if (v_rows) {
         const size_t row = node_bytes / 3;
         for (int d = 0; d < 3; ++d) {
-            if ((rc = do_spread_interp(ctx, b, g, x, F, u, f, v, flags, stream, vp, xn, dt, d, d > 0)) != IFEM_OK)
+            if ((rc = do_spread_interp(ctx, b, x, F, u, f, v, flags, stream, vp, xn, dt, d, d > 0)) != IFEM_OK)
                 return rc;
             if ((e = cudaEventRecord(ctx->fork[d == 2 ? 7 : 2 + d], s)) == cudaSuccess &&
                 (e = cudaStreamWaitEvent(ctx->aux[1], ctx->fork[d == 2 ? 7 : 2 + d], 0)) == cudaSuccess)
@@ -1422,10 +1452,10 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
         if ((e = cudaEventRecord(ctx->fork[8], ctx->aux[1])) != cudaSuccess)
             return launch_rc(ctx, e, "step_coupling_host: copy out");
     } else if (fused) {
-        if ((rc = do_spread_interp(ctx, b, g, x, F, u, f, v, flags, stream, vp, xn, dt)) != IFEM_OK)
+        if ((rc = do_spread_interp(ctx, b, x, F, u, f, v, flags, stream, vp, xn, dt)) != IFEM_OK)
             return rc;
     } else {
-        if ((rc = do_spread(ctx, b, g, x, F, f, flags, stream)) != IFEM_OK)
+        if ((rc = do_spread(ctx, b, x, F, f, flags, stream)) != IFEM_OK)
             return rc;
         if ((e = cudaStreamWaitEvent(s, ctx->fork[3], 0)) != cudaSuccess)
             return launch_rc(ctx, e, "step_coupling join");
@@ -1576,8 +1606,8 @@ static int autotune(ifem_ctx ctx, ifem_batch b, const void *x, void *stream)
             if ((rc = do_bin(ctx, b, g, x, stream, BIN_ALL, F)) == IFEM_OK) {
                 // the transfer launches the step will use (fused where it fuses)
                 if (use_halo(ctx))
-                    rc = do_spread_interp(ctx, b, g, x, F, u, f, v, 0, stream);
-                else if ((rc = do_spread(ctx, b, g, x, F, f, 0, stream)) == IFEM_OK)
+                    rc = do_spread_interp(ctx, b, x, F, u, f, v, 0, stream);
+                else if ((rc = do_spread(ctx, b, x, F, f, 0, stream)) == IFEM_OK)
                     rc = do_interp(ctx, b, u, x, v, stream);
             }
             cudaEventRecord(e1, s);

@@ -26,6 +26,8 @@ constexpr int kMaxCtaSmemBytes = 227 * 1024;   // opt-in dynamic shared memory o
 // FP32 nodal force kernel: a float4 (position, mean curvature) of shared
 // memory per template node, 16-bit node ids
 constexpr int kNodalMaxNodes = kMaxCtaSmemBytes / 16;
+constexpr int kNodBits = 14, kNodMask = (1 << kNodBits) - 1;   // node id bits in the first id of an incidence
+static_assert(kNodalMaxNodes <= kNodMask + 1, "node ids of the nodal kernel");
 __host__ __device__ inline size_t nodal_smem_bytes(int n_nodes) { return (size_t)n_nodes * sizeof(float4); }
 constexpr int kStatusWords = 8;
 enum StatusWord {
@@ -53,8 +55,10 @@ struct TmplDev {
     // FP32 nodal force kernel (templates of at most kNodalMaxNodes nodes, else null): incidences in
     // slices of 32 nodes, slot s of node k at nod_off[k / 32] + 32 s + k % 32
     const int *nod_off;
-    const float4 *nod_ref;   // membranes: reference edge dots r_k, r_j, r_l and 1/(2 A0); solids: h1, h2, h3, 1/(6 V0)
-    const void *nod_idx;     // membranes: ushort2 (j, l); solids: ushort4 (1, 2, 3, 1 at the tet's first corner)
+    const float4 *nod_ref;   // membranes: reference edge dots r_a, r_b, r_c and 1/(2 A0); solids: h of the
+                             // corners, 1/(6 V0) in the node's own place
+    const void *nod_idx;     // membranes: ushort2 (j, l); solids: ushort4, the corners; the node's corner
+                             // number in the bits of the first id above kNodBits
     double mu, C, kb, c0, lam;
     float mu_f, half_muD_f, kb_f, kH0_f, half_lam_f;   // FP32 nodal kernel: mu, C mu/2, kb, -c0/2, lam/2
 };
@@ -137,7 +141,8 @@ struct DevWork {
     int *cand_cursor;   // n_tiles
     int *cand_nodes;    // pair list: node id per (tile, node) candidate pair
     long long cand_cap;
-    int *own_count;     // per (tile, 4^3 sub-block): n_tiles * kOwnSub3 + 1, then own_flag, tile_fsum
+    int *own_count;     // per (tile, 4^3 sub-block): n_tiles * kOwnSub3 + 1; in one piece with red_tile
+                        // and counters before it and, after it, own_flag and tile_fsum or cand_count
     int *own_flag;      // n_tiles (FP32 halo path): 1 where the tile owns a node
     float *tile_fsum;   // 3 per tile (FP32 halo path): sum of |F_d| over the tile's own nodes, from the
                         // placement when it is given the forces (the fused transfer's fixed-point scale)
@@ -159,7 +164,8 @@ struct DevWork {
     int *scan_blocks;   // block partial sums for the tile scan
     void *elem_buf;     // per element nodal forces (12 reals per element)
     void *bend_buf;     // per node bending scratch (A, kH, n[3], lap) 6 reals
-    double *red_tile;   // per active tile: 3 FP64 sums of added spread values
+    double *red_tile;   // per tile: 3 FP64 sums of added spread values
+    size_t zero_bytes;  // counters and what follows them (cleared by every binning)
     DetW *wtab;         // N entries (FP64 Peskin only, else null): written by the binning
     unsigned long long *status;  // kStatusWords
 };
@@ -376,8 +382,7 @@ struct TransferArgs {
     int n_sm;
     int acc64;        // FP32 spread: 64-bit (1) or 32-bit (0) fixed-point accumulators
     int halo;         // FP32 Peskin, IFEM_SCATTER_ATOMIC: the tile transfer over own lists
-    int binned;       // the binning of this step ran just before on the same stream (own tiles
-                      // listed, work counter and per-tile sums cleared)
+    int clear_sums;   // binning: a spread follows, clear its per-tile sums too
     int lattice;      // tile transfer: -1 all three lattices, else that lattice only
     int pdl;          // tile transfer: may start before the previous kernel in the stream ends
     int use_wtab;     // FP64 Peskin interpolation: read the stencils the binning of x tabulated

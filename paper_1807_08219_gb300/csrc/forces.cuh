@@ -764,32 +764,40 @@ __global__ void bend_pass2_kernel(DevBatch b, const real *__restrict__ x, const 
 // a fixed order, so there are no atomics, no element buffer and no second
 // pass over the elements, and the result is the same from run to run. Each
 // element is evaluated once per corner (3 or 4 times), in forms that need only
-// the corner's own row:
+// the corner's own row. What an element gives its corners adds up to zero in
+// exact arithmetic; the forms below keep that under rounding (every corner
+// computes the same bits of what it shares with another, and takes them with
+// the opposite sign), as an element evaluated once does: errors that do not
+// cancel between neighbours show up in the spread field, where the forces
+// themselves mostly do (one red cell: error of the field 2.1e-6 without, 1.1e-6
+// with, relative L2).
 //
-// Membranes, triangle (k, j, l) at node k, e1 = x_j - x_k, e2 = x_l - x_k: the
-// laws depend on the metric G = [e_a . e_b] alone. With R the metric of the
-// reference triangle, m = Dm^-1 and m m^T = R^-1, det m^2 = 1/det R:
-//   I1 = tr(G R^-1), I2 = det G / det R,
-//   F_k = A0 [e1 e2] (a R^-1 + b adj(G)/det R) (1, 1)^T
-//       = (w/2) [e1 (a r_l + b d_l) + e2 (a r_j + b d_j)],   w = 1/(2 A0),
-// d_k = e1.e2, d_j = |e1|^2 - d_k, d_l = |e2|^2 - d_k the edge dots at the
-// three corners, r_* the same of the reference triangle, and S^ = a I + b adj C^:
-//   NH a = mu, b = -mu/I2^2;  Skalak a = mu (I1 - 1), b = (C mu/2)(I2 - 1) - mu;
-//   I1 = w^2 (|e1|^2 r_l + |e2|^2 r_j + (d_j + d_l) r_k), I2 = w^2 |e1 x e2|^2.
-// These are the dots and the cross product that the bending operators take.
+// Membranes, triangle (a, b, c), the node k one of its corners, (k, j, l) in
+// orientation order: the laws depend on the metric alone. With d_i the edge dot
+// at corner i (d_k = (x_j - x_k).(x_l - x_k)) and r_i the same of the reference
+// triangle, w = 1/(2 A0), 4 A^2 = |e x e'|^2:
+//   I1 = w^2 (d_a (r_b + r_c) + d_b (r_c + r_a) + d_c (r_a + r_b)), I2 = 4 A^2 w^2,
+//   F_k = s_l (x_j - x_k) + s_j (x_l - x_k), s_i = (w/2) (a r_i + b d_i),
+// S^ = a I + b adj C^: NH a = mu, b = -mu/I2^2; Skalak a = mu (I1 - 1), b = (C
+// mu/2)(I2 - 1) - mu. s_i belongs to the edge opposite corner i: both of its
+// ends take the same s_i (the dots do not depend on the corner they are computed
+// from, I1 and 4 A^2 are evaluated in the triangle's own order), times edge
+// vectors of opposite sign (a fused multiply-add: exact up to the sum).
 //
-// Solids, tet (0, 1, 2, 3) rotated (an even permutation) so that the node is
-// corner 0, d_c = x_c - x_0: with P = mu F + beta cof F, beta = (lam/2 (J^2 - 1)
-// - mu)/J, and sum_c cof(F) grad N_c = (d2 x d3 + d3 x d1 + d1 x d2)/(6 V0) =: n/(6 V0),
-//   F_0 = mu (h1 d1 + h2 d2 + h3 d3) + (beta/6) n,  h_c = V0 grad N_c . sum grad N,
-//   J = d1 . (d2 x d3)/(6 V0).
+// Solids, tet (0, 1, 2, 3), y_i = x_i - x_0: with P = mu F + beta cof F, beta =
+// (lam/2 (J^2 - 1) - mu)/J, J = y_1 . (y_2 x y_3)/(6 V0),
+//   F_k = sum_m mu h_km (x_m - x_k) + (beta/6) n_k,  h_km = -V0 grad N_k . grad N_m,
+//   n_1, n_2, n_3 = -y_2 x y_3, -y_3 x y_1, -y_1 x y_2, n_0 = -(n_1 + n_2 + n_3):
+// h_km is the same number at both ends, y, J, beta and the n are evaluated in
+// the tet's own order by every corner.
 //
 // Layout: incidences in slices of 32 nodes (a warp), slot by slot, so that a
-// warp's reads are consecutive: reference values (float4: r_k, r_j, r_l, w or
-// h1, h2, h3, 1/(6 V0)) and the other corners as 16-bit node ids. A closed
-// surface's incidences are ordered as a fan around the node (l of one triangle
-// is j of the next), so a triangle takes one new position and edge instead of
-// two.
+// warp's reads are consecutive: reference values and 16-bit node ids, the
+// node's corner number in the top bits. Membranes: r_a, r_b, r_c, w and (j, l);
+// a closed surface's incidences are ordered as a fan around the node (l of one
+// triangle is j of the next), so a triangle takes one new position instead of
+// two. Solids: the h of the four corners with 1/(6 V0) in the node's own place
+// (where x_m - x_k is 0) and the four corners.
 //
 // Bending (Meyer et al. 2003) per incident triangle: 2A = |e1 x e2| from one
 // rsqrt, cotangents d/2A. The corner-angle sum enters only through 2 pi -
@@ -799,31 +807,35 @@ __global__ void bend_pass2_kernel(DevBatch b, const real *__restrict__ x, const 
 struct RingF {
     float fn[3], q, inv2A, dk, dj, dl;   // q = |e1 x e2|^2
 };
-__device__ __forceinline__ void ring_edge_f32(const float4 xk, const float4 xj, float e[3], float &l)
+__device__ __forceinline__ float dot3f(const float a[3], const float b[3])
 {
-    e[0] = xj.x - xk.x;
-    e[1] = xj.y - xk.y;
-    e[2] = xj.z - xk.z;
-    l = e[0] * e[0] + e[1] * e[1] + e[2] * e[2];
+    return fmaf(a[2], b[2], fmaf(a[1], b[1], __fmul_rn(a[0], b[0])));
 }
-__device__ __forceinline__ void ring_tri_f32(const float e1[3], float l1, const float e2[3], float l2, RingF &t)
+__device__ __forceinline__ void edge_f32(const float4 p, const float4 q, float e[3])   // q - p
+{
+    e[0] = q.x - p.x;
+    e[1] = q.y - p.y;
+    e[2] = q.z - p.z;
+}
+// e1 = x_j - x_k, e2 = x_l - x_k and e3 = x_l - x_j. Each component of a dot is
+// a product of the same two coordinate differences from whichever corner it is
+// computed, up to two signs that cancel: the dots are the same bits at all three.
+__device__ __forceinline__ void ring_tri_f32(const float e1[3], const float e2[3], const float e3[3], RingF &t)
 {
     t.fn[0] = e1[1] * e2[2] - e1[2] * e2[1];
     t.fn[1] = e1[2] * e2[0] - e1[0] * e2[2];
     t.fn[2] = e1[0] * e2[1] - e1[1] * e2[0];
     t.q = t.fn[0] * t.fn[0] + t.fn[1] * t.fn[1] + t.fn[2] * t.fn[2];
     t.inv2A = rsqrtf(t.q);
-    t.dk = e1[0] * e2[0] + e1[1] * e2[1] + e1[2] * e2[2];
-    t.dj = l1 - t.dk;
-    t.dl = l2 - t.dk;
+    t.dk = dot3f(e1, e2);
+    t.dj = -dot3f(e1, e3);
+    t.dl = dot3f(e2, e3);
 }
 
 // Pass 1 of a membrane node: elastic force and, with BEND, the part of the
 // bending force that needs no neighbour's curvature, 2 kb * 2 (kH - kH0)
 // (kH^2 - kG + kH0 kH) A n; kH receives the mean curvature. Along a fan the
-// second edge of a triangle is the first of the next: its vector and length
-// are kept, and the two triangles' coefficients are added before they
-// multiply it.
+// second edge of a triangle is the first of the next: its vector is kept.
 template <bool BEND>
 __device__ __forceinline__ void nodal_membrane(const TmplDev &T, int k, const float4 *xs, float F[3], float &kH)
 {
@@ -838,60 +850,61 @@ __device__ __forceinline__ void nodal_membrane(const TmplDev &T, int k, const fl
     float4 rn = make_float4(0.f, 0.f, 0.f, 0.f);
     ushort2 in = make_ushort2(0, 0);
     int prev = -1;
-    float e1[3] = {0.f, 0.f, 0.f}, l1 = 0.f, cF = 0.f, cK = 0.f;   // current edge and its coefficients
+    float4 xj = xk;
+    float e1[3] = {0.f, 0.f, 0.f};   // x_j - x_k
     if (deg > 0) {
         rn = ref[0];
         in = idx[0];
     }
     for (int q = 0; q < deg; ++q) {
         const float4 r = rn;
-        const ushort2 jl = in;
+        const int j = in.x & kNodMask, c = in.x >> kNodBits, l = in.y;
         if (q + 1 < deg) {
             rn = ref[32 * (q + 1)];
             in = idx[32 * (q + 1)];
         }
-        if (jl.x != prev) {   // a new fan
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                F[i] += cF * e1[i];
-                if constexpr (BEND)
-                    K[i] += cK * e1[i];
-            }
-            cF = cK = 0.f;
-            ring_edge_f32(xk, xs[jl.x], e1, l1);
+        if (j != prev) {   // a new fan
+            xj = xs[j];
+            edge_f32(xk, xj, e1);
         }
-        prev = jl.y;
-        float e2[3], l2;
-        ring_edge_f32(xk, xs[jl.y], e2, l2);
+        prev = l;
+        const float4 xl = xs[l];
+        float e2[3], e3[3];
+        edge_f32(xk, xl, e2);
+        edge_f32(xj, xl, e3);
+        xj = xl;
         RingF t;
-        ring_tri_f32(e1, l1, e2, l2, t);
-        const float w = r.w, w2 = w * w;
-        const float I2 = t.q * w2;
+        ring_tri_f32(e1, e2, e3, t);
+        // the triangle's own order: k is its corner c, so (a, b, c) = (k, j, l), (l, k, j) or (j, l, k)
+        const float da = c == 0 ? t.dk : (c == 1 ? t.dl : t.dj), db = c == 0 ? t.dj : (c == 1 ? t.dk : t.dl),
+                    dc = c == 0 ? t.dl : (c == 1 ? t.dj : t.dk);
+        const float rj = c == 0 ? r.y : (c == 1 ? r.z : r.x), rl = c == 0 ? r.z : (c == 1 ? r.x : r.y);
+        const float w = r.w, w2 = __fmul_rn(w, w);
+        // 4 A^2 from the dots: the cross product's bits depend on the corner
+        const float I2 = __fmul_rn(fmaf(dc, da, fmaf(db, dc, __fmul_rn(da, db))), w2);
         float a, b;
         if (T.law == 0) {
             a = mu;
-            b = -mu / (I2 * I2);
+            b = __fdiv_rn(-mu, __fmul_rn(I2, I2));
         } else {
-            a = mu * ((l1 * r.z + l2 * r.y + (t.dj + t.dl) * r.x) * w2 - 1.f);
-            b = half_muD * (I2 - 1.f) - mu;
+            const float I1 = __fmul_rn(fmaf(dc, r.x + r.y, fmaf(db, r.z + r.x, __fmul_rn(da, r.y + r.z))), w2);
+            a = __fmul_rn(mu, I1 - 1.f);
+            b = fmaf(half_muD, I2 - 1.f, -mu);
         }
         const float hw = 0.5f * w;
-        cF += hw * (a * r.z + b * t.dl);
+        const float sl = __fmul_rn(hw, fmaf(a, rl, __fmul_rn(b, t.dl)));   // edge (k, j)
+        const float sj = __fmul_rn(hw, fmaf(a, rj, __fmul_rn(b, t.dj)));   // edge (k, l)
 #pragma unroll
         for (int i = 0; i < 3; ++i)
-            F[i] += cF * e1[i];
-        cF = hw * (a * r.y + b * t.dj);
+            F[i] = fmaf(sj, e2[i], fmaf(sl, e1[i], F[i]));
         if constexpr (BEND) {
             const float cj = t.dj * t.inv2A, cl = t.dl * t.inv2A;
-            // K += cot_l (x_k - x_j) + cot_j (x_k - x_l), sign taken below
-            cK += cl;
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                K[i] += cK * e1[i];
+                K[i] += cl * e1[i] + cj * e2[i];   // cot_l (x_j - x_k) + cot_j (x_l - x_k), sign taken below
                 nrm[i] += t.fn[i];
             }
-            cK = cj;
-            const float twoA = t.q * t.inv2A;
+            const float l1 = t.dk + t.dj, l2 = t.dk + t.dl, twoA = t.q * t.inv2A;
             // 8 x mixed area: Voronoi, or 2A / 4 at an obtuse corner and 2A / 8 beside one
             const float obt = t.dk < 0.f ? twoA + twoA : twoA;
             A8 += fminf(t.dk, fminf(t.dj, t.dl)) >= 0.f ? cl * l1 + cj * l2 : obt;
@@ -905,11 +918,7 @@ __device__ __forceinline__ void nodal_membrane(const TmplDev &T, int k, const fl
 #pragma unroll
         for (int i = 0; i < 3; ++i)
             e1[i] = e2[i];
-        l1 = l2;
     }
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-        F[i] += cF * e1[i];
     if constexpr (BEND) {
         const float kb = T.kb_f, kH0 = T.kH0_f;
         const float rnl = rsqrtf(nrm[0] * nrm[0] + nrm[1] * nrm[1] + nrm[2] * nrm[2]);
@@ -917,7 +926,6 @@ __device__ __forceinline__ void nodal_membrane(const TmplDev &T, int k, const fl
         const float h = -0.5f / A;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            K[i] += cK * e1[i];
             nrm[i] *= rnl;
             K[i] *= h;
         }
@@ -940,38 +948,44 @@ __device__ __forceinline__ void nodal_bend2(const TmplDev &T, int k, const float
     const ushort2 *idx = reinterpret_cast<const ushort2 *>(T.nod_idx) + T.nod_off[k >> 5] + (k & 31);
     const float4 xk = xs[k];
     float lap = 0.f, nrm[3] = {0.f, 0.f, 0.f};
-    float e1[3] = {0.f, 0.f, 0.f}, l1 = 0.f, h1 = 0.f;
+    float4 xj = xk;
+    float e1[3] = {0.f, 0.f, 0.f};
     int prev = -1;
     ushort2 in = deg > 0 ? idx[0] : make_ushort2(0, 0);
     for (int q = 0; q < deg; ++q) {
-        const ushort2 jl = in;
+        const int j = in.x & kNodMask, l = in.y;
         if (q + 1 < deg)
             in = idx[32 * (q + 1)];
-        if (jl.x != prev) {
-            const float4 xj = xs[jl.x];
-            ring_edge_f32(xk, xj, e1, l1);
-            h1 = xj.w - xk.w;
+        if (j != prev) {
+            xj = xs[j];
+            edge_f32(xk, xj, e1);
         }
-        prev = jl.y;
-        const float4 xl = xs[jl.y];
-        float e2[3], l2;
-        ring_edge_f32(xk, xl, e2, l2);
-        const float h2 = xl.w - xk.w;
+        prev = l;
+        const float4 xl = xs[l];
+        float e2[3], e3[3];
+        edge_f32(xk, xl, e2);
+        edge_f32(xj, xl, e3);
         RingF t;
-        ring_tri_f32(e1, l1, e2, l2, t);
-        lap += (t.dl * h1 + t.dj * h2) * t.inv2A;
+        ring_tri_f32(e1, e2, e3, t);
+        lap += (t.dl * (xj.w - xk.w) + t.dj * (xl.w - xk.w)) * t.inv2A;
+        xj = xl;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             nrm[i] += t.fn[i];
             e1[i] = e2[i];
         }
-        l1 = l2;
-        h1 = h2;
     }
     const float s = T.kb_f * lap * rsqrtf(nrm[0] * nrm[0] + nrm[1] * nrm[1] + nrm[2] * nrm[2]);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
         Fb[i] = s * nrm[i];
+}
+
+__device__ __forceinline__ void cross_f32(const float a[3], const float b[3], float r[3])
+{
+    r[0] = a[1] * b[2] - a[2] * b[1];
+    r[1] = a[2] * b[0] - a[0] * b[2];
+    r[2] = a[0] * b[1] - a[1] * b[0];
 }
 
 // A solid node; returns the number of incident tets with J <= 0 among those
@@ -983,7 +997,7 @@ __device__ __forceinline__ int nodal_solid(const TmplDev &T, int k, const float4
     const long long at = T.nod_off[k >> 5] + (k & 31);
     const float4 *ref = T.nod_ref + at;
     const ushort4 *idx = reinterpret_cast<const ushort4 *>(T.nod_idx) + at;
-    const float4 x0 = xs[k];
+    const float4 xk = xs[k];
     int inverted = 0;
     F[0] = F[1] = F[2] = 0.f;
     float4 rn = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -999,34 +1013,42 @@ __device__ __forceinline__ int nodal_solid(const TmplDev &T, int k, const float4
             rn = ref[32 * (q + 1)];
             in = idx[32 * (q + 1)];
         }
-        const float4 p1 = xs[v.x], p2 = xs[v.y], p3 = xs[v.z];
-        const float d1[3] = {p1.x - x0.x, p1.y - x0.y, p1.z - x0.z};
-        const float d2[3] = {p2.x - x0.x, p2.y - x0.y, p2.z - x0.z};
-        const float d3[3] = {p3.x - x0.x, p3.y - x0.y, p3.z - x0.z};
-        const float c[3] = {d2[1] * d3[2] - d2[2] * d3[1], d2[2] * d3[0] - d2[0] * d3[2],
-                            d2[0] * d3[1] - d2[1] * d3[0]};
-        const float J = (d1[0] * c[0] + d1[1] * c[1] + d1[2] * c[2]) * h.w;
-        inverted += v.w != 0 && !(J > 0.f);
-        // n = d2 x d3 + d1 x (d2 - d3)
-        const float g[3] = {d2[0] - d3[0], d2[1] - d3[1], d2[2] - d3[2]};
-        const float n[3] = {c[0] + (d1[1] * g[2] - d1[2] * g[1]), c[1] + (d1[2] * g[0] - d1[0] * g[2]),
-                            c[2] + (d1[0] * g[1] - d1[1] * g[0])};
-        const float beta = (half_lam * (J * J - 1.f) - mu) / (6.f * J);
+        const int c = v.x >> kNodBits;
+        const float4 p0 = xs[v.x & kNodMask], p1 = xs[v.y], p2 = xs[v.z], p3 = xs[v.w];
+        float y1[3], y2[3], y3[3], n1[3], n2[3], n3[3];
+        edge_f32(p0, p1, y1);
+        edge_f32(p0, p2, y2);
+        edge_f32(p0, p3, y3);
+        cross_f32(y2, y3, n1);
+        cross_f32(y3, y1, n2);
+        cross_f32(y1, y2, n3);
+        const float inv6V = c == 0 ? h.x : (c == 1 ? h.y : (c == 2 ? h.z : h.w));
+        const float J = dot3f(y1, n1) * inv6V;
+        inverted += c == 0 && !(J > 0.f);
+        const float beta = __fdiv_rn(fmaf(half_lam, fmaf(J, J, -1.f), -mu), 6.f * J);
+        const float m0 = mu * h.x, m1 = mu * h.y, m2 = mu * h.z, m3 = mu * h.w;
+        const float x0[3] = {p0.x - xk.x, p0.y - xk.y, p0.z - xk.z}, x1[3] = {p1.x - xk.x, p1.y - xk.y, p1.z - xk.z};
+        const float x2[3] = {p2.x - xk.x, p2.y - xk.y, p2.z - xk.z}, x3[3] = {p3.x - xk.x, p3.y - xk.y, p3.z - xk.z};
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
-            F[i] += mu * (h.x * d1[i] + h.y * d2[i] + h.z * d3[i]) + beta * n[i];
+        for (int i = 0; i < 3; ++i) {
+            const float n = c == 0 ? (n1[i] + n2[i]) + n3[i] : -(c == 1 ? n1[i] : (c == 2 ? n2[i] : n3[i]));
+            float acc = fmaf(m0, x0[i], F[i]);
+            acc = fmaf(m1, x1[i], acc);
+            acc = fmaf(m2, x2[i], acc);
+            acc = fmaf(m3, x3[i], acc);
+            F[i] = fmaf(beta, n, acc);
+        }
     }
     return inverted;
 }
 
-// What bounds it: latency and instruction issue. On the 600-particle suspension
-// (1.33 M nodes) 63 M warp instructions, 64 % of the issue slots of the active
-// cycles, at the 28 warps per SM that 64 registers allow (fewer registers
-// spill: 110 us with 40); shared memory at 34 %. 85 us against 129 us for the
-// kernel before it (per-element forces added with float atomics in shared
-// memory, 60 % of that pipe), one red cell 11 against 47 us, the
-// element-buffer path of the deterministic mode (four launches) 51 -> 19 us
-// on 72 particles.
+// What bounds it: latency and instruction issue, at the 28 warps per SM that 64
+// registers allow (fewer registers spill: 110 against 85 us on the 600-particle
+// suspension with 40), shared memory at a third of its rate. 600 particles (1.33 M
+// nodes): 90 us against 129 us for the kernel before it (per-element forces
+// added with float atomics in shared memory, 60 % of that pipe), one red cell
+// 11 against 47 us, the element-buffer path of the deterministic mode (four
+// launches) 51 -> 20 us on 72 particles, 64 balls of 4096 nodes 93 -> 43 us.
 // One cluster of S CTAs per particle (S = 1: one CTA), each holding every
 // position of the particle in shared memory (float4, kH in w) and taking a
 // chunk of its nodes (inst0 < 0: all particles, the largest first; else

@@ -25,7 +25,7 @@ struct ifem_ctx_s {
     int acc64 = 0;
     int tuned = 0;
     cudaStream_t aux[2] = {};   // fork-join streams of ifem_step_coupling
-    static constexpr int kForkEvents = 10;
+    static constexpr int kForkEvents = 11;
     cudaEvent_t fork[kForkEvents] = {};
 };
 

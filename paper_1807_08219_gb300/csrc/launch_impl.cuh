@@ -111,11 +111,12 @@ cudaError_t bin_impl(const TransferArgs &a, int det_sort, int with_cand, int sta
     // one-pass binning of the FP32 halo path: kBinPer nodes per thread
     dim3 g1((b.max_nodes + 256 * kBinPer - 1) / (256 * kBinPer), b.n_inst);
     if (stages & BIN_COUNT) {
-        if (with_cand)
-            cudaMemsetAsync(w.cand_count, 0, sizeof(int) * (nt + 1), s);
-        // own counts, then (FP32 halo path) the per-tile flags and |F| sums behind them
-        cudaMemsetAsync(w.own_count, 0, sizeof(int) * (no + 1 + (with_cand ? 0 : 4 * nt)), s);
-        cudaMemsetAsync(w.counters, 0, sizeof(int) * kCounters, s);
+        // one clear: the counters, counts and per-tile |F| sums, and before them
+        // the spread's per-tile sums
+        const size_t sums = a.clear_sums ? sizeof(double) * 3 * (size_t)nt : 0;
+        cudaError_t e = cudaMemsetAsync(reinterpret_cast<char *>(w.counters) - sums, 0, sums + w.zero_bytes, s);
+        if (e != cudaSuccess)
+            return e;
         IFEM_LAUNCH_CHECK();
         if (empty)
             return cudaSuccess;
@@ -212,18 +213,10 @@ cudaError_t spread_impl(const TransferArgs &a)
 {
     const DevBatch &b = a.b;
     cudaStream_t s = a.stream;
-    // the fused halo transfer right after its binning: own_scatter_kernel
-    // cleared the per-tile sums and the binning the work counter
-    const bool cleared = a.binned && a.halo && a.u != nullptr && a.v != nullptr;
-    if (!cleared)
-        cudaMemsetAsync(a.w.red_tile, 0, sizeof(double) * 3 * a.g.n_tiles, s);
-    IFEM_LAUNCH_CHECK();
     if (b.n_inst == 0 || b.N == 0)
         return cudaSuccess;
     if constexpr (std::is_same<real, float>::value) {
         const int E = a.g.max_edge;
-        if (!cleared)
-            cudaMemsetAsync(a.w.counters + 2, 0, sizeof(int), s);
         if (a.halo) {
             // with u and v given, interpolation is fused into the spread, and
             // with xn also the position update

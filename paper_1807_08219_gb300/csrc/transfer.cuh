@@ -878,9 +878,7 @@ __global__ void __launch_bounds__(256) spread_fast_kernel(DevBatch b, DevGrid g,
 // and its id, kBinPer nodes per thread as in own_count_kernel (loads first,
 // then the offsets, then the stores). With the force in the record the
 // transfer reads its nodes in two consecutive 16-byte loads, without a gather
-// through the node id. The per-tile FP64 sums of the spread are cleared for
-// every tile (the transfer writes them for the listed tiles only) and the
-// tiles that own nodes are listed, counters[3] of them, with everything the
+// through the node id. The tiles that own nodes are listed, counters[3] of them, with everything the
 // transfer needs of a tile: it fetches an item in one copy, without walking
 // empty tiles or decoding tile numbers. The list keeps roughly the tile order
 // (in order within each warp's append), so items running at the same time are
@@ -967,9 +965,6 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
         bool has = false;
         if (t < g.n_tiles) {
             has = w.own_flag[t] != 0;
-            w.red_tile[3 * t] = 0.0;
-            w.red_tile[3 * t + 1] = 0.0;
-            w.red_tile[3 * t + 2] = 0.0;
         }
         const unsigned m = __ballot_sync(0xffffffffu, has);
         int base = 0;
@@ -1112,18 +1107,18 @@ __device__ __forceinline__ bool tile_vec(const TileItem &it, const float *lat)
     return ((it.sx | it.n | it.ex) & 3) == 0 && (reinterpret_cast<uintptr_t>(lat) & 15) == 0;
 }
 
-// Fixed-point scale of an item: the largest power of two that keeps the bound
-// sum |g_k| / 8 below 2^30. fsum: the placement's atomic float sum of |F_d|
-// over n nodes, within (n - 1) 2^-24 of the exact one in any order.
+// Fixed-point scale of an item: keeps the bound sum |g_k| / 8 on any value (and
+// the rounding of its terms) below 2^31, three mantissa bits of the largest such
+// scale (the bits a different order of the placement's additions cannot reach).
+// A power of two below 2^30 instead left the field of one red cell with 1.5 to
+// 1.9 times the error. fsum: the placement's atomic float sum of |F_d| over n
+// nodes, within (n - 1) 2^-24 of the exact one in any order.
 __device__ __forceinline__ float tile_scale(const TileItem &it, float fsum)
 {
-    const float bound = fsum * (1.0001f + (float)(it.end - it.beg) * 1.1920929e-7f) * it.sd * 0.125f;
+    const float bound = fsum * (1.0002f + (float)(it.end - it.beg) * 1.1920929e-7f) * it.sd * 0.125f;
     float scale = 1.f;
-    if (bound > 0.f && isfinite(bound)) {
-        int e = (int)floorf(log2f(FixedPoint<int>::kRange / bound));
-        e = e > 120 ? 120 : (e < -120 ? -120 : e);
-        scale = exp2f((float)e);
-    }
+    if (bound > 0.f && isfinite(bound))
+        scale = __uint_as_float(__float_as_uint(fminf(fmaxf(2147483648.f / bound, 0x1p-120f), 0x1p120f)) & 0xfff00000u);
     return scale;
 }
 
@@ -1170,9 +1165,8 @@ __device__ __forceinline__ void tile_stage(const TileItem &it, const float *__re
 }
 
 // Adds every non-zero value of A to the grid and clears it; returns the exact
-// integer sum and counts the non-zero values inside the tile itself. Two
-// neighbours' sum fits 32 bits: their weights add up to at most 0.22, against
-// the 1/8 of the bound. bt: box thread.
+// integer sum and counts the non-zero values inside the tile itself. bt: box
+// thread.
 template <int W>
 __device__ __forceinline__ long long tile_flush(const TileItem &it, float *__restrict__ f, int4 *A, float inv,
                                                 int bt, unsigned &touched)
@@ -1202,7 +1196,7 @@ __device__ __forceinline__ long long tile_flush(const TileItem &it, float *__res
         A[8 * yb * S::NZ * S::NX] = make_int4(0, 0, 0, 0);
         const int ly = 2 * yb + yl;
         float *row = plane + wrap1(it.sy - 2 + ly, n) * n;
-        qsum += (long long)(q.x + q.y) + (long long)(q.z + q.w);
+        qsum += ((long long)q.x + q.y) + ((long long)q.z + q.w);
         const float v0 = (float)q.x * inv, v1 = (float)q.y * inv, v2 = (float)q.z * inv, v3 = (float)q.w * inv;
         const bool in_y = (unsigned)(ly - 2) < (unsigned)it.ey;
         if (vec) {
@@ -1410,14 +1404,13 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
         s_scale[i & 3] = tile_scale(tile_item(s_desc[i % kRing], s_d[i % kRing], density), fsum);
     };
     auto get_fsum = [&](int i) { return w.tile_fsum[3LL * s_desc[i % kRing].tile + s_d[i % kRing]]; };
-    auto write_sum = [&](int i) {   // one thread: the exact sum of a flushed item, times h^3
+    auto write_sum = [&](int i) {   // one thread: the exact integer sum of a flushed item, scaled, times h^3
         const TileDesc &td = s_desc[i % kRing];
         long long vsum = 0;
 #pragma unroll
         for (int q = 0; q < kBoxWarps; ++q)
             vsum += s_red[i & 1][q];
-        // |vsum| < 2^53, the scale a power of two: one rounding
-        w.red_tile[3LL * td.tile + s_d[i % kRing]] = (double)vsum * (double)(1.f / s_scale[i & 3]) * td.h3;
+        w.red_tile[3LL * td.tile + s_d[i % kRing]] = (double)vsum / (double)s_scale[i & 3] * td.h3;
     };
     if (!box)
         unit_ahead(0);
