@@ -18,18 +18,16 @@ a step.
 """
 from __future__ import annotations
 
-import numpy as np
 import torch
 
 from . import ifem as I
 
 
-def _node_box_scale(coupler) -> torch.Tensor:
-    """(n_b/L_b)^3 of each node's box, as a (1, N) tensor of the coupler's dtype."""
-    wl = coupler.wl
-    s = np.concatenate([np.full(wl.templates[i.tmpl].n_nodes, (wl.boxes[i.box].n / wl.boxes[i.box].L) ** 3)
-                        for i in wl.instances]) if wl.instances else np.zeros(0)
-    return torch.as_tensor(s, dtype=coupler.dtype, device=coupler.device)[None, :]
+def _times_box_scale(v, coupler) -> torch.Tensor:
+    """v times (n_b/L_b)^3 of each node's box, in place: one number where the boxes
+    share it, else the coupler's per-node row."""
+    scales = {(bx.n / bx.L) ** 3 for bx in coupler.wl.boxes}
+    return v.mul_(scales.pop() if len(scales) == 1 else coupler.node_box_scale())
 
 
 class SpreadFn(torch.autograd.Function):
@@ -48,7 +46,7 @@ class SpreadFn(torch.autograd.Function):
         cp = ctx.coupler
         v = cp.empty_nodes()
         I.ifem_interpolate(cp.ctx, cp.batch, cp.grid, g.contiguous(), x.contiguous(), v)
-        return v * _node_box_scale(cp), None, None
+        return _times_box_scale(v, cp), None, None
 
 
 class InterpFn(torch.autograd.Function):

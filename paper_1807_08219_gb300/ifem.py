@@ -386,6 +386,7 @@ class Coupler:
         self.N = ifem_batch_nodes(self.batch)
         self.G = ifem_grid_values(self.grid)
         self.box_off = [ifem_grid_box_offset(self.grid, b) for b in range(len(wl.boxes))]
+        self._box_scale = None
 
     # host <-> device helpers (layout conversions only)
     def nodes_to_device(self, a: np.ndarray):
@@ -414,6 +415,18 @@ class Coupler:
 
     def zeros_grid(self):
         return self.torch.zeros(self.G, dtype=self.dtype, device=self.device)
+
+    def node_box_scale(self):
+        """(n_b/L_b)^3 of each node's box, a (1, N) tensor made once (the copy has
+        arrived when the call returns, so any stream may read it)."""
+        if self._box_scale is None:
+            wl = self.wl
+            s = [np.full(wl.templates[i.tmpl].n_nodes, (wl.boxes[i.box].n / wl.boxes[i.box].L) ** 3)
+                 for i in wl.instances]
+            s = self.torch.as_tensor(np.concatenate(s) if s else np.zeros(0), dtype=self.dtype).to(self.device)
+            self.torch.cuda.synchronize(self.device)
+            self._box_scale = s[None, :]
+        return self._box_scale
 
     def close(self):
         if self.batch is not None:
