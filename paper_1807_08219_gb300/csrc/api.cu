@@ -409,6 +409,11 @@ static int nodal_upload(ifem_ctx ctx, ifem_tmpl t, int nv, const int32_t *el, co
 static int tmpl_upload(ifem_ctx ctx, ifem_tmpl t, int nv, const int32_t *el, const double *X,
                        const std::vector<double> &ref)
 {
+    double extent = 0.0;
+    for (size_t i = 0; i < 3 * (size_t)t->n_nodes; ++i)
+        extent = std::max(extent, std::fabs(X[i]));
+    if (extent > 0.0 && std::isfinite(extent))
+        t->vol_scale = (float)std::ldexp(1.0, -std::min(100, std::max(-100, std::ilogb(extent))));
     std::vector<float> reff(ref.begin(), ref.end());
     std::vector<int> off, idx;
     incidence(t->n_nodes, t->n_elems, nv, el, off, idx);
@@ -676,6 +681,7 @@ extern "C" int ifem_batch_create(ifem_ctx ctx, int n_tmpl, const ifem_tmpl *tmpl
         d.kb = s->kb;
         d.c0 = s->c0;
         d.lam = s->lam;
+        d.vol_scale = s->vol_scale;
         d.mu_f = (float)s->mu;
         d.half_muD_f = 0.5f * ((float)s->C * d.mu_f);
         d.kb_f = (float)s->kb;

@@ -60,6 +60,7 @@ struct TmplDev {
     const void *nod_idx;     // membranes: ushort2 (j, l); solids: ushort4, the corners; the node's corner
                              // number in the bits of the first id above kNodBits
     double mu, C, kb, c0, lam;
+    float vol_scale;         // power of two near 1 over the template's extent
     float mu_f, half_muD_f, kb_f, kH0_f, half_lam_f;   // FP32 nodal kernel: mu, C mu/2, kb, -c0/2, lam/2
 };
 

@@ -35,6 +35,7 @@ struct ifem_tmpl_s {
     int law;
     int n_nodes, n_elems;
     double mu, C, kb, c0, lam;
+    float vol_scale = 1.f;
     int *d_elems = nullptr;
     double *d_ref_d = nullptr;
     float *d_ref_f = nullptr;

@@ -366,6 +366,17 @@ cudaError_t volume_impl(const LagrangeArgs &a)
 {
     if (a.b.n_inst == 0)
         return cudaSuccess;
+    if constexpr (std::is_same<real, float>::value) {
+        const size_t sm = sizeof(float4) * (size_t)a.b.max_nodes;
+        if (sm + 1024 <= (size_t)kMaxCtaSmemBytes) {
+            cudaError_t e = cudaFuncSetAttribute(volume_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            if (e != cudaSuccess)
+                return e;
+            volume_f32_kernel<<<a.b.n_inst, kVolThreadsF, sm, a.stream>>>(a.b, (const float *)a.x, a.out);
+            IFEM_LAUNCH_CHECK();
+            return cudaSuccess;
+        }
+    }
     volume_kernel<real><<<a.b.n_inst, kVolThreads, 0, a.stream>>>(a.b, (const real *)a.x, a.out);
     IFEM_LAUNCH_CHECK();
     return cudaSuccess;
@@ -376,6 +387,17 @@ cudaError_t vcorr_impl(const LagrangeArgs &a)
 {
     if (a.b.n_inst == 0)
         return cudaSuccess;
+    if constexpr (std::is_same<real, float>::value) {
+        const size_t sm = 2 * sizeof(float4) * (size_t)a.b.max_nodes;
+        if (sm + 1024 <= (size_t)kMaxCtaSmemBytes) {
+            cudaError_t e = cudaFuncSetAttribute(vc_fused_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            if (e != cudaSuccess)
+                return e;
+            vc_fused_f32_kernel<<<a.b.n_inst, kVolThreadsF, sm, a.stream>>>(a.b, (float *)a.x, a.V0, a.out, a.status);
+            IFEM_LAUNCH_CHECK();
+            return cudaSuccess;
+        }
+    }
     dim3 gn((a.b.max_nodes + 255) / 256, a.b.n_inst);
     vc_alpha_kernel<real><<<gn, 256, 0, a.stream>>>(a.b, (const real *)a.x, a.alpha);
     IFEM_LAUNCH_CHECK();
