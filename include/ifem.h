@@ -101,13 +101,12 @@ typedef enum { IFEM_KERNEL_PESKIN4 = 0, IFEM_KERNEL_MLS27 = 1 } ifem_kernel;
 
 /* Summation order of the FP32 scatters (IFEM_FP64 is always deterministic).
  * Forces are a fixed-order sum per node over its incident elements in both.
- * DET: spreading sums each lattice value from the node lists of its own tile
- * (every node binned into each tile its stencil reaches), so repeated runs
- * give identical results.
- * ATOMIC: with PESKIN4, spreading visits each node
- * once, in the tile holding its cell, accumulates into the tile plus a
- * 2-cell halo (4 in x) and adds that to the grid with atomic L2 adds, so the
- * order in which neighbouring tiles' halos combine is not reproducible. */
+ * Spreading visits each node once, in the tile holding its cell, accumulates
+ * into the tile plus a 2-cell halo (4 in x) in fixed point and adds that to the
+ * grid. DET: where more than two tiles reach a value, their terms are added in a
+ * fixed order, so repeated runs give identical results (also MLS27 in either
+ * mode). ATOMIC: they are added with atomic L2 adds, so the order in which
+ * neighbouring tiles' halos combine is not reproducible. */
 typedef enum { IFEM_SCATTER_DET = 0, IFEM_SCATTER_ATOMIC = 1 } ifem_scatter;
 
 typedef enum { IFEM_LAW_NEO_HOOKE = 0, IFEM_LAW_SKALAK = 1 } ifem_membrane_law;
@@ -161,9 +160,8 @@ typedef struct {
                                    spread needs no per-tile candidate lists) */
     int64_t active_tiles;       /* tiles with at least one node pair */
     int64_t touched_cells;      /* non-zero lattice values added by spreads since the last sync
-                                   (FP32 path; the FP64 path rewrites every value of an active
-                                   tile; the FP32 ATOMIC Peskin spread counts the values inside
-                                   each node's own tile only) */
+                                   (FP32: counted inside each node's own tile only; the FP64 path
+                                   rewrites every value of an active tile) */
 } ifem_stats;
 
 /* ---------------------------------------------------------------- context */
@@ -376,10 +374,9 @@ int ifem_reduce(ifem_ctx ctx, ifem_batch b, const void *x, const void *F, const 
  * before the reductions (valid under CUDA-graph capture of `stream`); with
  * cfg.profile = 1 the stages run one after the other on `stream` instead
  * (forces, then binning, spreading, interpolation, reductions), so that
- * ifem_stage_times can attribute them. With IFEM_FP32, IFEM_SCATTER_ATOMIC
- * and IFEM_KERNEL_PESKIN4 the interpolation is fused into the spreading
- * kernel (each node's stencil weights serve both transfers), and the last
- * part of the binning waits for the forces: it also sums |F| per tile, which
+ * ifem_stage_times can attribute them. With IFEM_FP32 the interpolation is fused
+ * into the spreading kernel (each node's stencil weights serve both transfers),
+ * and the last part of the binning waits for the forces: it also sums |F| per tile, which
  * sets the spread accumulators' fixed-point scales. Results equal those of
  * the separate calls up to FP32 rounding. */
 int ifem_step_coupling(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, const void *u,

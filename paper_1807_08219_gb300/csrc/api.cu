@@ -95,10 +95,6 @@ extern "C" int ifem_ctx_create(const ifem_config *cfg, ifem_ctx *out)
     // pairs), 8 for the deterministic FP64 spread (its cost grows with the
     // candidates per tile times the values per tile)
     ctx->tile = cfg->tile ? cfg->tile : (cfg->precision == IFEM_FP64 ? 8 : 16);
-    // FP32 spread accumulator width (tuning knob): IFEM_SPREAD_ACC=64 selects
-    // 64-bit fixed point (slower shared-memory atomics), anything else 32-bit
-    if (const char *acc = std::getenv("IFEM_SPREAD_ACC"))
-        ctx->acc64 = std::string(acc) == "64" ? 1 : 0;
     if (cudaSetDevice(cfg->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess ||
         cudaMalloc((void **)&ctx->d_status, sizeof(unsigned long long) * kStatusWords) != cudaSuccess ||
@@ -761,7 +757,28 @@ extern "C" int ifem_batch_set_origins(ifem_batch b, const double *origins)
     return IFEM_OK;
 }
 
-static int use_halo(ifem_ctx ctx);
+static bool reproducible(ifem_ctx ctx);
+
+// Tile edge t and tiles per axis T of a box of n >= 8 cells for own lists: every
+// tile at least 4 cells, so that the halos on its two sides meet different cells,
+// and none larger than the box width of the edge asked for holds (tile_width).
+// The last tile takes the remainder, or is larger by it where it is below 4 and
+// fits, else the edge is one less.
+static void own_tiling(int n, int tile, int &t, int &T)
+{
+    const int most = tile_width(tile) - 4;
+    for (t = std::min(tile, n);; --t) {
+        const int r = n % t;
+        if (r == 0 || r >= 4) {
+            T = (n + t - 1) / t;
+            return;
+        }
+        if (t + r <= most) {
+            T = n / t;
+            return;
+        }
+    }
+}
 
 // Work buffers for (batch, grid, tile): box/tile tables, per-tile lists.
 static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
@@ -770,16 +787,19 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
     if (ws.grid == g && ws.tile == tile)
         return IFEM_OK;
     ws_free(ws);
+    const bool f32 = ctx->cfg.precision == IFEM_FP32;
     std::vector<BoxDev> boxes(g->n_boxes);
     long long nt = 0;
     int max_edge = 0;
     for (int i = 0; i < g->n_boxes; ++i) {
         BoxDev &B = boxes[i];
         B.n = g->n[i];
-        B.t = std::min(tile, B.n);
-        // candidate lists need tiles of at least 5 cells; own lists do not, and
-        // keep every tile within the tile edge
-        B.T = use_halo(ctx) ? (B.n + B.t - 1) / B.t : tiles_per_axis(B.n, B.t);
+        if (f32) {
+            own_tiling(B.n, tile, B.t, B.T);
+        } else {   // candidate lists: tiles of at least 5 cells
+            B.t = std::min(tile, B.n);
+            B.T = tiles_per_axis(B.n, B.t);
+        }
         B.tile_base = nt;
         B.grid_off = g->off[i];
         B.L = g->L[i];
@@ -806,40 +826,47 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
     long long N = b->N;
     const long long no = nt * kOwnSub3;
     int nb = (int)((no + kScanBlock - 1) / kScanBlock);
-    w.cand_cap = 8 * N;
     CK(alloc((void **)&ws.d_boxes, sizeof(BoxDev) * boxes.size()));
     CK(cudaMemcpy(ws.d_boxes, boxes.data(), sizeof(BoxDev) * boxes.size(), cudaMemcpyHostToDevice));
     // what a binning clears, in one piece: the spread's per-tile sums (by a
     // spread's binning only), then the counters and counts
-    const size_t zero_ints = kCounters + (size_t)(no + 1) + (use_halo(ctx) ? 4 * nt : nt + 1);
+    const size_t bin_ints = reproducible(ctx) ? 2 * kFsumBins * 3 * (size_t)nt : 0;
+    const size_t zero_ints =
+        kCounters + bin_ints + (size_t)(no + 1) + (!f32 ? nt + 1 : (reproducible(ctx) ? nt : 4 * nt));
     CK(alloc((void **)&w.red_tile, sizeof(double) * 3 * (size_t)nt + sizeof(int) * zero_ints));
     CK(cudaMemset(w.red_tile, 0, sizeof(double) * 3 * (size_t)nt));
     w.counters = reinterpret_cast<int *>(w.red_tile + 3 * nt);
     w.zero_bytes = sizeof(int) * zero_ints;
-    w.own_count = w.counters + kCounters;
-    CK(alloc((void **)&w.cand_off, sizeof(int) * (nt + 1)));
-    CK(alloc((void **)&w.cand_cursor, sizeof(int) * (nt + 1)));
-    CK(alloc((void **)&w.cand_nodes, sizeof(int) * (size_t)w.cand_cap));
-    if (use_halo(ctx)) {
+    w.tile_fbin = reinterpret_cast<unsigned long long *>(w.counters + kCounters);
+    w.own_count = w.counters + kCounters + bin_ints;
+    CK(alloc((void **)&w.own_cursor, sizeof(int) * (no + 1)));
+    const size_t Nn = (size_t)std::max<long long>(N, 1);
+    if (f32) {
         w.own_flag = w.own_count + no + 1;
         w.tile_fsum = reinterpret_cast<float *>(w.own_flag + nt);
+        CK(alloc((void **)&w.own_rec, 2 * sizeof(float4) * Nn));
+        CK(alloc((void **)&w.tile_desc, sizeof(TileDesc) * (size_t)(nt + 1)));
+        CK(alloc((void **)&w.tile_slot, sizeof(int) * (size_t)(nt + 1)));
+        CK(alloc((void **)&w.node_key, sizeof(int2) * Nn));
+        CK(alloc((void **)&w.node_rec, sizeof(float4) * Nn));
+        if (reproducible(ctx)) {   // a box per listed tile and lattice: at most one tile per node
+            CK(alloc((void **)&w.box_buf, tile_box_bytes(max_edge) * 3 * (size_t)std::min(nt, N)));
+            CK(alloc((void **)&w.field, sizeof(float) * (size_t)g->total));
+            CK(alloc((void **)&w.near_tile, sizeof(int2) * (size_t)(nt + 1)));
+        }
     } else {
         w.cand_count = w.own_count + no + 1;
-    }
-    CK(alloc((void **)&w.own_cursor, sizeof(int) * (no + 1)));
-    if (!use_halo(ctx)) {
+        w.cand_cap = 8 * N;
+        CK(alloc((void **)&w.cand_off, sizeof(int) * (nt + 1)));
+        CK(alloc((void **)&w.cand_cursor, sizeof(int) * (nt + 1)));
+        CK(alloc((void **)&w.cand_nodes, sizeof(int) * (size_t)w.cand_cap));
         CK(alloc((void **)&w.own_off, sizeof(int) * (no + 1)));
-        CK(alloc((void **)&w.own_nodes, sizeof(int) * (size_t)std::max<long long>(N, 1)));
-    } else {
-        CK(alloc((void **)&w.own_rec, 2 * sizeof(float4) * (size_t)std::max<long long>(N, 1)));
-        CK(alloc((void **)&w.tile_desc, sizeof(TileDesc) * (size_t)(nt + 1)));
-        CK(alloc((void **)&w.node_key, sizeof(int2) * (size_t)std::max<long long>(N, 1)));
-        CK(alloc((void **)&w.node_rec, sizeof(float4) * (size_t)std::max<long long>(N, 1)));
+        CK(alloc((void **)&w.own_nodes, sizeof(int) * Nn));
+        CK(alloc((void **)&w.active, sizeof(int) * (nt + 1)));
     }
     w.wtab = nullptr;
     if (ctx->cfg.precision == IFEM_FP64 && ctx->cfg.kernel == IFEM_KERNEL_PESKIN4)
         CK(alloc((void **)&w.wtab, sizeof(DetW) * (size_t)std::max<long long>(N, 1)));
-    CK(alloc((void **)&w.active, sizeof(int) * (nt + 1)));
     CK(alloc((void **)&w.scan_blocks, sizeof(int) * 2 * (nb + 1)));
     w.elem_buf = b->d_elem_buf;
     w.bend_buf = b->d_bend_buf;
@@ -879,13 +906,12 @@ static int launch_rc(ifem_ctx ctx, cudaError_t e, const char *what)
     return IFEM_OK;
 }
 
-// The FP32 Peskin spread of an IFEM_SCATTER_ATOMIC context uses the halo
-// scatter (own nodes only, L2 reductions); every other configuration the
-// owner-computes spread over candidate lists.
-static int use_halo(ifem_ctx ctx)
+// The FP32 spread that gives the same bits from run to run: IFEM_SCATTER_DET, and
+// the MLS kernel in both modes.
+static bool reproducible(ifem_ctx ctx)
 {
-    return ctx->cfg.precision == IFEM_FP32 && ctx->cfg.kernel == IFEM_KERNEL_PESKIN4 &&
-           ctx->cfg.scatter == IFEM_SCATTER_ATOMIC;
+    return ctx->cfg.precision == IFEM_FP32 &&
+           (ctx->cfg.scatter == IFEM_SCATTER_DET || ctx->cfg.kernel == IFEM_KERNEL_MLS27);
 }
 
 static TransferArgs transfer_args(ifem_ctx ctx, ifem_batch b, const void *x, const void *F, const void *u,
@@ -904,8 +930,9 @@ static TransferArgs transfer_args(ifem_ctx ctx, ifem_batch b, const void *x, con
     a.density = (flags & IFEM_SPREAD_FORCE) ? 0 : 1;
     a.support = ctx->cfg.mls_support;
     a.n_sm = ctx->n_sm;
-    a.acc64 = ctx->acc64;
-    a.halo = use_halo(ctx);
+    a.store = reproducible(ctx);
+    a.cleared = (flags & IFEM_SPREAD_OVERWRITE) != 0;
+    a.total = b->grid0->total;
     a.lattice = -1;
     a.stream = (cudaStream_t)stream;
     return a;
@@ -933,7 +960,7 @@ static int do_forces(ifem_ctx ctx, ifem_batch b, const void *x, void *F, const v
     return launch_rc(ctx, e, "forces");
 }
 
-// stages other than BIN_ALL: the FP32 halo path only. F (FP32 halo path):
+// stages other than BIN_ALL: FP32 only. F (FP32):
 // the placement also sums |F| per tile, which the tile transfer's spread
 // requires (every spread follows a binning given the same forces).
 // sums: a spread follows (the binning clears its per-tile sums, which an
@@ -946,8 +973,7 @@ static int do_bin(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, void *
         return rc;
     TransferArgs a = transfer_args(ctx, b, x, F, nullptr, nullptr, nullptr, 0, stream);
     a.clear_sums = sums;
-    cudaError_t e = ctx->cfg.precision == IFEM_FP64 ? launch_bin_f64(a, 1, 1, stages)
-                                                    : launch_bin_f32(a, 0, !use_halo(ctx), stages);
+    cudaError_t e = ctx->cfg.precision == IFEM_FP64 ? launch_bin_f64(a, stages) : launch_bin_f32(a, stages);
     return launch_rc(ctx, e, "binning");
 }
 
@@ -967,8 +993,8 @@ static int do_spread(ifem_ctx ctx, ifem_batch b, const void *x, const void *F, v
     return launch_rc(ctx, e, "spread");
 }
 
-// Spreading with the interpolation of the same step fused into it (the
-// halo-scatter configuration only): one launch per step for both transfers.
+// Spreading with the interpolation of the same step fused into it (FP32): one
+// launch per step for both transfers.
 // With xn given the launch also writes the position update from the
 // velocities it gathers (xn = x + dt (3/2 v - 1/2 vp)).
 static int do_spread_interp(ifem_ctx ctx, ifem_batch b, const void *x, const void *F, const void *u, void *f,
@@ -1289,7 +1315,7 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
         mark(ctx, 2, stream);
         if ((rc = do_overwrite(ctx, g, f, flags, stream)) != IFEM_OK)
             return rc;
-        ctx->ev_fused = use_halo(ctx);
+        ctx->ev_fused = ctx->cfg.precision == IFEM_FP32;
         if (ctx->ev_fused) {
             if ((rc = do_spread_interp(ctx, b, x, F, u, f, v, flags, stream, vp, xn, dt)) != IFEM_OK)
                 return rc;
@@ -1339,7 +1365,7 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
     //   s:    copy x[0:h] copy x[h:N] count, scan, wait(forces) placement ... spread+interp  sums of v, boxes  copy red  wait(copy v)
     //   aux0:   wait(x[0:h]) forces[0:h] wait(x[h:N]) forces[h:N] wait(placement) sums of x, F
     //   aux1:                                           wait(v) copy v ------------------/
-    const bool fused = use_halo(ctx) != 0;
+    const bool fused = ctx->cfg.precision == IFEM_FP32;
     if ((rc = ws_ensure(ctx, b, g, ctx->tile)) != IFEM_OK)
         return rc;
     // the clearing of f runs on aux1 beside the host copies, or beside the
@@ -1438,7 +1464,7 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
     // programmatic serialization: their CTAs start on the SMs that the
     // previous lattice's CTAs leave when its items run out (they read nothing
     // it writes), so the three launches share one tail instead of one each
-    const bool v_rows = fused && io && node_bytes > 0;
+    const bool v_rows = fused && !reproducible(ctx) && io && node_bytes > 0;
     if (v_rows) {
         const size_t row = node_bytes / 3;
         for (int d = 0; d < 3; ++d) {
@@ -1611,7 +1637,7 @@ static int autotune(ifem_ctx ctx, ifem_batch b, const void *x, void *stream)
             cudaEventRecord(e0, s);
             if ((rc = do_bin(ctx, b, g, x, stream, BIN_ALL, F)) == IFEM_OK) {
                 // the transfer launches the step will use (fused where it fuses)
-                if (use_halo(ctx))
+                if (ctx->cfg.precision == IFEM_FP32)
                     rc = do_spread_interp(ctx, b, x, F, u, f, v, 0, stream);
                 else if ((rc = do_spread(ctx, b, x, F, f, 0, stream)) == IFEM_OK)
                     rc = do_interp(ctx, b, u, x, v, stream);

@@ -21,6 +21,7 @@ constexpr int kOwnSub3 = kOwnSub * kOwnSub * kOwnSub;
 constexpr int kScanThreads = 512;  // tile-count scan: threads per block
 constexpr int kScanPer = 4;        // and values per thread
 constexpr int kScanBlock = kScanThreads * kScanPer;
+constexpr int kFsumBins = 8;       // DevWork::tile_fbin entries per sum
 constexpr int kCounters = 16;      // DevWork::counters entries
 constexpr int kMaxCtaSmemBytes = 227 * 1024;   // opt-in dynamic shared memory of one CTA
 // FP32 nodal force kernel: a float4 (position, mean curvature) of shared
@@ -125,17 +126,25 @@ struct DetW {
 };
 static_assert(sizeof(DetW) == 336, "DetW layout");
 
-// A tile with own nodes (FP32 halo path), as the transfer needs it.
+// A tile with own nodes (FP32), as the transfer needs it.
 struct alignas(16) TileDesc {
     int tile, n, beg, end;   // tile number, cells per box side, own records [beg, end)
     int start[3], edge[3];   // first cell and cells per axis
     long long grid_off;      // the box's offset in a grid field
     double h3;               // (L/n)^3
     float scale_f;           // (n/L)^3
-    int pad;
+    int slot;                // its place in the list
 };
 static_assert(sizeof(TileDesc) == 64, "TileDesc layout");
 
+// FP32 tile transfer: width of the shared boxes in y and z (4 more in x) for
+// tiles of at most max_edge cells, and bytes of a box.
+__host__ __device__ inline int tile_width(int max_edge) { return max_edge <= 8 ? 12 : (max_edge <= 12 ? 16 : 20); }
+__host__ __device__ inline size_t tile_box_bytes(int max_edge)
+{
+    const size_t w = tile_width(max_edge);
+    return 4 * (w + 4) * w * w;
+}
 struct DevWork {
     int *cand_count;    // n_tiles + 1
     int *cand_off;      // n_tiles + 1
@@ -144,24 +153,29 @@ struct DevWork {
     long long cand_cap;
     int *own_count;     // per (tile, 4^3 sub-block): n_tiles * kOwnSub3 + 1; in one piece with red_tile
                         // and counters before it and, after it, own_flag and tile_fsum or cand_count
-    int *own_flag;      // n_tiles (FP32 halo path): 1 where the tile owns a node
-    float *tile_fsum;   // 3 per tile (FP32 halo path): sum of |F_d| over the tile's own nodes, from the
-                        // placement when it is given the forces (the fused transfer's fixed-point scale)
-    int *own_off;       // n_tiles * kOwnSub3 + 1 offsets (not in the FP32 halo path)
-    int *own_cursor;    // fill cursors; local (per scan block) offsets in the FP32 halo path
+    int *own_flag;      // n_tiles (FP32): 1 where the tile owns a node
+    float *tile_fsum;   // 3 per tile (FP32): sum of |F_d| over the tile's own nodes, from the
+                        // placement when it is given the forces (the transfer's fixed-point scale)
+    unsigned long long *tile_fbin;   // the same for the reproducible spread: kFsumBins integers each
+    int *own_off;       // n_tiles * kOwnSub3 + 1 offsets (FP64)
+    int *own_cursor;    // fill cursors; local (per scan block) offsets in the FP32
     int *own_nodes;     // N entries: nodes grouped by the tile (and sub-block) of their cell (not in
-                        // the FP32 halo path)
-    float4 *own_rec;    // FP32 halo path, 2 per node in that grouping: fractional cell coordinates
+                        // the FP32)
+    float4 *own_rec;    // FP32, 2 per node in that grouping: fractional cell coordinates
                         // x, y, z of the node and, in w, its cell within the tile packed as 8-bit
                         // x | y << 8 | z << 16; its force and, in w, its id
-    int2 *node_key;     // N entries, by node (FP32 halo path): own-list key (-1: not binned) and
+    int2 *node_key;     // N entries, by node (FP32): own-list key (-1: not binned) and
                         // the node's rank among the nodes of that key
-    float4 *node_rec;   // N entries, by node (FP32 halo path): the first float4 of its own_rec entry
+    float4 *node_rec;   // N entries, by node (FP32): the first float4 of its own_rec entry
     int *active;        // tiles with candidate pairs
-    TileDesc *tile_desc;  // tiles with own nodes (FP32 halo path), counters[3] of them
+    TileDesc *tile_desc;  // tiles with own nodes (FP32), counters[3] of them
+    int *tile_slot;     // n_tiles (FP32): a tile's place in that list, or -1
+    int2 *near_tile;    // reproducible spread: tiles that a box reaches and their boxes, counters[9] of them
+    float *box_buf;     // reproducible spread: a box per listed tile and lattice
+    float *field;       // reproducible spread onto a field that is not cleared: the field it is spread into
     int *counters;      // kCounters: [0] n_active, [2] work counter, [3] tiles with own nodes,
                         // [4] total pairs, [5] total own nodes, [1] [6] [7] work counters of
-                        // one-lattice launches, [8] scan blocks finished
+                        // one-lattice launches, [8] scan blocks finished, [9] near_tile entries
     int *scan_blocks;   // block partial sums for the tile scan
     void *elem_buf;     // per element nodal forces (12 reals per element)
     void *bend_buf;     // per node bending scratch (A, kH, n[3], lap) 6 reals
@@ -381,8 +395,9 @@ struct TransferArgs {
     int density;
     double support;
     int n_sm;
-    int acc64;        // FP32 spread: 64-bit (1) or 32-bit (0) fixed-point accumulators
-    int halo;         // FP32 Peskin, IFEM_SCATTER_ATOMIC: the tile transfer over own lists
+    int store;        // FP32: reproducible spread through the boxes of every tile
+    int cleared;      // f is zero before the spread
+    long long total;  // values of the grid
     int clear_sums;   // binning: a spread follows, clear its per-tile sums too
     int lattice;      // tile transfer: -1 all three lattices, else that lattice only
     int pdl;          // tile transfer: may start before the previous kernel in the stream ends
@@ -410,10 +425,10 @@ cudaError_t launch_forces_f32(const ForcesArgs &a);
 cudaError_t launch_forces_f64(const ForcesArgs &a);
 // Binning in two parts: the clears, the count pass and the scan, then the
 // placement (which also sums |F| per tile when TransferArgs::F is given).
-// Only the FP32 halo path (with_cand = 0) takes them apart.
+// Only the FP32 binning takes them apart.
 enum BinStage { BIN_COUNT = 1, BIN_PLACE = 2, BIN_ALL = 3 };
-cudaError_t launch_bin_f32(const TransferArgs &a, int det_sort, int with_cand, int stages = BIN_ALL);
-cudaError_t launch_bin_f64(const TransferArgs &a, int det_sort, int with_cand, int stages = BIN_ALL);
+cudaError_t launch_bin_f32(const TransferArgs &a, int stages = BIN_ALL);
+cudaError_t launch_bin_f64(const TransferArgs &a, int stages = BIN_ALL);
 cudaError_t launch_spread_f32(const TransferArgs &a);
 cudaError_t launch_spread_f64(const TransferArgs &a);
 cudaError_t launch_interp_f32(const TransferArgs &a);

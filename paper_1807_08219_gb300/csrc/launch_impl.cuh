@@ -96,19 +96,23 @@ cudaError_t forces_impl(const ForcesArgs &a)
     return cudaSuccess;
 }
 
+// Binning. FP32: one-pass own lists (count, scan, placement; the stages can be
+// launched apart). FP64: candidate and own lists, the candidates sorted, and
+// the Peskin stencil table.
 template <typename real>
-cudaError_t bin_impl(const TransferArgs &a, int det_sort, int with_cand, int stages)
+cudaError_t bin_impl(const TransferArgs &a, int stages)
 {
     const DevBatch &b = a.b;
     const DevWork &w = a.w;
     const long long nt = a.g.n_tiles;
     cudaStream_t s = a.stream;
     const long long no = nt * kOwnSub3;
-    if (with_cand && stages != BIN_ALL)
+    constexpr bool f32 = std::is_same<real, float>::value;
+    if (!f32 && stages != BIN_ALL)
         return cudaErrorInvalidValue;
     const bool empty = b.n_inst == 0 || b.N == 0;
     dim3 gn((b.max_nodes + 255) / 256, b.n_inst);
-    // one-pass binning of the FP32 halo path: kBinPer nodes per thread
+    // one-pass binning: kBinPer nodes per thread
     dim3 g1((b.max_nodes + 256 * kBinPer - 1) / (256 * kBinPer), b.n_inst);
     if (stages & BIN_COUNT) {
         // one clear: the counters, counts and per-tile |F| sums, and before them
@@ -120,42 +124,33 @@ cudaError_t bin_impl(const TransferArgs &a, int det_sort, int with_cand, int sta
         IFEM_LAUNCH_CHECK();
         if (empty)
             return cudaSuccess;
-        if (with_cand) {
+        if constexpr (f32)
+            own_count_kernel<<<g1, 256, 0, s>>>(b, a.g, w, (const float *)a.x);
+        else
             bin_kernel<real, false><<<gn, 256, 0, s>>>(b, a.g, w, (const real *)a.x);
-        } else {
-            if constexpr (!std::is_same<real, float>::value)
-                return cudaErrorInvalidValue;   // the one-pass own lists are FP32 only
-            else
-                own_count_kernel<<<g1, 256, 0, s>>>(b, a.g, w, (const float *)a.x);
-        }
         IFEM_LAUNCH_CHECK();
         int nb = (int)((no + kScanBlock - 1) / kScanBlock);
-        // without candidate lists the local own offsets go to the cursors, and
-        // own_scatter_kernel writes the final offsets beside them
-        scan_local_kernel<<<nb, kScanThreads, 0, s>>>(with_cand ? nt : 0, no, w.cand_count, w.own_count, w.cand_off,
-                                                      with_cand ? w.own_off : w.own_cursor, w.scan_blocks,
+        // FP32: the local own offsets go to the cursors (own_scatter_kernel adds the block offsets)
+        scan_local_kernel<<<nb, kScanThreads, 0, s>>>(f32 ? 0 : nt, no, w.cand_count, w.own_count, w.cand_off,
+                                                      f32 ? w.own_cursor : w.own_off, w.scan_blocks,
                                                       w.counters + 8, w.counters + 4);
         IFEM_LAUNCH_CHECK();
     }
     if (empty || !(stages & BIN_PLACE))
         return cudaSuccess;
-    if (with_cand) {
+    if constexpr (f32) {
+        // enough threads for every tile as well as every node
+        const long long per_inst = ((nt + 255) / 256 + b.n_inst - 1) / b.n_inst;
+        dim3 gs((unsigned)std::max<long long>(g1.x, per_inst), b.n_inst);
+        own_scatter_kernel<<<gs, 256, 0, s>>>(b, a.g, w, (const float *)a.F, a.store);
+        IFEM_LAUNCH_CHECK();
+    } else {
         scan_finish_kernel<<<(unsigned)((no + 1 + 255) / 256), 256, 0, s>>>(nt, no, w);
         IFEM_LAUNCH_CHECK();
         bin_kernel<real, true><<<gn, 256, 0, s>>>(b, a.g, w, (const real *)a.x);
         IFEM_LAUNCH_CHECK();
-    } else {
-        // enough threads for every tile as well as every node
-        const long long per_inst = ((nt + 255) / 256 + b.n_inst - 1) / b.n_inst;
-        dim3 gs((unsigned)std::max<long long>(g1.x, per_inst), b.n_inst);
-        own_scatter_kernel<<<gs, 256, 0, s>>>(b, a.g, w, (const float *)a.F);
-        IFEM_LAUNCH_CHECK();
-    }
-    if (det_sort) {
         sort_segments_kernel<<<a.n_sm * 4, 512, 0, s>>>(w);
         IFEM_LAUNCH_CHECK();
-    }
-    if constexpr (std::is_same<real, double>::value) {
         if (a.kernel == 0 && w.wtab) {
             det_weights_kernel<<<(unsigned)((3 * b.N + 255) / 256), 256, 0, s>>>(b, a.g, w.wtab, (const double *)a.x);
             IFEM_LAUNCH_CHECK();
@@ -164,13 +159,13 @@ cudaError_t bin_impl(const TransferArgs &a, int det_sort, int with_cand, int sta
     return cudaSuccess;
 }
 
-// The FP32 Peskin tile transfer over the own lists of the binning just before
-// it: spreading (SPREAD), interpolation (INTERP) or both, with the position
-// update (AB2) on request. One resident wave of CTAs takes the items.
-template <int W, bool SPREAD, bool INTERP, bool AB2>
+// The FP32 tile transfer over the own lists of the binning just before it:
+// spreading (SPREAD), interpolation (INTERP) or both. One resident wave of CTAs
+// takes the items.
+template <int KER, int W, bool SPREAD, bool INTERP, bool STORE>
 cudaError_t launch_tile_w(const TransferArgs &a)
 {
-    auto kern = transfer_tile_kernel<W, SPREAD, INTERP, AB2>;
+    auto kern = transfer_tile_kernel<KER, W, SPREAD, INTERP, STORE>;
     constexpr int kKinds = (SPREAD ? 1 : 0) + (INTERP ? 1 : 0), T = TileShape<W>::kThreads;
     const size_t sm = (size_t)4 * TileShape<W>::kWords * 2 * kKinds;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -178,6 +173,13 @@ cudaError_t launch_tile_w(const TransferArgs &a)
         return e;
     int occ = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, T, sm);
+    float *f = (float *)a.f;
+    if (STORE && !a.cleared) {
+        f = a.w.field;
+        if ((e = cudaMemsetAsync(f, 0, sizeof(float) * (size_t)a.total, a.stream)) != cudaSuccess)
+            return e;
+        IFEM_LAUNCH_CHECK();
+    }
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     // programmatic dependent launch: the CTAs of this grid may start once
@@ -192,19 +194,31 @@ cudaError_t launch_tile_w(const TransferArgs &a)
     cfg.stream = a.stream;
     cfg.attrs = attr;
     cfg.numAttrs = a.pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, a.b, a.w, (const float *)a.x, (float *)a.f, a.density, (const float *)a.u,
-                              (float *)a.v, (const float *)a.vp, (float *)a.xn, (float)a.dt, a.lattice);
+    e = cudaLaunchKernelEx(&cfg, kern, a.b, a.w, (const float *)a.x, f, a.density, (const float *)a.u,
+                           (float *)a.v, (const float *)a.vp, (float *)a.xn, (float)a.dt, (float)(1.0 / a.support),
+                           a.lattice);
+    if (e != cudaSuccess || !STORE)
+        return e;
+    const long long units = 3 * std::min<long long>(a.g.n_tiles, 27 * a.b.N);
+    const long long blocks = std::min(units, 8LL * a.n_sm);   // all resident
+    tile_combine_kernel<W><<<(unsigned)blocks, kCombineThreads, 0, a.stream>>>(a.g, a.w, f);
+    IFEM_LAUNCH_CHECK();
+    if (!a.cleared) {
+        add_field_kernel<<<8 * a.n_sm, 256, 0, a.stream>>>((float *)a.f, f, a.total);
+        IFEM_LAUNCH_CHECK();
+    }
+    return cudaSuccess;
 }
-template <bool SPREAD, bool INTERP, bool AB2>
+template <int KER, bool SPREAD, bool INTERP, bool STORE>
 cudaError_t launch_tile(const TransferArgs &a)
 {
     switch (tile_width(a.g.max_edge)) {
     case 12:
-        return launch_tile_w<12, SPREAD, INTERP, AB2>(a);
+        return launch_tile_w<KER, 12, SPREAD, INTERP, STORE>(a);
     case 16:
-        return launch_tile_w<16, SPREAD, INTERP, AB2>(a);
+        return launch_tile_w<KER, 16, SPREAD, INTERP, STORE>(a);
     default:
-        return launch_tile_w<20, SPREAD, INTERP, AB2>(a);
+        return launch_tile_w<KER, 20, SPREAD, INTERP, STORE>(a);
     }
 }
 
@@ -216,24 +230,14 @@ cudaError_t spread_impl(const TransferArgs &a)
     if (b.n_inst == 0 || b.N == 0)
         return cudaSuccess;
     if constexpr (std::is_same<real, float>::value) {
-        const int E = a.g.max_edge;
-        if (a.halo) {
-            // with u and v given, interpolation is fused into the spread, and
-            // with xn also the position update
-            if (!(a.u && a.v))
-                return launch_tile<true, false, false>(a);
-            return a.xn ? launch_tile<true, true, true>(a) : launch_tile<true, true, false>(a);
-        }
-        size_t acc = a.acc64 ? sizeof(long long) : sizeof(int);
-        size_t sm = acc * 3 * (size_t)acc_stride(E, E, E);
-        auto kern = a.kernel == 0 ? (a.acc64 ? spread_fast_kernel<0, long long> : spread_fast_kernel<0, int>)
-                                  : (a.acc64 ? spread_fast_kernel<1, long long> : spread_fast_kernel<1, int>);
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        int occ = 1;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 256, sm);
-        occ = occ < 1 ? 1 : occ;
-        kern<<<a.n_sm * occ, 256, sm, s>>>(b, a.g, a.w, (const float *)a.x, (const float *)a.F, (float *)a.f,
-                                           a.density, (float)a.support);
+        // with u and v given, interpolation is fused into the spread (the MLS
+        // spread is reproducible in both scatter modes)
+        const bool fused = a.u != nullptr && a.v != nullptr;
+        if (a.kernel == 1)
+            return fused ? launch_tile<1, true, true, true>(a) : launch_tile<1, true, false, true>(a);
+        if (a.store)
+            return fused ? launch_tile<0, true, true, true>(a) : launch_tile<0, true, false, true>(a);
+        return fused ? launch_tile<0, true, true, false>(a) : launch_tile<0, true, false, false>(a);
     } else {
         if (a.kernel == 0) {
             // warp per (tile, lattice) over the binning's stencil table
@@ -273,25 +277,16 @@ cudaError_t interp_impl(const TransferArgs &a)
     if (b.n_inst == 0 || b.N == 0)
         return cudaSuccess;
     if constexpr (std::is_same<real, float>::value) {
-        unsigned grid = (unsigned)((3 * b.N + 255) / 256);
-        if (a.halo)
-            return launch_tile<false, true, false>(a);
-        if (a.kernel == 0)
-            interp_direct_kernel<0><<<grid, 256, 0, a.stream>>>(b, a.g, a.w, (const float *)a.u, (const float *)a.x,
-                                                               (float *)a.v, (float)a.support);
-        else
-            interp_direct_kernel<1><<<grid, 256, 0, a.stream>>>(b, a.g, a.w, (const float *)a.u, (const float *)a.x,
-                                                               (float *)a.v, (float)a.support);
+        return a.kernel == 0 ? launch_tile<0, false, true, false>(a) : launch_tile<1, false, true, false>(a);
     } else {
         unsigned grid = (unsigned)((b.N + 255) / 256);
         if (a.kernel == 0)
-            interp_kernel<real, true, 0><<<grid, 256, 0, a.stream>>>(b, a.g, a.w, (const real *)a.u,
-                                                                    (const real *)a.x, (real *)a.v, (real)a.support, 0,
+            interp_kernel<real, 0><<<grid, 256, 0, a.stream>>>(b, a.g, a.w, (const real *)a.u,
+                                                                    (const real *)a.x, (real *)a.v, (real)a.support,
                                                                     a.use_wtab && a.w.wtab != nullptr);
         else
-            interp_kernel<real, true, 1><<<grid, 256, 0, a.stream>>>(b, a.g, a.w, (const real *)a.u,
-                                                                    (const real *)a.x, (real *)a.v, (real)a.support, 0,
-                                                                    0);
+            interp_kernel<real, 1><<<grid, 256, 0, a.stream>>>(b, a.g, a.w, (const real *)a.u,
+                                                                    (const real *)a.x, (real *)a.v, (real)a.support, 0);
     }
     IFEM_LAUNCH_CHECK();
     return cudaSuccess;

@@ -150,7 +150,7 @@ __device__ __forceinline__ int agg_append(int *count, int *cursor, int *list, lo
     return slot;
 }
 
-// One-pass own-list binning (FP32 halo path): per node its rank within its
+// One-pass own-list binning (FP32): per node its rank within its
 // own-list key (the old value of the key's count, one atomic per group of
 // lanes with the same key) and its record -- fractional lattice coordinates
 // and cell within the tile, 8-bit x | y << 8 | z << 16 -- kept by node for
@@ -222,9 +222,8 @@ static __global__ void __launch_bounds__(256) own_count_kernel(DevBatch b, DevGr
 }
 
 // FILL = false: count candidate / own pairs per tile; FILL = true: write them
-// (paths with candidate lists; the FP32 halo path bins with own_count_kernel
-// and own_scatter_kernel). Block size must be a multiple of 32 (every lane
-// reaches the warp votes).
+// (FP64; FP32 bins with own_count_kernel and own_scatter_kernel). Block size
+// must be a multiple of 32 (every lane reaches the warp votes).
 template <typename real, bool FILL>
 __global__ void bin_kernel(DevBatch b, DevGrid g, DevWork w, const real *__restrict__ x)
 {
@@ -265,8 +264,8 @@ __global__ void bin_kernel(DevBatch b, DevGrid g, DevWork w, const real *__restr
 
 // Exclusive scan of the per-tile counts (two lists at once): block-local
 // scan, whose last block to finish scans the block sums -> add + cursors +
-// active lists (scan_finish_kernel; in the FP32 halo path
-// own_scatter_kernel adds the block offsets itself).
+// active lists (scan_finish_kernel; in FP32 own_scatter_kernel adds the block
+// offsets itself).
 
 __device__ inline int block_exclusive_scan(int v, int *sh, int &total)
 {
@@ -539,29 +538,6 @@ __device__ __forceinline__ void df_add_prod(DF &x, float a, float b)
     x.lo += pe;
 }
 
-// ---------------------------------------------------- spread, FP32 fast
-// One CTA per active tile, tiles taken from a global counter. Contributions
-// are accumulated in shared memory as fixed-point integers (Acc = int or
-// long long) with native integer atomics: integer addition is associative,
-// so the accumulated tile is independent of the order in which threads add
-// (the FP32 result is reproducible run to run). Per tile and lattice the
-// scale is a power of two chosen from a bound on the largest possible sum,
-// |f_J| <= wmax * sum_k |g_k| over the tile's candidates, so no sum can
-// overflow. Work units are (candidate node, lattice) pairs. Flush: one
-// read-modify-write per non-zero owned value, rows of x in lanes.
-template <typename Acc>
-struct FixedPoint;
-template <>
-struct FixedPoint<int> {
-    static constexpr float kRange = 1073741824.0f;  // 2^30
-    __device__ static __forceinline__ int conv(float v) { return __float2int_rn(v); }
-};
-template <>
-struct FixedPoint<long long> {
-    static constexpr float kRange = 1152921504606846976.0f;  // 2^60
-    __device__ static __forceinline__ long long conv(float v) { return __float2ll_rn(v); }
-};
-
 // The four Peskin weights of one axis share one square root: with
 // r = s - floor(s) in [0, 1) and q = sqrt(1 + 4r - 4r^2),
 //   phi(1 + r) = (3 - 2r - q)/8, phi(r) = (3 - 2r + q)/8,
@@ -585,8 +561,6 @@ __device__ __forceinline__ int peskin_axis_fast(float s, float ph[4])
     return (int)fl - 1;
 }
 
-__device__ __forceinline__ void acc_add(int *p, int v) { atomicAdd(p, v); }
-
 // Fire-and-forget adds performed at L2 (no value returned, so the SM does not
 // wait for the line): the tile flush adds its sums to the grid this way.
 __device__ __forceinline__ void red_add_v4(float *p, float a, float b, float c, float d)
@@ -598,17 +572,6 @@ __device__ __forceinline__ void red_add_v4(float *p, float a, float b, float c, 
 __device__ __forceinline__ void red_add(float *p, float a)
 {
     asm volatile("red.global.add.f32 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "f"(a) : "memory");
-}
-
-// Shared-memory pitches of a tile accumulator: odd row and plane pitches
-// spread the atomics of neighbouring nodes over the 32 banks.
-__host__ __device__ inline int acc_px(int ex) { return ex | 1; }
-__host__ __device__ inline int acc_pp(int ey, int px) { return (ey * px) | 1; }
-__host__ __device__ inline int acc_stride(int ex, int ey, int ez) { return ez * acc_pp(ey, acc_px(ex)); }
-// two's-complement addition through the unsigned 64-bit atomic
-__device__ __forceinline__ void acc_add(long long *p, long long v)
-{
-    atomicAdd(reinterpret_cast<unsigned long long *>(p), (unsigned long long)v);
 }
 
 // n-periodic wrap of an index that is normally already in (-n, 2n)
@@ -623,262 +586,46 @@ __device__ __forceinline__ int wrap_near(int v, int n)
     return v;
 }
 
-template <int KER, typename Acc>
-__global__ void __launch_bounds__(256) spread_fast_kernel(DevBatch b, DevGrid g, DevWork w,
-                                                          const float *__restrict__ x,
-                                                          const float *__restrict__ F, float *__restrict__ f,
-                                                          int density, float support)
+// Periodic wrap of a box coordinate in [-n, 2n): the boxes of a grid have
+// at least 8 cells and the halos at most 4, so one correction suffices.
+__device__ __forceinline__ int wrap1(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
+
+// A sum of non-negative floats that does not depend on their order: 64-bit
+// integers, one per 32 binades, in units of 2^(32 bin - 131), values rounded up
+// to them (at most 2^-4 of a value at the low end of a bin; 2^27 of the largest
+// values fit). A value that is not finite counts as the largest float.
+__device__ __forceinline__ void fsum_add(unsigned long long *bins, float v)
 {
-    extern __shared__ __align__(16) unsigned char spread_smem[];
-    Acc *acc = reinterpret_cast<Acc *>(spread_smem);
-    __shared__ float s_part[3][8];
-    __shared__ float s_scale[3];
-    __shared__ double s_red[3][8];
-    __shared__ int s_tile;
-    __shared__ TileInfo s_ti;
-    __shared__ BoxDev s_B;
-    const long long N = b.N;
-    const int n_active = w.counters[0];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        status_add(w.status, ST_PAIRS, (unsigned long long)w.cand_off[g.n_tiles]);
-        status_add(w.status, ST_ACTIVE, (unsigned long long)n_active);
+    if (!(v <= 3.402823466e38f))
+        v = 3.402823466e38f;
+    if (v == 0.f)
+        return;
+    const int bin = __float_as_int(v) >> 28;   // exponent field / 32
+    // the unit's reciprocal in two factors that are floats
+    const float q = ceilf(v * __int_as_float((127 + 67 - 16 * bin) << 23) * __int_as_float((127 + 64 - 16 * bin) << 23));
+    atomicAdd(bins + bin, (unsigned long long)q);
+}
+__device__ __forceinline__ float fsum_get(const unsigned long long *__restrict__ bins)
+{
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < kFsumBins; ++k) {
+        const unsigned long long q = bins[k];
+        if (q)
+            s += (double)q * __hiloint2double((1023 + 32 * k - 131) << 20, 0);
     }
-    // accumulators start at zero; the flush of every tile clears what it read
-    {
-        const int E = g.max_edge;
-        for (int i = threadIdx.x; i < 3 * acc_stride(E, E, E); i += blockDim.x)
-            acc[i] = 0;
-    }
-    for (;;) {
-        if (threadIdx.x == 0) {
-            int it = atomicAdd(&w.counters[2], 1);
-            s_tile = it < n_active ? w.active[it] : -1;
-            if (it < n_active) {
-                s_ti = decode_tile(g, s_tile);
-                s_B = g.boxes[s_ti.box];
-            }
-        }
-        __syncthreads();
-        const int tile = s_tile;
-        if (tile < 0)
-            break;
-        const int ex = s_ti.edge[0], ey = s_ti.edge[1], ez = s_ti.edge[2];
-        const int sx = s_ti.start[0], sy = s_ti.start[1], sz = s_ti.start[2];
-        const int px = acc_px(ex), pp = acc_pp(ey, px);
-        const int vol = ez * pp;   // per-lattice stride of the padded accumulator
-        const int n = s_B.n;
-        const float sd = density ? s_B.scale_f : 1.f;
-        const double h3 = 1.0 / s_B.scale;
-        const int beg = w.cand_off[tile], end = w.cand_off[tile + 1];
-        // bound on |sum| per lattice: wmax * sum_k |F_k,d| * sd
-        float gs0 = 0.f, gs1 = 0.f, gs2 = 0.f;
-        for (int q = beg + threadIdx.x; q < end; q += blockDim.x) {
-            const int node = w.cand_nodes[q];
-            gs0 += fabsf(F[node]);
-            gs1 += fabsf(F[N + node]);
-            gs2 += fabsf(F[2 * N + node]);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            gs0 += __shfl_down_sync(0xffffffffu, gs0, o);
-            gs1 += __shfl_down_sync(0xffffffffu, gs1, o);
-            gs2 += __shfl_down_sync(0xffffffffu, gs2, o);
-        }
-        if (lane == 0) {
-            s_part[0][wid] = gs0;
-            s_part[1][wid] = gs1;
-            s_part[2][wid] = gs2;
-        }
-        __syncthreads();
-        if (threadIdx.x < 3) {
-            float tot = 0.f;
-            for (int q = 0; q < nw; ++q)
-                tot += s_part[threadIdx.x][q];
-            // |phi| <= 1/8 (Peskin: (1/2)^3); MLS weights are non-negative, sum to 1
-            // and stay below 1/2 in practice; the bound sums over every candidate
-            // of the tile, far above what any single value receives
-            const float wmax = KER == 0 ? 0.125f : 0.5f;
-            float bound = tot * sd * wmax * 1.0001f;
-            float sc = 1.f;
-            if (bound > 0.f && isfinite(bound)) {
-                int e = (int)floorf(log2f(FixedPoint<Acc>::kRange / bound));
-                e = e > 120 ? 120 : (e < -120 ? -120 : e);
-                sc = exp2f((float)e);
-            }
-            s_scale[threadIdx.x] = sc;
-        }
-        __syncthreads();
-#pragma unroll 1
-        for (int d = 0; d < 3; ++d) {
-            Acc *accd = acc + d * vol;
-            const float gsc = sd * s_scale[d];
-            for (int q = beg + threadIdx.x; q < end; q += blockDim.x) {
-                const int node = w.cand_nodes[q];
-                const InstDev &I = b.inst[b.node_inst[node]];
-                const float gq = F[d * N + node] * gsc;
-                if constexpr (KER == 0) {
-                    float ph[3][4];
-                    int l[3][4];
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        const int I0 = I.I0[a];
-                        const float s = (I.f0[a] - (a == d ? 0.f : 0.5f)) + x[a * N + node] * s_B.inv_h_f;
-                        const int base = wrap_near(I0 + peskin_axis_fast(s, ph[a]), n);
-                        const int st = a == 0 ? sx : (a == 1 ? sy : sz);
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) {
-                            int idx = base + m;
-                            idx -= idx >= n ? n : 0;
-                            l[a][m] = idx - st;
-                        }
-                    }
-                    // validity bit masks; every slot runs, the atomic is predicated
-                    // (no divergent branches around the 64 slots)
-                    unsigned okx = 0, oky = 0, okz = 0;
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        okx |= (unsigned)((unsigned)l[0][m] < (unsigned)ex) << m;
-                        oky |= (unsigned)((unsigned)l[1][m] < (unsigned)ey) << m;
-                        okz |= (unsigned)((unsigned)l[2][m] < (unsigned)ez) << m;
-                    }
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const float wz = ph[2][c] * gq;
-#pragma unroll
-                        for (int bb = 0; bb < 4; ++bb) {
-                            const float wyz = ph[1][bb] * wz;
-                            const unsigned rowok = (okz >> c) & (oky >> bb) & 1u;
-                            const int row = l[2][c] * pp + l[1][bb] * px;
-#pragma unroll
-                            for (int a = 0; a < 4; ++a) {
-                                const Acc qv = FixedPoint<Acc>::conv(ph[0][a] * wyz);
-                                if (rowok & (okx >> a))
-                                    acc_add(accd + row + l[0][a], qv);
-                            }
-                        }
-                    }
-                } else {
-                    float s[3];
-#pragma unroll
-                    for (int a = 0; a < 3; ++a)
-                        s[a] = (I.f0[a] - (a == d ? 0.f : 0.5f)) + x[a * N + node] * s_B.inv_h_f;
-                    int base[3];
-                    float wt[27];
-                    if (!mls_weights<float>(s, support, base, wt)) {
-                        status_add(w.status, ST_DOMAIN, 1);
-                        continue;
-                    }
-                    int l[3][3];
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        const int bw = wrap_near(I.I0[a] + base[a], n);
-                        const int st = a == 0 ? sx : (a == 1 ? sy : sz);
-#pragma unroll
-                        for (int m = 0; m < 3; ++m) {
-                            int idx = bw + m;
-                            idx -= idx >= n ? n : 0;
-                            l[a][m] = idx - st;
-                        }
-                    }
-                    int J = 0;
-#pragma unroll
-                    for (int c = 0; c < 3; ++c)
-#pragma unroll
-                        for (int bb = 0; bb < 3; ++bb)
-#pragma unroll
-                            for (int a = 0; a < 3; ++a, ++J)
-                                if ((unsigned)l[2][c] < (unsigned)ez && (unsigned)l[1][bb] < (unsigned)ey &&
-                                    (unsigned)l[0][a] < (unsigned)ex)
-                                    acc_add(accd + l[2][c] * pp + l[1][bb] * px + l[0][a],
-                                            FixedPoint<Acc>::conv(wt[J] * gq));
-                }
-            }
-        }
-        __syncthreads();
-        // flush: per lattice, every row (z, y) of the tile, x in quads when the
-        // rows are 16-byte aligned; non-zero sums are added to the grid with
-        // L2 reductions (each value belongs to this tile only) and cleared
-        const long long n3 = (long long)n * n * n;
-        unsigned touched = 0;
-        // quads need 16-byte aligned rows: box field base, n, tile start and
-        // edge all multiples of 4 floats
-        const bool vec = ((sx | n | ex) & 3) == 0 &&
-                         ((reinterpret_cast<uintptr_t>(f + s_B.grid_off)) & 15) == 0;
-        const int nq = vec ? (ex >> 2) : ex;
-        const int items = ey * ez * nq;
-#pragma unroll 1
-        for (int d = 0; d < 3; ++d) {
-            const float inv = 1.f / s_scale[d];
-            DF part{0.f, 0.f};
-            float *fd = f + s_B.grid_off + d * n3;
-            Acc *ad = acc + d * vol;
-            for (int item = threadIdx.x; item < items; item += blockDim.x) {
-                const int r = item / nq, qx = item - r * nq;
-                const int lz = r / ey, ly = r - lz * ey;
-                Acc *src = ad + lz * pp + ly * px;
-                float *dst = fd + ((long long)(sz + lz) * n + (sy + ly)) * n + sx;
-                if (vec) {
-                    const int x0 = qx << 2;
-                    const Acc q0 = src[x0], q1 = src[x0 + 1], q2 = src[x0 + 2], q3 = src[x0 + 3];
-                    if ((q0 | q1 | q2 | q3) != 0) {
-                        src[x0] = 0;
-                        src[x0 + 1] = 0;
-                        src[x0 + 2] = 0;
-                        src[x0 + 3] = 0;
-                        const float v0 = (float)q0 * inv, v1 = (float)q1 * inv, v2 = (float)q2 * inv,
-                                    v3 = (float)q3 * inv;
-                        red_add_v4(dst + x0, v0, v1, v2, v3);
-                        df_add(part, v0);
-                        df_add(part, v1);
-                        df_add(part, v2);
-                        df_add(part, v3);
-                        touched += (q0 != 0) + (q1 != 0) + (q2 != 0) + (q3 != 0);
-                    }
-                } else {
-                    const Acc q = src[qx];
-                    if (q != 0) {
-                        src[qx] = 0;
-                        const float v = (float)q * inv;
-                        red_add(dst + qx, v);
-                        df_add(part, v);
-                        ++touched;
-                    }
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float hi = __shfl_down_sync(0xffffffffu, part.hi, o);
-                const float lo = __shfl_down_sync(0xffffffffu, part.lo, o);
-                df_add(part, hi);
-                part.lo += lo;
-            }
-            if (lane == 0)
-                s_red[d][wid] = (double)part.hi + (double)part.lo;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            touched += __shfl_down_sync(0xffffffffu, touched, o);
-        if (lane == 0)
-            status_add(w.status, ST_TOUCHED, touched);
-        __syncthreads();
-        if (threadIdx.x < 3) {
-            double v = 0.0;
-            for (int q = 0; q < nw; ++q)
-                v += s_red[threadIdx.x][q];
-            w.red_tile[3LL * tile + threadIdx.x] = v * h3;
-        }
-        // the next iteration's barrier orders these reads before s_red is rewritten
-    }
+    return (float)s;
 }
 
-// FP32 halo path, after the scan: every binned node goes to its slot (the
+// FP32, after the scan: every binned node goes to its slot (the
 // scanned offset of its key plus its rank from own_count_kernel) as one
 // 32-byte record: what own_count_kernel kept of it, its force (0 without F)
 // and its id, kBinPer nodes per thread as in own_count_kernel (loads first,
 // then the offsets, then the stores). With the force in the record the
 // transfer reads its nodes in two consecutive 16-byte loads, without a gather
-// through the node id. The tiles that own nodes are listed, counters[3] of them, with everything the
+// through the node id. The tiles that own nodes are listed (tile_slot: a
+// tile's place in the list, or -1; for a reproducible spread also the tiles that
+// a box reaches, near_tile, counters[9] of them), counters[3] of them, with everything the
 // transfer needs of a tile: it fetches an item in one copy, without walking
 // empty tiles or decoding tile numbers. The list keeps roughly the tile order
 // (in order within each warp's append), so items running at the same time are
@@ -893,7 +640,7 @@ __global__ void __launch_bounds__(256) spread_fast_kernel(DevBatch b, DevGrid g,
 // not fixed; the transfer's bound allows for it).
 // Grid: as own_count_kernel along x and y, at least n_tiles threads in all.
 static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, DevGrid g, DevWork w,
-                                                                 const float *__restrict__ F)
+                                                                 const float *__restrict__ F, int det)
 {
     const InstDev I = b.inst[blockIdx.y];
     const long long N = b.N;
@@ -953,8 +700,12 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
             }
             if (tile >= 0 && (lane == 31 || next != tile)) {
 #pragma unroll
-                for (int d = 0; d < 3; ++d)
-                    atomicAdd(&w.tile_fsum[3LL * tile + d], fa[j][d]);
+                for (int d = 0; d < 3; ++d) {
+                    if (det)
+                        fsum_add(w.tile_fbin + kFsumBins * (3LL * tile + d), fa[j][d]);
+                    else
+                        atomicAdd(&w.tile_fsum[3LL * tile + d], fa[j][d]);
+                }
             }
         }
     }
@@ -971,6 +722,9 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
         if (lane == 0 && m)
             base = atomicAdd(&w.counters[3], __popc(m));
         base = __shfl_sync(0xffffffffu, base, 0);
+        const int slot = base + __popc(m & ((1u << lane) - 1u));
+        if (t < g.n_tiles)
+            w.tile_slot[t] = has ? slot : -1;
         if (has) {
             const TileInfo ti = decode_tile(g, t);
             const BoxDev &B = g.boxes[ti.box];
@@ -988,16 +742,38 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
             td.grid_off = B.grid_off;
             td.h3 = 1.0 / B.scale;
             td.scale_f = B.scale_f;
-            td.pad = 0;
-            w.tile_desc[base + __popc(m & ((1u << lane) - 1u))] = td;
+            td.slot = slot;
+            w.tile_desc[slot] = td;
+        }
+        if (det) {   // tiles reached by a box: those with nodes in them or in a neighbour
+            bool near = false;
+            int box = 0;
+            if (t < g.n_tiles) {
+                box = box_of_tile(g, t);
+                const BoxDev &B = g.boxes[box];
+                const int T = B.T, local = (int)(t - B.tile_base);
+                const int jx = local % T, jy = (local / T) % T, jz = local / (T * T);
+                int any = 0;
+#pragma unroll
+                for (int k = 0; k < 27; ++k)
+                    any |= w.own_flag[B.tile_base + (wrap1(jz + k / 9 - 1, T) * T + wrap1(jy + k / 3 % 3 - 1, T)) * T +
+                                      wrap1(jx + k % 3 - 1, T)];
+                near = any != 0;
+            }
+            const unsigned mn = __ballot_sync(0xffffffffu, near);
+            if (lane == 0 && mn)
+                base = atomicAdd(&w.counters[9], __popc(mn));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (near)
+                w.near_tile[base + __popc(mn & ((1u << lane) - 1u))] = make_int2((int)t, box);
         }
     }
 }
 
-// ------------------------------- tile transfer, FP32 Peskin, own nodes only
-// IFEM_SCATTER_ATOMIC, Peskin kernel: spreading, interpolation, or both fused
-// (Algorithm steps 2 and 4 use the same stencil weights of the same
-// positions), with the position update of Eq. Bashforth_eqn on request. Work
+// --------------------------------------- tile transfer, FP32, own nodes only
+// Spreading, interpolation, or both fused (Algorithm steps 2 and 4 use the same
+// stencil weights of the same positions), with the position update of Eq.
+// Bashforth_eqn on request, for both kernels and scatter modes. Work
 // item = (tile, lattice) over the tiles with own nodes (own_scatter_kernel),
 // taken from a global counter. Each node is visited only by the tile that
 // holds its cell. Boxes of shared memory cover the tile plus a halo, 2 cells
@@ -1012,9 +788,13 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
 // item i (one (node, lattice) unit per thread: the Peskin weights, v_d = sum
 // phi u_d from U, 64 contributions added to A with shared-memory reductions),
 // the box warps copy the velocities of item i + 1 into the other U (cp.async)
-// and flush the other A, of item i - 1: every non-zero value is added to the
-// grid with an L2 reduction (the halos of neighbouring tiles combine there;
-// the order of a value's terms across tiles is not fixed) and cleared. One
+// and flush the other A, of item i - 1, and clear it. IFEM_SCATTER_ATOMIC with
+// the Peskin kernel: every non-zero value is added to the grid with an L2
+// reduction (the halos of neighbouring tiles combine there; the order of a
+// value's terms across tiles is not fixed). Otherwise (STORE), onto a cleared
+// field, only values that at most two boxes reach are added like that; the
+// others go to a buffer, and tile_combine_kernel writes the sum of their terms in
+// a fixed order, so that repeated runs give the same bits. One
 // barrier per item. With the copy, the node loop and the flush one after the
 // other, each waited out its own memory latency.
 //
@@ -1034,7 +814,7 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
 // 32 lanes are on 32 different banks at every step wherever their nodes lie.
 // (In plain z-y-x order the lanes' banks are random: 2.7 wavefronts per load
 // and 3.4 per reduction on the 600-particle suspension, by a count over its
-// stencils.) The weights are rotated into that order once per unit; the
+// stencils.) The Peskin weights are rotated into that order once per unit; the
 // interpolation adds its terms in pairs that no rotation separates, so v does
 // not depend on the lane.
 
@@ -1058,10 +838,6 @@ __device__ __forceinline__ void cp_async4(unsigned dst, const void *src)
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Periodic wrap of a box coordinate in [-n, 2n): the boxes of a grid have
-// at least 8 cells and the halos at most 4, so one correction suffices.
-__device__ __forceinline__ int wrap1(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
-
 // Work counter of a launch: the three lattices of each listed tile, in list
 // order (lattice < 0, counters[2]), or lattice d of each listed tile
 // (counters[1], [6], [7] for d = 0, 1, 2), so that one launch per lattice
@@ -1076,7 +852,6 @@ __device__ __forceinline__ int *tile_counter(const DevWork &w, int lattice)
 // one (x >> 2, z, y & 1) and walks y in kYStep phases; two phases where that
 // measured faster (64 boxes of odd sizes, 16-cell tiles: 243 against 284 us;
 // 600 particles 292 against 291).
-__host__ __device__ inline int tile_width(int max_edge) { return max_edge <= 8 ? 12 : (max_edge <= 12 ? 16 : 20); }
 template <int W>
 struct TileShape {
     static constexpr int NX = W / 4 + 1, NZ = W / 4, NY = W / 2;
@@ -1090,7 +865,7 @@ struct TileShape {
 };
 
 struct TileItem {
-    int tile, d, beg, end;
+    int tile, slot, d, beg, end;
     int sx, sy, sz, ex, ey, ez;
     int n;
     long long grid_off;
@@ -1098,7 +873,7 @@ struct TileItem {
 };
 __device__ __forceinline__ TileItem tile_item(const TileDesc &td, int d, int density)
 {
-    return TileItem{td.tile, d, td.beg, td.end, td.start[0], td.start[1], td.start[2], td.edge[0], td.edge[1],
+    return TileItem{td.tile, td.slot, d, td.beg, td.end, td.start[0], td.start[1], td.start[2], td.edge[0], td.edge[1],
                     td.edge[2], td.n, td.grid_off, density ? td.scale_f : 1.f};
 }
 // 16-byte access to the grid's quads: n, the tile's start and edge multiples of 4, the lattice aligned.
@@ -1113,9 +888,12 @@ __device__ __forceinline__ bool tile_vec(const TileItem &it, const float *lat)
 // A power of two below 2^30 instead left the field of one red cell with 1.5 to
 // 1.9 times the error. fsum: the placement's atomic float sum of |F_d| over n
 // nodes, within (n - 1) 2^-24 of the exact one in any order.
+// An MLS weight is taken to be at most 1 (0.49 with the default support).
+template <int KER>
 __device__ __forceinline__ float tile_scale(const TileItem &it, float fsum)
 {
-    const float bound = fsum * (1.0002f + (float)(it.end - it.beg) * 1.1920929e-7f) * it.sd * 0.125f;
+    const float n = (float)(it.end - it.beg);
+    const float bound = fsum * (1.0002f + n * 1.1920929e-7f) * it.sd * (KER == 0 ? 0.125f : 1.f);
     float scale = 1.f;
     if (bound > 0.f && isfinite(bound))
         scale = __uint_as_float(__float_as_uint(fminf(fmaxf(2147483648.f / bound, 0x1p-120f), 0x1p120f)) & 0xfff00000u);
@@ -1165,11 +943,14 @@ __device__ __forceinline__ void tile_stage(const TileItem &it, const float *__re
 }
 
 // Adds every non-zero value of A to the grid and clears it; returns the exact
-// integer sum and counts the non-zero values inside the tile itself. bt: box
-// thread.
-template <int W>
-__device__ __forceinline__ long long tile_flush(const TileItem &it, float *__restrict__ f, int4 *A, float inv,
-                                                int bt, unsigned &touched)
+// integer sum and counts the non-zero values inside the tile itself. STORE:
+// values that three or more boxes can reach, those within 2 cells of a tile's
+// faces along two axes or three, go to the item's box of the buffer instead, in
+// A's own order, zero or not; the others have at most two terms, whose sum from
+// zero is the same in either order. bt: box thread.
+template <int W, bool STORE>
+__device__ __forceinline__ long long tile_flush(const TileItem &it, float *__restrict__ f, float *__restrict__ buf,
+                                                int4 *A, float inv, int bt, unsigned &touched)
 {
     using S = TileShape<W>;
     const int n = it.n;
@@ -1185,22 +966,42 @@ __device__ __forceinline__ long long tile_flush(const TileItem &it, float *__res
     const bool in_xz = in_z && (unsigned)(4 * gx - 4) < (unsigned)it.ex;
     if (vec)
         plane += wrap1(it.sx - 4 + 4 * gx, n);
+    // STORE: cells of the quad that are near a face along x, and the row along z
+    const bool face_z = lz < 4 || lz >= it.ez;
+    unsigned face_x = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        face_x |= (4 * gx + c < 6 || 4 * gx + c >= it.ex + 2) ? 1u << c : 0u;
+    float4 *out = reinterpret_cast<float4 *>(buf + (3LL * it.slot + it.d) * S::kWords) + bt;
     long long qsum = 0;
     A += bt;
 #pragma unroll
     for (int k = 0; k < S::NY / S::kYStep; ++k) {
-        const int yb = y0 + k * S::kYStep;
-        const int4 q = A[8 * yb * S::NZ * S::NX];
-        if ((q.x | q.y | q.z | q.w) == 0)
+        const int yb = y0 + k * S::kYStep, at = 8 * yb * S::NZ * S::NX, ly = 2 * yb + yl;
+        const int4 q = A[at];
+        const bool zero = (q.x | q.y | q.z | q.w) == 0;
+        float v0 = (float)q.x * inv, v1 = (float)q.y * inv, v2 = (float)q.z * inv, v3 = (float)q.w * inv;
+        if constexpr (STORE) {
+            const bool face_y = ly < 4 || ly >= it.ey;
+            if ((face_y && face_z) || ((face_y || face_z) && face_x)) {
+                if (ly < it.ey + 4)
+                    out[at] = make_float4(v0, v1, v2, v3);
+                const unsigned keep = face_y && face_z ? 0u : ~face_x;
+                v0 = keep & 1u ? v0 : 0.f;
+                v1 = keep & 2u ? v1 : 0.f;
+                v2 = keep & 4u ? v2 : 0.f;
+                v3 = keep & 8u ? v3 : 0.f;
+            }
+        }
+        if (zero)
             continue;
-        A[8 * yb * S::NZ * S::NX] = make_int4(0, 0, 0, 0);
-        const int ly = 2 * yb + yl;
+        A[at] = make_int4(0, 0, 0, 0);
         float *row = plane + wrap1(it.sy - 2 + ly, n) * n;
         qsum += ((long long)q.x + q.y) + ((long long)q.z + q.w);
-        const float v0 = (float)q.x * inv, v1 = (float)q.y * inv, v2 = (float)q.z * inv, v3 = (float)q.w * inv;
         const bool in_y = (unsigned)(ly - 2) < (unsigned)it.ey;
         if (vec) {
-            red_add_v4(row, v0, v1, v2, v3);
+            if (!STORE || v0 != 0.f || v1 != 0.f || v2 != 0.f || v3 != 0.f)
+                red_add_v4(row, v0, v1, v2, v3);
             if (in_xz && in_y)
                 touched += min((unsigned)q.x, 1u) + min((unsigned)q.y, 1u) + min((unsigned)q.z, 1u) +
                            min((unsigned)q.w, 1u);
@@ -1210,7 +1011,8 @@ __device__ __forceinline__ long long tile_flush(const TileItem &it, float *__res
 #pragma unroll
             for (int c = 0; c < 4; ++c)
                 if (qc[c] != 0) {
-                    red_add(row + wrap1(it.sx - 4 + 4 * gx + c, n), vc[c]);
+                    if (!STORE || vc[c] != 0.f)
+                        red_add(row + wrap1(it.sx - 4 + 4 * gx + c, n), vc[c]);
                     touched += in_z && in_y && (unsigned)(4 * gx + c - 4) < (unsigned)it.ex;
                 }
         }
@@ -1239,13 +1041,92 @@ __device__ __forceinline__ void rotate4(float p[4], int r)
     p[3] = two ? a1 : a3;
 }
 
+// mls_weights in FP32, every operation's rounding stated: the same bits in each
+// kernel that uses it. y: the points' distances from the node per axis (cells),
+// wt: z-outer, x-inner. The cubic's outer piece is 4/3 (1 - r)^3; the moments
+// are summed along x, then y, then z (a third of the products of a sum over the
+// 27 points).
+__device__ __forceinline__ bool mls_weights_f32(const float y[3][3], float inv_support, float wt[27])
+{
+    float A00 = 0.f, A10 = 0.f, A11 = 0.f, A20 = 0.f, A21 = 0.f, A22 = 0.f, A30 = 0.f, A31 = 0.f, A32 = 0.f, A33 = 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        float B00 = 0.f, B10 = 0.f, B11 = 0.f, B20 = 0.f, B21 = 0.f, B22 = 0.f;   // of the plane
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const float yz = fmaf(y[2][c], y[2][c], __fmul_rn(y[1][b], y[1][b]));
+            float s0 = 0.f, s1 = 0.f, s2 = 0.f;   // of the row
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const float r = __fmul_rn(sqrtf(fmaf(y[0][a], y[0][a], yz)), inv_support);
+                const float q = fmaxf(__fadd_rn(1.f, -r), 0.f), qq = __fmul_rn(q, q);
+                const float W = r <= 0.5f ? fmaf(-4.f * q, __fmul_rn(r, r), 2.f / 3.f) : __fmul_rn(4.f / 3.f * q, qq);
+                wt[(c * 3 + b) * 3 + a] = W;
+                const float Wy = __fmul_rn(W, y[0][a]);
+                s0 = __fadd_rn(s0, W);
+                s1 = __fadd_rn(s1, Wy);
+                s2 = fmaf(Wy, y[0][a], s2);
+            }
+            const float t0 = __fmul_rn(s0, y[1][b]);
+            B00 = __fadd_rn(B00, s0);
+            B10 = __fadd_rn(B10, s1);
+            B11 = __fadd_rn(B11, s2);
+            B20 = __fadd_rn(B20, t0);
+            B21 = fmaf(s1, y[1][b], B21);
+            B22 = fmaf(t0, y[1][b], B22);
+        }
+        const float t0 = __fmul_rn(B00, y[2][c]);
+        A00 = __fadd_rn(A00, B00);
+        A10 = __fadd_rn(A10, B10);
+        A11 = __fadd_rn(A11, B11);
+        A20 = __fadd_rn(A20, B20);
+        A21 = __fadd_rn(A21, B21);
+        A22 = __fadd_rn(A22, B22);
+        A30 = __fadd_rn(A30, t0);
+        A31 = fmaf(B10, y[2][c], A31);
+        A32 = fmaf(B20, y[2][c], A32);
+        A33 = fmaf(t0, y[2][c], A33);
+    }
+    // A z = e1 by A = L D L^T with unit L; the pivots are those of the Cholesky factor, squared
+    const float d0 = A00, i0 = __frcp_rn(d0);
+    const float l10 = __fmul_rn(A10, i0), l20 = __fmul_rn(A20, i0), l30 = __fmul_rn(A30, i0);
+    const float d1 = fmaf(-l10, A10, A11), i1 = __frcp_rn(d1);
+    const float u21 = fmaf(-l20, A10, A21), u31 = fmaf(-l30, A10, A31);
+    const float l21 = __fmul_rn(u21, i1), l31 = __fmul_rn(u31, i1);
+    const float d2 = fmaf(-l21, u21, fmaf(-l20, A20, A22)), i2 = __frcp_rn(d2);
+    const float u32 = fmaf(-l31, u21, fmaf(-l30, A20, A32));
+    const float l32 = __fmul_rn(u32, i2);
+    const float d3 = fmaf(-l32, u32, fmaf(-l31, u31, fmaf(-l30, A30, A33)));
+    if (!(d0 > 0.f && d1 > 0.f && d2 > 0.f && d3 > 0.f))
+        return false;
+    const float f1 = -l10, f2 = fmaf(-l21, f1, -l20), f3 = fmaf(-l32, f2, fmaf(-l31, f1, -l30));
+    const float z3 = __fmul_rn(f3, __frcp_rn(d3));
+    const float z2 = fmaf(-l32, z3, __fmul_rn(f2, i2));
+    const float z1 = fmaf(-l31, z3, fmaf(-l21, z2, __fmul_rn(f1, i1)));
+    const float z0 = fmaf(-l30, z3, fmaf(-l20, z2, fmaf(-l10, z1, i0)));
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const float zz = fmaf(z2, y[1][b], fmaf(z3, y[2][c], z0));
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                wt[(c * 3 + b) * 3 + a] = __fmul_rn(wt[(c * 3 + b) * 3 + a], fmaf(z1, y[0][a], zz));
+        }
+    return true;
+}
+
 // One (node, lattice) unit: spreads into A, interpolates from U, or both
 // (gq: the node's force times the item's fixed-point scale).
-template <int W, bool SPREAD, bool INTERP, bool AB2>
+// MLS units take their 27 points in plain order: the weights (a 4 x 4 moment
+// system, mls_weights_f32) cost more than the banks. 48 mixed cells in a 101^3
+// grid, transfers of a step: 202 us with a spread over candidate lists that
+// evaluated a node's weights in each of its tiles, plus the interpolation; 93 us.
+template <int KER, int W, bool SPREAD, bool INTERP>
 __device__ __forceinline__ void tile_node(const TileItem &cur, const DevWork &w, const TileUnit &un, float gsc,
                                           const unsigned char *U, unsigned sA, float *__restrict__ v,
                                           const float *__restrict__ x, const float *__restrict__ vp,
-                                          float *__restrict__ xn, float dt, long long N)
+                                          float *__restrict__ xn, float dt, float inv_support, long long N)
 {
     using S = TileShape<W>;
     const int lane = threadIdx.x & 31, d = cur.d;
@@ -1253,9 +1134,60 @@ __device__ __forceinline__ void tile_node(const TileItem &cur, const DevWork &w,
     const float gq = (d == 0 ? un.fn.x : (d == 1 ? un.fn.y : un.fn.z)) * gsc;
     const unsigned pk = __float_as_uint(un.rec.w);
     const float fr[3] = {un.rec.x, un.rec.y, un.rec.z};
-    float ph[3][4];
     int l0[3];
     bool inside = true;
+    auto put = [&](float out) {
+        const long long i = d * N + node;
+        v[i] = out;
+        if (xn)   // Eq. Bashforth_eqn
+            xn[i] = ab2_value(x[i], out, vp[i], dt);
+    };
+    if constexpr (KER == 1) {
+        float y[3][3], wt[27];
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            const float s = ax == d ? fr[ax] : fr[ax] - 0.5f;   // from the node's cell
+            const float base = floorf(s + 0.5f) - 1.f;
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+                y[ax][m] = (base + (float)m) - s;
+            l0[ax] = (int)((pk >> (8 * ax)) & 255u) + (int)base + 2;
+            inside = inside && (unsigned)l0[ax] <= (unsigned)(ax == 0 ? cur.ex : (ax == 1 ? cur.ey : cur.ez)) + 1u;
+        }
+        const bool regular = mls_weights_f32(y, inv_support, wt);
+        if (!inside || !regular) {   // a singular moment matrix (or an inconsistent record: never expected)
+            status_add(w.status, ST_DOMAIN, SPREAD && INTERP ? 2 : 1);   // once per transfer
+            if constexpr (INTERP)
+                put(0.f);
+            return;
+        }
+        int xo[3], yo[3], zo[3];
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            const int lx = l0[0] + 2 + m, ly = l0[1] + m, lz = l0[2] + m;
+            xo[m] = 4 * (lx & 3) + 128 * (lx >> 2);
+            zo[m] = 16 * (lz & 3) + 128 * S::NX * (lz >> 2);
+            yo[m] = 64 * (ly & 1) + 128 * S::NX * S::NZ * (ly >> 1);
+        }
+        float out = 0.f;
+        int J = 0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int bb = 0; bb < 3; ++bb)
+#pragma unroll
+                for (int a = 0; a < 3; ++a, ++J) {
+                    const int o = zo[c] + yo[bb] + xo[a];
+                    if constexpr (INTERP)
+                        out = fmaf(wt[J], *reinterpret_cast<const float *>(U + o), out);
+                    if constexpr (SPREAD)
+                        red_shared_add_nc(sA + (unsigned)o, __float2int_rn(__fmul_rn(wt[J], gq)));
+                }
+        if constexpr (INTERP)
+            put(out);
+        return;
+    }
+    float ph[3][4];
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
         // lattice d sits at the cell coordinate, the other two half a
@@ -1324,22 +1256,16 @@ __device__ __forceinline__ void tile_node(const TileItem &cur, const DevWork &w,
         if constexpr (INTERP)
             p[t0] = __fmul_rn(ph[0][t0], __fadd_rn(__fadd_rn(qz[0], qz[2]), __fadd_rn(qz[1], qz[3])));
     }
-    if constexpr (INTERP) {
-        const float out = __fadd_rn(__fadd_rn(p[0], p[2]), __fadd_rn(p[1], p[3]));
-        const long long i = d * N + node;
-        v[i] = out;
-        if constexpr (AB2)
-            xn[i] = ab2_value(x[i], out, vp[i], dt);
-    }
+    if constexpr (INTERP)
+        put(__fadd_rn(__fadd_rn(p[0], p[2]), __fadd_rn(p[1], p[3])));
 }
 
-template <int W, bool SPREAD, bool INTERP, bool AB2>
+template <int KER, int W, bool SPREAD, bool INTERP, bool STORE>
 __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
     transfer_tile_kernel(DevBatch b, DevWork w, const float *__restrict__ x, float *__restrict__ f, int density,
                          const float *__restrict__ u, float *__restrict__ v, const float *__restrict__ vp,
-                         float *__restrict__ xn, float dt, int lattice)
+                         float *__restrict__ xn, float dt, float inv_support, int lattice)
 {
-    static_assert(INTERP || !AB2, "the position update needs the interpolation");
     using S = TileShape<W>;
     constexpr int kBox = 4 * S::kWords, kBoxWarps = S::kBoxThreads / 32, kRing = 8;
     extern __shared__ __align__(128) unsigned char tile_smem[];
@@ -1401,9 +1327,12 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
             un = tile_unit(w, td.beg + nt);
     };
     auto put_scale = [&](int i, float fsum) {   // one thread
-        s_scale[i & 3] = tile_scale(tile_item(s_desc[i % kRing], s_d[i % kRing], density), fsum);
+        s_scale[i & 3] = tile_scale<KER>(tile_item(s_desc[i % kRing], s_d[i % kRing], density), fsum);
     };
-    auto get_fsum = [&](int i) { return w.tile_fsum[3LL * s_desc[i % kRing].tile + s_d[i % kRing]]; };
+    auto get_fsum = [&](int i) {
+        const long long at = 3LL * s_desc[i % kRing].tile + s_d[i % kRing];
+        return STORE ? fsum_get(w.tile_fbin + kFsumBins * at) : w.tile_fsum[at];
+    };
     auto write_sum = [&](int i) {   // one thread: the exact integer sum of a flushed item, scaled, times h^3
         const TileDesc &td = s_desc[i % kRing];
         long long vsum = 0;
@@ -1437,14 +1366,14 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
                 const unsigned char *Ui = U + (i & 1) * kBox;
                 const unsigned sA = smem_u32(A) + (unsigned)((i & 1) * kBox);
                 if (q < cur.end)
-                    tile_node<W, SPREAD, INTERP, AB2>(cur, w, mine, gsc, Ui, sA, v, x, vp, xn, dt, N);
+                    tile_node<KER, W, SPREAD, INTERP>(cur, w, mine, gsc, Ui, sA, v, x, vp, xn, dt, inv_support, N);
                 if (more) {
 #pragma unroll 1
                     for (q += S::kNodeThreads; q < cur.end; q += S::kNodeThreads) {
                         mine = un;
                         if (q + S::kNodeThreads < cur.end)
                             un = tile_unit(w, q + S::kNodeThreads);
-                        tile_node<W, SPREAD, INTERP, AB2>(cur, w, mine, gsc, Ui, sA, v, x, vp, xn, dt, N);
+                        tile_node<KER, W, SPREAD, INTERP>(cur, w, mine, gsc, Ui, sA, v, x, vp, xn, dt, inv_support, N);
                     }
                     unit_ahead(i + 1);
                 }
@@ -1466,8 +1395,9 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
                 // this flush's sum is written during the next item, by a node
                 // thread; the next item's scale by a thread of the second warp
                 const TileItem old = tile_item(s_desc[(i - 1) % kRing], s_d[(i - 1) % kRing], density);
-                long long qsum = tile_flush<W>(old, f, reinterpret_cast<int4 *>(A + ((i - 1) & 1) * kBox),
-                                               1.f / s_scale[(i - 1) & 3], bt, touched);
+                int4 *box_A = reinterpret_cast<int4 *>(A + ((i - 1) & 1) * kBox);
+                const float inv = 1.f / s_scale[(i - 1) & 3];
+                long long qsum = tile_flush<W, STORE>(old, f, w.box_buf, box_A, inv, bt, touched);
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1)
                     qsum += __shfl_down_sync(0xffffffffu, qsum, o);
@@ -1494,88 +1424,170 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
     }
 }
 
-// ------------------------------------------------- interp, FP32 direct
-// Thread per (node, lattice) unit over the nodes in tile order (spatial
-// locality for the L1/L2-cached gathers): v = sum_z phi_z sum_y phi_y
-// sum_x phi_x u, one square root per axis, 32-bit row offsets.
-template <int KER>
-__global__ void __launch_bounds__(256, 6) interp_direct_kernel(DevBatch b, DevGrid g, DevWork w,
-                                                            const float *__restrict__ u,
-                                                            const float *__restrict__ x, float *__restrict__ v,
-                                                            float support)
+// The reproducible spread's second half: the values of the cleared field f that
+// three or more boxes can reach (tile_flush), each the sum of its boxes' terms
+// in a fixed order. Unit = (tile, lattice). Every tile has at least 4 cells per
+// axis (own_tiling), so a value near a face has one neighbour there, along two
+// axes or three of them; along an axis of one or two tiles the neighbour is the
+// tile itself or the same one on both sides, with different cells of its box.
+// Bound by the loads' latency: an item has its 4 or 8 loads in flight together
+// (two cells of x each where the grid's quads are aligned), and what a unit
+// needs to know of its tile and neighbours is read during the unit before it.
+// 16% of a 16-cell tile's values come here: 10 us for 72 mixed cells in a 128^3
+// grid, after 46 of the transfer. Storing whole boxes and summing every value took
+// 27 (47 when only their non-zero quads were written and read, by a mask). The
+// spread over candidate lists that this replaces (every tile visits each node
+// whose stencil reaches it) took 106 after an interpolation of 37.
+struct CombineUnit {
+    int slot[27], start[3], edge[3], prev[3], n;   // neighbours' boxes; first cell, cells, the previous tile's cells
+    long long off;
+};
+constexpr int kCombineThreads = 128;
+
+// P: cells of an item along x
+template <int W, int P>
+__device__ __forceinline__ void combine_unit(const CombineUnit &un, const float *__restrict__ boxes, float *__restrict__ fd)
 {
-    const int total = w.counters[5];
-    const long long unit = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (unit >= 3LL * total)
-        return;
-    const int d = (int)(unit / total);
-    const int node = w.own_nodes[unit - (long long)d * total];
-    const InstDev I = b.inst[b.node_inst[node]];
-    const BoxDev B = g.boxes[I.box];
-    const long long N = b.N;
-    const int n = B.n;
-    const float *ud = u + B.grid_off + (long long)d * n * n * n;
-    float out = 0.f;
-    if constexpr (KER == 0) {
-        float ph[3][4];
-        int ix[4], iy[4], iz[4];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            int I0;
-            float s = LatCoord<float>::get(I, B, a, x[a * N + node], mac_off(d, a), I0);
-            int base = wrap_near(I0 + peskin_axis_fast(s, ph[a]), n);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                int idx = base + m;
-                idx -= idx >= n ? n : 0;
-                if (a == 0) ix[m] = idx;
-                else if (a == 1) iy[m] = idx;
-                else iz[m] = idx;
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            float accz = 0.f;
-#pragma unroll
-            for (int bb = 0; bb < 4; ++bb) {
-                const float *row = ud + (iz[c] * n + iy[bb]) * n;
-                float accy = ph[0][0] * __ldg(row + ix[0]);
-#pragma unroll
-                for (int a = 1; a < 4; ++a)
-                    accy += ph[0][a] * __ldg(row + ix[a]);
-                accz += ph[1][bb] * accy;
-            }
-            out += ph[2][c] * accz;
-        }
-    } else {
-        float s[3];
-        int I0[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            s[a] = LatCoord<float>::get(I, B, a, x[a * N + node], mac_off(d, a), I0[a]);
-        int base[3];
-        float wt[27];
-        if (!mls_weights<float>(s, support, base, wt)) {
-            status_add(w.status, ST_DOMAIN, 1);
+    using S = TileShape<W>;
+    const int n = un.n, ex = un.edge[0], ey = un.edge[1], ez = un.edge[2];
+    // rows near a face along y and z: all of x; rows near one of them: the two ends of x
+    const int nx = ex / P, ends = 4 / P, both = 16 * nx, one_z = 4 * (ey - 4), one = one_z + 4 * (ez - 4);
+    auto near = [](int k, int e) { return k < 2 ? k : e - 4 + k; };
+    // neighbour along an axis, and the cell in the neighbour's box (halo h)
+    auto side = [](int c, int e) { return c < 2 ? -1 : (c >= e - 2 ? 1 : 0); };
+    auto other = [](int c, int e, int prev, int h) { return c < 2 ? c + prev + h : c - e + h; };
+    auto word_x = [](int l) { return 32 * (l >> 2) + (l & 3); };
+    auto word_y = [](int l) { return 32 * S::NX * S::NZ * (l >> 1) + 16 * (l & 1); };
+    auto word_z = [](int l) { return 32 * S::NX * (l >> 2) + 4 * (l & 3); };
+    for (int i = threadIdx.x; i < both + ends * one; i += kCombineThreads) {
+        int x, y, z;
+        if (i < both) {
+            const int r = i / nx;
+            x = P * (i - r * nx);
+            z = near(r & 3, ez);
+            y = near(r >> 2, ey);
         } else {
-            int ix[3], iy[3], iz[3];
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                ix[m] = wrap_near(I0[0] + base[0] + m, n);
-                iy[m] = wrap_near(I0[1] + base[1] + m, n);
-                iz[m] = wrap_near(I0[2] + base[2] + m, n);
+            const int j = i - both, k = j & (ends - 1), r = j / ends;
+            x = P == 2 ? (k ? ex - 2 : 0) : near(k, ex);
+            if (r < one_z) {
+                z = near(r & 3, ez);
+                y = 2 + (r >> 2);
+            } else {
+                y = near((r - one_z) & 3, ey);
+                z = 2 + ((r - one_z) >> 2);
             }
-            int J = 0;
-#pragma unroll
-            for (int c = 0; c < 3; ++c)
-#pragma unroll
-                for (int bb = 0; bb < 3; ++bb)
-#pragma unroll
-                    for (int a = 0; a < 3; ++a, ++J)
-                        out += wt[J] * __ldg(ud + (iz[c] * n + iy[bb]) * n + ix[a]);
         }
+        const int o[3] = {side(x, ex), side(y, ey), side(z, ez)};
+        const int wx[2] = {word_x(x + 4), word_x(other(x, ex, un.prev[0], 4))};
+        const int wy[2] = {word_y(y + 2), word_y(other(y, ey, un.prev[1], 2))};
+        const int wz[2] = {word_z(z + 2), word_z(other(z, ez, un.prev[2], 2))};
+        float2 q[8];
+        bool any = false;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {   // own box first
+            const int kx = k & 1, ky = k >> 1 & 1, kz = k >> 2;
+            const int slot = un.slot[13 + kx * o[0] + 3 * ky * o[1] + 9 * kz * o[2]];
+            q[k] = make_float2(0.f, 0.f);
+            if (slot >= 0 && !(kx && !o[0]) && !(ky && !o[1]) && !(kz && !o[2])) {
+                const float *p = boxes + 3LL * S::kWords * slot + (kx ? wx[1] : wx[0]) + (ky ? wy[1] : wy[0]) +
+                                 (kz ? wz[1] : wz[0]);
+                any = true;
+                if (P == 2)
+                    q[k] = __ldg(reinterpret_cast<const float2 *>(p));
+                else
+                    q[k].x = __ldg(p);
+            }
+        }
+        if (!any)
+            continue;
+        float2 acc = q[0];
+#pragma unroll
+        for (int k = 1; k < 8; ++k) {
+            acc.x += q[k].x;
+            acc.y += q[k].y;
+        }
+        float *out = fd + ((long long)(un.start[2] + z) * n + un.start[1] + y) * n + un.start[0] + x;
+        if (P == 2)
+            *reinterpret_cast<float2 *>(out) = acc;
+        else
+            *out = acc.x;
     }
-    v[d * N + node] = out;
+}
+
+template <int W>
+__global__ void __launch_bounds__(kCombineThreads, 8)
+    tile_combine_kernel(DevGrid g, DevWork w, float *__restrict__ f)
+{
+    using S = TileShape<W>;
+    __shared__ CombineUnit s_unit[2];
+    const int units = 3 * w.counters[9], lane = threadIdx.x;
+    // first warp: lane k < 27 a neighbour's slot, lanes 27 to 29 an axis, lane 30 the box
+    int3 got;
+    long long off = 0;
+    auto near_of = [&](int unit) {
+        return unit < units ? w.near_tile[unit / 3] : make_int2(-1, 0);   // tile, box
+    };
+    auto read = [&](int2 near) {
+        if (near.x < 0)
+            return;
+        const BoxDev &B = g.boxes[near.y];
+        const int T = B.T, local = (int)(near.x - B.tile_base);
+        const int j[3] = {local % T, (local / T) % T, local / (T * T)};
+        if (lane < 27) {
+            const int jx = wrap1(j[0] + lane % 3 - 1, T), jy = wrap1(j[1] + lane / 3 % 3 - 1, T);
+            const int jz = wrap1(j[2] + lane / 9 - 1, T);
+            got.x = w.tile_slot[B.tile_base + (jz * T + jy) * T + jx];
+        } else if (lane < 30) {
+            const int ja = lane == 27 ? j[0] : (lane == 28 ? j[1] : j[2]);
+            got = make_int3(tile_start(ja, B.t), tile_edge(ja, B.t, T, B.n), tile_edge(wrap1(ja - 1, T), B.t, T, B.n));
+        } else if (lane == 30) {
+            got.x = B.n;
+            off = B.grid_off;
+        }
+    };
+    auto keep = [&](CombineUnit &u) {
+        if (lane < 27) {
+            u.slot[lane] = got.x;
+        } else if (lane < 30) {
+            u.start[lane - 27] = got.x;
+            u.edge[lane - 27] = got.y;
+            u.prev[lane - 27] = got.z;
+        } else if (lane == 30) {
+            u.n = got.x;
+            u.off = off;
+        }
+    };
+    int2 next = make_int2(-1, 0);
+    if (threadIdx.x < 32) {
+        read(near_of(blockIdx.x));
+        next = near_of(blockIdx.x + gridDim.x);
+        keep(s_unit[0]);
+    }
+    __syncthreads();
+    for (int unit = blockIdx.x, buf = 0; unit < units; unit += gridDim.x, buf ^= 1) {
+        if (threadIdx.x < 32) {
+            read(next);
+            next = near_of(unit + 2 * gridDim.x);
+        }
+        const CombineUnit &un = s_unit[buf];
+        const int d = unit % 3, n = un.n;
+        float *fd = f + un.off + (long long)d * n * n * n;
+        const float *boxes = w.box_buf + (long long)d * S::kWords;
+        if (((un.start[0] | n | un.edge[0] | un.prev[0]) & 3) == 0 && (reinterpret_cast<uintptr_t>(fd) & 15) == 0)
+            combine_unit<W, 2>(un, boxes, fd);
+        else
+            combine_unit<W, 1>(un, boxes, fd);
+        if (threadIdx.x < 32)
+            keep(s_unit[buf ^ 1]);
+        __syncthreads();
+    }
+}
+
+// f += a field (the reproducible spread onto a field that is not cleared)
+static __global__ void __launch_bounds__(256) add_field_kernel(float *__restrict__ f, const float *__restrict__ a, long long total)
+{
+    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < total; i += 256LL * gridDim.x)
+        f[i] += a[i];
 }
 
 // ---------------------------------------- spread, FP64 deterministic, MLS
@@ -1853,21 +1865,18 @@ static __global__ void __launch_bounds__(32 * kDetWarps) spread_det_warp_kernel(
     }
 }
 
-// ------------------------------------------------------------- interp
-// Thread per node (in tile order for locality). DET: the oracle's order,
-// acc = acc + ((phi_x*phi_y)*phi_z)*u from 0, z-outer, x-inner. Fast FP32:
-// separable sum_z phi_z sum_y phi_y sum_x phi_x u.
-template <typename real, bool DET, int KER>
+// ------------------------------------------------------- interp, FP64
+// Thread per node, in the oracle's order: acc = acc + ((phi_x*phi_y)*phi_z)*u
+// from 0, z-outer, x-inner.
+template <typename real, int KER>
 __global__ void __launch_bounds__(256) interp_kernel(DevBatch b, DevGrid g, DevWork w,
                                                      const real *__restrict__ u, const real *__restrict__ x,
-                                                     real *__restrict__ v, real support, int use_order,
-                                                     int use_wtab)
+                                                     real *__restrict__ v, real support, int use_wtab)
 {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    // in tile order only the binned nodes are listed (non-finite ones are not)
-    if (idx >= (use_order ? (long long)w.counters[5] : b.N))
+    if (idx >= b.N)
         return;
-    const int node = use_order ? w.own_nodes[idx] : (int)idx;
+    const int node = (int)idx;
     const InstDev I = b.inst[b.node_inst[node]];
     const BoxDev B = g.boxes[I.box];
     const long long N = b.N;
@@ -1881,8 +1890,7 @@ __global__ void __launch_bounds__(256) interp_kernel(DevBatch b, DevGrid g, DevW
         finite = finite && isfinite(xl[a]);
     }
     if (!finite) {
-        if (!use_order)
-            status_add(w.status, ST_DOMAIN, 1);
+        status_add(w.status, ST_DOMAIN, 1);
 #pragma unroll
         for (int d = 0; d < 3; ++d)
             v[d * N + node] = xl[0] + xl[1] + xl[2];
@@ -1921,34 +1929,17 @@ __global__ void __launch_bounds__(256) interp_kernel(DevBatch b, DevGrid g, DevW
                     else iz[m] = wi;
                 }
             }
-            if (DET) {
-                real acc = real(0);
+            real acc = real(0);
 #pragma unroll
-                for (int c = 0; c < 4; ++c)
+            for (int c = 0; c < 4; ++c)
 #pragma unroll
-                    for (int bb = 0; bb < 4; ++bb)
+                for (int bb = 0; bb < 4; ++bb)
 #pragma unroll
-                        for (int a = 0; a < 4; ++a) {
-                            real wgt = (ph[0][a] * ph[1][bb]) * ph[2][c];
-                            acc = acc + wgt * ud[((long long)iz[c] * n + iy[bb]) * n + ix[a]];
-                        }
-                out = acc;
-            } else {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    real accz = real(0);
-#pragma unroll
-                    for (int bb = 0; bb < 4; ++bb) {
-                        const real *row = ud + ((long long)iz[c] * n + iy[bb]) * n;
-                        real accy = ph[0][0] * __ldg(row + ix[0]);
-#pragma unroll
-                        for (int a = 1; a < 4; ++a)
-                            accy += ph[0][a] * __ldg(row + ix[a]);
-                        accz += ph[1][bb] * accy;
+                    for (int a = 0; a < 4; ++a) {
+                        real wgt = (ph[0][a] * ph[1][bb]) * ph[2][c];
+                        acc = acc + wgt * ud[((long long)iz[c] * n + iy[bb]) * n + ix[a]];
                     }
-                    out += ph[2][c] * accz;
-                }
-            }
+            out = acc;
         } else {
             real s[3];
             int I0[3];
