@@ -832,7 +832,7 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
     // spread's binning only), then the counters and counts
     const size_t bin_ints = reproducible(ctx) ? 2 * kFsumBins * 3 * (size_t)nt : 0;
     const size_t zero_ints =
-        kCounters + bin_ints + (size_t)(no + 1) + (!f32 ? nt + 1 : (reproducible(ctx) ? nt : 4 * nt));
+        kCounters + bin_ints + (size_t)(no + 1) + (!f32 ? 4 * nt + 1 : (reproducible(ctx) ? nt : 4 * nt));
     CK(alloc((void **)&w.red_tile, sizeof(double) * 3 * (size_t)nt + sizeof(int) * zero_ints));
     CK(cudaMemset(w.red_tile, 0, sizeof(double) * 3 * (size_t)nt));
     w.counters = reinterpret_cast<int *>(w.red_tile + 3 * nt);
@@ -856,17 +856,19 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
         }
     } else {
         w.cand_count = w.own_count + no + 1;
+        w.red_done = w.cand_count + nt + 1;
+        CK(alloc((void **)&w.red_part, sizeof(double) * 24 * (size_t)nt));
         w.cand_cap = 8 * N;
         CK(alloc((void **)&w.cand_off, sizeof(int) * (nt + 1)));
         CK(alloc((void **)&w.cand_cursor, sizeof(int) * (nt + 1)));
         CK(alloc((void **)&w.cand_nodes, sizeof(int) * (size_t)w.cand_cap));
         CK(alloc((void **)&w.own_off, sizeof(int) * (no + 1)));
         CK(alloc((void **)&w.own_nodes, sizeof(int) * Nn));
-        CK(alloc((void **)&w.active, sizeof(int) * (nt + 1)));
+        CK(alloc((void **)&w.active, sizeof(int) * kTileClasses * (size_t)nt));
     }
     w.wtab = nullptr;
     if (ctx->cfg.precision == IFEM_FP64 && ctx->cfg.kernel == IFEM_KERNEL_PESKIN4)
-        CK(alloc((void **)&w.wtab, sizeof(DetW) * (size_t)std::max<long long>(N, 1)));
+        CK(alloc((void **)&w.wtab, sizeof(DetW) * Nn));
     CK(alloc((void **)&w.scan_blocks, sizeof(int) * 2 * (nb + 1)));
     w.elem_buf = b->d_elem_buf;
     w.bend_buf = b->d_bend_buf;

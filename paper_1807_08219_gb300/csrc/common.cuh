@@ -21,6 +21,7 @@ constexpr int kOwnSub3 = kOwnSub * kOwnSub * kOwnSub;
 constexpr int kScanThreads = 512;  // tile-count scan: threads per block
 constexpr int kScanPer = 4;        // and values per thread
 constexpr int kScanBlock = kScanThreads * kScanPer;
+constexpr int kTileClasses = 4;    // DevWork::active lists
 constexpr int kFsumBins = 8;       // DevWork::tile_fbin entries per sum
 constexpr int kCounters = 16;      // DevWork::counters entries
 constexpr int kMaxCtaSmemBytes = 227 * 1024;   // opt-in dynamic shared memory of one CTA
@@ -114,17 +115,15 @@ struct DevGrid {
     const BoxDev *boxes;
 };
 
-// FP64 Peskin stencil of one node on the three MAC lattices (deterministic
-// FP64 path), computed once per binning from the positions: per lattice d
-// and axis a the wrapped first stencil index base[d][a] and the four weights
-// ph[d][a][m]; lo[a] is the wrapped cell index c - 2, the low corner of the
-// reach of all three lattices.
-struct DetW {
-    double ph[3][3][4];
-    int base[3][3];
-    int lo[3];
+// FP64 Peskin stencil of a node: along each axis of the two offsets its
+// lattices have there (0 for the lattice of that component, 1/2 for the other
+// two), the wrapped first index and the four weights.
+struct alignas(16) DetW {
+    double ph[3][2][4];
+    int base[3][2];
+    int pad[2];
 };
-static_assert(sizeof(DetW) == 336, "DetW layout");
+static_assert(sizeof(DetW) == 224, "DetW layout");
 
 // A tile with own nodes (FP32), as the transfer needs it.
 struct alignas(16) TileDesc {
@@ -167,18 +166,21 @@ struct DevWork {
     int2 *node_key;     // N entries, by node (FP32): own-list key (-1: not binned) and
                         // the node's rank among the nodes of that key
     float4 *node_rec;   // N entries, by node (FP32): the first float4 of its own_rec entry
-    int *active;        // tiles with candidate pairs
+    int *active;        // tiles with candidate pairs, kTileClasses lists of n_tiles entries
     TileDesc *tile_desc;  // tiles with own nodes (FP32), counters[3] of them
     int *tile_slot;     // n_tiles (FP32): a tile's place in that list, or -1
     int2 *near_tile;    // reproducible spread: tiles that a box reaches and their boxes, counters[9] of them
     float *box_buf;     // reproducible spread: a box per listed tile and lattice
     float *field;       // reproducible spread onto a field that is not cleared: the field it is spread into
-    int *counters;      // kCounters: [0] n_active, [2] work counter, [3] tiles with own nodes,
+    int *counters;      // kCounters: [2] work counter, [3] tiles with own nodes,
                         // [4] total pairs, [5] total own nodes, [1] [6] [7] work counters of
-                        // one-lattice launches, [8] scan blocks finished, [9] near_tile entries
+                        // one-lattice launches, [8] scan blocks finished, [9] near_tile entries,
+                        // [10] to [13] active tiles per class
     int *scan_blocks;   // block partial sums for the tile scan
     void *elem_buf;     // per element nodal forces (12 reals per element)
     void *bend_buf;     // per node bending scratch (A, kH, n[3], lap) 6 reals
+    double *red_part;   // FP64 Peskin: 8 octants' sums per long list and lattice, and
+    int *red_done;      // how many of them are there
     double *red_tile;   // per tile: 3 FP64 sums of added spread values
     size_t zero_bytes;  // counters and what follows them (cleared by every binning)
     DetW *wtab;         // N entries (FP64 Peskin only, else null): written by the binning

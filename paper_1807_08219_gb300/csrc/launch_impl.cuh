@@ -145,11 +145,11 @@ cudaError_t bin_impl(const TransferArgs &a, int stages)
         own_scatter_kernel<<<gs, 256, 0, s>>>(b, a.g, w, (const float *)a.F, a.store);
         IFEM_LAUNCH_CHECK();
     } else {
-        scan_finish_kernel<<<(unsigned)((no + 1 + 255) / 256), 256, 0, s>>>(nt, no, w);
+        scan_finish_kernel<<<(unsigned)((no + 1 + 255) / 256), 256, 0, s>>>(nt, no, w, a.n_sm);
         IFEM_LAUNCH_CHECK();
         bin_kernel<real, true><<<gn, 256, 0, s>>>(b, a.g, w, (const real *)a.x);
         IFEM_LAUNCH_CHECK();
-        sort_segments_kernel<<<a.n_sm * 4, 512, 0, s>>>(w);
+        sort_segments_kernel<<<a.n_sm * 4, 512, 0, s>>>(a.g, w);
         IFEM_LAUNCH_CHECK();
         if (a.kernel == 0 && w.wtab) {
             det_weights_kernel<<<(unsigned)((3 * b.N + 255) / 256), 256, 0, s>>>(b, a.g, w.wtab, (const double *)a.x);
@@ -240,7 +240,7 @@ cudaError_t spread_impl(const TransferArgs &a)
         return fused ? launch_tile<0, true, true, false>(a) : launch_tile<0, true, false, false>(a);
     } else {
         if (a.kernel == 0) {
-            // warp per (tile, lattice) over the binning's stencil table
+            // a warp per (tile, lattice) or octant of one, over the binning's stencil table
             if (!a.w.wtab)
                 return cudaErrorInvalidValue;
             // as many warps per CTA (up to kDetWarps) as the largest tile's
@@ -279,13 +279,13 @@ cudaError_t interp_impl(const TransferArgs &a)
     if constexpr (std::is_same<real, float>::value) {
         return a.kernel == 0 ? launch_tile<0, false, true, false>(a) : launch_tile<1, false, true, false>(a);
     } else {
-        unsigned grid = (unsigned)((b.N + 255) / 256);
+        unsigned grid = (unsigned)((b.N + kInterpThreads - 1) / kInterpThreads);
         if (a.kernel == 0)
-            interp_kernel<real, 0><<<grid, 256, 0, a.stream>>>(b, a.g, a.w, (const real *)a.u,
+            interp_kernel<real, 0><<<grid, kInterpThreads, 0, a.stream>>>(b, a.g, a.w, (const real *)a.u,
                                                                     (const real *)a.x, (real *)a.v, (real)a.support,
                                                                     a.use_wtab && a.w.wtab != nullptr);
         else
-            interp_kernel<real, 1><<<grid, 256, 0, a.stream>>>(b, a.g, a.w, (const real *)a.u,
+            interp_kernel<real, 1><<<grid, kInterpThreads, 0, a.stream>>>(b, a.g, a.w, (const real *)a.u,
                                                                     (const real *)a.x, (real *)a.v, (real)a.support, 0);
     }
     IFEM_LAUNCH_CHECK();

@@ -364,9 +364,40 @@ static __global__ void scan_local_kernel(long long n1, long long n2, const int *
 }
 
 // n1 tiles (candidate lists), n2 own sub-blocks. Adds the block offsets,
-// sets the fill cursors, writes the terminal offsets and the list of tiles
-// with candidates (order irrelevant: tiles are processed independently).
-static __global__ void scan_finish_kernel(long long n1, long long n2, DevWork w)
+// sets the fill cursors, writes the terminal offsets and the lists of tiles
+// with candidates, by class of their number, most first: a warp takes up to
+// 0.1 us a candidate, so the few long lists of a dense spot, begun last, were
+// the tail of the FP64 spread.
+// Class 0, lists that several warps walk (spread_det_warp_kernel), begins at 0.6
+// of the candidates that a quarter of an SM has to walk in all: a unit longer
+// than that would be the spread's length.
+__device__ __forceinline__ int tile_class(int count, int limit)
+{
+    return count >= limit ? 0 : (2 * count >= limit ? 1 : (4 * count >= limit ? 2 : 3));
+}
+struct ActiveTiles {
+    int count[kTileClasses], total;
+    __device__ explicit ActiveTiles(const DevWork &w) : total(0)
+    {
+#pragma unroll
+        for (int k = 0; k < kTileClasses; ++k)
+            total += count[k] = w.counters[10 + k];
+    }
+    __device__ int tile(const DevGrid &g, const DevWork &w, int i) const
+    {
+        const int *list = w.active;
+#pragma unroll
+        for (int k = 0; k < kTileClasses - 1; ++k)
+            if (i >= count[k]) {
+                i -= count[k];
+                list += g.n_tiles;
+            } else {
+                break;
+            }
+        return list[i];
+    }
+};
+static __global__ void scan_finish_kernel(long long n1, long long n2, DevWork w, int n_sm)
 {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long n = n1 > n2 ? n1 : n2;
@@ -390,26 +421,30 @@ static __global__ void scan_finish_kernel(long long n1, long long n2, DevWork w)
         w.cand_cursor[i] = o1;
     }
     const unsigned act = __activemask();
-    const unsigned m1 = __ballot_sync(act, c1 > 0);
     const int lane = threadIdx.x & 31;
     const int leader = __ffs(act) - 1;
-    int b1 = 0;
-    if (lane == leader && m1)
-        b1 = atomicAdd(&w.counters[0], __popc(m1));
-    b1 = __shfl_sync(act, b1, leader);
-    if (c1 > 0)
-        w.active[b1 + __popc(m1 & ((1u << lane) - 1u))] = (int)i;
+    const int limit = max(256, (int)(9LL * w.counters[4] / (20 * n_sm)));   // 3 lattices, 4 quarters
+#pragma unroll
+    for (int k = 0; k < kTileClasses; ++k) {
+        const unsigned m = __ballot_sync(act, c1 > 0 && tile_class(c1, limit) == k);
+        int at = 0;
+        if (lane == leader && m)
+            at = atomicAdd(&w.counters[10 + k], __popc(m));
+        at = __shfl_sync(act, at, leader);
+        if (m >> lane & 1u)
+            w.active[k * n1 + at + __popc(m & ((1u << lane) - 1u))] = (int)i;
+    }
 }
 
 // Deterministic mode: sort each tile's candidate list by node id (bitonic
 // sort in shared memory). Lists longer than kSortCap are flagged.
 constexpr int kSortCap = 4096;
-static __global__ void sort_segments_kernel(DevWork w)
+static __global__ void sort_segments_kernel(DevGrid g, DevWork w)
 {
     __shared__ int key[kSortCap];
-    const int n_active = w.counters[0];
-    for (int it = blockIdx.x; it < n_active; it += gridDim.x) {
-        const int tile = w.active[it];
+    const ActiveTiles active(w);
+    for (int it = blockIdx.x; it < active.total; it += gridDim.x) {
+        const int tile = active.tile(g, w, it);
         const int beg = w.cand_off[tile], len = w.cand_off[tile + 1] - beg;
         if (len > kSortCap) {
             if (threadIdx.x == 0)
@@ -455,47 +490,33 @@ __device__ __forceinline__ long long peskin_axis(real s, real ph[4])
     return i0;
 }
 
-// FP64 Peskin stencils of every node on the three lattices (thread per
-// (node, lattice)), computed once after binning: the deterministic spread
-// stages its candidates from this table instead of re-evaluating them for
-// every tile a node reaches, and the step's interpolation reads it too. The
-// values are those of peskin_axis<double> on the same coordinates (same
-// expressions, same compilation), bit for bit. Non-finite nodes are never
-// binned and their entries are left unwritten.
+// FP64 Peskin stencils of every node, thread per (node, axis): the weights of
+// the two offsets that the lattices have along the axis (the same expressions as
+// the gather and the spread, same compilation), bit for bit. Bound by the FP64
+// pipe: 24 weights a node, where the three lattices' nine axes took 36 (133 k
+// nodes 230 us, 135 now). Non-finite nodes are never binned and never read.
 static __global__ void det_weights_kernel(DevBatch b, DevGrid g, DetW *__restrict__ wt, const double *__restrict__ x)
 {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long N = b.N;
     if (t >= 3 * N)
         return;
-    const long long node = t / 3;
-    const int d = (int)(t - 3 * node);
-    const InstDev I = b.inst[b.node_inst[node]];
-    const BoxDev B = g.boxes[I.box];
-    double xl[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-        xl[a] = x[a * N + node];
-    if (!(isfinite(xl[0]) && isfinite(xl[1]) && isfinite(xl[2])))
+    const int a = (int)(t / N);
+    const long long node = t - a * N;
+    const InstDev &I = b.inst[b.node_inst[node]];
+    const BoxDev &B = g.boxes[I.box];
+    const double xa = x[t];
+    if (!isfinite(xa))
         return;
     DetW &W = wt[node];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
+    for (int o = 0; o < 2; ++o) {
         int I0;
-        const double sa = LatCoord<double>::get(I, B, a, xl[a], (double)mac_off(d, a), I0);
         double ph[4];
-        W.base[d][a] = wrapi(peskin_axis<double>(sa, ph), B.n);
+        W.base[a][o] = wrapi(peskin_axis<double>(LatCoord<double>::get(I, B, a, xa, o ? 0.5 : 0.0, I0), ph), B.n);
 #pragma unroll
         for (int m = 0; m < 4; ++m)
-            W.ph[d][a][m] = ph[m];
-    }
-    if (d == 0) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            int I0;
-            const double sc = LatCoord<double>::get(I, B, a, xl[a], 0.0, I0);
-            W.lo[a] = wrapi((long long)floor(sc) - 2, B.n);
-        }
+            W.ph[a][o][m] = ph[m];
     }
 }
 
@@ -1618,13 +1639,14 @@ static __global__ void __launch_bounds__(kDetThreads, 2) spread_det_mls_kernel(D
     __shared__ DetCand cand[kDetChunk];
     __shared__ double red_sh[3][kDetThreads / 32];
     const long long N = b.N;
-    const int n_active = w.counters[0];
+    const ActiveTiles active(w);
+    const int n_active = active.total;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         status_add(w.status, ST_PAIRS, (unsigned long long)w.cand_off[g.n_tiles]);
         status_add(w.status, ST_ACTIVE, (unsigned long long)n_active);
     }
     for (int it = blockIdx.x; it < n_active; it += gridDim.x) {
-        const int tile = w.active[it];
+        const int tile = active.tile(g, w, it);
         const TileInfo ti = decode_tile(g, tile);
         const BoxDev B = g.boxes[ti.box];
         const int ex = ti.edge[0], ey = ti.edge[1], ez = ti.edge[2];
@@ -1749,29 +1771,41 @@ static __global__ void __launch_bounds__(kDetThreads, 2) spread_det_mls_kernel(D
     }
 }
 
-// FP64 deterministic Peskin spread, one warp per (tile, lattice) unit. The
-// unit's owned values sit in a shared-memory accumulator loaded from f; the
-// warp walks the tile's candidates in ascending node order, spreading each
-// candidate's 64 stencil points over its lanes (two points per lane, on
-// distinct cells since every box has at least 8 cells per axis), with a warp
-// barrier between candidates, so every value receives its terms in the
-// oracle's node order, f = f + ((phi_x phi_y) phi_z) g. Every lane carries
-// FP64 work on every candidate whose stencil it meets inside the tile (this
-// GPU's FP64 pipe is charged per warp instruction, whatever the active
-// lanes). Stencils come from the binning's table (det_weights_kernel).
-constexpr int kDetWarps = 4;   // units (warps) per CTA at most
-constexpr int kDetStage = 32;  // candidates staged per round
-struct DetStage {
+// FP64 deterministic Peskin spread, one warp per unit = (tile, lattice), the
+// longest candidate lists first; the longest (tile_class 0) are walked by 8 warps,
+// one per octant of the tile. The unit's owned values sit in a shared-memory
+// accumulator loaded from f; the warp walks the tile's candidates in ascending
+// node order, f = f + ((phi_x phi_y) phi_z) g, those whose points miss the unit
+// left out 32 at a time, with a warp barrier between candidates, so every value
+// receives its terms in the oracle's order. A candidate's points inside the unit
+// (40% of them for 8-cell tiles) are dealt to consecutive lanes: 1.25 rounds of
+// three products and an addition, 1.64 with a fixed lane per point. kDetAhead
+// candidates' weights are computed before the first of them is added; the next
+// candidates' stencils are copied from the binning's table (det_weights_kernel)
+// meanwhile.
+// Bound by the FP64 pipe, which is charged per warp instruction whatever the
+// active lanes: 19 cycles on an SM, 64 between two of one warp, of about 6 a
+// candidate; and at the end by the longest walks, about 700 cycles a candidate.
+// 133 k nodes in 120^3, 8-cell tiles: 530 us; 788 with a lane fixed to each point,
+// whole tiles in any order and each candidate's chain of products on the way of
+// the next. 36 k nodes, a solid's tiles with up to 2200 candidates: 518 to 225.
+// Other ways tried on the first: lanes that own cells by their residues mod 4, 2,
+// without barriers, 640 (6.2 FP64 instructions a candidate for 4.9); the terms
+// tabulated once per node, 182, and only added here, 672.
+constexpr int kDetWarps = 4;    // units (warps) per CTA at most
+constexpr int kDetAhead = 4;
+constexpr int kDetStage = 32;   // candidates staged at a time, two stages
+struct alignas(16) DetStage {
     double ph[3][4];
     double g;
-    int base[3];
-    int pad;
+    unsigned box;   // first cell (6 bits an axis), first point (2), points - 1 (2); top bit: none
+    unsigned inv;   // 2^15 / points along x and, above it, along y
 };
 // Shared memory of one warp: the accumulator of the largest tile + staging.
 __host__ __device__ inline size_t det_warp_bytes(int max_edge)
 {
     const size_t e3 = (size_t)max_edge * max_edge * max_edge;
-    return e3 * sizeof(double) + kDetStage * sizeof(DetStage);
+    return ((e3 + 1) & ~(size_t)1) * sizeof(double) + 2 * (kDetStage + kDetAhead) * sizeof(DetStage);
 }
 
 static __global__ void __launch_bounds__(32 * kDetWarps) spread_det_warp_kernel(DevBatch b, DevGrid g, DevWork w,
@@ -1779,79 +1813,138 @@ static __global__ void __launch_bounds__(32 * kDetWarps) spread_det_warp_kernel(
                                                                               double *__restrict__ f, int density)
 {
     extern __shared__ __align__(16) unsigned char det_smem[];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const size_t e3 = (size_t)g.max_edge * g.max_edge * g.max_edge;
-    double *acc = reinterpret_cast<double *>(det_smem) + wid * e3;
-    DetStage *st = reinterpret_cast<DetStage *>(reinterpret_cast<double *>(det_smem) + nw * e3) + wid * kDetStage;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    DetStage *stages = reinterpret_cast<DetStage *>(det_smem + wid * det_warp_bytes(g.max_edge));
+    double *acc = reinterpret_cast<double *>(stages + 2 * (kDetStage + kDetAhead));
     const long long N = b.N;
-    const int n_active = w.counters[0];
+    const ActiveTiles active(w);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         status_add(w.status, ST_PAIRS, (unsigned long long)w.cand_off[g.n_tiles]);
-        status_add(w.status, ST_ACTIVE, (unsigned long long)n_active);
+        status_add(w.status, ST_ACTIVE, (unsigned long long)active.total);
     }
-    // this lane's stencil points: (a, bb, c0) and (a, bb, c0 + 2)
-    const int a = lane & 3, bb = (lane >> 2) & 3, c0 = lane >> 4;
-    const long long n_units = 3LL * n_active;
-    for (long long unit = (long long)blockIdx.x * nw + wid; unit < n_units; unit += (long long)gridDim.x * nw) {
-        const int tile = w.active[unit / 3];
-        const int d = (int)(unit - 3 * (unit / 3));
+    const int n_split = 24 * active.count[0], n_units = n_split + 3 * (active.total - active.count[0]);
+    const int n_warps = gridDim.x * (blockDim.x >> 5);
+    // each warp's first unit is given, long and short ones spread over the SMs
+    // evenly; the rest are fetched
+    for (int unit = wid * gridDim.x + blockIdx.x; unit < n_units;) {
+        const bool split = unit < n_split;
+        const int whole = split ? unit >> 3 : unit - (n_split / 8) * 7;   // (place in the list, lattice)
+        const int tile = active.tile(g, w, whole / 3), d = whole % 3;
         const TileInfo ti = decode_tile(g, tile);
-        const BoxDev B = g.boxes[ti.box];
-        const int ex = ti.edge[0], ey = ti.edge[1], ez = ti.edge[2];
-        const int sx = ti.start[0], sy = ti.start[1], sz = ti.start[2];
-        const int n = B.n, vol = ex * ey * ez;
-        double *fd = f + B.grid_off + (long long)d * n * n * n;
-        for (int i = lane; i < vol; i += 32) {
-            const int lx = i % ex, ly = (i / ex) % ey, lz = i / (ex * ey);
-            acc[i] = fd[((long long)(sz + lz) * n + sy + ly) * n + sx + lx];
+        const BoxDev &B = g.boxes[ti.box];
+        int s[3], e[3];   // the unit's first cell and cells
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const int lo = split && (unit >> a & 1) ? ti.edge[a] >> 1 : 0;
+            e[a] = (split && !(unit >> a & 1) ? ti.edge[a] >> 1 : ti.edge[a]) - lo;
+            s[a] = ti.start[a] + lo;
         }
+        const int n = B.n, ex = e[0], ey = e[1], ez = e[2], vol = ex * ey * ez;
         const double scale = density ? B.scale : 1.0;
+        double *fd = f + B.grid_off + (long long)d * n * n * n + ((long long)s[2] * n + s[1]) * n + s[0];
         const int beg = w.cand_off[tile], end = w.cand_off[tile + 1];
-        for (int c = beg; c < end; c += kDetStage) {
-            const int nc = min(kDetStage, end - c);
-            __syncwarp();
-            if (lane < nc) {
-                const int node = w.cand_nodes[c + lane];
-                const DetW &Wn = w.wtab[node];
-                DetStage &S = st[lane];
+
+        // stages candidate node (-1: none) of each lane whose points meet the unit, in
+        // order, and then entries without points up to a multiple of kDetAhead; returns
+        // their number
+        auto issue = [&](int node, DetStage *st) {
+            bool in = node >= 0;
+            unsigned box = 0, num_a[3] = {1, 1, 1};
+            const DetW &W = w.wtab[max(node, 0)];
+            if (in) {
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    S.base[q] = Wn.base[d][q];
-#pragma unroll
-                    for (int m = 0; m < 4; ++m)
-                        S.ph[q][m] = Wn.ph[d][q][m];
+                for (int a = 0; a < 3; ++a) {
+                    int r = W.base[a][a == d ? 0 : 1] - s[a];
+                    if (r >= e[a])
+                        r -= n;
+                    // a box of one tile holds all points, past its last cell from the first on
+                    const int lo = max(r, 0), k = e[a] == n ? 4 : min(r + 4, e[a]) - lo;
+                    in = in && k > 0;
+                    num_a[a] = (unsigned)max(k, 1);
+                    box |= (unsigned)lo << (6 * a) | (unsigned)((lo - r) & 3) << (18 + 2 * a) |
+                           ((num_a[a] - 1) & 3) << (24 + 2 * a);
                 }
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, in);
+            const int num = __popc(m), slot = __popc(m & ((1u << lane) - 1u));
+            if (in) {
+                DetStage &S = st[slot];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const double *ph = W.ph[a][a == d ? 0 : 1];
+                    cp_async16(smem_u32(&S.ph[a][0]), ph);
+                    cp_async16(smem_u32(&S.ph[a][2]), ph + 2);
+                }
+                S.box = box;
+                S.inv = (32768u + num_a[0] - 1) / num_a[0] | ((32768u + num_a[1] - 1) / num_a[1]) << 16;
                 S.g = F[d * N + node] * scale;
             }
+            if (lane < kDetAhead)
+                st[num + lane].box = 1u << 31;
+            return num;
+        };
+        auto node_at = [&](int c) { return c + lane < end ? w.cand_nodes[c + lane] : -1; };
+        int num = issue(node_at(beg), stages), ahead = node_at(beg + 32);
+        for (int i = lane; i < vol; i += 32) {
+            const int x = i % ex, y = i / ex % ey, z = i / (ex * ey);
+            acc[i] = fd[((long long)z * n + y) * n + x];
+        }
+        for (int c = beg, buf = 0; c < end; c += 32, buf ^= 1) {
+            const DetStage *st = stages + buf * (kDetStage + kDetAhead);
+            const int count = num;
+            cp_async_wait_all();
             __syncwarp();
-            for (int j = 0; j < nc; ++j) {
-                const DetStage &S = st[j];
-                // tile-relative cell of each point (base is wrapped into [0, n))
-                int lx = S.base[0] + a - sx, ly = S.base[1] + bb - sy;
-                int lz0 = S.base[2] + c0 - sz, lz1 = lz0 + 2;
-                lx += lx < 0 ? n : (lx >= n ? -n : 0);
-                ly += ly < 0 ? n : (ly >= n ? -n : 0);
-                lz0 += lz0 < 0 ? n : (lz0 >= n ? -n : 0);
-                lz1 += lz1 < 0 ? n : (lz1 >= n ? -n : 0);
-                if ((unsigned)lx < (unsigned)ex && (unsigned)ly < (unsigned)ey) {
-                    const double t = S.ph[0][a] * S.ph[1][bb];
-                    if ((unsigned)lz0 < (unsigned)ez) {
-                        const int i = (lz0 * ey + ly) * ex + lx;
-                        acc[i] = acc[i] + (t * S.ph[2][c0]) * S.g;
-                    }
-                    if ((unsigned)lz1 < (unsigned)ez) {
-                        const int i = (lz1 * ey + ly) * ex + lx;
-                        acc[i] = acc[i] + (t * S.ph[2][c0 + 2]) * S.g;
+            num = issue(ahead, stages + (buf ^ 1) * (kDetStage + kDetAhead));
+            ahead = node_at(c + 64);
+            for (int j = 0; j < count; j += kDetAhead) {
+                int at[kDetAhead][2];
+                double wg[kDetAhead][2];
+#pragma unroll
+                for (int q = 0; q < kDetAhead; ++q) {
+                    at[q][0] = at[q][1] = -1;
+                    const DetStage &S = st[j + q];
+                    const unsigned box = S.box, inv = S.inv;
+                    if (box >> 31)   // the same for the warp
+                        continue;
+                    const int kx = (box >> 24 & 3) + 1, ky = (box >> 26 & 3) + 1;
+                    const int points = kx * ky * (int)((box >> 28 & 3) + 1);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int p = lane + 32 * h;
+                        if (p < points) {
+                            const int r = (int)(p * (inv & 0xffffu)) >> 15, lz = (int)(r * (inv >> 16)) >> 15;
+                            const int lx = p - r * kx, ly = r - lz * ky;
+                            int x = (int)(box & 63) + lx, y = (int)(box >> 6 & 63) + ly, z = (int)(box >> 12 & 63) + lz;
+                            x -= x >= ex ? ex : 0;   // (a box of one tile)
+                            y -= y >= ey ? ey : 0;
+                            z -= z >= ez ? ez : 0;
+                            at[q][h] = (z * ey + y) * ex + x;
+                            const double t = S.ph[0][(box >> 18 & 3) + lx] * S.ph[1][(box >> 20 & 3) + ly];
+                            wg[q][h] = (t * S.ph[2][(box >> 22 & 3) + lz]) * S.g;
+                        }
                     }
                 }
-                __syncwarp();
+#pragma unroll
+                for (int q = 0; q < kDetAhead; ++q) {
+                    double s0 = 0.0, s1 = 0.0;   // both loads before the stores
+                    if (at[q][0] >= 0)
+                        s0 = acc[at[q][0]];
+                    if (at[q][1] >= 0)
+                        s1 = acc[at[q][1]];
+                    if (at[q][0] >= 0)
+                        acc[at[q][0]] = s0 + wg[q][0];
+                    if (at[q][1] >= 0)
+                        acc[at[q][1]] = s1 + wg[q][1];
+                    __syncwarp();
+                }
             }
+            __syncwarp();   // the stage is free
         }
         // write back; the unit's FP64 sum of the values it added
         double part = 0.0;
         for (int i = lane; i < vol; i += 32) {
-            const int lx = i % ex, ly = (i / ex) % ey, lz = i / (ex * ey);
-            double *p = fd + ((long long)(sz + lz) * n + sy + ly) * n + sx + lx;
+            const int x = i % ex, y = i / ex % ey, z = i / (ex * ey);
+            double *p = fd + ((long long)z * n + y) * n + x;
             const double old = *p;
             *p = acc[i];
             part += acc[i] - old;
@@ -1859,17 +1952,38 @@ static __global__ void __launch_bounds__(32 * kDetWarps) spread_det_warp_kernel(
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
             part += __shfl_down_sync(0xffffffffu, part, o);
-        if (lane == 0)
-            w.red_tile[3LL * tile + d] = part * (1.0 / B.scale);
-        __syncwarp();
+        if (lane == 0) {
+            part *= 1.0 / B.scale;
+            bool last = true;
+            if (split) {   // the octants' sums are added in their order, by the last to finish
+                double *parts = w.red_part + 8 * whole;
+                parts[unit & 7] = part;
+                __threadfence();
+                last = atomicAdd(&w.red_done[whole], 1) == 7;
+                if (last) {
+                    __threadfence();
+                    part = 0.0;
+                    for (int k = 0; k < 8; ++k)
+                        part += __ldcg(&parts[k]);
+                }
+            }
+            if (last)
+                w.red_tile[3LL * tile + d] = part;
+            unit = n_warps + atomicAdd(&w.counters[2], 1);
+        }
+        unit = __shfl_sync(0xffffffffu, unit, 0);
     }
 }
 
 // ------------------------------------------------------- interp, FP64
 // Thread per node, in the oracle's order: acc = acc + ((phi_x*phi_y)*phi_z)*u
-// from 0, z-outer, x-inner.
+// from 0, z-outer, x-inner. Bound by the FP64 pipe (200 warp instructions a
+// lattice of 32 nodes). One lattice after the other and 64 threads a CTA: 133 k
+// nodes 174 us, 36 k 45, where all three unrolled (their shared stencils kept in
+// registers) in CTAs of 256 took 223 and 61.
+constexpr int kInterpThreads = 64;
 template <typename real, int KER>
-__global__ void __launch_bounds__(256) interp_kernel(DevBatch b, DevGrid g, DevWork w,
+__global__ void __launch_bounds__(kInterpThreads) interp_kernel(DevBatch b, DevGrid g, DevWork w,
                                                      const real *__restrict__ u, const real *__restrict__ x,
                                                      real *__restrict__ v, real support, int use_wtab)
 {
@@ -1896,7 +2010,7 @@ __global__ void __launch_bounds__(256) interp_kernel(DevBatch b, DevGrid g, DevW
             v[d * N + node] = xl[0] + xl[1] + xl[2];
         return;
     }
-#pragma unroll
+#pragma unroll 1
     for (int d = 0; d < 3; ++d) {
         const real *ud = u + B.grid_off + d * n3;
         real out = real(0);
@@ -1912,10 +2026,10 @@ __global__ void __launch_bounds__(256) interp_kernel(DevBatch b, DevGrid g, DevW
             for (int a = 0; a < 3; ++a) {
                 long long i0;
                 if (wt) {
-                    i0 = wt->base[d][a];
+                    i0 = wt->base[a][a == d ? 0 : 1];
 #pragma unroll
                     for (int m = 0; m < 4; ++m)
-                        ph[a][m] = (real)wt->ph[d][a][m];
+                        ph[a][m] = (real)wt->ph[a][a == d ? 0 : 1][m];
                 } else {
                     int I0;
                     real s = LatCoord<real>::get(I, B, a, xl[a], (real)mac_off(d, a), I0);
