@@ -88,9 +88,11 @@ cudaError_t forces_impl(const ForcesArgs &a)
     IFEM_LAUNCH_CHECK();
     if (!a.hvp && b.any_bending) {
         real *bb = (real *)a.w.bend_buf;
-        bend_pass1_kernel<real><<<gn, blk, 0, s>>>(b, x, bb);
+        bend_tri_kernel<real><<<ge, blk, 0, s>>>(b, x, ebuf);
         IFEM_LAUNCH_CHECK();
-        bend_pass2_kernel<real><<<gn, blk, 0, s>>>(b, x, bb, F);
+        bend_pass1_kernel<real><<<gn, blk, 0, s>>>(b, x, ebuf, bb);
+        IFEM_LAUNCH_CHECK();
+        bend_pass2_kernel<real><<<gn, blk, 0, s>>>(b, ebuf, bb, F);
         IFEM_LAUNCH_CHECK();
     }
     return cudaSuccess;

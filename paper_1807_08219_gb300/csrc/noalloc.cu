@@ -38,10 +38,13 @@ cudaError_t launch(const DevBatch &b, const real *x, real *F, unsigned char *scr
     node_gather_kernel<real><<<gn, 256, 0, s>>>(b, ebuf, F);
     if ((e = cudaGetLastError()) != cudaSuccess || !b.any_bending)
         return e;
-    bend_pass1_kernel<real><<<gn, 256, 0, s>>>(b, x, bbuf);
+    bend_tri_kernel<real><<<ge, 256, 0, s>>>(b, x, ebuf);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
-    bend_pass2_kernel<real><<<gn, 256, 0, s>>>(b, x, bbuf, F);
+    bend_pass1_kernel<real><<<gn, 256, 0, s>>>(b, x, ebuf, bbuf);
+    if ((e = cudaGetLastError()) != cudaSuccess)
+        return e;
+    bend_pass2_kernel<real><<<gn, 256, 0, s>>>(b, ebuf, bbuf, F);
     return cudaGetLastError();
 }
 
