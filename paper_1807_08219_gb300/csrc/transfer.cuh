@@ -1312,6 +1312,11 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
     // travels during item i, the descriptor of item i + 2 is copied during it
     const int n_items = w.counters[3] * (lattice < 0 ? 3 : 1);
     int *counter = tile_counter(w, lattice);
+    // Fewer than 3 items per CTA: strided over the CTAs, so that the longest CTA
+    // has as few as can be and no counter is waited for (one cell in 128^3, 150
+    // items for 304 CTAs: 17.7 us with three each, 8.4 now). Else each CTA begins with three neighbours (of
+    // one tile, mostly) and takes the rest as it gets to them.
+    const bool few = n_items < 3 * (int)gridDim.x;
     int ahead = 0;   // its lane 0: number of the next item to be copied
     auto fetch = [&](int it, int i) {
         const int q = lattice < 0 ? it / 3 : it, slot = i % kRing;
@@ -1322,13 +1327,16 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
                        reinterpret_cast<const char *>(w.tile_desc + q) + 16 * lane);
     };
     if (threadIdx.x < 32) {
-        int first = 0;
-        if (lane == 0)
-            first = atomicAdd(counter, 3);   // the first items of a CTA are neighbours
-        first = __shfl_sync(0xffffffffu, first, 0);
-        ahead = first + 2;
+        int first = blockIdx.x;
+        if (!few) {
+            if (lane == 0)
+                first = atomicAdd(counter, 3);
+            first = __shfl_sync(0xffffffffu, first, 0);
+        }
+        const int step = few ? gridDim.x : 1;
+        ahead = first + 2 * step;
         fetch(first, 0);
-        fetch(first + 1, 1);
+        fetch(first + step, 1);
         cp_async_wait_all();
     }
     __syncthreads();
@@ -1406,7 +1414,7 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
                 if (threadIdx.x < 32) {
                     fetch(__shfl_sync(0xffffffffu, ahead, 0), i + 2);
                     if (lane == 0)
-                        ahead = atomicAdd(counter, 1);
+                        ahead = few ? n_items : atomicAdd(counter, 1);
                 }
                 if (INTERP && s_d[(i + 1) % kRing] >= 0)
                     tile_stage<W>(tile_item(s_desc[(i + 1) % kRing], s_d[(i + 1) % kRing], density), u,
