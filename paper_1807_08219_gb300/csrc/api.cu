@@ -1428,6 +1428,9 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
     // forces and its placement (which sums the forces per tile) after them
     if ((rc = do_bin(ctx, b, g, x, stream, fused ? BIN_COUNT : BIN_ALL)) != IFEM_OK)
         return rc;
+    // (before the placement, so that nothing stands between it and the transfer)
+    if (clear_f && (e = cudaStreamWaitEvent(s, ctx->fork[10], 0)) != cudaSuccess)
+        return launch_rc(ctx, e, "step_coupling join");
     if (fused) {
         if ((e = cudaStreamWaitEvent(s, ctx->fork[1], 0)) != cudaSuccess)
             return launch_rc(ctx, e, "step_coupling join");
@@ -1457,8 +1460,6 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
             return launch_rc(ctx, e, "step_coupling fork");
     }
     if (!fused && (e = cudaStreamWaitEvent(s, ctx->fork[1], 0)) != cudaSuccess)
-        return launch_rc(ctx, e, "step_coupling join");
-    if (clear_f && (e = cudaStreamWaitEvent(s, ctx->fork[10], 0)) != cudaSuccess)
         return launch_rc(ctx, e, "step_coupling join");
     // with host arrays and the fused transfer, one launch per lattice: row d
     // of v goes back to the host on aux1 as soon as lattice d's launch ends,

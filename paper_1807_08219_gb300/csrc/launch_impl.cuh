@@ -98,6 +98,26 @@ cudaError_t forces_impl(const ForcesArgs &a)
     return cudaSuccess;
 }
 
+// Launch whose start overlaps the end of the kernel before it in the stream (the
+// kernel itself waits, pdl_wait): of a small step's chain of short kernels the
+// launches' gaps, 1 to 3 us each, are a third (one capsule, 64^3: 42 us, 33 with
+// the scan, the transfer and tile_combine_kernel launched so; CHAIN_FIGURES).
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 // Binning. FP32: one-pass own lists (count, scan, placement; the stages can be
 // launched apart). FP64: candidate and own lists, the candidates sorted, and
 // the Peskin stencil table.
@@ -133,10 +153,10 @@ cudaError_t bin_impl(const TransferArgs &a, int stages)
         IFEM_LAUNCH_CHECK();
         int nb = (int)((no + kScanBlock - 1) / kScanBlock);
         // FP32: the local own offsets go to the cursors (own_scatter_kernel adds the block offsets)
-        scan_local_kernel<<<nb, kScanThreads, 0, s>>>(f32 ? 0 : nt, no, w.cand_count, w.own_count, w.cand_off,
-                                                      f32 ? w.own_cursor : w.own_off, w.scan_blocks,
-                                                      w.counters + 8, w.counters + 4);
-        IFEM_LAUNCH_CHECK();
+        if ((e = launch_after(scan_local_kernel, nb, kScanThreads, 0, s, f32 ? 0 : nt, no, w.cand_count, w.own_count,
+                              w.cand_off, f32 ? w.own_cursor : w.own_off, w.scan_blocks, w.counters + 8,
+                              w.counters + 4)) != cudaSuccess)
+            return e;
     }
     if (empty || !(stages & BIN_PLACE))
         return cudaSuccess;
@@ -195,7 +215,7 @@ cudaError_t launch_tile_w(const TransferArgs &a)
     cfg.dynamicSmemBytes = sm;
     cfg.stream = a.stream;
     cfg.attrs = attr;
-    cfg.numAttrs = a.pdl ? 1 : 0;
+    cfg.numAttrs = a.pdl || (a.lattice < 0 && f == a.f) ? 1 : 0;
     e = cudaLaunchKernelEx(&cfg, kern, a.b, a.w, (const float *)a.x, f, a.density, (const float *)a.u,
                            (float *)a.v, (const float *)a.vp, (float *)a.xn, (float)a.dt, (float)(1.0 / a.support),
                            a.lattice);
@@ -203,8 +223,9 @@ cudaError_t launch_tile_w(const TransferArgs &a)
         return e;
     const long long units = 3 * std::min<long long>(a.g.n_tiles, 27 * a.b.N);
     const long long blocks = std::min(units, 8LL * a.n_sm);   // all resident
-    tile_combine_kernel<W><<<(unsigned)blocks, kCombineThreads, 0, a.stream>>>(a.g, a.w, f);
-    IFEM_LAUNCH_CHECK();
+    if ((e = launch_after(tile_combine_kernel<W>, (unsigned)blocks, kCombineThreads, 0, a.stream, a.g, a.w, f)) !=
+        cudaSuccess)
+        return e;
     if (!a.cleared) {
         add_field_kernel<<<8 * a.n_sm, 256, 0, a.stream>>>((float *)a.f, f, a.total);
         IFEM_LAUNCH_CHECK();

@@ -150,6 +150,12 @@ __device__ __forceinline__ int agg_append(int *count, int *cursor, int *list, lo
     return slot;
 }
 
+// Programmatic dependent launch: a kernel launched so (launch_after) may start
+// once every CTA of the one before it has triggered, and waits for that one's end
+// and its stores before it reads them. Without the attribute both do nothing.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // One-pass own-list binning (FP32): per node its rank within its
 // own-list key (the old value of the key's count, one atomic per group of
 // lanes with the same key) and its record -- fractional lattice coordinates
@@ -164,6 +170,7 @@ __device__ __forceinline__ int agg_append(int *count, int *cursor, int *list, lo
 constexpr int kBinPer = 4;
 static __global__ void __launch_bounds__(256) own_count_kernel(DevBatch b, DevGrid g, DevWork w, const float *__restrict__ x)
 {
+    pdl_trigger();
     const InstDev I = b.inst[blockIdx.y];
     const BoxDev B = g.boxes[I.box];
     const long long N = b.N;
@@ -305,6 +312,7 @@ static __global__ void scan_local_kernel(long long n1, long long n2, const int *
                                          const int *__restrict__ c2, int *__restrict__ o1, int *__restrict__ o2,
                                          int *__restrict__ bsum, int *__restrict__ ticket, int *__restrict__ totals)
 {
+    pdl_wait();
     __shared__ int sh[33];
     __shared__ int last;
     long long base = (long long)blockIdx.x * kScanBlock + (long long)threadIdx.x * kScanPer;
@@ -663,6 +671,7 @@ __device__ __forceinline__ float fsum_get(const unsigned long long *__restrict__
 static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, DevGrid g, DevWork w,
                                                                  const float *__restrict__ F, int det)
 {
+    pdl_trigger();
     const InstDev I = b.inst[blockIdx.y];
     const long long N = b.N;
     const int lane = threadIdx.x & 31;
@@ -1304,10 +1313,12 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
     // next lattice of the same step, which reads nothing this one writes) may
     // start at once: the grid is sized to be resident, so its CTAs take the
     // SMs that this grid's CTAs leave when the items run out
-    asm volatile("griddepcontrol.launch_dependents;");
+    pdl_trigger();
     if constexpr (SPREAD)
         for (int i = threadIdx.x; i < 2 * kBox / 16; i += S::kThreads)
             reinterpret_cast<int4 *>(A)[i] = make_int4(0, 0, 0, 0);
+    if (lattice < 0)
+        pdl_wait();   // for the binning's placement
     // the first box warp takes the items: the counter's answer for item i + 3
     // travels during item i, the descriptor of item i + 2 is copied during it
     const int n_items = w.counters[3] * (lattice < 0 ? 3 : 1);
@@ -1547,6 +1558,7 @@ template <int W>
 __global__ void __launch_bounds__(kCombineThreads, 8)
     tile_combine_kernel(DevGrid g, DevWork w, float *__restrict__ f)
 {
+    pdl_wait();
     using S = TileShape<W>;
     __shared__ CombineUnit s_unit[2];
     const int units = 3 * w.counters[9], lane = threadIdx.x;
