@@ -920,6 +920,7 @@ static TransferArgs transfer_args(ifem_ctx ctx, ifem_batch b, const void *x, con
                                   void *f, void *v, int flags, void *stream)
 {
     TransferArgs a{};
+    a.cache = &ctx->launch_cache;
     a.b = dev_batch(b);
     a.g = dev_grid(b);
     a.w = b->ws.w;
@@ -946,6 +947,7 @@ static int do_forces(ifem_ctx ctx, ifem_batch b, const void *x, void *F, const v
                      int inst0 = 0, int inst_n = 0)
 {
     ForcesArgs a{};
+    a.cache = &ctx->launch_cache;
     a.inst0 = inst0;
     a.inst_n = inst_n;
     a.b = dev_batch(b);
@@ -968,13 +970,14 @@ static int do_forces(ifem_ctx ctx, ifem_batch b, const void *x, void *F, const v
 // sums: a spread follows (the binning clears its per-tile sums, which an
 // interpolation's binning leaves for ifem_reduce).
 static int do_bin(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, void *stream, int stages = BIN_ALL,
-                  const void *F = nullptr, int sums = 1)
+                  const void *F = nullptr, int sums = 1, void *clear_f = nullptr)
 {
     int rc = ws_ensure(ctx, b, g, ctx->tile);
     if (rc != IFEM_OK)
         return rc;
-    TransferArgs a = transfer_args(ctx, b, x, F, nullptr, nullptr, nullptr, 0, stream);
+    TransferArgs a = transfer_args(ctx, b, x, F, nullptr, clear_f, nullptr, 0, stream);
     a.clear_sums = sums;
+    a.clear_f = clear_f != nullptr;
     cudaError_t e = ctx->cfg.precision == IFEM_FP64 ? launch_bin_f64(a, stages) : launch_bin_f32(a, stages);
     return launch_rc(ctx, e, "binning");
 }
@@ -1289,6 +1292,8 @@ static cudaError_t copy_nodes_in(ifem_ctx ctx, ifem_batch b, const void *xh, voi
                              3, cudaMemcpyHostToDevice, s);
 }
 
+constexpr size_t kSmallField = size_t(8) << 20;   // bytes (step_impl)
+
 // One coupling step; with xn given (the caller checked vp, dt and aliasing)
 // also the position update from the interpolated velocities; with io given
 // the host copies in and out around it.
@@ -1373,7 +1378,10 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
     // the clearing of f runs on aux1 beside the host copies, or beside the
     // forces and the binning: then launched after the forces, whose blocks
     // leave it room (before them it takes every SM and they wait)
-    const bool clear_f = (flags & IFEM_SPREAD_OVERWRITE) != 0;
+    // (a small field is cleared with the binning counters: 8 MB take 2 us there, less than
+    // the fork, the launch and the join)
+    const bool small_f = (flags & IFEM_SPREAD_OVERWRITE) && !io && (size_t)g->total * real_size(ctx) <= kSmallField;
+    const bool clear_f = (flags & IFEM_SPREAD_OVERWRITE) && !small_f;
     if ((e = cudaEventRecord(ctx->fork[0], s)) != cudaSuccess)
         return launch_rc(ctx, e, "step_coupling fork");
     auto start_clear = [&]() -> int {
@@ -1426,7 +1434,7 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
         return launch_rc(ctx, e, "step_coupling fork");
     // with the fused transfer the binning's count and scan run beside the
     // forces and its placement (which sums the forces per tile) after them
-    if ((rc = do_bin(ctx, b, g, x, stream, fused ? BIN_COUNT : BIN_ALL)) != IFEM_OK)
+    if ((rc = do_bin(ctx, b, g, x, stream, fused ? BIN_COUNT : BIN_ALL, nullptr, 1, small_f ? f : nullptr)) != IFEM_OK)
         return rc;
     // (before the placement, so that nothing stands between it and the transfer)
     if (clear_f && (e = cudaStreamWaitEvent(s, ctx->fork[10], 0)) != cudaSuccess)

@@ -371,7 +371,14 @@ struct LatCoord<float> {
 };
 
 // ------------------------------------------------------------- launchers
+// Launch parameters that depend on the device only, asked for once per context (0: not yet).
+struct LaunchCache {
+    int tile_ctas[2][3][2][2][2];   // transfer_tile_kernel<KER, W, SPREAD, INTERP, STORE>: resident CTAs per SM
+    int nodal[2];                   // forces_nodal_f32_kernel<CLUSTER>: shared memory allowed
+};
+
 struct ForcesArgs {
+    LaunchCache *cache;
     DevBatch b;
     DevWork w;
     const void *x;
@@ -385,6 +392,7 @@ struct ForcesArgs {
 };
 
 struct TransferArgs {
+    LaunchCache *cache;
     DevBatch b;
     DevGrid g;
     DevWork w;
@@ -399,6 +407,7 @@ struct TransferArgs {
     int n_sm;
     int store;        // FP32: reproducible spread through the boxes of every tile
     int cleared;      // f is zero before the spread
+    int clear_f;      // the binning clears f too
     long long total;  // values of the grid
     int clear_sums;   // binning: a spread follows, clear its per-tile sums too
     int lattice;      // tile transfer: -1 all three lattices, else that lattice only

@@ -14,6 +14,7 @@ using namespace ifem;
 struct ifem_ctx_s {
     ifem_config cfg;
     int n_sm = 0;
+    ifem::LaunchCache launch_cache{};
     int tile = 8;
     std::string err;
     unsigned long long *d_status = nullptr;

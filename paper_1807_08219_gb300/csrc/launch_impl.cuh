@@ -31,7 +31,7 @@ namespace ifem {
 // blocks measured slower throughout: 600 particles 102 us with 192 threads).
 template <typename real>   // float (a template so that kernels_f64.cu compiles no FP32 kernel)
 static cudaError_t launch_nodal_forces(const DevBatch &b, const float *x, float *F, unsigned long long *status,
-                                       int inst0, int n, int n_sm, cudaStream_t s)
+                                       int inst0, int n, int n_sm, LaunchCache *cache, cudaStream_t s)
 {
     const int S = 16 * n <= n_sm ? 8 : (2 * n <= n_sm ? 4 : (2 * n <= 3 * n_sm ? 2 : 1));
     const int chunk = ((b.max_nodes + S - 1) / S + 31) & ~31;
@@ -39,9 +39,13 @@ static cudaError_t launch_nodal_forces(const DevBatch &b, const float *x, float 
     const int threads = ((chunk + rounds - 1) / rounds + 31) & ~31;
     const size_t sm = nodal_smem_bytes(b.max_nodes);
     auto kern = S > 1 ? forces_nodal_f32_kernel<true> : forces_nodal_f32_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess)
-        return e;
+    if (!cache->nodal[S > 1]) {   // the largest size: contexts share the function's attribute
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)nodal_smem_bytes(kNodalMaxNodes));
+        if (e != cudaSuccess)
+            return e;
+        cache->nodal[S > 1] = 1;
+    }
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -70,7 +74,7 @@ cudaError_t forces_impl(const ForcesArgs &a)
             const int n = a.inst_n > 0 ? a.inst_n : b.n_inst;
             if (a.inst0 < 0 || a.inst0 + n > b.n_inst)
                 return cudaErrorInvalidValue;
-            return launch_nodal_forces<real>(b, x, F, a.w.status, a.inst0, n, a.n_sm, s);
+            return launch_nodal_forces<real>(b, x, F, a.w.status, a.inst0, n, a.n_sm, a.cache, s);
         }
     }
     if (a.inst0 != 0 || (a.inst_n != 0 && a.inst_n != b.n_inst))
@@ -100,16 +104,16 @@ cudaError_t forces_impl(const ForcesArgs &a)
 
 // Launch whose start overlaps the end of the kernel before it in the stream (the
 // kernel itself waits, pdl_wait): of a small step's chain of short kernels the
-// launches' gaps, 1 to 3 us each, are a third (one capsule, 64^3: 42 us, 33 with
-// the scan, the transfer and tile_combine_kernel launched so; CHAIN_FIGURES).
+// launches gaps, 1 to 3 us each, are a quarter (one capsule, 64^3: 42 us, 32
+// with the whole chain launched so).
 template <typename... P, typename... A>
-cudaError_t launch_after(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args)
+cudaError_t launch_after(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, A... args)
 {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
@@ -140,17 +144,21 @@ cudaError_t bin_impl(const TransferArgs &a, int stages)
         // one clear: the counters, counts and per-tile |F| sums, and before them
         // the spread's per-tile sums
         const size_t sums = a.clear_sums ? sizeof(double) * 3 * (size_t)nt : 0;
-        cudaError_t e = cudaMemsetAsync(reinterpret_cast<char *>(w.counters) - sums, 0, sums + w.zero_bytes, s);
-        if (e != cudaSuccess)
-            return e;
+        const size_t words = (sums + w.zero_bytes) / sizeof(int);
+        cudaError_t e = cudaSuccess;
+        const size_t f_words = a.clear_f ? (size_t)a.total * sizeof(real) / sizeof(int) : 0;
+        clear_kernel<<<(unsigned)std::min<size_t>((words + f_words + 255) / 256, 8 * a.n_sm), 256, 0, s>>>(
+            w.counters - sums / sizeof(int), words, (int *)a.f, f_words);
         IFEM_LAUNCH_CHECK();
         if (empty)
             return cudaSuccess;
-        if constexpr (f32)
-            own_count_kernel<<<g1, 256, 0, s>>>(b, a.g, w, (const float *)a.x);
-        else
+        if constexpr (f32) {
+            if ((e = launch_after(own_count_kernel, g1, 256, 0, s, b, a.g, w, (const float *)a.x)) != cudaSuccess)
+                return e;
+        } else {
             bin_kernel<real, false><<<gn, 256, 0, s>>>(b, a.g, w, (const real *)a.x);
-        IFEM_LAUNCH_CHECK();
+            IFEM_LAUNCH_CHECK();
+        }
         int nb = (int)((no + kScanBlock - 1) / kScanBlock);
         // FP32: the local own offsets go to the cursors (own_scatter_kernel adds the block offsets)
         if ((e = launch_after(scan_local_kernel, nb, kScanThreads, 0, s, f32 ? 0 : nt, no, w.cand_count, w.own_count,
@@ -164,8 +172,8 @@ cudaError_t bin_impl(const TransferArgs &a, int stages)
         // enough threads for every tile as well as every node
         const long long per_inst = ((nt + 255) / 256 + b.n_inst - 1) / b.n_inst;
         dim3 gs((unsigned)std::max<long long>(g1.x, per_inst), b.n_inst);
-        own_scatter_kernel<<<gs, 256, 0, s>>>(b, a.g, w, (const float *)a.F, a.store);
-        IFEM_LAUNCH_CHECK();
+        if (cudaError_t e = launch_after(own_scatter_kernel, gs, 256, 0, s, b, a.g, w, (const float *)a.F, a.store))
+            return e;
     } else {
         scan_finish_kernel<<<(unsigned)((no + 1 + 255) / 256), 256, 0, s>>>(nt, no, w, a.n_sm);
         IFEM_LAUNCH_CHECK();
@@ -190,11 +198,15 @@ cudaError_t launch_tile_w(const TransferArgs &a)
     auto kern = transfer_tile_kernel<KER, W, SPREAD, INTERP, STORE>;
     constexpr int kKinds = (SPREAD ? 1 : 0) + (INTERP ? 1 : 0), T = TileShape<W>::kThreads;
     const size_t sm = (size_t)4 * TileShape<W>::kWords * 2 * kKinds;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess)
-        return e;
-    int occ = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, T, sm);
+    cudaError_t e = cudaSuccess;
+    int &occ = a.cache->tile_ctas[KER][W / 4 - 3][SPREAD][INTERP][STORE];
+    if (occ == 0) {
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
+            return e;
+        int ctas = 1;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kern, T, sm);
+        occ = ctas < 1 ? 1 : ctas;
+    }
     float *f = (float *)a.f;
     if (STORE && !a.cleared) {
         f = a.w.field;
@@ -210,7 +222,7 @@ cudaError_t launch_tile_w(const TransferArgs &a)
     // writes
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(a.n_sm * (occ < 1 ? 1 : occ));
+    cfg.gridDim = dim3(a.n_sm * occ);
     cfg.blockDim = dim3(T);
     cfg.dynamicSmemBytes = sm;
     cfg.stream = a.stream;

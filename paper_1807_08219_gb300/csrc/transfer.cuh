@@ -156,6 +156,19 @@ __device__ __forceinline__ int agg_append(int *count, int *cursor, int *list, lo
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Clears a binning's counters and counts, and the field to be spread into where
+// that is small (a kernel, not a memset, for own_count_kernel to follow without a
+// gap).
+static __global__ void __launch_bounds__(256) clear_kernel(int *__restrict__ p, size_t words, int *__restrict__ f,
+                                                           size_t f_words)
+{
+    pdl_trigger();
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < words; i += (size_t)gridDim.x * 256)
+        p[i] = 0;
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < f_words; i += (size_t)gridDim.x * 256)
+        f[i] = 0;
+}
+
 // One-pass own-list binning (FP32): per node its rank within its
 // own-list key (the old value of the key's count, one atomic per group of
 // lanes with the same key) and its record -- fractional lattice coordinates
@@ -190,6 +203,7 @@ static __global__ void __launch_bounds__(256) own_count_kernel(DevBatch b, DevGr
             xa[j][2] = x[2 * N + node[j]];
         }
     }
+    pdl_wait();   // for the clearing (which began after the positions were there)
     bool ok[kBinPer];
     int key[kBinPer];
 #pragma unroll
@@ -312,6 +326,7 @@ static __global__ void scan_local_kernel(long long n1, long long n2, const int *
                                          const int *__restrict__ c2, int *__restrict__ o1, int *__restrict__ o2,
                                          int *__restrict__ bsum, int *__restrict__ ticket, int *__restrict__ totals)
 {
+    pdl_trigger();
     pdl_wait();
     __shared__ int sh[33];
     __shared__ int last;
@@ -672,6 +687,7 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
                                                                  const float *__restrict__ F, int det)
 {
     pdl_trigger();
+    pdl_wait();   // for the scan
     const InstDev I = b.inst[blockIdx.y];
     const long long N = b.N;
     const int lane = threadIdx.x & 31;
