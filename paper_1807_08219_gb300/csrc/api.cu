@@ -1292,7 +1292,8 @@ static cudaError_t copy_nodes_in(ifem_ctx ctx, ifem_batch b, const void *xh, voi
                              3, cudaMemcpyHostToDevice, s);
 }
 
-constexpr size_t kSmallField = size_t(8) << 20;   // bytes (step_impl)
+constexpr size_t kSmallField = size_t(8) << 20;   // bytes of f (step_impl)
+constexpr size_t kRowsFrom = size_t(5) << 19;     // bytes of v (step_impl)
 
 // One coupling step; with xn given (the caller checked vp, dt and aliasing)
 // also the position update from the interpolated velocities; with io given
@@ -1474,8 +1475,12 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
     // beside the later lattices. Lattices 1 and 2 are launched with
     // programmatic serialization: their CTAs start on the SMs that the
     // previous lattice's CTAs leave when its items run out (they read nothing
-    // it writes), so the three launches share one tail instead of one each
-    const bool v_rows = fused && !reproducible(ctx) && io && node_bytes > 0;
+    // it writes), so the three launches share one tail instead of one each. Only
+    // where a row takes longer than a launch (three launches against one, us):
+    // 16 MB of v 671 to 735, 3.6 MB 167 to 170, 1.3 MB 126 to 123, 0.6 MB 93 to 87;
+    // the reproducible spread, whose second half would run per lattice too, 1.5 MB
+    // 243 to 221
+    const bool v_rows = fused && !reproducible(ctx) && io && node_bytes >= kRowsFrom;
     if (v_rows) {
         const size_t row = node_bytes / 3;
         for (int d = 0; d < 3; ++d) {
