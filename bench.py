@@ -46,9 +46,8 @@ REF_BUDGET_S = 150.0   # --impl reference: warm-up + timed oracle steps
 # reported for that workload only; set an entry to None when its kernel changes.
 NCU_TRAFFIC = {"spread+interp": None, "spread": None, "interp": None, "forces": None, "bin": None}
 # The unit that bounds each kernel in that capture and its fraction of peak (context for the HBM
-# fraction: the fused transfer kernel is latency-bound at 12 warps per SM, with the L1 load/store
-# pipe the busiest unit; the forces kernel is bound by shared-memory wavefronts).
-NCU_LIMITER = {"forces": ("shared-memory wavefronts", 0.598)}
+# fraction); an entry only while its capture is the current kernel's.
+NCU_LIMITER = {}
 
 
 def peaks():
@@ -658,11 +657,11 @@ def main():
     if not args.no_cpu:
         cpu = cpu_baseline_parallel(wl)
         cpu["single_thread"] = cpu_baseline_sample(wl)
-    # bin (halo path: count + rank, scan, placement + list of tiles with own nodes; candidate path:
-    # count, 2 scans, fill), forces, spread and interp (one fused launch on the halo path), 2 reductions
-    launches_per_step = (3 if fused else 4) + 1 + (1 if fused else 2) + 2
+    # bin (clear, count + rank, scan, placement + list of tiles with own nodes), forces, spread +
+    # interp in one launch (a second one adds up the reproducible spread's boxes), 2 reductions
+    launches_per_step = 4 + 1 + 1 + 2
     if scatter == I.IFEM_SCATTER_DET:
-        launches_per_step += 3
+        launches_per_step += 1
     line = {
         "metric": METRIC, "value": value, "unit": "nodes/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": t_ms, "higher_is_better": True, "scaling": "weak",
