@@ -89,6 +89,7 @@ struct BoxDev {
     double L;
     double inv_h;          // n / L
     double scale;          // (n/L)^3
+    double h3;             // 1 / scale
     float inv_h_f;         // FP32 copies for the FP32 kernels (no FP64 pipe use)
     float scale_f;
 };

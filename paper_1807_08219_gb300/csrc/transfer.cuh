@@ -786,7 +786,7 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
                 td.edge[a] = ti.edge[a];
             }
             td.grid_off = B.grid_off;
-            td.h3 = 1.0 / B.scale;
+            td.h3 = B.h3;
             td.scale_f = B.scale_f;
             td.slot = slot;
             w.tile_desc[slot] = td;
@@ -928,22 +928,26 @@ __device__ __forceinline__ bool tile_vec(const TileItem &it, const float *lat)
     return ((it.sx | it.n | it.ex) & 3) == 0 && (reinterpret_cast<uintptr_t>(lat) & 15) == 0;
 }
 
-// Fixed-point scale of an item: keeps the bound sum |g_k| / 8 on any value (and
-// the rounding of its terms) below 2^31, three mantissa bits of the largest such
-// scale (the bits a different order of the placement's additions cannot reach).
-// A power of two below 2^30 instead left the field of one red cell with 1.5 to
-// 1.9 times the error. fsum: the placement's atomic float sum of |F_d| over n
-// nodes, within (n - 1) 2^-24 of the exact one in any order.
+// Fixed-point unit (y) of an item and its reciprocal (x), the scale: keep the
+// bound sum |g_k| / 8 on any value (and the rounding of its terms) below 2^31.
+// The unit is the smallest such one rounded up to three mantissa bits (the bits a
+// different order of the placement's additions cannot reach), so that integers
+// become values by an exact product (an FP64 division of each item's sum by the
+// scale held up one of the node warps that the item waits for: steps of 600 mixed
+// cells 460 us, of 64 boxes 418, now 453 and 407). A power of two instead left the field of one red cell with 1.5 to 1.9 times
+// the error. fsum: the placement's atomic float sum of |F_d| over n nodes, within
+// (n - 1) 2^-24 of the exact one in any order.
 // An MLS weight is taken to be at most 1 (0.49 with the default support).
 template <int KER>
-__device__ __forceinline__ float tile_scale(const TileItem &it, float fsum)
+__device__ __forceinline__ float2 tile_scale(const TileItem &it, float fsum)
 {
     const float n = (float)(it.end - it.beg);
     const float bound = fsum * (1.0002f + n * 1.1920929e-7f) * it.sd * (KER == 0 ? 0.125f : 1.f);
-    float scale = 1.f;
-    if (bound > 0.f && isfinite(bound))
-        scale = __uint_as_float(__float_as_uint(fminf(fmaxf(2147483648.f / bound, 0x1p-120f), 0x1p120f)) & 0xfff00000u);
-    return scale;
+    if (!(bound > 0.f && isfinite(bound)))
+        return make_float2(1.f, 1.f);
+    const float least = fminf(fmaxf(bound * 0x1p-31f, 0x1p-120f), 0x1p120f);
+    const float unit = __uint_as_float((__float_as_uint(least) + 0xfffffu) & 0xfff00000u);
+    return make_float2(1.f / unit, unit);
 }
 
 // Copies the velocity box of an item's lattice into U asynchronously: quads
@@ -1319,7 +1323,7 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
     extern __shared__ __align__(128) unsigned char tile_smem[];
     unsigned char *U = tile_smem, *A = tile_smem + (INTERP ? 2 * kBox : 0);
     __shared__ long long s_red[2][kBoxWarps];
-    __shared__ float s_scale[4];   // fixed-point scale of item i in i % 4
+    __shared__ float2 s_scale[4];   // fixed-point scale and unit of item i in i % 4
     // items i of this CTA in slot i % kRing: lattice (-1: none) and descriptor
     __shared__ int s_d[kRing];
     __shared__ __align__(16) TileDesc s_desc[kRing];
@@ -1397,7 +1401,7 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
 #pragma unroll
         for (int q = 0; q < kBoxWarps; ++q)
             vsum += s_red[i & 1][q];
-        w.red_tile[3LL * td.tile + s_d[i % kRing]] = (double)vsum / (double)s_scale[i & 3] * td.h3;
+        w.red_tile[3LL * td.tile + s_d[i % kRing]] = (double)vsum * (double)s_scale[i & 3].y * td.h3;
     };
     if (!box)
         unit_ahead(0);
@@ -1413,7 +1417,7 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
                 write_sum(i - 2);
             if (valid) {
                 const TileItem cur = tile_item(s_desc[i % kRing], s_d[i % kRing], density);
-                const float gsc = SPREAD ? cur.sd * s_scale[i & 3] : 0.f;
+                const float gsc = SPREAD ? cur.sd * s_scale[i & 3].x : 0.f;
                 TileUnit mine = un;
                 int q = cur.beg + nt;
                 const bool more = q + S::kNodeThreads < cur.end;
@@ -1454,7 +1458,7 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
                 // thread; the next item's scale by a thread of the second warp
                 const TileItem old = tile_item(s_desc[(i - 1) % kRing], s_d[(i - 1) % kRing], density);
                 int4 *box_A = reinterpret_cast<int4 *>(A + ((i - 1) & 1) * kBox);
-                const float inv = 1.f / s_scale[(i - 1) & 3];
+                const float inv = s_scale[(i - 1) & 3].y;
                 long long qsum = tile_flush<W, STORE>(old, f, w.box_buf, box_A, inv, bt, touched);
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1)
