@@ -936,7 +936,7 @@ static TransferArgs transfer_args(ifem_ctx ctx, ifem_batch b, const void *x, con
     a.n_sm = ctx->n_sm;
     a.store = reproducible(ctx);
     a.cleared = (flags & IFEM_SPREAD_OVERWRITE) != 0;
-    a.total = b->grid0->total;
+    a.total = b->ws.grid->total;   // the call's grid, which need not be the batch's first
     a.lattice = -1;
     a.stream = (cudaStream_t)stream;
     return a;
