@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -556,8 +557,10 @@ extern "C" int ifem_grid_create(ifem_ctx ctx, int n_boxes, const int32_t *n, con
     for (int b = 0; b < n_boxes; ++b)
         if (n[b] < 8 || n[b] > 1024 || !(L[b] > 0.0) || !std::isfinite(L[b]))
             return fail(ctx, IFEM_ERR_ARG, "grid: box sides must be 8..1024 cells with L > 0");
+    static std::atomic<unsigned long long> serials{0};
     ifem_grid g = new ifem_grid_s();
     g->ctx = ctx;
+    g->serial = ++serials;
     g->n_boxes = n_boxes;
     g->n.assign(n, n + n_boxes);
     g->L.assign(L, L + n_boxes);
@@ -715,7 +718,7 @@ static void ws_free(Workspace &ws)
     for (void *p : ws.allocs)
         cudaFree(p);
     ws.allocs.clear();
-    ws.grid = nullptr;
+    ws.grid = 0;
     ws.tile = 0;
 }
 
@@ -784,7 +787,7 @@ static void own_tiling(int n, int tile, int &t, int &T)
 static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
 {
     Workspace &ws = b->ws;
-    if (ws.grid == g && ws.tile == tile)
+    if (ws.grid == g->serial && ws.tile == tile)
         return IFEM_OK;
     ws_free(ws);
     const bool f32 = ctx->cfg.precision == IFEM_FP32;
@@ -874,7 +877,9 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
     w.elem_buf = b->d_elem_buf;
     w.bend_buf = b->d_bend_buf;
     w.status = ctx->d_status;
-    ws.grid = g;
+    ws.grid = g->serial;
+    ws.n_boxes = g->n_boxes;
+    ws.total = g->total;
     ws.tile = tile;
     ws.n_tiles = nt;
     ws.max_edge = max_edge;
@@ -884,7 +889,7 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
 static DevGrid dev_grid(ifem_batch b)
 {
     DevGrid d{};
-    d.n_boxes = b->ws.grid->n_boxes;
+    d.n_boxes = b->ws.n_boxes;
     d.n_tiles = b->ws.n_tiles;
     d.max_edge = b->ws.max_edge;
     d.boxes = b->ws.d_boxes;
@@ -936,7 +941,7 @@ static TransferArgs transfer_args(ifem_ctx ctx, ifem_batch b, const void *x, con
     a.n_sm = ctx->n_sm;
     a.store = reproducible(ctx);
     a.cleared = (flags & IFEM_SPREAD_OVERWRITE) != 0;
-    a.total = b->ws.grid->total;   // the call's grid, which need not be the batch's first
+    a.total = b->ws.total;   // the call's grid, which need not be the batch's first
     a.lattice = -1;
     a.stream = (cudaStream_t)stream;
     return a;

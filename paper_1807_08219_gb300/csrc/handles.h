@@ -49,6 +49,7 @@ struct ifem_tmpl_s {
 
 struct ifem_grid_s {
     ifem_ctx ctx;
+    unsigned long long serial;   // of this process; an address can come back with another grid
     int n_boxes;
     std::vector<int> n;
     std::vector<double> L;
@@ -57,7 +58,9 @@ struct ifem_grid_s {
 };
 
 struct Workspace {
-    ifem_grid grid = nullptr;
+    unsigned long long grid = 0;   // serial of the grid it was made for (0: none), and
+    int n_boxes = 0;               // that grid's boxes
+    long long total = 0;           // and values
     int tile = 0;
     long long n_tiles = 0;
     int max_edge = 0;

@@ -72,3 +72,33 @@ def test_another_grid(precision, kernel, scatter, first, call, overwrite, step):
         assert bool((got[0][0] == got[1][0]).all())
     else:
         assert float((got[0][0].double() - got[1][0].double()).norm()) < 1e-5 * got[1][1]
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_grid_at_the_address_of_a_destroyed_one(precision):
+    """The batch's tiles follow the grid, not its handle's address."""
+    from paper_1807_08219_gb300 import ifem as I
+    w = _workload(precision)
+    cp = I.Coupler(dataclasses.replace(w, boxes=[W.Box(64, 1.0)]), precision=precision)
+    try:
+        calls = [[64, 48], [64, 24]] if precision == 0 else [[48], [33]]
+        first = I.ifem_grid_create(cp.ctx, calls[0], [1.0] * len(calls[0]))
+        _calls(cp, first, False, 0)
+        at = first.value
+        I.ifem_grid_destroy(first)
+        grids = []
+        while len(grids) < 64 and (not grids or grids[-1].value != at):
+            grids.append(I.ifem_grid_create(cp.ctx, calls[1], [1.0] * len(calls[1])))
+        if grids[-1].value != at:
+            pytest.skip("the allocator did not give the address back")
+        got = _calls(cp, grids[-1], False, 0)[0]
+        for g in grids[:-1]:
+            I.ifem_grid_destroy(g)
+        again = I.Coupler(dataclasses.replace(w, boxes=[W.Box(n, 1.0) for n in calls[1]]), precision=precision)
+        try:
+            assert bool((got == _calls(again, again.grid, False, 0)[0]).all())
+        finally:
+            again.close()
+        I.ifem_grid_destroy(grids[-1])
+    finally:
+        cp.close()
