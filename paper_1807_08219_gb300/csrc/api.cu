@@ -1037,6 +1037,7 @@ static int do_ab2(ifem_ctx ctx, ifem_batch b, const void *x, const void *v, cons
                   void *stream)
 {
     LagrangeArgs a{};
+    a.cache = &ctx->launch_cache;
     a.b = dev_batch(b);
     a.x = const_cast<void *>(x);
     a.x_out = xn;
@@ -1109,6 +1110,7 @@ extern "C" int ifem_spread(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *
 static LagrangeArgs lagrange_args(ifem_ctx ctx, ifem_batch b, void *x, void *stream)
 {
     LagrangeArgs a{};
+    a.cache = &ctx->launch_cache;
     a.b = dev_batch(b);
     a.x = x;
     a.status = ctx->d_status;

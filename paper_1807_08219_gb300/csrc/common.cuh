@@ -375,7 +375,8 @@ struct LatCoord<float> {
 // Launch parameters that depend on the device only, asked for once per context (0: not yet).
 struct LaunchCache {
     int tile_ctas[2][3][2][2][2];   // transfer_tile_kernel<KER, W, SPREAD, INTERP, STORE>: resident CTAs per SM
-    int nodal[2];                   // forces_nodal_f32_kernel<CLUSTER>: shared memory allowed
+    int nodal[2], volume, vcorr, det_warp;   // forces_nodal_f32_kernel<CLUSTER>, volume_f32_kernel,
+                                    // vc_fused_f32_kernel, spread_det_warp_kernel: shared memory allowed
 };
 
 struct ForcesArgs {
@@ -469,6 +470,7 @@ cudaError_t launch_interp_cc_f64(const TransferArgs &a, int ncomp);
 
 // Lagrangian update: AB2 positions, volumes, membrane volume correction.
 struct LagrangeArgs {
+    LaunchCache *cache;
     DevBatch b;
     void *x;
     void *x_out;      // AB2 result (null: in place)

@@ -17,6 +17,20 @@ namespace ifem {
             return e_;                           \
     } while (0)
 
+// Allows a kernel its largest dynamic shared memory, once per context. The limit
+// belongs to the function, which all contexts and threads share: set to what one
+// launch needs, another thread's smaller batch could lower it before that launch.
+template <typename Kernel>
+static cudaError_t allow_smem(Kernel kern, size_t largest, int &done)
+{
+    if (done)
+        return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)largest);
+    done = e == cudaSuccess;
+    return e;
+}
+constexpr size_t kVolSmemBytes = kMaxCtaSmemBytes - 1024;   // beside the volume kernels' own arrays
+
 // FP32 nodal forces of particles [inst0, inst0 + n): a cluster of S CTAs per
 // particle. With few particles one CTA each leaves most SMs idle; with many,
 // each doubling only stages the positions once more. Times in us, S = 1, 2, 4, 8:
@@ -39,13 +53,8 @@ static cudaError_t launch_nodal_forces(const DevBatch &b, const float *x, float 
     const int threads = ((chunk + rounds - 1) / rounds + 31) & ~31;
     const size_t sm = nodal_smem_bytes(b.max_nodes);
     auto kern = S > 1 ? forces_nodal_f32_kernel<true> : forces_nodal_f32_kernel<false>;
-    if (!cache->nodal[S > 1]) {   // the largest size: contexts share the function's attribute
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)nodal_smem_bytes(kNodalMaxNodes));
-        if (e != cudaSuccess)
-            return e;
-        cache->nodal[S > 1] = 1;
-    }
+    if (cudaError_t e = allow_smem(kern, nodal_smem_bytes(kNodalMaxNodes), cache->nodal[S > 1]))
+        return e;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -285,7 +294,8 @@ cudaError_t spread_impl(const TransferArgs &a)
             if (warps < 1)
                 return cudaErrorInvalidValue;
             const size_t sm = per_warp * warps;
-            cudaFuncSetAttribute(spread_det_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            if (cudaError_t e = allow_smem(spread_det_warp_kernel, kMaxCtaSmemBytes, a.cache->det_warp))
+                return e;
             int occ = 1;
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, spread_det_warp_kernel, 32 * warps, sm);
             occ = occ < 1 ? 1 : occ;
@@ -398,9 +408,8 @@ cudaError_t volume_impl(const LagrangeArgs &a)
         return cudaSuccess;
     if constexpr (std::is_same<real, float>::value) {
         const size_t sm = sizeof(float4) * (size_t)a.b.max_nodes;
-        if (sm + 1024 <= (size_t)kMaxCtaSmemBytes) {
-            cudaError_t e = cudaFuncSetAttribute(volume_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess)
+        if (sm <= kVolSmemBytes) {
+            if (cudaError_t e = allow_smem(volume_f32_kernel, kVolSmemBytes, a.cache->volume))
                 return e;
             volume_f32_kernel<<<a.b.n_inst, kVolThreadsF, sm, a.stream>>>(a.b, (const float *)a.x, a.out);
             IFEM_LAUNCH_CHECK();
@@ -419,9 +428,8 @@ cudaError_t vcorr_impl(const LagrangeArgs &a)
         return cudaSuccess;
     if constexpr (std::is_same<real, float>::value) {
         const size_t sm = 2 * sizeof(float4) * (size_t)a.b.max_nodes;
-        if (sm + 1024 <= (size_t)kMaxCtaSmemBytes) {
-            cudaError_t e = cudaFuncSetAttribute(vc_fused_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess)
+        if (sm <= kVolSmemBytes) {
+            if (cudaError_t e = allow_smem(vc_fused_f32_kernel, kVolSmemBytes, a.cache->vcorr))
                 return e;
             vc_fused_f32_kernel<<<a.b.n_inst, kVolThreadsF, sm, a.stream>>>(a.b, (float *)a.x, a.V0, a.out, a.status);
             IFEM_LAUNCH_CHECK();
