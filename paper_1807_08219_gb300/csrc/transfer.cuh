@@ -1341,6 +1341,12 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
             reinterpret_cast<int4 *>(A)[i] = make_int4(0, 0, 0, 0);
     if (lattice < 0)
         pdl_wait();   // for the binning's placement
+    if constexpr (INTERP)
+        if (xn && w.counters[5] != N)   // the update of nodes that are not binned, as ab2_kernel does it
+            for (long long k = (long long)blockIdx.x * S::kThreads + threadIdx.x; k < N; k += (long long)gridDim.x * S::kThreads)
+                if (w.node_key[k].x < 0)
+                    for (int d = 0; d < 3; ++d)
+                        xn[d * N + k] = ab2_value(x[d * N + k], v[d * N + k], vp[d * N + k], dt);
     // the first box warp takes the items: the counter's answer for item i + 3
     // travels during item i, the descriptor of item i + 2 is copied during it
     const int n_items = w.counters[3] * (lattice < 0 ? 3 : 1);
