@@ -937,7 +937,7 @@ __device__ __forceinline__ bool tile_vec(const TileItem &it, const float *lat)
 // cells 460 us, of 64 boxes 418, now 453 and 407). A power of two instead left the field of one red cell with 1.5 to 1.9 times
 // the error. fsum: the placement's atomic float sum of |F_d| over n nodes, within
 // (n - 1) 2^-24 of the exact one in any order.
-// An MLS weight is taken to be at most 1 (0.49 with the default support).
+// An MLS weight is at most 1 (mls_weights_f32).
 template <int KER>
 __device__ __forceinline__ float2 tile_scale(const TileItem &it, float fsum)
 {
@@ -1097,6 +1097,10 @@ __device__ __forceinline__ void rotate4(float p[4], int r)
 // are summed along x, then y, then z (a third of the products of a sum over the
 // 27 points). A distance is r2 * rsqrt(r2): with sqrtf the transfer of 48 mixed
 // cells in 101^3 took 83 us, 74 now; the velocities' error, 1.9e-7, is the same.
+// False where the moment matrix is singular: a pivot that is not positive, or a
+// weight above 1. The weights of a regular matrix are at most 1 for every support
+// (0.49 for the default sqrt(3)); rounding gives larger ones where the condition
+// number passes 1e6 or so, which happens for supports below 1.25 (5e3 at 1.25).
 __device__ __forceinline__ bool mls_weights_f32(const float y[3][3], float inv_support, float wt[27])
 {
     float A00 = 0.f, A10 = 0.f, A11 = 0.f, A20 = 0.f, A21 = 0.f, A22 = 0.f, A30 = 0.f, A31 = 0.f, A32 = 0.f, A33 = 0.f;
@@ -1165,6 +1169,13 @@ __device__ __forceinline__ bool mls_weights_f32(const float y[3][3], float inv_s
             for (int a = 0; a < 3; ++a)
                 wt[(c * 3 + b) * 3 + a] = __fmul_rn(wt[(c * 3 + b) * 3 + a], fmaf(z1, y[0][a], zz));
         }
+    if (inv_support > 0.75f) {
+        float most = 0.f;
+#pragma unroll
+        for (int J = 0; J < 27; ++J)
+            most = fmaxf(most, fabsf(wt[J]));
+        return most <= 1.0001f;
+    }
     return true;
 }
 

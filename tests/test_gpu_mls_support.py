@@ -1,0 +1,46 @@
+"""FP32 MLS transfers with small supports, where some moment matrices are singular
+or nearly so: nodes that do not get regular weights are counted and left out of
+both transfers, so that the spread stays the transpose of the interpolation
+(<f, u> h^3 = sum F v, to 1e-5 of sum |F| max |u|: FP32 weights and the fixed point of
+the spread, one node to most tiles, are each within a few 1e-7)."""
+import numpy as np
+import pytest
+
+import ifem_workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("support", [0.8, 0.95, 1.0, 1.02, 1.05, 1.1, 1.2, 1.3, 1.4, 0.0])
+def test_transfers_stay_transposes(support):
+    import torch
+    from paper_1807_08219_gb300 import ifem as I
+    n, rng = 64, np.random.default_rng(11)
+    t = W.make("C1").templates[0]
+    # half of the nodes near grid points, faces or centres of cells, at any distance down to 1e-6 cells
+    p = n * rng.random((t.n_nodes, 3))
+    p[::2] = np.round(2.0 * p[::2]) / 2.0 + rng.standard_normal(p[::2].shape) * 10.0 ** -rng.integers(1, 7, (len(p[::2]), 1))
+    ctx = I.ifem_ctx_create(I.IFEM_FP32, I.IFEM_KERNEL_MLS27, I.IFEM_SCATTER_DET, 6, support)
+    tm = I.ifem_tmpl_create_membrane(ctx, t.elems, t.X, I.IFEM_LAW_NEO_HOOKE, 1.0, 1.0, 0.0)
+    grid = I.ifem_grid_create(ctx, [n], [1.0])
+    batch = I.ifem_batch_create(ctx, [tm], [(0, 0, np.zeros(3))], grid)
+    try:
+        dev = torch.device("cuda")
+        x = torch.as_tensor((p / n).T, dtype=torch.float32, device=dev).contiguous()
+        F = torch.as_tensor(rng.standard_normal(x.shape), dtype=torch.float32, device=dev)
+        u = torch.as_tensor(rng.standard_normal(3 * n ** 3), dtype=torch.float32, device=dev)
+        f, v = torch.empty_like(u), torch.empty_like(x)
+        I.ifem_spread(ctx, batch, grid, x, F, f, I.IFEM_SPREAD_OVERWRITE)
+        lost = I.ifem_sync_status(ctx, raise_on_error=False)[1]["domain_errors"]
+        I.ifem_interpolate(ctx, batch, grid, u, x, v)
+        assert I.ifem_sync_status(ctx, raise_on_error=False)[1]["domain_errors"] == lost
+        assert int((v == 0).sum()) >= lost and (lost == 0 if support == 0 or support > 1.25 else lost > 0)
+        both = float((f.double() * u.double()).sum()) / n ** 3, float((F.double() * v.double()).sum())
+        size = float(F.double().abs().sum() * u.double().abs().max())
+        assert abs(both[0] - both[1]) < 1e-5 * size
+        assert float(v.abs().max()) < 27 * float(u.abs().max())
+    finally:
+        I.ifem_batch_destroy(batch)
+        I.ifem_grid_destroy(grid)
+        I.ifem_tmpl_destroy(tm)
+        I.ifem_ctx_destroy(ctx)
