@@ -855,7 +855,6 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
         CK(alloc((void **)&w.node_rec, sizeof(float4) * Nn));
         if (reproducible(ctx)) {   // a box per listed tile and lattice: at most one tile per node
             CK(alloc((void **)&w.box_buf, tile_box_bytes(max_edge) * 3 * (size_t)std::min(nt, N)));
-            CK(alloc((void **)&w.field, sizeof(float) * (size_t)g->total));
             CK(alloc((void **)&w.near_tile, sizeof(int2) * (size_t)(nt + 1)));
         }
     } else {
@@ -1662,7 +1661,7 @@ static int autotune(ifem_ctx ctx, ifem_batch b, const void *x, void *stream)
             if ((rc = do_bin(ctx, b, g, x, stream, BIN_ALL, F)) == IFEM_OK) {
                 // the transfer launches the step will use (fused where it fuses)
                 if (ctx->cfg.precision == IFEM_FP32)
-                    rc = do_spread_interp(ctx, b, x, F, u, f, v, 0, stream);
+                    rc = do_spread_interp(ctx, b, x, F, u, f, v, IFEM_SPREAD_OVERWRITE, stream);
                 else if ((rc = do_spread(ctx, b, x, F, f, 0, stream)) == IFEM_OK)
                     rc = do_interp(ctx, b, u, x, v, stream);
             }

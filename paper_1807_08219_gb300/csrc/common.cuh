@@ -172,7 +172,6 @@ struct DevWork {
     int *tile_slot;     // n_tiles (FP32): a tile's place in that list, or -1
     int2 *near_tile;    // reproducible spread: tiles that a box reaches and their boxes, counters[9] of them
     float *box_buf;     // reproducible spread: a box per listed tile and lattice
-    float *field;       // reproducible spread onto a field that is not cleared: the field it is spread into
     int *counters;      // kCounters: [2] work counter, [3] tiles with own nodes,
                         // [4] total pairs, [5] total own nodes, [1] [6] [7] work counters of
                         // one-lattice launches, [8] scan blocks finished, [9] near_tile entries,
@@ -408,7 +407,7 @@ struct TransferArgs {
     double support;
     int n_sm;
     int store;        // FP32: reproducible spread through the boxes of every tile
-    int cleared;      // f is zero before the spread
+    int cleared;      // f is zero before the spread (else the reproducible spread adds to it)
     int clear_f;      // the binning clears f too
     long long total;  // values of the grid
     int clear_sums;   // binning: a spread follows, clear its per-tile sums too

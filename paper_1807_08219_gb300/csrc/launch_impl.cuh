@@ -217,12 +217,7 @@ cudaError_t launch_tile_w(const TransferArgs &a)
         occ = ctas < 1 ? 1 : ctas;
     }
     float *f = (float *)a.f;
-    if (STORE && !a.cleared) {
-        f = a.w.field;
-        if ((e = cudaMemsetAsync(f, 0, sizeof(float) * (size_t)a.total, a.stream)) != cudaSuccess)
-            return e;
-        IFEM_LAUNCH_CHECK();
-    }
+    const int add = !a.cleared;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     // programmatic dependent launch: the CTAs of this grid may start once
@@ -236,22 +231,15 @@ cudaError_t launch_tile_w(const TransferArgs &a)
     cfg.dynamicSmemBytes = sm;
     cfg.stream = a.stream;
     cfg.attrs = attr;
-    cfg.numAttrs = a.pdl || (a.lattice < 0 && f == a.f) ? 1 : 0;
+    cfg.numAttrs = a.pdl || a.lattice < 0 ? 1 : 0;
     e = cudaLaunchKernelEx(&cfg, kern, a.b, a.w, (const float *)a.x, f, a.density, (const float *)a.u,
                            (float *)a.v, (const float *)a.vp, (float *)a.xn, (float)a.dt, (float)(1.0 / a.support),
-                           a.lattice);
+                           a.lattice, add);
     if (e != cudaSuccess || !STORE)
         return e;
     const long long units = 3 * std::min<long long>(a.g.n_tiles, 27 * a.b.N);
     const long long blocks = std::min(units, 8LL * a.n_sm);   // all resident
-    if ((e = launch_after(tile_combine_kernel<W>, (unsigned)blocks, kCombineThreads, 0, a.stream, a.g, a.w, f)) !=
-        cudaSuccess)
-        return e;
-    if (!a.cleared) {
-        add_field_kernel<<<8 * a.n_sm, 256, 0, a.stream>>>((float *)a.f, f, a.total);
-        IFEM_LAUNCH_CHECK();
-    }
-    return cudaSuccess;
+    return launch_after(tile_combine_kernel<W>, (unsigned)blocks, kCombineThreads, 0, a.stream, a.g, a.w, f, add);
 }
 template <int KER, bool SPREAD, bool INTERP, bool STORE>
 cudaError_t launch_tile(const TransferArgs &a)

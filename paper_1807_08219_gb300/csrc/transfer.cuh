@@ -613,6 +613,11 @@ __device__ __forceinline__ void red_add_v4(float *p, float a, float b, float c, 
                  "f"(b), "f"(c), "f"(d)
                  : "memory");
 }
+__device__ __forceinline__ void red_add_v2(float *p, float a, float b)
+{
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(__cvta_generic_to_global(p)), "f"(a), "f"(b)
+                 : "memory");
+}
 __device__ __forceinline__ void red_add(float *p, float a)
 {
     asm volatile("red.global.add.f32 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "f"(a) : "memory");
@@ -837,10 +842,11 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
 // and flush the other A, of item i - 1, and clear it. IFEM_SCATTER_ATOMIC with
 // the Peskin kernel: every non-zero value is added to the grid with an L2
 // reduction (the halos of neighbouring tiles combine there; the order of a
-// value's terms across tiles is not fixed). Otherwise (STORE), onto a cleared
-// field, only values that at most two boxes reach are added like that; the
-// others go to a buffer, and tile_combine_kernel writes the sum of their terms in
-// a fixed order, so that repeated runs give the same bits. One
+// value's terms across tiles is not fixed). Otherwise (STORE) only values whose
+// terms have no order are added like that: on a cleared field those that at most
+// two boxes reach, else (add) those that one does. The others go to a buffer, and
+// tile_combine_kernel sums their terms in a fixed order and writes the sum or adds
+// it, so that repeated runs give the same bits. One
 // barrier per item. With the copy, the node loop and the flush one after the
 // other, each waited out its own memory latency.
 //
@@ -997,10 +1003,11 @@ __device__ __forceinline__ void tile_stage(const TileItem &it, const float *__re
 // values that three or more boxes can reach, those within 2 cells of a tile's
 // faces along two axes or three, go to the item's box of the buffer instead, in
 // A's own order, zero or not; the others have at most two terms, whose sum from
-// zero is the same in either order. bt: box thread.
+// zero is the same in either order. add (f is not cleared): values that two boxes
+// can reach, near a face along one axis, go there too. bt: box thread.
 template <int W, bool STORE>
 __device__ __forceinline__ long long tile_flush(const TileItem &it, float *__restrict__ f, float *__restrict__ buf,
-                                                int4 *A, float inv, int bt, unsigned &touched)
+                                                int4 *A, float inv, int bt, bool add, unsigned &touched)
 {
     using S = TileShape<W>;
     const int n = it.n;
@@ -1033,10 +1040,11 @@ __device__ __forceinline__ long long tile_flush(const TileItem &it, float *__res
         float v0 = (float)q.x * inv, v1 = (float)q.y * inv, v2 = (float)q.z * inv, v3 = (float)q.w * inv;
         if constexpr (STORE) {
             const bool face_y = ly < 4 || ly >= it.ey;
-            if ((face_y && face_z) || ((face_y || face_z) && face_x)) {
+            const bool any = add || face_y || face_z, whole = add ? face_y || face_z : face_y && face_z;
+            if (whole || (any && face_x)) {
                 if (ly < it.ey + 4)
                     out[at] = make_float4(v0, v1, v2, v3);
-                const unsigned keep = face_y && face_z ? 0u : ~face_x;
+                const unsigned keep = whole ? 0u : ~face_x;
                 v0 = keep & 1u ? v0 : 0.f;
                 v1 = keep & 2u ? v1 : 0.f;
                 v2 = keep & 4u ? v2 : 0.f;
@@ -1327,7 +1335,7 @@ template <int KER, int W, bool SPREAD, bool INTERP, bool STORE>
 __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
     transfer_tile_kernel(DevBatch b, DevWork w, const float *__restrict__ x, float *__restrict__ f, int density,
                          const float *__restrict__ u, float *__restrict__ v, const float *__restrict__ vp,
-                         float *__restrict__ xn, float dt, float inv_support, int lattice)
+                         float *__restrict__ xn, float dt, float inv_support, int lattice, int add)
 {
     using S = TileShape<W>;
     constexpr int kBox = 4 * S::kWords, kBoxWarps = S::kBoxThreads / 32, kRing = 8;
@@ -1476,7 +1484,7 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
                 const TileItem old = tile_item(s_desc[(i - 1) % kRing], s_d[(i - 1) % kRing], density);
                 int4 *box_A = reinterpret_cast<int4 *>(A + ((i - 1) & 1) * kBox);
                 const float inv = s_scale[(i - 1) & 3].y;
-                long long qsum = tile_flush<W, STORE>(old, f, w.box_buf, box_A, inv, bt, touched);
+                long long qsum = tile_flush<W, STORE>(old, f, w.box_buf, box_A, inv, bt, add != 0, touched);
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1)
                     qsum += __shfl_down_sync(0xffffffffu, qsum, o);
@@ -1505,32 +1513,45 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
 
 // The reproducible spread's second half: the values of the cleared field f that
 // three or more boxes can reach (tile_flush), each the sum of its boxes' terms
-// in a fixed order. Unit = (tile, lattice). Every tile has at least 4 cells per
+// in a fixed order; with add those that two or more can reach, the sum added to f.
+// Unit = (tile, lattice). Every tile has at least 4 cells per
 // axis (own_tiling), so a value near a face has one neighbour there, along two
 // axes or three of them; along an axis of one or two tiles the neighbour is the
 // tile itself or the same one on both sides, with different cells of its box.
-// Bound by the loads' latency: an item has its 4 or 8 loads in flight together
-// (two cells of x each where the grid's quads are aligned), and what a unit
-// needs to know of its tile and neighbours is read during the unit before it.
-// 16% of a 16-cell tile's values come here: 10 us for 72 mixed cells in a 128^3
-// grid, after 46 of the transfer. Storing whole boxes and summing every value took
-// 27 (47 when only their non-zero quads were written and read, by a mask). The
-// spread over candidate lists that this replaces (every tile visits each node
-// whose stencil reaches it) took 106 after an interpolation of 37.
+// Bound by the loads' latency: an item, two cells of x, has its 4 or 8 loads in
+// flight together, and what a unit needs to know of its tile and neighbours is read
+// during the unit before it. 16% of a 16-cell tile's values come here (58% with
+// add): 10 us for 72 mixed cells in a 128^3 grid, after 46 of the transfer. Storing
+// whole boxes and summing every value took 27 (47 when only their non-zero quads were
+// written and read, by a mask); single values where the grid's quads are not aligned
+// made a step of 64 boxes of any size 606 us, 566 in pairs. The spread over candidate
+// lists that this replaces (every tile visits each node whose stencil reaches it)
+// took 106 after an interpolation of 37.
+// add: adding the sums of the reached tiles' values where they belong. Clearing a
+// second field, spreading into it and adding it reads and writes every value of every
+// box: steps of one red cell in 256^3 203 us, 49 now; 72 mixed cells, 128^3, 125 and
+// 117; 600, 256^3, 701 and 635; 64 boxes 777 and 705.
 struct CombineUnit {
     int slot[27], start[3], edge[3], prev[3], n;   // neighbours' boxes; first cell, cells, the previous tile's cells
     long long off;
 };
 constexpr int kCombineThreads = 128;
 
-// P: cells of an item along x
-template <int W, int P>
-__device__ __forceinline__ void combine_unit(const CombineUnit &un, const float *__restrict__ boxes, float *__restrict__ fd)
+// An item is two cells along x, or one at the end of an odd row. EVEN: the tile and
+// the one before it have an even number of cells along x, so that both cells lie in
+// one pair of every box; else the x neighbours' values are loaded one by one (the
+// two cells may even have different ones), the others in pairs from even cells on.
+template <int W, bool EVEN>
+__device__ __forceinline__ void combine_unit(const CombineUnit &un, const float *__restrict__ boxes, float *__restrict__ fd,
+                                             bool add)
 {
     using S = TileShape<W>;
     const int n = un.n, ex = un.edge[0], ey = un.edge[1], ez = un.edge[2];
-    // rows near a face along y and z: all of x; rows near one of them: the two ends of x
-    const int nx = ex / P, ends = 4 / P, both = 16 * nx, one_z = 4 * (ey - 4), one = one_z + 4 * (ez - 4);
+    const bool vec = ((un.start[0] | n) & 1) == 0 && (reinterpret_cast<uintptr_t>(fd) & 7) == 0;
+    // rows near a face along y and z: all of x; rows near one of them: the two ends of x.
+    // add: rows near a face along y or z: all of x; the others: the ends
+    const int nx = (ex + 1) / 2, one_z = 4 * (ey - 4), one = one_z + 4 * (ez - 4);
+    const int whole = nx * (add ? 16 + one : 16), part = 2 * (add ? (ey - 4) * (ez - 4) : one);
     auto near = [](int k, int e) { return k < 2 ? k : e - 4 + k; };
     // neighbour along an axis, and the cell in the neighbour's box (halo h)
     auto side = [](int c, int e) { return c < 2 ? -1 : (c >= e - 2 ? 1 : 0); };
@@ -1538,26 +1559,34 @@ __device__ __forceinline__ void combine_unit(const CombineUnit &un, const float 
     auto word_x = [](int l) { return 32 * (l >> 2) + (l & 3); };
     auto word_y = [](int l) { return 32 * S::NX * S::NZ * (l >> 1) + 16 * (l & 1); };
     auto word_z = [](int l) { return 32 * S::NX * (l >> 2) + 4 * (l & 3); };
-    for (int i = threadIdx.x; i < both + ends * one; i += kCombineThreads) {
-        int x, y, z;
-        if (i < both) {
-            const int r = i / nx;
-            x = P * (i - r * nx);
+    for (int i = threadIdx.x; i < whole + part; i += kCombineThreads) {
+        int x, y, z, r;   // r: the row, first the 16 near both, then those near one, then the others
+        if (i < whole) {
+            r = i / nx;
+            x = 2 * (i - r * nx);
+        } else {
+            const int j = i - whole;
+            r = (j >> 1) + (add ? 16 + one : 16);
+            x = j & 1 ? ex - 2 : 0;
+        }
+        if (r < 16) {
             z = near(r & 3, ez);
             y = near(r >> 2, ey);
+        } else if (r < 16 + one_z) {
+            z = near(r & 3, ez);
+            y = 2 + ((r - 16) >> 2);
+        } else if (r < 16 + one) {
+            y = near((r - 16 - one_z) & 3, ey);
+            z = 2 + ((r - 16 - one_z) >> 2);
         } else {
-            const int j = i - both, k = j & (ends - 1), r = j / ends;
-            x = P == 2 ? (k ? ex - 2 : 0) : near(k, ex);
-            if (r < one_z) {
-                z = near(r & 3, ez);
-                y = 2 + (r >> 2);
-            } else {
-                y = near((r - one_z) & 3, ey);
-                z = 2 + ((r - one_z) >> 2);
-            }
+            z = (r - 16 - one) / (ey - 4);
+            y = 2 + r - 16 - one - z * (ey - 4);
+            z += 2;
         }
-        const int o[3] = {side(x, ex), side(y, ey), side(z, ez)};
+        const bool two = EVEN || x + 1 < ex;
+        const int o[3] = {side(x, ex), side(y, ey), side(z, ez)}, o1 = EVEN ? o[0] : (two ? side(x + 1, ex) : 0);
         const int wx[2] = {word_x(x + 4), word_x(other(x, ex, un.prev[0], 4))};
+        const int wx1[2] = {word_x(x + 5), word_x(other(x + 1, ex, un.prev[0], 4))};
         const int wy[2] = {word_y(y + 2), word_y(other(y, ey, un.prev[1], 2))};
         const int wz[2] = {word_z(z + 2), word_z(other(z, ez, un.prev[2], 2))};
         float2 q[8];
@@ -1565,17 +1594,25 @@ __device__ __forceinline__ void combine_unit(const CombineUnit &un, const float 
 #pragma unroll
         for (int k = 0; k < 8; ++k) {   // own box first
             const int kx = k & 1, ky = k >> 1 & 1, kz = k >> 2;
-            const int slot = un.slot[13 + kx * o[0] + 3 * ky * o[1] + 9 * kz * o[2]];
+            const int at = 13 + 3 * ky * o[1] + 9 * kz * o[2];
+            const float *p = boxes + (ky ? wy[1] : wy[0]) + (kz ? wz[1] : wz[0]);
+            const bool there = !(ky && !o[1]) && !(kz && !o[2]);
             q[k] = make_float2(0.f, 0.f);
-            if (slot >= 0 && !(kx && !o[0]) && !(ky && !o[1]) && !(kz && !o[2])) {
-                const float *p = boxes + 3LL * S::kWords * slot + (kx ? wx[1] : wx[0]) + (ky ? wy[1] : wy[0]) +
-                                 (kz ? wz[1] : wz[0]);
-                any = true;
-                if (P == 2)
-                    q[k] = __ldg(reinterpret_cast<const float2 *>(p));
-                else
-                    q[k].x = __ldg(p);
+            const int slot = un.slot[at + kx * o[0]];
+            const bool first = there && slot >= 0 && !(kx && !o[0]);
+            if (EVEN || (!kx && !(x & 1))) {   // an odd row's last pair ends outside the tile: a cell of the box
+                if (first)
+                    q[k] = __ldg(reinterpret_cast<const float2 *>(p + 3LL * S::kWords * slot + (kx ? wx[1] : wx[0])));
+            } else {
+                const int slot1 = un.slot[at + kx * o1];
+                if (first)
+                    q[k].x = __ldg(p + 3LL * S::kWords * slot + (kx ? wx[1] : wx[0]));
+                if (two && there && slot1 >= 0 && !(kx && !o1)) {
+                    q[k].y = __ldg(p + 3LL * S::kWords * slot1 + (kx ? wx1[1] : wx1[0]));
+                    any = true;
+                }
             }
+            any |= first;
         }
         if (!any)
             continue;
@@ -1586,16 +1623,29 @@ __device__ __forceinline__ void combine_unit(const CombineUnit &un, const float 
             acc.y += q[k].y;
         }
         float *out = fd + ((long long)(un.start[2] + z) * n + un.start[1] + y) * n + un.start[0] + x;
-        if (P == 2)
+        if (add) {   // one term a value; by reductions, so that calls on other streams may add to f too
+            if (vec && two && !(x & 1)) {
+                if (acc.x != 0.f || acc.y != 0.f)
+                    red_add_v2(out, acc.x, acc.y);
+            } else {
+                if (acc.x != 0.f)
+                    red_add(out, acc.x);
+                if (two && acc.y != 0.f)
+                    red_add(out + 1, acc.y);
+            }
+        } else if (vec && two && !(x & 1)) {
             *reinterpret_cast<float2 *>(out) = acc;
-        else
+        } else {
             *out = acc.x;
+            if (two)
+                out[1] = acc.y;
+        }
     }
 }
 
 template <int W>
 __global__ void __launch_bounds__(kCombineThreads, 8)
-    tile_combine_kernel(DevGrid g, DevWork w, float *__restrict__ f)
+    tile_combine_kernel(DevGrid g, DevWork w, float *__restrict__ f, int add)
 {
     pdl_wait();
     using S = TileShape<W>;
@@ -1653,21 +1703,14 @@ __global__ void __launch_bounds__(kCombineThreads, 8)
         const int d = unit % 3, n = un.n;
         float *fd = f + un.off + (long long)d * n * n * n;
         const float *boxes = w.box_buf + (long long)d * S::kWords;
-        if (((un.start[0] | n | un.edge[0] | un.prev[0]) & 3) == 0 && (reinterpret_cast<uintptr_t>(fd) & 15) == 0)
-            combine_unit<W, 2>(un, boxes, fd);
+        if (((un.edge[0] | un.prev[0]) & 1) == 0)
+            combine_unit<W, true>(un, boxes, fd, add != 0);
         else
-            combine_unit<W, 1>(un, boxes, fd);
+            combine_unit<W, false>(un, boxes, fd, add != 0);
         if (threadIdx.x < 32)
             keep(s_unit[buf ^ 1]);
         __syncthreads();
     }
-}
-
-// f += a field (the reproducible spread onto a field that is not cleared)
-static __global__ void __launch_bounds__(256) add_field_kernel(float *__restrict__ f, const float *__restrict__ a, long long total)
-{
-    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < total; i += 256LL * gridDim.x)
-        f[i] += a[i];
 }
 
 // ---------------------------------------- spread, FP64 deterministic, MLS
