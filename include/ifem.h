@@ -229,10 +229,16 @@ int ifem_batch_set_origins(ifem_batch b, const double *origins);
  * If ctx was created with tile = 0 and has not been tuned yet, first run the
  * tile autotuner: binning + spreading + interpolation of b at positions x
  * (device node array, required then) are timed with CUDA events on `stream`
- * for tile edges {8, 12, 16} (FP32) or {6, 8, 10} (FP64), and the fastest is
+ * for tile edges {8, 12, 16} (FP32) or {6, 8, 10, 12} (FP64), and the fastest is
  * kept (ifem_ctx_tile). Autotuning allocates temporary buffers and
  * synchronises: call it outside stream capture. Without ifem_prepare, a
- * context with tile = 0 uses 16 (FP32) or 8 (FP64). */
+ * context with tile = 0 uses 16 (FP32) or 8 (FP64).
+ * Device memory: about 60 bytes (FP32) or 260 (FP64) per node and 1.3 KB per
+ * tile; with the reproducible FP32 spread (IFEM_SCATTER_DET, or MLS27) also each
+ * tile's cells and halo, for at most as many tiles as nodes: 3 x 38 KB for tiles
+ * of up to 16 cells a side (3 x 20 KB up to 12, 3 x 9 KB up to 8) while that is at
+ * most 4 GB in all, else a third of it (the lattices are then taken one after the
+ * other), in managed memory where the device has no room left. */
 int ifem_prepare(ifem_ctx ctx, ifem_batch b, const void *x, void *stream);
 
 /* --------------------------------------------------------------- compute */

@@ -783,6 +783,13 @@ static void own_tiling(int n, int tile, int &t, int &T)
     }
 }
 
+// Boxes of the reproducible spread's three lattices at a time up to this memory (37000
+// tiles of 16 cells, 540^3). Beyond it, and where the device has no room for them, one
+// lattice after the other takes a third of the memory (38 KB a tile, whose cells take
+// 49 KB of a field) and four more launches: 60 red cells in 512^3 390 and 431 us, 1500
+// mixed cells in 400^3 1664 and 1685, 72 in 128^3 96 and 133.
+constexpr size_t kBoxBytes = size_t(4) << 30;
+
 // Work buffers for (batch, grid, tile): box/tile tables, per-tile lists.
 static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
 {
@@ -853,8 +860,25 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
         CK(alloc((void **)&w.tile_slot, sizeof(int) * (size_t)(nt + 1)));
         CK(alloc((void **)&w.node_key, sizeof(int2) * Nn));
         CK(alloc((void **)&w.node_rec, sizeof(float4) * Nn));
-        if (reproducible(ctx)) {   // a box per listed tile and lattice: at most one tile per node
-            CK(alloc((void **)&w.box_buf, tile_box_bytes(max_edge) * 3 * (size_t)std::min(nt, N)));
+        if (reproducible(ctx)) {
+            // a box per listed tile, at most one tile per node, for each lattice or for the three in
+            // turn; last, in memory that may lie on the host, so that what a grid and its fields leave
+            // of the device is enough
+            const size_t one = tile_box_bytes(max_edge) * (size_t)std::min(nt, N);
+            w.box_lattices = 3 * one <= kBoxBytes ? 3 : 1;
+            cudaError_t e = alloc((void **)&w.box_buf, one * w.box_lattices);
+            if (e == cudaErrorMemoryAllocation && w.box_lattices == 3) {
+                cudaGetLastError();
+                w.box_lattices = 1;
+                e = alloc((void **)&w.box_buf, one);
+            }
+            if (e == cudaErrorMemoryAllocation) {
+                cudaGetLastError();
+                e = cudaMallocManaged((void **)&w.box_buf, std::max<size_t>(one, 16));
+                if (e == cudaSuccess)
+                    ws.allocs.push_back(w.box_buf);
+            }
+            CK(e);
             CK(alloc((void **)&w.near_tile, sizeof(int2) * (size_t)(nt + 1)));
         }
     } else {

@@ -171,7 +171,8 @@ struct DevWork {
     TileDesc *tile_desc;  // tiles with own nodes (FP32), counters[3] of them
     int *tile_slot;     // n_tiles (FP32): a tile's place in that list, or -1
     int2 *near_tile;    // reproducible spread: tiles that a box reaches and their boxes, counters[9] of them
-    float *box_buf;     // reproducible spread: a box per listed tile and lattice
+    float *box_buf;     // reproducible spread: a box per listed tile and, with box_lattices = 3, lattice;
+    int box_lattices;   // with 1 the lattices take it in turn
     int *counters;      // kCounters: [2] work counter, [3] tiles with own nodes,
                         // [4] total pairs, [5] total own nodes, [1] [6] [7] work counters of
                         // one-lattice launches, [8] scan blocks finished, [9] near_tile entries,

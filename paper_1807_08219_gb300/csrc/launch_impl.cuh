@@ -232,14 +232,27 @@ cudaError_t launch_tile_w(const TransferArgs &a)
     cfg.stream = a.stream;
     cfg.attrs = attr;
     cfg.numAttrs = a.pdl || a.lattice < 0 ? 1 : 0;
-    e = cudaLaunchKernelEx(&cfg, kern, a.b, a.w, (const float *)a.x, f, a.density, (const float *)a.u,
-                           (float *)a.v, (const float *)a.vp, (float *)a.xn, (float)a.dt, (float)(1.0 / a.support),
-                           a.lattice, add);
-    if (e != cudaSuccess || !STORE)
-        return e;
-    const long long units = 3 * std::min<long long>(a.g.n_tiles, 27 * a.b.N);
+    auto transfer = [&](int lattice) {
+        return cudaLaunchKernelEx(&cfg, kern, a.b, a.w, (const float *)a.x, f, a.density, (const float *)a.u,
+                                  (float *)a.v, (const float *)a.vp, (float *)a.xn, (float)a.dt,
+                                  (float)(1.0 / a.support), lattice, add);
+    };
+    if (!STORE)
+        return transfer(a.lattice);
+    // one lattice after the other where the buffer holds the boxes of one: each waits
+    // for the combination of the one before
+    const bool apart = a.w.box_lattices == 1;
+    if (apart)
+        cfg.numAttrs = 0;
+    const long long units = (apart ? 1 : 3) * std::min<long long>(a.g.n_tiles, 27 * a.b.N);
     const long long blocks = std::min(units, 8LL * a.n_sm);   // all resident
-    return launch_after(tile_combine_kernel<W>, (unsigned)blocks, kCombineThreads, 0, a.stream, a.g, a.w, f, add);
+    auto combine = apart ? tile_combine_kernel<W, 1> : tile_combine_kernel<W, 3>;
+    for (int d = apart ? 0 : -1; d < (apart ? 3 : 0); ++d)
+        if ((e = transfer(d)) != cudaSuccess ||
+            (e = launch_after(combine, (unsigned)blocks, kCombineThreads, 0, a.stream, a.g, a.w, f, add,
+                              d)) != cudaSuccess)
+            return e;
+    return cudaSuccess;
 }
 template <int KER, bool SPREAD, bool INTERP, bool STORE>
 cudaError_t launch_tile(const TransferArgs &a)

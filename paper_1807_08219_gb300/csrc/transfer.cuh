@@ -1004,7 +1004,8 @@ __device__ __forceinline__ void tile_stage(const TileItem &it, const float *__re
 // faces along two axes or three, go to the item's box of the buffer instead, in
 // A's own order, zero or not; the others have at most two terms, whose sum from
 // zero is the same in either order. add (f is not cleared): values that two boxes
-// can reach, near a face along one axis, go there too. bt: box thread.
+// can reach, near a face along one axis, go there too. buf: the item's place in the
+// buffer. bt: box thread.
 template <int W, bool STORE>
 __device__ __forceinline__ long long tile_flush(const TileItem &it, float *__restrict__ f, float *__restrict__ buf,
                                                 int4 *A, float inv, int bt, bool add, unsigned &touched)
@@ -1029,7 +1030,7 @@ __device__ __forceinline__ long long tile_flush(const TileItem &it, float *__res
 #pragma unroll
     for (int c = 0; c < 4; ++c)
         face_x |= (4 * gx + c < 6 || 4 * gx + c >= it.ex + 2) ? 1u << c : 0u;
-    float4 *out = reinterpret_cast<float4 *>(buf + (3LL * it.slot + it.d) * S::kWords) + bt;
+    float4 *out = reinterpret_cast<float4 *>(buf) + bt;
     long long qsum = 0;
     A += bt;
 #pragma unroll
@@ -1484,7 +1485,8 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
                 const TileItem old = tile_item(s_desc[(i - 1) % kRing], s_d[(i - 1) % kRing], density);
                 int4 *box_A = reinterpret_cast<int4 *>(A + ((i - 1) & 1) * kBox);
                 const float inv = s_scale[(i - 1) & 3].y;
-                long long qsum = tile_flush<W, STORE>(old, f, w.box_buf, box_A, inv, bt, add != 0, touched);
+                float *buf = w.box_buf + ((long long)w.box_lattices * old.slot + (w.box_lattices == 3 ? old.d : 0)) * S::kWords;
+                long long qsum = tile_flush<W, STORE>(old, f, buf, box_A, inv, bt, add != 0, touched);
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1)
                     qsum += __shfl_down_sync(0xffffffffu, qsum, o);
@@ -1514,7 +1516,7 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
 // The reproducible spread's second half: the values of the cleared field f that
 // three or more boxes can reach (tile_flush), each the sum of its boxes' terms
 // in a fixed order; with add those that two or more can reach, the sum added to f.
-// Unit = (tile, lattice). Every tile has at least 4 cells per
+// Unit = (tile, lattice); L = 1: of the lattice given. Every tile has at least 4 cells per
 // axis (own_tiling), so a value near a face has one neighbour there, along two
 // axes or three of them; along an axis of one or two tiles the neighbour is the
 // tile itself or the same one on both sides, with different cells of its box.
@@ -1541,11 +1543,14 @@ constexpr int kCombineThreads = 128;
 // the one before it have an even number of cells along x, so that both cells lie in
 // one pair of every box; else the x neighbours' values are loaded one by one (the
 // two cells may even have different ones), the others in pairs from even cells on.
-template <int W, bool EVEN>
+// L: lattices whose boxes are kept (DevWork::box_lattices; known when compiled, 117 us
+// for a step of 72 mixed cells with add, 125 with the product at run time).
+template <int W, int L, bool EVEN>
 __device__ __forceinline__ void combine_unit(const CombineUnit &un, const float *__restrict__ boxes, float *__restrict__ fd,
                                              bool add)
 {
     using S = TileShape<W>;
+    constexpr long long kStride = (long long)L * S::kWords;   // between the boxes of two tiles
     const int n = un.n, ex = un.edge[0], ey = un.edge[1], ez = un.edge[2];
     const bool vec = ((un.start[0] | n) & 1) == 0 && (reinterpret_cast<uintptr_t>(fd) & 7) == 0;
     // rows near a face along y and z: all of x; rows near one of them: the two ends of x.
@@ -1602,13 +1607,13 @@ __device__ __forceinline__ void combine_unit(const CombineUnit &un, const float 
             const bool first = there && slot >= 0 && !(kx && !o[0]);
             if (EVEN || (!kx && !(x & 1))) {   // an odd row's last pair ends outside the tile: a cell of the box
                 if (first)
-                    q[k] = __ldg(reinterpret_cast<const float2 *>(p + 3LL * S::kWords * slot + (kx ? wx[1] : wx[0])));
+                    q[k] = __ldg(reinterpret_cast<const float2 *>(p + kStride * slot + (kx ? wx[1] : wx[0])));
             } else {
                 const int slot1 = un.slot[at + kx * o1];
                 if (first)
-                    q[k].x = __ldg(p + 3LL * S::kWords * slot + (kx ? wx[1] : wx[0]));
+                    q[k].x = __ldg(p + kStride * slot + (kx ? wx[1] : wx[0]));
                 if (two && there && slot1 >= 0 && !(kx && !o1)) {
-                    q[k].y = __ldg(p + 3LL * S::kWords * slot1 + (kx ? wx1[1] : wx1[0]));
+                    q[k].y = __ldg(p + kStride * slot1 + (kx ? wx1[1] : wx1[0]));
                     any = true;
                 }
             }
@@ -1643,19 +1648,19 @@ __device__ __forceinline__ void combine_unit(const CombineUnit &un, const float 
     }
 }
 
-template <int W>
+template <int W, int L>
 __global__ void __launch_bounds__(kCombineThreads, 8)
-    tile_combine_kernel(DevGrid g, DevWork w, float *__restrict__ f, int add)
+    tile_combine_kernel(DevGrid g, DevWork w, float *__restrict__ f, int add, int lattice)
 {
     pdl_wait();
     using S = TileShape<W>;
     __shared__ CombineUnit s_unit[2];
-    const int units = 3 * w.counters[9], lane = threadIdx.x;
+    const int units = L * w.counters[9], lane = threadIdx.x;
     // first warp: lane k < 27 a neighbour's slot, lanes 27 to 29 an axis, lane 30 the box
     int3 got;
     long long off = 0;
     auto near_of = [&](int unit) {
-        return unit < units ? w.near_tile[unit / 3] : make_int2(-1, 0);   // tile, box
+        return unit < units ? w.near_tile[unit / L] : make_int2(-1, 0);   // tile, box
     };
     auto read = [&](int2 near) {
         if (near.x < 0)
@@ -1700,13 +1705,13 @@ __global__ void __launch_bounds__(kCombineThreads, 8)
             next = near_of(unit + 2 * gridDim.x);
         }
         const CombineUnit &un = s_unit[buf];
-        const int d = unit % 3, n = un.n;
+        const int d = L == 3 ? unit % 3 : lattice, n = un.n;
         float *fd = f + un.off + (long long)d * n * n * n;
-        const float *boxes = w.box_buf + (long long)d * S::kWords;
+        const float *boxes = w.box_buf + (L == 3 ? (long long)d * S::kWords : 0);
         if (((un.edge[0] | un.prev[0]) & 1) == 0)
-            combine_unit<W, true>(un, boxes, fd, add != 0);
+            combine_unit<W, L, true>(un, boxes, fd, add != 0);
         else
-            combine_unit<W, false>(un, boxes, fd, add != 0);
+            combine_unit<W, L, false>(un, boxes, fd, add != 0);
         if (threadIdx.x < 32)
             keep(s_unit[buf ^ 1]);
         __syncthreads();
