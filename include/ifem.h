@@ -333,7 +333,8 @@ int ifem_indicator_source(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x
 int ifem_ab2_update(ifem_ctx ctx, ifem_batch b, void *x, const void *v, const void *v_prev, double dt,
                     void *stream);
 
-/* Current volume of every particle, FP64 in both precisions: membranes by the
+/* Current volume of every particle, to FP64 accuracy in both precisions (the
+ * elements of larger FP32 meshes are evaluated in float pairs): membranes by the
  * polyhedron formula of Sec. "Conservation of Volume for Membranes",
  *   V = 1/18 sum_faces [x1.(x2 x x3) + x2.(x3 x x1) + x3.(x1 x x2)],
  * solids as the sum of their tets' signed volumes det(Ds)/6. x: device node
@@ -349,7 +350,8 @@ int ifem_volumes(ifem_ctx ctx, ifem_batch b, const void *x, double *vol, void *s
  *   A L^3 + B L^2 + C L + D = 0, A = 1/18 sum alpha.(alpha x alpha),
  *   B = 1/6 sum x.(alpha x alpha), C = 1/6 sum alpha.(x x x) (all cyclic over
  *   each face's nodes), D = V(x) - V0.
- * The cubic's sums and Lambda are FP64 in both precisions; with IFEM_FP32
+ * The cubic's sums and Lambda have FP64 accuracy in both precisions (A, B, C of
+ * FP32 positions to a few 1e-16, from float pairs); with IFEM_FP32
  * positions alpha comes from FP32 cross products of the ring's edge vectors
  * (equal to the formula above on a closed ring), and since the cubic is built
  * from that same alpha the corrected volume still meets V0. V0: device double array of n_inst

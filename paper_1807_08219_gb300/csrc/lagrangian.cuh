@@ -2,7 +2,8 @@
 // Adams-Bashforth position update (Eq. Bashforth_eqn), per-particle volumes
 // and the membrane volume correction of Sec. "Conservation of Volume for
 // Membranes" (after Mendez et al. 2014). Positions are the particles' local
-// offsets; volumes and the correction's sums are FP64 in both precisions.
+// offsets; volumes and the correction's sums have FP64 accuracy in both precisions
+// (for FP32 positions by float pairs, see below).
 #pragma once
 #include "forces.cuh"
 #include "transfer.cuh"
@@ -78,12 +79,22 @@ __global__ void __launch_bounds__(kVolThreads) volume_kernel(DevBatch b, const r
 }
 
 // ------------------------------------------------ FP32 positions, float pairs
-// Volumes and the correction's sums of FP32 positions to FP64 accuracy without
-// the FP64 pipe (two lane operations a cycle and SM on this GPU, conversions
+// Volumes and the correction's sums of FP32 positions to FP64 accuracy with little
+// of the FP64 pipe (two lane operations a cycle and SM on this GPU, conversions
 // included): a triple product of float vectors as an unevaluated float pair.
 // Products are exact (by FMA), sums carry their error term. Inputs are scaled by
 // powers of two (TmplDev::vol_scale) so that the error terms stay in range for
 // particles of any unit.
+// A pair holds 2^-48 of a term. What is left of that in a volume falls with the
+// square root of the number of elements, to what FP64 leaves from kPairElems of them
+// on, if the sums themselves are FP64 (each element's below kPairFew elements, four
+// as a pair from there; vol_totals). Relative error of the volume, rms over random
+// affine maps and noise, FP64 and pairs: 80 triangles 0.8 and 1.9e-16, 320 0.7 and
+// 1.0e-16, 1280 0.7 and 0.9e-16 (red cells 0.8 and 0.8e-16), 2058 tets 0.7 and
+// 0.8e-16, 5120 triangles 0.8 and 0.7e-16; pairs summed as pairs up to the block 3 to
+// 5e-16 throughout. Below, volumes take the FP64 pipe.
+constexpr int kPairElems = 1024, kPairFew = 4096;
+
 __device__ __forceinline__ DF df_cross_comp(float a1, float b2, float a2, float b1)   // a1 b2 - a2 b1
 {
     const float p = __fmul_rn(a1, b2), pe = fmaf(a1, b2, -p), q = __fmul_rn(a2, b1), qe = fmaf(a2, b1, -q);
@@ -92,17 +103,37 @@ __device__ __forceinline__ DF df_cross_comp(float a1, float b2, float a2, float 
     const float h = s + e;
     return DF{h, e - (h - s)};
 }
-__device__ __forceinline__ DF df_triple(const float a[3], const float b[3], const float c[3])   // a . (b x c)
+// x + y as a sum and its error
+__device__ __forceinline__ float two_sum(float x, float y, float &err)
 {
-    DF t{0.f, 0.f};
+    const float s = x + y, b = s - x;
+    err = (x - (s - b)) + (y - b);
+    return s;
+}
+// a . (b x c) + rest: the products' high parts are summed exactly, what is below
+// them (eight terms and rest) with its error, so that half an ulp of the low part
+// is nearly all that is lost
+__device__ __forceinline__ DF df_triple(const float a[3], const float b[3], const float c[3], float rest)
+{
+    float h = 0.f, l = rest, m = 0.f;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const int j = (i + 1) % 3, k = (i + 2) % 3;
         const DF u = df_cross_comp(b[j], c[k], b[k], c[j]);
-        const float p = __fmul_rn(u.hi, a[i]);
-        df_add_df(t, DF{p, fmaf(u.hi, a[i], -p) + u.lo * a[i]});
+        const float p = __fmul_rn(u.hi, a[i]), pe = fmaf(u.hi, a[i], -p);
+        float e, e1, e2;
+        h = i ? two_sum(h, p, e) : p;
+        l = two_sum(l, pe, e1);
+        l = two_sum(l, __fmul_rn(u.lo, a[i]), e2);
+        m += e1 + e2;
+        if (i) {
+            l = two_sum(l, e, e1);
+            m += e1;
+        }
     }
-    return t;
+    float e;
+    h = two_sum(h, l, e);
+    return DF{h, e + m};
 }
 // y - x as an exact float pair h + l (l is mostly 0)
 __device__ __forceinline__ void df_edge(const float x[3], const float y[3], float h[3], float l[3])
@@ -129,9 +160,7 @@ __device__ __forceinline__ DF df_face(const float p[3][3])
     float h1[3], l1[3], h2[3], l2[3];
     df_edge(p[0], p[1], h1, l1);
     df_edge(p[0], p[2], h2, l2);
-    DF t = df_triple(p[0], h1, h2);
-    df_add(t, dot_cross_f32(p[0], l1, h2) + dot_cross_f32(p[0], h1, l2));
-    return t;
+    return df_triple(p[0], h1, h2, dot_cross_f32(p[0], l1, h2) + dot_cross_f32(p[0], h1, l2));
 }
 // det of a tet's edges x_i - x_0, the same way
 __device__ __forceinline__ DF df_tet(const float x[4][3])
@@ -140,29 +169,61 @@ __device__ __forceinline__ DF df_tet(const float x[4][3])
 #pragma unroll
     for (int c = 0; c < 3; ++c)
         df_edge(x[0], x[1 + c], h[c], l[c]);
-    DF t = df_triple(h[0], h[1], h[2]);
+    float rest = 0.f;
 #pragma unroll
     for (int c = 0; c < 3; ++c)
-        df_add(t, dot_cross_f32(l[c], h[(c + 1) % 3], h[(c + 2) % 3]));
-    return t;
+        rest += dot_cross_f32(l[c], h[(c + 1) % 3], h[(c + 2) % 3]);
+    return df_triple(h[0], h[1], h[2], rest);
 }
 
 constexpr int kVolThreadsF = 512;
 
-// Fixed-order block total of float pairs, in FP64 (every thread gets it).
-__device__ __forceinline__ double df_block_sum(DF v, double *sh)
+// A thread's sum of float pairs: so many as a pair, those in FP64.
+struct PairSum {
+    DF p{0.f, 0.f};
+    double s = 0.0;
+    int n = 0;
+    __device__ __forceinline__ void add(DF t) { df_add_df(p, t); }
+    __device__ __forceinline__ void add(DF t, int every)
+    {
+        df_add_df(p, t);
+        if (++n == every)
+            flush();
+    }
+    __device__ __forceinline__ void flush()
+    {
+        s += (double)p.hi;
+        s += (double)p.lo;
+        p = DF{0.f, 0.f};
+        n = 0;
+    }
+};
+
+// Fixed-order block totals of Q FP64 values per thread, a warp each (every thread
+// gets them).
+template <int Q>
+__device__ __forceinline__ void vol_totals(const double (&v)[Q], double (*sh)[kVolThreadsF], double (&tot)[Q])
 {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        df_add_df(v, DF{__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o)});
-    __syncthreads();   // sh may still be read from an earlier total
-    if ((threadIdx.x & 31) == 0)
-        sh[threadIdx.x >> 5] = (double)v.hi + (double)v.lo;
+    for (int q = 0; q < Q; ++q)
+        sh[q][threadIdx.x] = v[q];
     __syncthreads();
-    double r = 0.0;
-    for (int q = 0; q < kVolThreadsF / 32; ++q)
-        r += sh[q];
-    return r;
+    if (wid < Q) {
+        double r = 0.0;
+        for (int k = lane; k < kVolThreadsF; k += 32)
+            r += sh[wid][k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            r += __shfl_down_sync(0xffffffffu, r, o);
+        __syncwarp();   // the warp has read its row
+        if (lane == 0)
+            sh[wid][0] = r;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+        tot[q] = sh[q][0];
 }
 
 // Stages an instance's positions, scaled, in shared memory.
@@ -186,29 +247,48 @@ __device__ __forceinline__ double vol_unscale(float scale, int power)   // scale
     const double r = 1.0 / (double)scale;
     return power == 2 ? r * r : (power == 3 ? r * r * r : r);
 }
+// Adds an element's six-fold volume: p its corners, E its template's elements.
+__device__ __forceinline__ void vol_add(PairSum &s, int kind, int E, const float p[4][3])
+{
+    if (E >= kPairElems) {
+        s.add(kind == 0 ? df_face(p) : df_tet(p), E >= kPairFew ? 4 : 1);
+        return;
+    }
+    double q[3][3], t[3];   // a face's corners, or a tet's edges
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            q[c][a] = kind == 0 ? (double)p[c][a] : (double)p[c + 1][a] - (double)p[0][a];
+    cross3d(q[1], q[2], t);
+    s.s += dot3d(q[0], t);
+}
 
 // Block per instance, FP32 positions (templates whose positions fit shared
-// memory): the formulas of volume_kernel. 200 capsules of 2562 nodes: 16 us
-// against 58 us in FP64.
+// memory): the formulas of volume_kernel. 200 capsules of 2562 nodes: 18 us
+// against 59 us in FP64; of 642 nodes 10 and 19.
 static __global__ void __launch_bounds__(kVolThreadsF) volume_f32_kernel(DevBatch b, const float *__restrict__ x,
                                                                          double *__restrict__ vol)
 {
     extern __shared__ __align__(16) float4 vol_xs[];
-    __shared__ double sh[kVolThreadsF / 32];
+    __shared__ double sh[1][kVolThreadsF];
     const InstDev I = b.inst[blockIdx.x];
     const TmplDev &T = b.tmpl[I.tmpl];
     vol_stage(I, x, b.N, T.vol_scale, vol_xs);
-    DF s{0.f, 0.f};
+    const int nv = T.kind == 0 ? 3 : 4;
+    PairSum s;
     for (int e = threadIdx.x; e < T.n_elems; e += kVolThreadsF) {
         float p[4][3];
-        const int nv = T.kind == 0 ? 3 : 4;
         for (int c = 0; c < nv; ++c)
             vol_get(vol_xs, T.elems[nv * e + c], p[c]);
-        df_add_df(s, T.kind == 0 ? df_face(p) : df_tet(p));
+        vol_add(s, T.kind, T.n_elems, p);
     }
-    const double r = df_block_sum(s, sh);
+    s.flush();
+    const double v[1] = {s.s};
+    double r[1];
+    vol_totals(v, sh, r);
     if (threadIdx.x == 0)
-        vol[blockIdx.x] = r * vol_unscale(T.vol_scale, 3) / 6.0;
+        vol[blockIdx.x] = r[0] * vol_unscale(T.vol_scale, 3) / 6.0;
 }
 
 // Thread per (instance, node) of a membrane: alpha_I = -(1/12) sum over the
@@ -373,15 +453,19 @@ __global__ void __launch_bounds__(kVolThreads) vc_correct_kernel(DevBatch b, rea
 // whose positions and alphas fit shared memory): alpha_I as in vc_alpha_kernel
 // (12 alpha = -acc, acc an FP32 sum of edge cross products, kept as it is), the
 // cubic's sums in float pairs with the factors 1/12 taken out, Newton in FP64,
-// x_I = x_I + Lambda alpha_I to one rounding. 200 capsules of 2562 nodes: 73 us
-// against 203 us for vc_alpha_kernel and vc_correct_kernel in FP64.
+// x_I = x_I + Lambda alpha_I to one rounding. D is what Lambda's error comes from
+// (a volume to 1e-16 less a close one), so A, B and C are kept as pairs up to the
+// block. Lambda differs from the FP64 kernels' by what FP64 leaves (1e-13 for a
+// volume off by 1e-3). 200 capsules of 2562 nodes: 61 us against 203 us for
+// vc_alpha_kernel and vc_correct_kernel in FP64; of 642 nodes 29 and 64, 162 nodes
+// 23 and 31.
 static __global__ void __launch_bounds__(kVolThreadsF) vc_fused_f32_kernel(DevBatch b, float *__restrict__ x,
                                                                            const double *__restrict__ V0,
                                                                            double *__restrict__ lambda,
                                                                            unsigned long long *status)
 {
     extern __shared__ __align__(16) float4 vol_xs[];
-    __shared__ double sh[kVolThreadsF / 32];
+    __shared__ double sh[4][kVolThreadsF];
     __shared__ double sL;
     const InstDev I = b.inst[blockIdx.x];
     const TmplDev &T = b.tmpl[I.tmpl];
@@ -395,7 +479,7 @@ static __global__ void __launch_bounds__(kVolThreadsF) vc_fused_f32_kernel(DevBa
     const float sx = T.vol_scale, sa = sx * sx;
     float4 *xs = vol_xs, *as = vol_xs + nn;   // positions and the alphas' sums, scaled
     vol_stage(I, x, N, sx, xs);
-    DF sA{0.f, 0.f}, sB{0.f, 0.f}, sC{0.f, 0.f}, sV{0.f, 0.f};
+    PairSum sA, sB, sC, sV;
     for (int k = threadIdx.x; k < nn; k += kVolThreadsF) {
         const float4 xk = xs[k];
         const float pk[3] = {xk.x, xk.y, xk.z};
@@ -418,29 +502,36 @@ static __global__ void __launch_bounds__(kVolThreadsF) vc_fused_f32_kernel(DevBa
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const float p = __fmul_rn(acc[a], acc[a]);
-            df_add_df(sC, DF{p, fmaf(acc[a], acc[a], -p)});
+            sC.add(DF{p, fmaf(acc[a], acc[a], -p)});
         }
     }
     __syncthreads();
     for (int e = threadIdx.x; e < T.n_elems; e += kVolThreadsF) {
-        float p[3][3], q[3][3];
+        float p[4][3], q[3][3];
         for (int c = 0; c < 3; ++c) {
             const int v = T.elems[3 * e + c];
             vol_get(xs, v, p[c]);
             vol_get(as, v, q[c]);
         }
         // the cyclic terms: the three of A and of V are equal, B takes all
-        df_add_df(sV, df_face(p));
-        df_add_df(sA, df_triple(q[0], q[1], q[2]));
-        df_add_df(sB, df_triple(p[0], q[1], q[2]));
-        df_add_df(sB, df_triple(p[1], q[2], q[0]));
-        df_add_df(sB, df_triple(p[2], q[0], q[1]));
+        vol_add(sV, 0, T.n_elems, p);
+        sA.add(df_triple(q[0], q[1], q[2], 0.f));
+        sB.add(df_triple(p[0], q[1], q[2], 0.f));
+        sB.add(df_triple(p[1], q[2], q[0], 0.f));
+        sB.add(df_triple(p[2], q[0], q[1], 0.f));
     }
+    sA.flush();
+    sB.flush();
+    sC.flush();
+    sV.flush();
+    const double v[4] = {sA.s, sB.s, sC.s, sV.s};
+    double tot[4];
+    vol_totals(v, sh, tot);
     const double ux = vol_unscale(sx, 1), ua = vol_unscale(sa, 1), g = -1.0 / 12.0;
-    const double A = df_block_sum(sA, sh) * (ua * ua * ua) * (g * g * g) / 6.0;
-    const double B = df_block_sum(sB, sh) * (ux * ua * ua) * (g * g) / 6.0;
-    const double C = -2.0 * df_block_sum(sC, sh) * (ua * ua) * (g * g);
-    const double D = df_block_sum(sV, sh) * (ux * ux * ux) / 6.0 - V0[blockIdx.x];
+    const double A = tot[0] * (ua * ua * ua) * (g * g * g) / 6.0;
+    const double B = tot[1] * (ux * ua * ua) * (g * g) / 6.0;
+    const double C = -2.0 * tot[2] * (ua * ua) * (g * g);
+    const double D = tot[3] * (ux * ux * ux) / 6.0 - V0[blockIdx.x];
     if (threadIdx.x == 0) {
         const double L = vc_newton(A, B, C, D, status);
         sL = L;

@@ -29,7 +29,9 @@ static cudaError_t allow_smem(Kernel kern, size_t largest, int &done)
     done = e == cudaSuccess;
     return e;
 }
-constexpr size_t kVolSmemBytes = kMaxCtaSmemBytes - 1024;   // beside the volume kernels' own arrays
+// beside the kernels' own arrays (vol_totals)
+constexpr size_t kVolSmemBytes = kMaxCtaSmemBytes - 8 * kVolThreadsF - 1024;
+constexpr size_t kVcorrSmemBytes = kMaxCtaSmemBytes - 4 * 8 * kVolThreadsF - 1024;
 
 // FP32 nodal forces of particles [inst0, inst0 + n): a cluster of S CTAs per
 // particle. With few particles one CTA each leaves most SMs idle; with many,
@@ -409,7 +411,8 @@ cudaError_t volume_impl(const LagrangeArgs &a)
         return cudaSuccess;
     if constexpr (std::is_same<real, float>::value) {
         const size_t sm = sizeof(float4) * (size_t)a.b.max_nodes;
-        if (sm <= kVolSmemBytes) {
+        // all in FP64: volume_kernel's smaller blocks (200 capsules of 162 nodes 8 us, 12)
+        if (sm <= kVolSmemBytes && a.b.max_elems >= kPairElems) {
             if (cudaError_t e = allow_smem(volume_f32_kernel, kVolSmemBytes, a.cache->volume))
                 return e;
             volume_f32_kernel<<<a.b.n_inst, kVolThreadsF, sm, a.stream>>>(a.b, (const float *)a.x, a.out);
@@ -429,8 +432,8 @@ cudaError_t vcorr_impl(const LagrangeArgs &a)
         return cudaSuccess;
     if constexpr (std::is_same<real, float>::value) {
         const size_t sm = 2 * sizeof(float4) * (size_t)a.b.max_nodes;
-        if (sm <= kVolSmemBytes) {
-            if (cudaError_t e = allow_smem(vc_fused_f32_kernel, kVolSmemBytes, a.cache->vcorr))
+        if (sm <= kVcorrSmemBytes) {
+            if (cudaError_t e = allow_smem(vc_fused_f32_kernel, kVcorrSmemBytes, a.cache->vcorr))
                 return e;
             vc_fused_f32_kernel<<<a.b.n_inst, kVolThreadsF, sm, a.stream>>>(a.b, (float *)a.x, a.V0, a.out, a.status);
             IFEM_LAUNCH_CHECK();
