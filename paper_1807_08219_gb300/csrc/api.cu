@@ -344,16 +344,33 @@ static int nodal_upload(ifem_ctx ctx, ifem_tmpl t, int nv, const int32_t *el, co
             width = std::max(width, off[k + 1] - off[k]);
         base[s + 1] = base[s] + 32 * width;
     }
-    const int per = nv == 3 ? 2 : 4;
-    std::vector<float4> r(base[slices], make_float4(0.f, 0.f, 0.f, 0.f));
-    std::vector<unsigned short> id((size_t)base[slices] * per, 0);
-    std::vector<int2> pairs;
-    std::vector<int> order;
     auto sub = [&](int i, int j, double d[3]) {
         for (int a = 0; a < 3; ++a)
             d[a] = X[3 * (size_t)i + a] - X[3 * (size_t)j + a];
     };
     auto dot = [](const double *p, const double *q) { return p[0] * q[0] + p[1] * q[1] + p[2] * q[2]; };
+    // edge dot products at a triangle's corners
+    auto corner_dots = [&](const int32_t *v, double d[3]) {
+        for (int i = 0; i < 3; ++i) {
+            double p[3], q[3];
+            sub(v[(i + 1) % 3], v[i], p);
+            sub(v[(i + 2) % 3], v[i], q);
+            d[i] = dot(p, q);
+        }
+    };
+    for (int e = 0; nv == 3 && e < t->n_elems; ++e) {
+        double d[3];
+        corner_dots(el + 3 * (size_t)e, d);
+        const double A2 = 4.0 * ref[5 * (size_t)e + 4] * ref[5 * (size_t)e + 4];
+        t->obtuse = std::max(t->obtuse, (std::fabs(d[0] * d[1]) + std::fabs(d[1] * d[2]) + std::fabs(d[2] * d[0])) / A2);
+    }
+    if (t->obtuse > kObtuseMost)
+        return IFEM_OK;
+    const int per = nv == 3 ? 2 : 4;
+    std::vector<float4> r(base[slices], make_float4(0.f, 0.f, 0.f, 0.f));
+    std::vector<unsigned short> id((size_t)base[slices] * per, 0);
+    std::vector<int2> pairs;
+    std::vector<int> order;
     for (int k = 0; k < nn; ++k) {
         const int deg = off[k + 1] - off[k];
         if (nv == 3) {
@@ -372,14 +389,9 @@ static int nodal_upload(ifem_ctx ctx, ifem_tmpl t, int nv, const int32_t *el, co
                 const int32_t *v = el + 3 * (size_t)e;
                 id[2 * at] = (unsigned short)(pairs[order[s]].x | c << kNodBits);
                 id[2 * at + 1] = (unsigned short)pairs[order[s]].y;
-                float d[3];
-                for (int i = 0; i < 3; ++i) {
-                    double p[3], q[3];
-                    sub(v[(i + 1) % 3], v[i], p);
-                    sub(v[(i + 2) % 3], v[i], q);
-                    d[i] = (float)dot(p, q);
-                }
-                r[at] = make_float4(d[0], d[1], d[2], (float)(0.5 / ref[5 * (size_t)e + 4]));
+                double d[3];
+                corner_dots(v, d);
+                r[at] = make_float4((float)d[0], (float)d[1], (float)d[2], (float)(0.5 / ref[5 * (size_t)e + 4]));
             } else {
                 const double *g = ref.data() + 10 * (size_t)e;   // grad N_1..3, V0
                 double gr[4][3];
@@ -657,6 +669,10 @@ extern "C" int ifem_batch_create(ifem_ctx ctx, int n_tmpl, const ifem_tmpl *tmpl
     b->N = N;
     b->n_elems = E;
     b->nodal_ok = b->max_nodes <= kNodalMaxNodes;
+    for (int t = 0; t < n_tmpl; ++t) {
+        b->nodal_ok = b->nodal_ok && tmpls[t]->obtuse <= kObtuseMost;
+        b->any_obtuse = b->any_obtuse || tmpls[t]->obtuse > kObtuseSum;
+    }
     split_origins(b, grid);
     std::vector<TmplDev> td(n_tmpl);
     for (int t = 0; t < n_tmpl; ++t) {

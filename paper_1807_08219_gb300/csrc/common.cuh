@@ -30,6 +30,7 @@ constexpr int kMaxCtaSmemBytes = 227 * 1024;   // opt-in dynamic shared memory o
 constexpr int kNodalMaxNodes = kMaxCtaSmemBytes / 16;
 constexpr int kNodBits = 14, kNodMask = (1 << kNodBits) - 1;   // node id bits in the first id of an incidence
 static_assert(kNodalMaxNodes <= kNodMask + 1, "node ids of the nodal kernel");
+constexpr double kObtuseSum = 2.5, kObtuseMost = 64.0;   // forces.cuh, nodal path
 __host__ __device__ inline size_t nodal_smem_bytes(int n_nodes) { return (size_t)n_nodes * sizeof(float4); }
 constexpr int kStatusWords = 8;
 enum StatusWord {
@@ -103,6 +104,7 @@ struct DevBatch {
     long long n_elems_total;
     int any_bending;       // some membrane template has kb != 0
     int nodal_ok;          // every template fits the FP32 nodal force kernel
+    int any_obtuse;        // and some need its OBTUSE form
     const InstDev *inst;
     const TmplDev *tmpl;
     const int *node_inst;
@@ -375,7 +377,7 @@ struct LatCoord<float> {
 // Launch parameters that depend on the device only, asked for once per context (0: not yet).
 struct LaunchCache {
     int tile_ctas[2][3][2][2][2];   // transfer_tile_kernel<KER, W, SPREAD, INTERP, STORE>: resident CTAs per SM
-    int nodal[2], volume, vcorr, det_warp;   // forces_nodal_f32_kernel<CLUSTER>, volume_f32_kernel,
+    int nodal[2][2], volume, vcorr, det_warp;   // forces_nodal_f32_kernel<CLUSTER, OBTUSE>, volume_f32_kernel,
                                     // vc_fused_f32_kernel, spread_det_warp_kernel: shared memory allowed
 };
 

@@ -843,6 +843,16 @@ __global__ void area_normal_kernel(DevBatch b, const real *__restrict__ x, real 
 // h_km is the same number at both ends, y, J, beta and the n are evaluated in
 // the tet's own order by every corner.
 //
+// 4 A^2 comes from the dots, d_a d_b + d_b d_c + d_c d_a, whose error grows with the
+// square of 1/sin of an obtuse angle, where that of the cross product grows with
+// 1/sin. Batches with templates whose reference triangles have it above
+// kObtuseSum times the result (105 degrees) take OBTUSE, which takes the cross
+// product there (error of single triangles' forces at 150 degrees, 15% deformed: 6e-6
+// with the dots, 1.1e-6; in the reference triangle's plane, as the general path, 0.9
+// to 1.4e-6); it costs 8% (600 particles 92 us, 99), so others do without (at 100
+// degrees, 1.84, the errors are equal). Beyond kObtuseMost (160 degrees) I1
+// cancels too: the general path.
+//
 // Layout: incidences in slices of 32 nodes (a warp), slot by slot, so that a
 // warp's reads are consecutive: reference values and 16-bit node ids, the
 // node's corner number in the top bits. Membranes: r_a, r_b, r_c, w and (j, l);
@@ -884,11 +894,24 @@ __device__ __forceinline__ void ring_tri_f32(const float e1[3], const float e2[3
     t.dl = dot3f(e2, e3);
 }
 
+// |p x q|^2, every operation's rounding stated: the same bits for p, q of either sign
+__device__ __forceinline__ float cross2_f32(const float p[3], const float q[3])
+{
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int j = (i + 1) % 3, k = (i + 2) % 3;
+        const float n = fmaf(p[j], q[k], -__fmul_rn(p[k], q[j]));
+        s = fmaf(n, n, s);
+    }
+    return s;
+}
+
 // Pass 1 of a membrane node: elastic force and, with BEND, the part of the
 // bending force that needs no neighbour's curvature, 2 kb * 2 (kH - kH0)
 // (kH^2 - kG + kH0 kH) A n; kH receives the mean curvature. Along a fan the
 // second edge of a triangle is the first of the next: its vector is kept.
-template <bool BEND>
+template <bool BEND, bool OBTUSE>
 __device__ __forceinline__ void nodal_membrane(const TmplDev &T, int k, const float4 *xs, float F[3], float &kH)
 {
     const float mu = T.mu_f, half_muD = T.half_muD_f;
@@ -932,8 +955,23 @@ __device__ __forceinline__ void nodal_membrane(const TmplDev &T, int k, const fl
                     dc = c == 0 ? t.dl : (c == 1 ? t.dj : t.dk);
         const float rj = c == 0 ? r.y : (c == 1 ? r.z : r.x), rl = c == 0 ? r.z : (c == 1 ? r.x : r.y);
         const float w = r.w, w2 = __fmul_rn(w, w);
-        // 4 A^2 from the dots: the cross product's bits depend on the corner
-        const float I2 = __fmul_rn(fmaf(dc, da, fmaf(db, dc, __fmul_rn(da, db))), w2);
+        float S = fmaf(dc, da, fmaf(db, dc, __fmul_rn(da, db)));   // 4 A^2
+        if constexpr (OBTUSE) {
+            // the products cancel in a triangle with an obtuse corner: there from the
+            // edges of its first corner, whose cross product every corner computes
+            // alike, up to its sign
+            const float least = fminf(da, fminf(db, dc));
+            if (least < 0.f && 16.f * __fmul_rn(least, least) > S) {
+                float p[3], q2[3];
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    p[i] = c == 0 ? e1[i] : (c == 1 ? e2[i] : e3[i]);
+                    q2[i] = c == 0 ? e2[i] : (c == 1 ? e3[i] : e1[i]);
+                }
+                S = cross2_f32(p, q2);
+            }
+        }
+        const float I2 = __fmul_rn(S, w2);
         float a, b;
         if (T.law == 0) {
             a = mu;
@@ -1107,7 +1145,7 @@ __device__ __forceinline__ int nodal_solid(const TmplDev &T, int k, const float4
 // particles inst0, inst0 + 1, ...); kH goes to every CTA of the cluster between the passes.
 // The row of F is kept in global memory between the passes (read back by the
 // thread that wrote it).
-template <bool CLUSTER>
+template <bool CLUSTER, bool OBTUSE>
 static __global__ void __launch_bounds__(512, 2) forces_nodal_f32_kernel(DevBatch b, const float *__restrict__ x,
                                                                       float *__restrict__ F,
                                                                       unsigned long long *status, int inst0, int S)
@@ -1147,7 +1185,7 @@ static __global__ void __launch_bounds__(512, 2) forces_nodal_f32_kernel(DevBatc
     if (T.kb_f == 0.f) {
         for (int k = k0 + (int)threadIdx.x; k < k1; k += blockDim.x) {
             float f[3], kH;
-            nodal_membrane<false>(T, k, xs, f, kH);
+            nodal_membrane<false, OBTUSE>(T, k, xs, f, kH);
 #pragma unroll
             for (int a = 0; a < 3; ++a)
                 Fp[a * N + k] = f[a];
@@ -1156,7 +1194,7 @@ static __global__ void __launch_bounds__(512, 2) forces_nodal_f32_kernel(DevBatc
     }
     for (int k = k0 + (int)threadIdx.x; k < k1; k += blockDim.x) {
         float f[3], kH;
-        nodal_membrane<true>(T, k, xs, f, kH);
+        nodal_membrane<true, OBTUSE>(T, k, xs, f, kH);
 #pragma unroll
         for (int a = 0; a < 3; ++a)
             Fp[a * N + k] = f[a];

@@ -36,6 +36,7 @@ struct ifem_tmpl_s {
     int n_nodes, n_elems;
     double mu, C, kb, c0, lam;
     float vol_scale = 1.f;
+    double obtuse = 1.0;   // largest sum of |d_i d_j| over 4 A0^2 of a membrane's triangles
     int *d_elems = nullptr;
     double *d_ref_d = nullptr;
     float *d_ref_f = nullptr;
@@ -77,7 +78,7 @@ struct ifem_batch_s {
     long long N = 0;
     long long n_elems = 0;
     int max_nodes = 0, max_elems = 0;
-    int any_bending = 0, nodal_ok = 0;
+    int any_bending = 0, nodal_ok = 0, any_obtuse = 0;
     int max_box = 0;
     ifem_grid grid0 = nullptr;
     InstDev *d_inst = nullptr;
@@ -126,6 +127,7 @@ inline DevBatch dev_batch(ifem_batch b)
     d.n_elems_total = b->n_elems;
     d.any_bending = b->any_bending;
     d.nodal_ok = b->nodal_ok;
+    d.any_obtuse = b->any_obtuse;
     d.inst = b->d_inst;
     d.tmpl = b->d_tmpl;
     d.node_inst = b->d_node_inst;

@@ -54,8 +54,9 @@ static cudaError_t launch_nodal_forces(const DevBatch &b, const float *x, float 
     const int rounds = (chunk + 511) / 512;
     const int threads = ((chunk + rounds - 1) / rounds + 31) & ~31;
     const size_t sm = nodal_smem_bytes(b.max_nodes);
-    auto kern = S > 1 ? forces_nodal_f32_kernel<true> : forces_nodal_f32_kernel<false>;
-    if (cudaError_t e = allow_smem(kern, nodal_smem_bytes(kNodalMaxNodes), cache->nodal[S > 1]))
+    auto kern = b.any_obtuse ? (S > 1 ? forces_nodal_f32_kernel<true, true> : forces_nodal_f32_kernel<false, true>)
+                             : (S > 1 ? forces_nodal_f32_kernel<true, false> : forces_nodal_f32_kernel<false, false>);
+    if (cudaError_t e = allow_smem(kern, nodal_smem_bytes(kNodalMaxNodes), cache->nodal[S > 1][b.any_obtuse != 0]))
         return e;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
