@@ -851,24 +851,24 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
     DevWork &w = ws.w;
     w = DevWork{};
     long long N = b->N;
-    const long long no = nt * kOwnSub3;
-    int nb = (int)((no + kScanBlock - 1) / kScanBlock);
+    const long long no = f32 ? nt * kOwnSub3 : 0;   // own lists: FP32
+    const int nb = (int)((std::max(nt, no) + kScanBlock - 1) / kScanBlock);
     CK(alloc((void **)&ws.d_boxes, sizeof(BoxDev) * boxes.size()));
     CK(cudaMemcpy(ws.d_boxes, boxes.data(), sizeof(BoxDev) * boxes.size(), cudaMemcpyHostToDevice));
     // what a binning clears, in one piece: the spread's per-tile sums (by a
     // spread's binning only), then the counters and counts
     const size_t bin_ints = reproducible(ctx) ? 2 * kFsumBins * 3 * (size_t)nt : 0;
     const size_t zero_ints =
-        kCounters + bin_ints + (size_t)(no + 1) + (!f32 ? 4 * nt + 1 : (reproducible(ctx) ? nt : 4 * nt));
+        kCounters + bin_ints + (size_t)(f32 ? no + 1 + (reproducible(ctx) ? nt : 4 * nt) : 4 * nt + 1);
     CK(alloc((void **)&w.red_tile, sizeof(double) * 3 * (size_t)nt + sizeof(int) * zero_ints));
     CK(cudaMemset(w.red_tile, 0, sizeof(double) * 3 * (size_t)nt));
     w.counters = reinterpret_cast<int *>(w.red_tile + 3 * nt);
     w.zero_bytes = sizeof(int) * zero_ints;
     w.tile_fbin = reinterpret_cast<unsigned long long *>(w.counters + kCounters);
-    w.own_count = w.counters + kCounters + bin_ints;
-    CK(alloc((void **)&w.own_cursor, sizeof(int) * (no + 1)));
     const size_t Nn = (size_t)std::max<long long>(N, 1);
     if (f32) {
+        w.own_count = w.counters + kCounters + bin_ints;
+        CK(alloc((void **)&w.own_cursor, sizeof(int) * (no + 1)));
         w.own_flag = w.own_count + no + 1;
         w.tile_fsum = reinterpret_cast<float *>(w.own_flag + nt);
         CK(alloc((void **)&w.own_rec, 2 * sizeof(float4) * Nn));
@@ -898,21 +898,19 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
             CK(alloc((void **)&w.near_tile, sizeof(int2) * (size_t)(nt + 1)));
         }
     } else {
-        w.cand_count = w.own_count + no + 1;
+        w.cand_count = w.counters + kCounters;
         w.red_done = w.cand_count + nt + 1;
         CK(alloc((void **)&w.red_part, sizeof(double) * 24 * (size_t)nt));
         w.cand_cap = 8 * N;
         CK(alloc((void **)&w.cand_off, sizeof(int) * (nt + 1)));
         CK(alloc((void **)&w.cand_cursor, sizeof(int) * (nt + 1)));
         CK(alloc((void **)&w.cand_nodes, sizeof(int) * (size_t)w.cand_cap));
-        CK(alloc((void **)&w.own_off, sizeof(int) * (no + 1)));
-        CK(alloc((void **)&w.own_nodes, sizeof(int) * Nn));
         CK(alloc((void **)&w.active, sizeof(int) * kTileClasses * (size_t)nt));
     }
     w.wtab = nullptr;
     if (ctx->cfg.precision == IFEM_FP64 && ctx->cfg.kernel == IFEM_KERNEL_PESKIN4)
         CK(alloc((void **)&w.wtab, sizeof(DetW) * Nn));
-    CK(alloc((void **)&w.scan_blocks, sizeof(int) * 2 * (nb + 1)));
+    CK(alloc((void **)&w.scan_blocks, sizeof(int) * (nb + 1)));
     w.elem_buf = b->d_elem_buf;
     w.bend_buf = b->d_bend_buf;
     w.status = ctx->d_status;

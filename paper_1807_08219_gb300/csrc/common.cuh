@@ -153,17 +153,15 @@ struct DevWork {
     int *cand_cursor;   // n_tiles
     int *cand_nodes;    // pair list: node id per (tile, node) candidate pair
     long long cand_cap;
-    int *own_count;     // per (tile, 4^3 sub-block): n_tiles * kOwnSub3 + 1; in one piece with red_tile
-                        // and counters before it and, after it, own_flag and tile_fsum or cand_count
+    int *own_count;     // FP32, per (tile, 4^3 sub-block): n_tiles * kOwnSub3 + 1; then own_flag and
+                        // tile_fsum. One piece with red_tile and counters before it (FP64: cand_count
+                        // and red_done follow those)
     int *own_flag;      // n_tiles (FP32): 1 where the tile owns a node
     float *tile_fsum;   // 3 per tile (FP32): sum of |F_d| over the tile's own nodes, from the
                         // placement when it is given the forces (the transfer's fixed-point scale)
     unsigned long long *tile_fbin;   // the same for the reproducible spread: kFsumBins integers each
-    int *own_off;       // n_tiles * kOwnSub3 + 1 offsets (FP64)
-    int *own_cursor;    // fill cursors; local (per scan block) offsets in the FP32
-    int *own_nodes;     // N entries: nodes grouped by the tile (and sub-block) of their cell (not in
-                        // the FP32)
-    float4 *own_rec;    // FP32, 2 per node in that grouping: fractional cell coordinates
+    int *own_cursor;    // FP32: offsets of the own lists within their scan block
+    float4 *own_rec;    // FP32, 2 per node, by tile and sub-block: fractional cell coordinates
                         // x, y, z of the node and, in w, its cell within the tile packed as 8-bit
                         // x | y << 8 | z << 16; its force and, in w, its id
     int2 *node_key;     // N entries, by node (FP32): own-list key (-1: not binned) and
@@ -176,7 +174,7 @@ struct DevWork {
     float *box_buf;     // reproducible spread: a box per listed tile and, with box_lattices = 3, lattice;
     int box_lattices;   // with 1 the lattices take it in turn
     int *counters;      // kCounters: [2] work counter, [3] tiles with own nodes,
-                        // [4] total pairs, [5] total own nodes, [1] [6] [7] work counters of
+                        // [4] total pairs (FP64), [5] total own nodes (FP32), [1] [6] [7] work counters of
                         // one-lattice launches, [8] scan blocks finished, [9] near_tile entries,
                         // [10] to [13] active tiles per class
     int *scan_blocks;   // block partial sums for the tile scan

@@ -135,8 +135,7 @@ cudaError_t launch_after(void (*kern)(P...), dim3 grid, unsigned block, size_t s
 }
 
 // Binning. FP32: one-pass own lists (count, scan, placement; the stages can be
-// launched apart). FP64: candidate and own lists, the candidates sorted, and
-// the Peskin stencil table.
+// launched apart). FP64: candidate lists, sorted, and the Peskin stencil table.
 template <typename real>
 cudaError_t bin_impl(const TransferArgs &a, int stages)
 {
@@ -144,7 +143,6 @@ cudaError_t bin_impl(const TransferArgs &a, int stages)
     const DevWork &w = a.w;
     const long long nt = a.g.n_tiles;
     cudaStream_t s = a.stream;
-    const long long no = nt * kOwnSub3;
     constexpr bool f32 = std::is_same<real, float>::value;
     if (!f32 && stages != BIN_ALL)
         return cudaErrorInvalidValue;
@@ -171,11 +169,12 @@ cudaError_t bin_impl(const TransferArgs &a, int stages)
             bin_kernel<real, false><<<gn, 256, 0, s>>>(b, a.g, w, (const real *)a.x);
             IFEM_LAUNCH_CHECK();
         }
-        int nb = (int)((no + kScanBlock - 1) / kScanBlock);
-        // FP32: the local own offsets go to the cursors (own_scatter_kernel adds the block offsets)
-        if ((e = launch_after(scan_local_kernel, nb, kScanThreads, 0, s, f32 ? 0 : nt, no, w.cand_count, w.own_count,
-                              w.cand_off, f32 ? w.own_cursor : w.own_off, w.scan_blocks, w.counters + 8,
-                              w.counters + 4)) != cudaSuccess)
+        // FP32: the local offsets go to the cursors (own_scatter_kernel adds the block offsets)
+        const long long n = f32 ? nt * kOwnSub3 : nt;
+        const unsigned nb = (unsigned)((n + kScanBlock - 1) / kScanBlock);
+        if ((e = launch_after(scan_local_kernel, nb, kScanThreads, 0, s, n, f32 ? w.own_count : w.cand_count,
+                              f32 ? w.own_cursor : w.cand_off, w.scan_blocks, w.counters + 8,
+                              w.counters + (f32 ? 5 : 4))) != cudaSuccess)
             return e;
     }
     if (empty || !(stages & BIN_PLACE))
@@ -187,7 +186,7 @@ cudaError_t bin_impl(const TransferArgs &a, int stages)
         if (cudaError_t e = launch_after(own_scatter_kernel, gs, 256, 0, s, b, a.g, w, (const float *)a.F, a.store))
             return e;
     } else {
-        scan_finish_kernel<<<(unsigned)((no + 1 + 255) / 256), 256, 0, s>>>(nt, no, w, a.n_sm);
+        scan_finish_kernel<<<(unsigned)((nt + 1 + 255) / 256), 256, 0, s>>>(nt, w, a.n_sm);
         IFEM_LAUNCH_CHECK();
         bin_kernel<real, true><<<gn, 256, 0, s>>>(b, a.g, w, (const real *)a.x);
         IFEM_LAUNCH_CHECK();

@@ -4,14 +4,16 @@
 //
 // Binning. Every node is assigned the cell c = floor(x n/L) of its box. For
 // both kernels and all three MAC lattices its stencil lies inside cells
-// c-2 .. c+2 per axis. Boxes are cut into tiles (edge t, the last tile per
-// axis t..t+4 cells, never fewer than 5), so the stencil meets at most two
-// tiles per axis. The binning writes
-//   cand lists: for every tile, the nodes whose stencil meets it (spread);
-//   own lists:  for every tile, the nodes whose cell lies in it (interp).
-// Spreading is owner-computes: the CTA that owns a tile accumulates every
-// contribution that lands in it and writes each touched value once, so no
-// global atomics are needed and no value is written by two CTAs.
+// c-2 .. c+2 per axis. Boxes are cut into tiles, so large that a stencil meets at
+// most two of them per axis.
+// FP32: tiles of 4 to 16 cells a side and own lists: for every tile, the nodes whose
+// cell lies in it. A tile's own nodes are spread and interpolated in shared boxes of
+// the tile and its halo, which are added to the grid (transfer_tile_kernel; in a
+// fixed order where the spread is reproducible, tile_combine_kernel).
+// FP64: tiles of 5 cells or more (the last per axis up to t + 4) and candidate
+// lists: for every tile, the nodes whose stencil meets it, by node number. Spreading
+// is owner-computes: every value is accumulated by one thread at a time in the order
+// of the nodes and written once, without atomics. Interpolation gathers per node.
 #pragma once
 #include <type_traits>
 
@@ -242,7 +244,7 @@ static __global__ void __launch_bounds__(256) own_count_kernel(DevBatch b, DevGr
     }
 }
 
-// FILL = false: count candidate / own pairs per tile; FILL = true: write them
+// FILL = false: count candidate pairs per tile; FILL = true: write them
 // (FP64; FP32 bins with own_count_kernel and own_scatter_kernel). Block size
 // must be a multiple of 32 (every lane reaches the warp votes).
 template <typename real, bool FILL>
@@ -270,8 +272,6 @@ __global__ void bin_kernel(DevBatch b, DevGrid g, DevWork w, const real *__restr
         tl[a][1] = tile_of(hi, B.t, B.T);
         nt[a] = tl[a][0] == tl[a][1] ? 1 : 2;
     }
-    int r[3];
-    agg_append<FILL>(w.own_count, w.own_cursor, w.own_nodes, own_key(B, c, r), ok, node);
 #pragma unroll
     for (int slot = 0; slot < 8; ++slot) {
         const int ix = slot & 1, iy = (slot >> 1) & 1, iz = slot >> 2;
@@ -283,10 +283,10 @@ __global__ void bin_kernel(DevBatch b, DevGrid g, DevWork w, const real *__restr
     }
 }
 
-// Exclusive scan of the per-tile counts (two lists at once): block-local
-// scan, whose last block to finish scans the block sums -> add + cursors +
-// active lists (scan_finish_kernel; in FP32 own_scatter_kernel adds the block
-// offsets itself).
+// Exclusive scan of the counts (FP32: per own sub-block, FP64: candidates per
+// tile): block-local scan, whose last block to finish scans the block sums -> add +
+// cursors + active lists (scan_finish_kernel, FP64; in FP32 own_scatter_kernel adds
+// the block offsets itself).
 
 __device__ inline int block_exclusive_scan(int v, int *sh, int &total)
 {
@@ -322,42 +322,32 @@ __device__ inline int block_exclusive_scan(int v, int *sh, int &total)
     return r;
 }
 
-static __global__ void scan_local_kernel(long long n1, long long n2, const int *__restrict__ c1,
-                                         const int *__restrict__ c2, int *__restrict__ o1, int *__restrict__ o2,
-                                         int *__restrict__ bsum, int *__restrict__ ticket, int *__restrict__ totals)
+static __global__ void scan_local_kernel(long long n, const int *__restrict__ count, int *__restrict__ off,
+                                         int *__restrict__ bsum, int *__restrict__ ticket, int *__restrict__ total)
 {
     pdl_trigger();
     pdl_wait();
     __shared__ int sh[33];
     __shared__ int last;
-    long long base = (long long)blockIdx.x * kScanBlock + (long long)threadIdx.x * kScanPer;
-    int v1[kScanPer], v2[kScanPer], s1 = 0, s2 = 0;
+    const long long base = (long long)blockIdx.x * kScanBlock + (long long)threadIdx.x * kScanPer;
+    int v[kScanPer], s = 0;
 #pragma unroll
     for (int q = 0; q < kScanPer; ++q) {
-        long long i = base + q;
-        v1[q] = i < n1 ? c1[i] : 0;
-        v2[q] = i < n2 ? c2[i] : 0;
-        s1 += v1[q];
-        s2 += v2[q];
+        v[q] = base + q < n ? count[base + q] : 0;
+        s += v[q];
     }
-    int t1, t2;
-    int e1 = block_exclusive_scan(s1, sh, t1);
-    int e2 = block_exclusive_scan(s2, sh, t2);
+    int t;
+    int e = block_exclusive_scan(s, sh, t);
 #pragma unroll
     for (int q = 0; q < kScanPer; ++q) {
-        long long i = base + q;
-        if (i < n1)
-            o1[i] = e1;
-        if (i < n2)
-            o2[i] = e2;
-        e1 += v1[q];
-        e2 += v2[q];
+        if (base + q < n)
+            off[base + q] = e;
+        e += v[q];
     }
     // block sums out, then a ticket: the block that takes the last one sees
     // every block's sum (fence before the ticket, L2 loads after it)
     if (threadIdx.x == 0) {
-        bsum[2 * blockIdx.x] = t1;
-        bsum[2 * blockIdx.x + 1] = t2;
+        bsum[blockIdx.x] = t;
         __threadfence();
         last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
     }
@@ -366,29 +356,22 @@ static __global__ void scan_local_kernel(long long n1, long long n2, const int *
         return;
     __threadfence();
     const int nb = (int)gridDim.x;
-    int run1 = 0, run2 = 0;
+    int run = 0;
     for (int b0 = 0; b0 < nb; b0 += blockDim.x) {
         const int i = b0 + threadIdx.x;
-        const int u1 = i < nb ? __ldcg(&bsum[2 * i]) : 0, u2 = i < nb ? __ldcg(&bsum[2 * i + 1]) : 0;
-        int w1, w2;
-        const int x1 = block_exclusive_scan(u1, sh, w1);
-        const int x2 = block_exclusive_scan(u2, sh, w2);
-        if (i < nb) {
-            bsum[2 * i] = x1 + run1;
-            bsum[2 * i + 1] = x2 + run2;
-        }
-        run1 += w1;
-        run2 += w2;
+        const int u = i < nb ? __ldcg(&bsum[i]) : 0;
+        int w;
+        const int x = block_exclusive_scan(u, sh, w);
+        if (i < nb)
+            bsum[i] = x + run;
+        run += w;
     }
-    if (threadIdx.x == 0) {
-        totals[0] = run1;
-        totals[1] = run2;
-    }
+    if (threadIdx.x == 0)
+        *total = run;
 }
 
-// n1 tiles (candidate lists), n2 own sub-blocks. Adds the block offsets,
-// sets the fill cursors, writes the terminal offsets and the lists of tiles
-// with candidates, by class of their number, most first: a warp takes up to
+// n tiles (candidate lists). Adds the block offsets, sets the fill cursors,
+// writes the terminal offset and the lists of tiles with candidates, by class of their number, most first: a warp takes up to
 // 0.1 us a candidate, so the few long lists of a dense spot, begun last, were
 // the tail of the FP64 spread.
 // Class 0, lists that several warps walk (spread_det_warp_kernel), begins at 0.6
@@ -420,26 +403,17 @@ struct ActiveTiles {
         return list[i];
     }
 };
-static __global__ void scan_finish_kernel(long long n1, long long n2, DevWork w, int n_sm)
+static __global__ void scan_finish_kernel(long long n, DevWork w, int n_sm)
 {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long n = n1 > n2 ? n1 : n2;
     if (i > n)
         return;
-    const int blk = (int)(i / kScanBlock);
-    if (i == n1)
-        w.cand_off[n1] = w.counters[4];
-    if (i == n2)
-        w.own_off[n2] = w.counters[5];
-    if (i < n2) {
-        const int o2 = w.own_off[i] + w.scan_blocks[2 * blk + 1];
-        w.own_off[i] = o2;
-        w.own_cursor[i] = o2;
-    }
     int c1 = 0;
-    if (i < n1) {
+    if (i == n) {
+        w.cand_off[n] = w.counters[4];
+    } else {
         c1 = w.cand_count[i];
-        const int o1 = w.cand_off[i] + w.scan_blocks[2 * blk];
+        const int o1 = w.cand_off[i] + w.scan_blocks[i / kScanBlock];
         w.cand_off[i] = o1;
         w.cand_cursor[i] = o1;
     }
@@ -455,7 +429,7 @@ static __global__ void scan_finish_kernel(long long n1, long long n2, DevWork w,
             at = atomicAdd(&w.counters[10 + k], __popc(m));
         at = __shfl_sync(act, at, leader);
         if (m >> lane & 1u)
-            w.active[k * n1 + at + __popc(m & ((1u << lane) - 1u))] = (int)i;
+            w.active[k * n + at + __popc(m & ((1u << lane) - 1u))] = (int)i;
     }
 }
 
@@ -719,7 +693,7 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
     int off[kBinPer];
 #pragma unroll
     for (int j = 0; j < kBinPer; ++j)
-        off[j] = kr[j].x >= 0 ? w.own_cursor[kr[j].x] + w.scan_blocks[2 * (kr[j].x / kScanBlock) + 1] : 0;
+        off[j] = kr[j].x >= 0 ? w.own_cursor[kr[j].x] + w.scan_blocks[kr[j].x / kScanBlock] : 0;
 #pragma unroll
     for (int j = 0; j < kBinPer; ++j) {
         if (kr[j].x >= 0) {
@@ -783,8 +757,8 @@ static __global__ void __launch_bounds__(256) own_scatter_kernel(DevBatch b, Dev
             TileDesc td;
             td.tile = (int)t;
             td.n = B.n;
-            td.beg = w.own_cursor[i] + w.scan_blocks[2 * (i / kScanBlock) + 1];
-            td.end = t + 1 < g.n_tiles ? w.own_cursor[j] + w.scan_blocks[2 * (j / kScanBlock) + 1] : w.counters[5];
+            td.beg = w.own_cursor[i] + w.scan_blocks[i / kScanBlock];
+            td.end = t + 1 < g.n_tiles ? w.own_cursor[j] + w.scan_blocks[j / kScanBlock] : w.counters[5];
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 td.start[a] = ti.start[a];
