@@ -1011,14 +1011,19 @@ static int do_forces(ifem_ctx ctx, ifem_batch b, const void *x, void *F, const v
 // the placement also sums |F| per tile, which the tile transfer's spread
 // requires (every spread follows a binning given the same forces).
 // sums: a spread follows (the binning clears its per-tile sums, which an
-// interpolation's binning leaves for ifem_reduce).
+// interpolation's binning leaves for ifem_reduce). v, vp, xn, dt (FP32): the
+// placement writes the position update of nodes that are in no tile.
 static int do_bin(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, void *stream, int stages = BIN_ALL,
-                  const void *F = nullptr, int sums = 1, void *clear_f = nullptr)
+                  const void *F = nullptr, int sums = 1, void *clear_f = nullptr, void *v = nullptr,
+                  const void *vp = nullptr, void *xn = nullptr, double dt = 0.0)
 {
     int rc = ws_ensure(ctx, b, g, ctx->tile);
     if (rc != IFEM_OK)
         return rc;
-    TransferArgs a = transfer_args(ctx, b, x, F, nullptr, clear_f, nullptr, 0, stream);
+    TransferArgs a = transfer_args(ctx, b, x, F, nullptr, clear_f, v, 0, stream);
+    a.vp = vp;
+    a.xn = xn;
+    a.dt = dt;
     a.clear_sums = sums;
     a.clear_f = clear_f != nullptr;
     cudaError_t e = ctx->cfg.precision == IFEM_FP64 ? launch_bin_f64(a, stages) : launch_bin_f32(a, stages);
@@ -1363,7 +1368,7 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
         if ((rc = do_forces(ctx, b, x, F, nullptr, 0, stream)) != IFEM_OK)
             return rc;
         mark(ctx, 0, stream);
-        if ((rc = do_bin(ctx, b, g, x, stream, BIN_ALL, F)) != IFEM_OK)
+        if ((rc = do_bin(ctx, b, g, x, stream, BIN_ALL, F, 1, nullptr, v, vp, xn, dt)) != IFEM_OK)
             return rc;
         mark(ctx, 2, stream);
         if ((rc = do_overwrite(ctx, g, f, flags, stream)) != IFEM_OK)
@@ -1488,7 +1493,7 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
     if (fused) {
         if ((e = cudaStreamWaitEvent(s, ctx->fork[1], 0)) != cudaSuccess)
             return launch_rc(ctx, e, "step_coupling join");
-        if ((rc = do_bin(ctx, b, g, x, stream, BIN_PLACE, F)) != IFEM_OK)
+        if ((rc = do_bin(ctx, b, g, x, stream, BIN_PLACE, F, 1, nullptr, v, vp, xn, dt)) != IFEM_OK)
             return rc;
     }
     // the x/F sums, after the forces and the binning, on aux0 beside the transfers

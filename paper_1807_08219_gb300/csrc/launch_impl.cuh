@@ -183,7 +183,9 @@ cudaError_t bin_impl(const TransferArgs &a, int stages)
         // enough threads for every tile as well as every node
         const long long per_inst = ((nt + 255) / 256 + b.n_inst - 1) / b.n_inst;
         dim3 gs((unsigned)std::max<long long>(g1.x, per_inst), b.n_inst);
-        if (cudaError_t e = launch_after(own_scatter_kernel, gs, 256, 0, s, b, a.g, w, (const float *)a.F, a.store))
+        if (cudaError_t e = launch_after(own_scatter_kernel, gs, 256, 0, s, b, a.g, w, (const float *)a.F, a.store,
+                                         (const float *)a.x, (const float *)a.v, (const float *)a.vp, (float *)a.xn,
+                                         (float)a.dt))
             return e;
     } else {
         scan_finish_kernel<<<(unsigned)((nt + 1 + 255) / 256), 256, 0, s>>>(nt, w, a.n_sm);
