@@ -106,7 +106,11 @@ typedef enum { IFEM_KERNEL_PESKIN4 = 0, IFEM_KERNEL_MLS27 = 1 } ifem_kernel;
  * grid. DET: where more than two tiles reach a value, their terms are added in a
  * fixed order, so repeated runs give identical results (also MLS27 in either
  * mode). ATOMIC: they are added with atomic L2 adds, so the order in which
- * neighbouring tiles' halos combine is not reproducible. */
+ * neighbouring tiles' halos combine is not reproducible.
+ * The fixed point has 32 bits, scaled by the forces of each tile. With the
+ * environment variable IFEM_SPREAD_ACC = 64 when a context is created, its
+ * reproducible FP32 spreads use 64 bits (slower): forces 1e6 times smaller than
+ * others in their tile keep FP32 accuracy. */
 typedef enum { IFEM_SCATTER_DET = 0, IFEM_SCATTER_ATOMIC = 1 } ifem_scatter;
 
 typedef enum { IFEM_LAW_NEO_HOOKE = 0, IFEM_LAW_SKALAK = 1 } ifem_membrane_law;

@@ -96,6 +96,9 @@ extern "C" int ifem_ctx_create(const ifem_config *cfg, ifem_ctx *out)
     // pairs), 8 for the deterministic FP64 spread (its cost grows with the
     // candidates per tile times the values per tile)
     ctx->tile = cfg->tile ? cfg->tile : (cfg->precision == IFEM_FP64 ? 8 : 16);
+    // accumulator width of the reproducible FP32 spread
+    if (const char *acc = std::getenv("IFEM_SPREAD_ACC"))
+        ctx->acc64 = std::string(acc) == "64" ? 1 : 0;
     if (cudaSetDevice(cfg->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess ||
         cudaMalloc((void **)&ctx->d_status, sizeof(unsigned long long) * kStatusWords) != cudaSuccess ||
@@ -977,6 +980,7 @@ static TransferArgs transfer_args(ifem_ctx ctx, ifem_batch b, const void *x, con
     a.support = ctx->cfg.mls_support;
     a.n_sm = ctx->n_sm;
     a.store = reproducible(ctx);
+    a.acc64 = ctx->acc64;
     a.cleared = (flags & IFEM_SPREAD_OVERWRITE) != 0;
     a.total = b->ws.total;   // the call's grid, which need not be the batch's first
     a.lattice = -1;

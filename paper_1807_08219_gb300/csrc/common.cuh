@@ -375,6 +375,7 @@ struct LatCoord<float> {
 // Launch parameters that depend on the device only, asked for once per context (0: not yet).
 struct LaunchCache {
     int tile_ctas[2][3][2][2][2];   // transfer_tile_kernel<KER, W, SPREAD, INTERP, STORE>: resident CTAs per SM
+    int wide_ctas[2][3];            // spread_wide_kernel<KER, W>
     int nodal[2][2], volume, vcorr, det_warp;   // forces_nodal_f32_kernel<CLUSTER, OBTUSE>, volume_f32_kernel,
                                     // vc_fused_f32_kernel, spread_det_warp_kernel: shared memory allowed
 };
@@ -408,6 +409,7 @@ struct TransferArgs {
     double support;
     int n_sm;
     int store;        // FP32: reproducible spread through the boxes of every tile
+    int acc64;        // with 64-bit accumulators
     int cleared;      // f is zero before the spread (else the reproducible spread adds to it)
     int clear_f;      // the binning clears f too
     long long total;  // values of the grid

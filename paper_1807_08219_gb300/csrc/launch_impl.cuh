@@ -243,6 +243,16 @@ cudaError_t launch_tile_w(const TransferArgs &a)
     };
     if (!STORE)
         return transfer(a.lattice);
+    const size_t wide = a.acc64 ? (size_t)8 * TileShape<W>::kWords : 0;
+    auto kwide = spread_wide_kernel<KER, W>;
+    int &wide_ctas = a.cache->wide_ctas[KER][W / 4 - 3];
+    if (wide && wide_ctas == 0) {
+        if ((e = cudaFuncSetAttribute(kwide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide)) != cudaSuccess ||
+            (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wide_ctas, kwide, TileShape<W>::kBoxThreads, wide)) !=
+                cudaSuccess)
+            return e;
+        wide_ctas = std::max(wide_ctas, 1);
+    }
     // one lattice after the other where the buffer holds the boxes of one: each waits
     // for the combination of the one before
     const bool apart = a.w.box_lattices == 1;
@@ -252,10 +262,15 @@ cudaError_t launch_tile_w(const TransferArgs &a)
     const long long blocks = std::min(units, 8LL * a.n_sm);   // all resident
     auto combine = apart ? tile_combine_kernel<W, 1> : tile_combine_kernel<W, 3>;
     for (int d = apart ? 0 : -1; d < (apart ? 3 : 0); ++d)
-        if ((e = transfer(d)) != cudaSuccess ||
+        if ((e = !wide ? transfer(d)
+                       : launch_after(kwide, a.n_sm * wide_ctas, TileShape<W>::kBoxThreads, wide, a.stream, a.w, f,
+                                      a.density, (float)(1.0 / a.support), d, add)) != cudaSuccess ||
             (e = launch_after(combine, (unsigned)blocks, kCombineThreads, 0, a.stream, a.g, a.w, f, add,
                               d)) != cudaSuccess)
             return e;
+    if constexpr (STORE && INTERP)
+        if (wide)
+            return launch_tile_w<KER, W, false, true, false>(a);
     return cudaSuccess;
 }
 template <int KER, bool SPREAD, bool INTERP, bool STORE>

@@ -864,6 +864,31 @@ __device__ __forceinline__ void red_shared_add_nc(unsigned a, int v)
     asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(a), "r"(v));
 }
 
+// Accumulator width of the spread: red_add of a value in fixed point at a byte offset
+// of the box of 32-bit words, and the box's quads.
+template <typename Acc>
+struct TileAcc;
+template <>
+struct TileAcc<int> {
+    using Quad = int4;
+    static __device__ __forceinline__ void add(unsigned A, int off, float v)
+    {
+        red_shared_add_nc(A + (unsigned)off, __float2int_rn(v));
+    }
+    static __device__ __forceinline__ unsigned some(int q) { return min((unsigned)q, 1u); }
+};
+template <>
+struct TileAcc<long long> {
+    struct alignas(16) Quad {
+        long long x, y, z, w;
+    };
+    static __device__ __forceinline__ void add(unsigned A, int off, float v)
+    {
+        asm volatile("red.shared.add.u64 [%0], %1;" ::"r"(A + 2u * (unsigned)off), "l"(__float2ll_rn(v)));
+    }
+    static __device__ __forceinline__ unsigned some(long long q) { return q != 0; }
+};
+
 __device__ __forceinline__ void cp_async16(unsigned dst, const void *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(__cvta_generic_to_global(src))
@@ -992,9 +1017,10 @@ __device__ __forceinline__ void tile_stage(const TileItem &it, const float *__re
 // zero is the same in either order. add (f is not cleared): values that two boxes
 // can reach, near a face along one axis, go there too. buf: the item's place in the
 // buffer. bt: box thread.
-template <int W, bool STORE>
+template <int W, bool STORE, typename Acc = int>
 __device__ __forceinline__ long long tile_flush(const TileItem &it, float *__restrict__ f, float *__restrict__ buf,
-                                                int4 *A, float inv, int bt, bool add, unsigned &touched)
+                                                typename TileAcc<Acc>::Quad *A, float inv, int bt, bool add,
+                                                unsigned &touched)
 {
     using S = TileShape<W>;
     const int n = it.n;
@@ -1022,7 +1048,7 @@ __device__ __forceinline__ long long tile_flush(const TileItem &it, float *__res
 #pragma unroll
     for (int k = 0; k < S::NY / S::kYStep; ++k) {
         const int yb = y0 + k * S::kYStep, at = 8 * yb * S::NZ * S::NX, ly = 2 * yb + yl;
-        const int4 q = A[at];
+        const typename TileAcc<Acc>::Quad q = A[at];
         const bool zero = (q.x | q.y | q.z | q.w) == 0;
         float v0 = (float)q.x * inv, v1 = (float)q.y * inv, v2 = (float)q.z * inv, v3 = (float)q.w * inv;
         if constexpr (STORE) {
@@ -1040,7 +1066,7 @@ __device__ __forceinline__ long long tile_flush(const TileItem &it, float *__res
         }
         if (zero)
             continue;
-        A[at] = make_int4(0, 0, 0, 0);
+        A[at] = {0, 0, 0, 0};
         float *row = plane + wrap1(it.sy - 2 + ly, n) * n;
         qsum += ((long long)q.x + q.y) + ((long long)q.z + q.w);
         const bool in_y = (unsigned)(ly - 2) < (unsigned)it.ey;
@@ -1048,10 +1074,10 @@ __device__ __forceinline__ long long tile_flush(const TileItem &it, float *__res
             if (!STORE || v0 != 0.f || v1 != 0.f || v2 != 0.f || v3 != 0.f)
                 red_add_v4(row, v0, v1, v2, v3);
             if (in_xz && in_y)
-                touched += min((unsigned)q.x, 1u) + min((unsigned)q.y, 1u) + min((unsigned)q.z, 1u) +
-                           min((unsigned)q.w, 1u);
+                touched += TileAcc<Acc>::some(q.x) + TileAcc<Acc>::some(q.y) + TileAcc<Acc>::some(q.z) +
+                           TileAcc<Acc>::some(q.w);
         } else {
-            const int qc[4] = {q.x, q.y, q.z, q.w};
+            const Acc qc[4] = {q.x, q.y, q.z, q.w};
             const float vc[4] = {v0, v1, v2, v3};
 #pragma unroll
             for (int c = 0; c < 4; ++c)
@@ -1180,7 +1206,7 @@ __device__ __forceinline__ bool mls_weights_f32(const float y[3][3], float inv_s
 // system, mls_weights_f32) cost more than the banks. 48 mixed cells in a 101^3
 // grid, transfers of a step: 202 us with a spread over candidate lists that
 // evaluated a node's weights in each of its tiles, plus the interpolation; 85 us.
-template <int KER, int W, bool SPREAD, bool INTERP>
+template <int KER, int W, bool SPREAD, bool INTERP, typename Acc = int>
 __device__ __forceinline__ void tile_node(const TileItem &cur, const DevWork &w, const TileUnit &un, float gsc,
                                           const unsigned char *U, unsigned sA, float *__restrict__ v,
                                           const float *__restrict__ x, const float *__restrict__ vp,
@@ -1239,7 +1265,7 @@ __device__ __forceinline__ void tile_node(const TileItem &cur, const DevWork &w,
                     if constexpr (INTERP)
                         out = fmaf(wt[J], *reinterpret_cast<const float *>(U + o), out);
                     if constexpr (SPREAD)
-                        red_shared_add_nc(sA + (unsigned)o, __float2int_rn(__fmul_rn(wt[J], gq)));
+                        TileAcc<Acc>::add(sA, o, __fmul_rn(wt[J], gq));
                 }
         if constexpr (INTERP)
             put(out);
@@ -1304,11 +1330,10 @@ __device__ __forceinline__ void tile_node(const TileItem &cur, const DevWork &w,
             }
             if constexpr (SPREAD) {
                 const float gz = gx * ph[2][t1];
-                const unsigned aa = sA + (unsigned)oa, ab = sA + (unsigned)ob;
-                red_shared_add_nc(aa, __float2int_rn(py0 * gz));
-                red_shared_add_nc(aa + kRow2, __float2int_rn(py2 * gz));
-                red_shared_add_nc(ab, __float2int_rn(py1 * gz));
-                red_shared_add_nc(ab + kRow2, __float2int_rn(py3 * gz));
+                TileAcc<Acc>::add(sA, oa, py0 * gz);
+                TileAcc<Acc>::add(sA, oa + kRow2, py2 * gz);
+                TileAcc<Acc>::add(sA, ob, py1 * gz);
+                TileAcc<Acc>::add(sA, ob + kRow2, py3 * gz);
             }
         }
         if constexpr (INTERP)
@@ -1491,6 +1516,58 @@ __global__ void __launch_bounds__(TileShape<W>::kThreads, TileShape<W>::kCtas)
         if (lane == 0)
             status_add(w.status, ST_TOUCHED, touched);
     }
+}
+
+// The reproducible spread with 64-bit accumulators, on request (ifem_ctx_create): small
+// forces beside large ones keep their digits. One box, a CTA per item, whose threads
+// first take its nodes and then flush it: twice the memory leaves no room for the box
+// that would be worked on meanwhile. Interpolation is a launch of its own. 27 bits of
+// scale more than tile_scale's, so that the sum of a whole box fits 64 bits. Steps of 72
+// mixed cells, 128^3: 226 us (95 with 32 bits); 48 with MLS, 101^3: 205 (110).
+template <int KER, int W>
+__global__ void __launch_bounds__(TileShape<W>::kBoxThreads)
+    spread_wide_kernel(DevWork w, float *__restrict__ f, int density, float inv_support, int lattice, int add)
+{
+    using S = TileShape<W>;
+    using Quad = TileAcc<long long>::Quad;
+    constexpr int T = S::kBoxThreads;
+    extern __shared__ __align__(128) unsigned char tile_smem[];
+    Quad *A = reinterpret_cast<Quad *>(tile_smem);
+    __shared__ long long s_red[T / 32];
+    for (int i = threadIdx.x; i < S::kWords / 4; i += T)
+        A[i] = {0, 0, 0, 0};
+    pdl_wait();   // for the binning's placement
+    const int per_tile = lattice < 0 ? 3 : 1, n_items = per_tile * w.counters[3];
+    unsigned touched = 0;
+    for (int i = blockIdx.x; i < n_items; i += gridDim.x) {
+        const TileDesc td = w.tile_desc[i / per_tile];
+        const TileItem it = tile_item(td, lattice < 0 ? i % 3 : lattice, density);
+        const float2 sc = tile_scale<KER>(it, fsum_get(w.tile_fbin + kFsumBins * (3LL * it.tile + it.d)));
+        const float unit = fmaxf(sc.y * 0x1p-27f, 0x1p-120f);
+        __syncthreads();   // the box is clear
+        for (int q = it.beg + (int)threadIdx.x; q < it.end; q += T)
+            tile_node<KER, W, true, false, long long>(it, w, tile_unit(w, q), it.sd * (1.f / unit), nullptr, smem_u32(A),
+                                                      nullptr, nullptr, nullptr, nullptr, 0.f, inv_support, 0);
+        asm volatile("" ::: "memory");   // the reductions stay before the barrier
+        __syncthreads();
+        float *buf = w.box_buf + ((long long)w.box_lattices * it.slot + (w.box_lattices == 3 ? it.d : 0)) * S::kWords;
+        long long qsum = tile_flush<W, true, long long>(it, f, buf, A, unit, threadIdx.x, add != 0, touched);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            qsum += __shfl_down_sync(0xffffffffu, qsum, o);
+        if ((threadIdx.x & 31) == 0)
+            s_red[threadIdx.x >> 5] = qsum;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            long long vsum = 0;
+            for (int k = 0; k < T / 32; ++k)
+                vsum += s_red[k];
+            w.red_tile[3LL * it.tile + it.d] = (double)vsum * (double)unit * td.h3;
+        }
+    }
+    touched = __reduce_add_sync(0xffffffffu, touched);
+    if ((threadIdx.x & 31) == 0)
+        status_add(w.status, ST_TOUCHED, touched);
 }
 
 // The reproducible spread's second half: the values of the cleared field f that
