@@ -836,6 +836,7 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
         B.scale = B.inv_h * B.inv_h * B.inv_h;
         B.h3 = 1.0 / B.scale;
         B.inv_h_f = (float)B.inv_h;
+        B.inv_h_lo = (float)(B.inv_h - (double)B.inv_h_f);
         B.scale_f = (float)B.scale;
         nt += (long long)B.T * B.T * B.T;
         for (int j = 0; j < B.T; ++j)

@@ -91,7 +91,8 @@ struct BoxDev {
     double inv_h;          // n / L
     double scale;          // (n/L)^3
     double h3;             // 1 / scale
-    float inv_h_f;         // FP32 copies for the FP32 kernels (no FP64 pipe use)
+    float inv_h_f;         // FP32 copies for the FP32 kernels (no FP64 pipe use), and
+    float inv_h_lo;        // what inv_h_f rounds off
     float scale_f;
 };
 
@@ -370,6 +371,14 @@ struct LatCoord<float> {
         return (I.f0[a] - o) + x * B.inv_h_f;
     }
 };
+
+// x + y as a sum and its error
+__device__ __forceinline__ float two_sum(float x, float y, float &err)
+{
+    const float s = x + y, b = s - x;
+    err = (x - (s - b)) + (y - b);
+    return s;
+}
 
 // ------------------------------------------------------------- launchers
 // Launch parameters that depend on the device only, asked for once per context (0: not yet).

@@ -103,13 +103,6 @@ __device__ __forceinline__ DF df_cross_comp(float a1, float b2, float a2, float 
     const float h = s + e;
     return DF{h, e - (h - s)};
 }
-// x + y as a sum and its error
-__device__ __forceinline__ float two_sum(float x, float y, float &err)
-{
-    const float s = x + y, b = s - x;
-    err = (x - (s - b)) + (y - b);
-    return s;
-}
 // a . (b x c) + rest: the products' high parts are summed exactly, what is below
 // them (eight terms and rest) with its error, so that half an ulp of the low part
 // is nearly all that is lost

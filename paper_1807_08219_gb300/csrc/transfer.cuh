@@ -171,6 +171,19 @@ static __global__ void __launch_bounds__(256) clear_kernel(int *__restrict__ p, 
         f[i] = 0;
 }
 
+// A node's lattice coordinate f0 + x n/L from the cell that begins at fl, with what
+// the coordinate itself, tens of cells, rounds off: that was most of the error of the
+// interpolation. A little outside [0, 1) where the rounded coordinate is in the next
+// cell: stencils from there are the same to second order, and within the boxes up to
+// the limits set here (coordinates of 1e5 cells and more).
+__device__ __forceinline__ float node_frac(float f0, float x, const BoxDev &B, float fl)
+{
+    const float p = __fmul_rn(x, B.inv_h_f), pe = fmaf(x, B.inv_h_lo, fmaf(x, B.inv_h_f, -p));
+    float e;
+    const float s = two_sum(f0, p, e);
+    return fminf(fmaxf((s - fl) + (e + pe), -0.015625f), 1.015625f);
+}
+
 // One-pass own-list binning (FP32): per node its rank within its
 // own-list key (the old value of the key's count, one atomic per group of
 // lanes with the same key) and its record -- fractional lattice coordinates
@@ -219,8 +232,11 @@ static __global__ void __launch_bounds__(256) own_count_kernel(DevBatch b, DevGr
         key[j] = own_key(B, c, r);
         if (ok[j]) {
             const unsigned pk = (unsigned)r[0] | ((unsigned)r[1] << 8) | ((unsigned)r[2] << 16);
-            w.node_rec[node[j]] = make_float4(sl[0] - floorf(sl[0]), sl[1] - floorf(sl[1]), sl[2] - floorf(sl[2]),
-                                              __uint_as_float(pk));
+            float fr[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                fr[a] = node_frac(I.f0[a], xa[j][a], B, floorf(sl[a]));
+            w.node_rec[node[j]] = make_float4(fr[0], fr[1], fr[2], __uint_as_float(pk));
         }
     }
     // every lane takes part in the votes and shuffles (invalid lanes form
@@ -565,7 +581,7 @@ __device__ __forceinline__ void df_add_prod(DF &x, float a, float b)
 // Used by the FP32 kernels; the FP64 kernels evaluate phi point by point.
 __device__ __forceinline__ void peskin_frac(float r, float ph[4])
 {
-    const float t = 1.f + 4.f * r - 4.f * r * r;   // in [1, 2] for r in [0, 1)
+    const float t = 1.f + 4.f * r - 4.f * r * r;   // in [1, 2] for r in [0, 1), at least 0.93 for node_frac's
     const float q = t * rsqrtf(t);
     ph[0] = (3.f - 2.f * r - q) * 0.125f;
     ph[1] = (3.f - 2.f * r + q) * 0.125f;
