@@ -1349,6 +1349,10 @@ static cudaError_t copy_nodes_in(ifem_ctx ctx, ifem_batch b, const void *xh, voi
 
 constexpr size_t kSmallField = size_t(8) << 20;   // bytes of f (step_impl)
 constexpr size_t kRowsFrom = size_t(5) << 19;     // bytes of v (step_impl)
+// Nodes of an FP64 MLS step from which the spread waits for the interpolation, us beside
+// it and after it: 20 k nodes 2745 and 2613, 10 k 2494 and 2087, 3.9 k 707 and 729, 2.2 k
+// (one solid, whose longest list is the spread) 1205 and 1386.
+constexpr long long kApartFrom = 8192;
 
 // One coupling step; with xn given (the caller checked vp, dt and aliasing)
 // also the position update from the interpolated velocities; with io given
@@ -1524,6 +1528,11 @@ static int step_impl(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, con
             return launch_rc(ctx, e, "step_coupling fork");
     }
     if (!fused && (e = cudaStreamWaitEvent(s, ctx->fork[1], 0)) != cudaSuccess)
+        return launch_rc(ctx, e, "step_coupling join");
+    // FP64 MLS: above kApartFrom nodes the spread waits for the interpolation, whose
+    // blocks keep half of its blocks off the SMs while they last
+    if (!fused && ctx->cfg.kernel == IFEM_KERNEL_MLS27 && b->N >= kApartFrom &&
+        (e = cudaStreamWaitEvent(s, ctx->fork[3], 0)) != cudaSuccess)
         return launch_rc(ctx, e, "step_coupling join");
     // with host arrays and the fused transfer, one launch per lattice: row d
     // of v goes back to the host on aux1 as soon as lattice d's launch ends,

@@ -104,3 +104,28 @@ def test_small_and_large_fields(precision, n, graph):
         assert torch.equal(f, ref)
     finally:
         cp.close()
+
+
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("count", [3, 4])   # 7686 and 10248 nodes
+def test_fp64_mls_order(count, graph):
+    """Spread beside the interpolation and after it: the bits of the separate calls."""
+    import torch
+    from paper_1807_08219_gb300 import ifem as I
+    w = _workload(count, 48)
+    cp = I.Coupler(w, precision=I.IFEM_FP64, kernel=I.IFEM_KERNEL_MLS27, tile=6)
+    try:
+        g = torch.Generator(device=cp.device).manual_seed(1)
+        u = torch.randn(cp.G, generator=g, device=cp.device, dtype=cp.dtype)
+        x, f = cp.nodes_to_device(w.x_local_all()), cp.zeros_grid()
+        F, v, F2, v2, f2 = cp.empty_nodes(), cp.empty_nodes(), cp.empty_nodes(), cp.empty_nodes(), cp.zeros_grid()
+        torch.cuda.synchronize()
+        _replayed(lambda s: I.ifem_step_coupling(cp.ctx, cp.batch, cp.grid, x, u, F, f, v, None, I.IFEM_SPREAD_OVERWRITE, s),
+                  (lambda: [t.fill_(np.nan) for t in (F, v, f)]) if graph else None)
+        I.ifem_compute_forces(cp.ctx, cp.batch, x, F2)
+        I.ifem_spread(cp.ctx, cp.batch, cp.grid, x, F2, f2, 0)
+        I.ifem_interpolate(cp.ctx, cp.batch, cp.grid, u, x, v2)
+        I.ifem_sync_status(cp.ctx)
+        assert torch.equal(F, F2) and torch.equal(v, v2) and torch.equal(f, f2)
+    finally:
+        cp.close()
