@@ -605,15 +605,17 @@ extern "C" int64_t ifem_grid_box_offset(ifem_grid g, int b)
 }
 
 // ------------------------------------------------------------ batch
-static void split_origins(ifem_batch b, ifem_grid g)
+// Origins in cells of the boxes that b->split_n and split_L give.
+static void split_origins(ifem_batch b)
 {
     for (size_t i = 0; i < b->h_inst.size(); ++i) {
         InstDev &I = b->h_inst[i];
-        double inv_h = (double)g->n[I.box] / g->L[I.box];
+        const int n = b->split_n[I.box];
+        double inv_h = (double)n / b->split_L[I.box];
         for (int a = 0; a < 3; ++a) {
             double s0 = I.origin[a] * inv_h;
             double fl = std::floor(s0);
-            I.I0[a] = (int)((long long)fl % g->n[I.box]);
+            I.I0[a] = (int)((long long)fl % n);
             I.f0[a] = (float)(s0 - fl);
         }
     }
@@ -676,7 +678,9 @@ extern "C" int ifem_batch_create(ifem_ctx ctx, int n_tmpl, const ifem_tmpl *tmpl
         b->nodal_ok = b->nodal_ok && tmpls[t]->obtuse <= kObtuseMost;
         b->any_obtuse = b->any_obtuse || tmpls[t]->obtuse > kObtuseSum;
     }
-    split_origins(b, grid);
+    b->split_n = grid->n;
+    b->split_L = grid->L;
+    split_origins(b);
     std::vector<TmplDev> td(n_tmpl);
     for (int t = 0; t < n_tmpl; ++t) {
         ifem_tmpl s = tmpls[t];
@@ -772,7 +776,7 @@ extern "C" int ifem_batch_set_origins(ifem_batch b, const double *origins)
                 return fail(ctx, IFEM_ERR_ARG, "set_origins: non-finite origin");
             b->h_inst[i].origin[a] = origins[3 * i + a];
         }
-    split_origins(b, b->grid0);
+    split_origins(b);
     CK(cudaSetDevice(ctx->cfg.device));
     if (!b->h_inst.empty())
         CK(cudaMemcpy(b->d_inst, b->h_inst.data(), sizeof(InstDev) * b->h_inst.size(), cudaMemcpyHostToDevice));
@@ -817,6 +821,16 @@ static int ws_ensure(ifem_ctx ctx, ifem_batch b, ifem_grid g, int tile)
         return IFEM_OK;
     ws_free(ws);
     const bool f32 = ctx->cfg.precision == IFEM_FP32;
+    // FP32 keeps the origins in cells: of this grid's boxes from here on
+    bool other = false;
+    for (const InstDev &I : b->h_inst)
+        other = other || b->split_n[I.box] != g->n[I.box] || b->split_L[I.box] != g->L[I.box];
+    if (f32 && other) {
+        b->split_n = g->n;
+        b->split_L = g->L;
+        split_origins(b);
+        CK(cudaMemcpy(b->d_inst, b->h_inst.data(), sizeof(InstDev) * b->h_inst.size(), cudaMemcpyHostToDevice));
+    }
     std::vector<BoxDev> boxes(g->n_boxes);
     long long nt = 0;
     int max_edge = 0;

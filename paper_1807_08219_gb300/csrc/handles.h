@@ -81,6 +81,8 @@ struct ifem_batch_s {
     int max_nodes = 0, max_elems = 0;
     int any_bending = 0, nodal_ok = 0, any_obtuse = 0;
     int max_box = 0;
+    std::vector<int> split_n;      // cells and sides of the boxes in whose cells the FP32
+    std::vector<double> split_L;   // origins are kept (InstDev::I0, f0)
     ifem_grid grid0 = nullptr;
     InstDev *d_inst = nullptr;
     TmplDev *d_tmpl = nullptr;

@@ -1,6 +1,5 @@
 """Calls on a grid other than the one the batch was created on. Every call takes
-its own grid of the context: a coarser or a finer one (IFEM_FP64), or one with
-further boxes (IFEM_FP32, whose origins are kept in cells of the first grid).
+its own grid of the context: a coarser or a finer one, or one with further boxes.
 The field lies between margins that hold a marker: what a call clears, adds and
 writes ends with the grid of the call. Fields equal those of a batch created on
 that grid: the same bits where the order of a value's terms is fixed, else
@@ -51,6 +50,7 @@ def _calls(cp, grid, step, flags):
 @pytest.mark.parametrize("overwrite", [False, True])
 @pytest.mark.parametrize("precision,kernel,scatter,first,call", [
     (1, 0, 0, [64], [40]), (1, 0, 0, [40], [64]), (1, 1, 0, [48], [33]), (1, 1, 0, [33], [48]),
+    (0, 0, 0, [64], [40]), (0, 0, 1, [40], [64]), (0, 1, 0, [48], [33]),
     (0, 0, 0, [64], [64, 24]), (0, 0, 1, [64], [64, 24]), (0, 1, 0, [64], [64, 24]),
     (0, 0, 0, [64, 24], [64]), (0, 0, 1, [64, 24], [64]), (0, 1, 0, [64, 24], [64]),
     (0, 0, 0, [64, 160], [64]), (0, 0, 0, [64], [64, 160])])   # above 8 MB a step clears another way
@@ -81,7 +81,7 @@ def test_grid_at_the_address_of_a_destroyed_one(precision):
     w = _workload(precision)
     cp = I.Coupler(dataclasses.replace(w, boxes=[W.Box(64, 1.0)]), precision=precision)
     try:
-        calls = [[64, 48], [64, 24]] if precision == 0 else [[48], [33]]
+        calls = [[48], [33]]
         first = I.ifem_grid_create(cp.ctx, calls[0], [1.0] * len(calls[0]))
         _calls(cp, first, False, 0)
         at = first.value
