@@ -1135,10 +1135,10 @@ __device__ __forceinline__ int nodal_solid(const TmplDev &T, int k, const float4
 // What bounds it: latency and instruction issue, at the 28 warps per SM that 64
 // registers allow (fewer registers spill: 110 against 85 us on the 600-particle
 // suspension with 40), shared memory at a third of its rate. 600 particles (1.33 M
-// nodes): 90 us against 129 us for the kernel before it (per-element forces
+// nodes): 92 us against 129 us for the kernel before it (per-element forces
 // added with float atomics in shared memory, 60 % of that pipe), one red cell
 // 11 against 47 us, the element-buffer path of the deterministic mode (four
-// launches) 51 -> 20 us on 72 particles, 64 balls of 4096 nodes 93 -> 43 us.
+// launches) 51 -> 20 us on 72 particles, 64 balls of 4096 nodes 93 -> 48 us.
 // One cluster of S CTAs per particle (S = 1: one CTA), each holding every
 // position of the particle in shared memory (float4, kH in w) and taking a
 // chunk of its nodes (inst0 < 0: all particles, the largest first; else

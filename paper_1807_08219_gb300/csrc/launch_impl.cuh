@@ -36,13 +36,13 @@ constexpr size_t kVcorrSmemBytes = kMaxCtaSmemBytes - 4 * 8 * kVolThreadsF - 102
 // FP32 nodal forces of particles [inst0, inst0 + n): a cluster of S CTAs per
 // particle. With few particles one CTA each leaves most SMs idle; with many,
 // each doubling only stages the positions once more. Times in us, S = 1, 2, 4, 8:
-//   one red cell (2562 nodes)     29  19  14  11
-//   16 balls of 4096 nodes        62  31  18  21
-//   64 balls of 4096 nodes        64  36  31  35
-//   72 red cells and platelets    30  21  19  30
-//   200 capsules of 2562 nodes    46  44  54  83
-//   300 red cells                 47  52  84 121
-//   600 red cells and platelets   85  87 132 212
+//   one red cell (2562 nodes)     31  20  15  11
+//   16 balls of 4096 nodes       107  57  31  26
+//   64 balls of 4096 nodes       108  57  48  52
+//   72 red cells and platelets    32  21  21  34
+//   200 capsules of 2562 nodes    50  45  56  83
+//   300 red cells                 51  55  82 121
+//   600 red cells and platelets   92  97 138 226
 // Nodes per thread: as few rounds as 512 threads allow, evenly filled (smaller
 // blocks measured slower throughout: 600 particles 102 us with 192 threads).
 template <typename real>   // float (a template so that kernels_f64.cu compiles no FP32 kernel)
