@@ -408,6 +408,7 @@ def time_extras(wl, I, torch, dev, flush, T, reps=20, warm=3):
     G = cp.zeros_grid()
     vol = torch.empty(len(wl.instances), dtype=torch.float64, device=dev)
     I.ifem_volumes(cp.ctx, cp.batch, x0, vol, s)
+    torch.cuda.synchronize()   # the copy runs on another stream
     V0 = vol.clone()
     lam = torch.empty_like(vol)
     u = cp.grid_to_device(wl.u)
