@@ -54,3 +54,24 @@ def test_faces_and_far_cells(kernel):
         x[1::3] = np.nextafter(x[1::3].astype(np.float32), np.float32(np.inf))
         v = _velocities(x, n, kernel, 0, u, np.zeros(3))
         assert np.abs(v - 1.0).max() < 1e-5
+
+
+@pytest.mark.parametrize("case", ["C1", "C2"])
+def test_smooth_fields(case):
+    """Velocities from a smooth field: relative L2 5.5e-8 against FP64 (the rounding of v
+    itself is 2.5e-8, of its sums about 4e-8; weights that do not sum to 1 to the last
+    bit would add 4e-8)."""
+    from paper_1807_08219_gb300 import ifem as I
+    w = W.make(case)
+    xl = w.x_local_all(np.float32).astype(np.float64)
+    got = []
+    for precision in (0, 1):
+        cp = I.Coupler(w, precision=precision)
+        try:
+            u = cp.grid_to_device([q.astype(np.float32).astype(np.float64) for q in w.u])
+            v = cp.empty_nodes()
+            I.ifem_interpolate(cp.ctx, cp.batch, cp.grid, u, cp.nodes_to_device(xl), v)
+            got.append(cp.nodes_to_host(v))
+        finally:
+            cp.close()
+    assert np.linalg.norm(got[0] - got[1]) < 5.5e-8 * np.linalg.norm(got[1])
