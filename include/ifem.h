@@ -160,9 +160,9 @@ typedef struct {
     int64_t domain_errors;      /* non-finite positions / singular MLS matrices */
     int64_t capacity_errors;    /* per-tile list longer than the kernel's limit */
     int64_t timeouts;           /* bounded waits that expired */
-    int64_t pairs;              /* (tile, node) pairs of the last binning (0 when the
-                                   spread needs no per-tile candidate lists) */
-    int64_t active_tiles;       /* tiles with at least one node pair */
+    int64_t pairs;              /* (tile, node) pairs of the last binning (IFEM_FP64; 0 in
+                                   IFEM_FP32, whose spreads need no per-tile candidate lists) */
+    int64_t active_tiles;       /* tiles with at least one such pair (IFEM_FP64; 0 in IFEM_FP32) */
     int64_t touched_cells;      /* non-zero lattice values added by spreads since the last sync
                                    (FP32: counted inside each node's own tile only; the FP64 path
                                    rewrites every value of an active tile) */
@@ -400,10 +400,10 @@ int ifem_step_coupling(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *x, c
  * with v the velocities this step interpolates. Arguments as
  * ifem_step_coupling, plus v_prev (device node array, the previous step's
  * velocities; pass v_prev = a copy of v for a forward-Euler first step) and
- * x_new (device node array receiving the new local positions). Where the
- * step fuses the interpolation into the spreading kernel (IFEM_FP32,
- * IFEM_SCATTER_ATOMIC, IFEM_KERNEL_PESKIN4) the same kernel also writes x_new
- * from each velocity it gathers, so v is never read back; elsewhere the update
+ * x_new (device node array receiving the new local positions). With IFEM_FP32
+ * the kernel that spreads and interpolates also writes x_new from each velocity
+ * it gathers, so v is never read back (nodes whose positions are not finite, which
+ * it does not visit, get theirs from the binning); with IFEM_FP64 the update
  * runs after the interpolation on its stream. x_new equals ifem_ab2_update on
  * a copy of x with the v this call writes (bit for bit). x_new may not overlap
  * x, v, v_prev or F, nor v_prev overlap v (IFEM_ERR_ARG); IFEM_ERR_ARG for a
@@ -423,10 +423,11 @@ int ifem_step_coupling_ab2(ifem_ctx ctx, ifem_batch b, ifem_grid g, const void *
  * arrays must stay valid, and v_host and red_host are filled, only once
  * `stream` has passed this point. Host arrays should be pinned
  * (cudaHostAlloc); pageable memory works outside graph capture but copies
- * without overlap. With IFEM_FP32, IFEM_SCATTER_ATOMIC and a batch of two or
+ * without overlap. With IFEM_FP32 and a batch of two or
  * more particles the positions arrive in two halves (by particle) and each
- * half's element forces start as soon as it has landed; with the Peskin
- * kernel the fused spreading and interpolation then run as one launch per
+ * half's element forces start as soon as it has landed; with IFEM_SCATTER_ATOMIC,
+ * the Peskin kernel and 2.5 MB of v or more the fused spreading and interpolation
+ * then run as one launch per
  * lattice, and row d of v goes back to the host as soon as lattice d is done
  * (rows 0 and 1 beside the later lattices, row 2 beside the sums of v and the
  * boxes); lattices 1 and 2 are launched with programmatic serialization, so
