@@ -11,7 +11,7 @@ import ifem_workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("support", [0.8, 0.95, 1.0, 1.02, 1.05, 1.1, 1.2, 1.3, 1.4, 0.0])
+@pytest.mark.parametrize("support", [0.8, 0.95, 1.0, 1.02, 1.05, 1.1, 1.2, 1.3, 1.4, 1.72, 1.725, 0.0])
 def test_transfers_stay_transposes(support):
     import torch
     from paper_1807_08219_gb300 import ifem as I
